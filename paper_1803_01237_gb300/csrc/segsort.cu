@@ -2,15 +2,14 @@
 // bucket ranges, the local merge).
 //
 // Design for sm_103a:
-//  * A segment of at most 14336 keys is sorted by one CTA on chip: its keys are
-//    read from HBM once into shared memory; a counting pass on a 10-bit digit
-//    that interpolates the segment's [min, max] key range splits them into
-//    1024 groups in key order; every key's final slot is its group's start plus
-//    the number of keys of its group below it in (key, input position) order;
-//    the keys are written once (16 B of HBM traffic per key).  Three CTA shapes
-//    by segment size (128, 256, 512 threads).  A segment whose largest group is
-//    above kTinyGroup keys (heavy duplicates, skew) goes to a stable LSD kernel
-//    (8-bit digit passes over a 16-bit index permutation).
+//  * A segment of at most 14336 keys is sorted by one CTA on chip (k_chip): its
+//    keys (and payload) are copied from HBM once into shared memory, counted
+//    into groups that follow their distribution, ordered inside the groups as
+//    32-bit words in registers, and written once (16 B of HBM traffic per key).
+//    Three CTA shapes by segment size (128, 256, 1024 threads).  The few
+//    segments it cannot order that way (large groups of distinct keys closer
+//    than its words resolve) go to k_small_msd and from there to a stable LSD
+//    kernel (8-bit digit passes over a 16-bit index permutation).
 //  * A larger segment takes one read pass for statistics (digit counts and the
 //    OR/AND of its keys) and one stable scatter on its first-split
 //    digit (its top varying byte, or an interpolation of the key range the
@@ -109,7 +108,7 @@ size_t segsort_ws_bytes(uint64_t N, uint64_t nseg) {
     b += align_up(d.ml * 8 * 4, 256) + align_up(d.ml * 4, 256);       // large_mask, any_large
     b += align_up(d.tiles * kRadix * 4, 256);                         // tile_off
     b += align_up(64 * 4, 256);                                       // counters
-    b += 8 * align_up(d.list * 4, 256);                               // class lists, fallback, slow lists
+    b += 7 * align_up(d.list * 4, 256);                               // class lists, fallback, slow lists
     b += align_up(8 * (d.list / 1024 + 2) * 4, 256);                  // blk
     return b;
 }
@@ -152,7 +151,6 @@ SegSortWs segsort_ws_carve(void* base, uint64_t N, uint64_t nseg, uint32_t* err)
     w.counters = (uint32_t*)take(64 * 4);
     for (int i = 0; i < 3; ++i) w.list[i] = (uint32_t*)take(d.list * 4);
     w.fb_list = (uint32_t*)take(d.list * 4);
-    w.slow_list = (uint32_t*)take(d.list * 4);
     for (int i = 0; i < 3; ++i) w.slow_keys[i] = (uint32_t*)take(d.list * 4);
     w.blk = (uint32_t*)take(8 * (d.list / 1024 + 2) * 4);
     w.err = err;
@@ -295,9 +293,8 @@ __device__ __forceinline__ void block_rank(DigitOf digit_of, uint32_t count, uin
 }
 
 // ---------------------------------------------------------------------------
-// On-chip sort of segments with min_n < n <= max_n keys (n <= CAP), taken
-// from `list` (compact ids, count at *nlist) or, when list is null, from all
-// nseg segments.  The keys are read once into shared memory.  One counting
+// On-chip sort of the segments k_chip leaves, with min_n < n <= max_n keys
+// (n <= CAP), taken from `list` (compact ids, count at *nlist).  The keys are read once into shared memory.  One counting
 // pass on a 10-bit digit (the segment's key range interpolated onto 1024
 // groups) splits them into groups that come in key order; inside a group the
 // atomics leave an arbitrary order, and each key's final slot is its group's
@@ -667,197 +664,6 @@ __global__ __launch_bounds__(THREADS) void k_small_msd(
     }
 }
 
-// ---------------------------------------------------------------------------
-// The same on-chip sort for segments of up to CAP = THREADS * ITEMS keys
-// (ITEMS <= 16) with the keys, digits and group slots held in registers:
-// one counting pass on the 10-bit digit, a scatter that stores each key and
-// its input position at its group slot, and a rank only for keys whose group
-// holds more than one key (a singleton's slot is its final position).  About
-// half the shared-memory traffic of k_small_msd.  A segment with a group
-// larger than kTinyGroup is appended to slow_list for k_small_msd.  It runs
-// the middle size class (up to 4096 keys, 256 threads); for the smallest
-// class the shared-memory kernel measured faster (more CTAs per SM).
-// ---------------------------------------------------------------------------
-template <int CAP>
-constexpr size_t reg_sort_smem() {
-    return (size_t)CAP * 8 + (size_t)CAP * 2 + 2 * (kChipRadix + 1) * 4 + 32 * 4 + 2 * 32 * 8 + 64;
-}
-
-template <bool PAY, int THREADS, int CAP>
-__global__ __launch_bounds__(THREADS) void k_small_reg(
-    const uint64_t* kin, uint64_t* kout, const uint32_t* pin, uint32_t* pout, const uint64_t* __restrict__ seg_lo,
-    const uint64_t* __restrict__ seg_hi, const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist,
-    uint64_t nseg, uint32_t min_n, uint32_t max_n, uint64_t flip_in, uint64_t flip_out,
-    uint32_t* __restrict__ slow_list, uint32_t* __restrict__ slow_count) {
-    constexpr int ITEMS = CAP / THREADS;
-    static_assert(CAP % THREADS == 0 && ITEMS <= 16 && CAP <= 4096 && kChipRadix <= 4096, "register sort shape");
-    constexpr int WARPS = THREADS / 32;
-    extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t* s_key = (uint64_t*)smem;                     // CAP: keys by group slot, then in final order
-    uint16_t* s_idx = (uint16_t*)(s_key + CAP);            // CAP: their input positions
-    uint32_t* s_start = (uint32_t*)(s_idx + CAP);          // kChipRadix+1: counts, then group starts
-    uint32_t* s_run = s_start + (kChipRadix + 1);          // kChipRadix+1: running slots
-    uint32_t* s_warp = s_run + (kChipRadix + 1);           // 32
-    uint64_t* s_red = (uint64_t*)(((uintptr_t)(s_warp + 32) + 7) & ~(uintptr_t)7);  // 2*32
-
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const uint64_t count = list ? (uint64_t)*nlist : nseg;
-    for (uint64_t k = blockIdx.x; k < count; k += gridDim.x) {
-        const uint64_t s = list ? (uint64_t)list[k] : k;
-        const uint64_t base = seg_lo[s];
-        const uint64_t n64 = seg_hi[s] - base;
-        if (n64 <= min_n || n64 > max_n) continue;  // uniform per CTA
-        const uint32_t n = (uint32_t)n64;
-        uint64_t key[ITEMS];
-        uint64_t kmin = ~0ull, kmax = 0;
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            const uint32_t e = tid + i * THREADS;
-            key[i] = e < n ? kin[base + e] ^ flip_in : 0ull;
-            if (e < n) { kmin = min(kmin, key[i]); kmax = max(kmax, key[i]); }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            kmin = min(kmin, (uint64_t)__shfl_xor_sync(0xffffffffu, kmin, o));
-            kmax = max(kmax, (uint64_t)__shfl_xor_sync(0xffffffffu, kmax, o));
-        }
-        if (lane == 0) { s_red[w] = kmin; s_red[32 + w] = kmax; }
-        for (int d = tid; d < kChipRadix; d += THREADS) s_start[d] = 0;
-        __syncthreads();
-        {
-            uint64_t a = ~0ull, b = 0;
-            for (int i = 0; i < WARPS; ++i) { a = min(a, s_red[i]); b = max(b, s_red[32 + i]); }
-            kmin = a;
-            kmax = b;
-        }
-        if (kmin == kmax) {  // all keys equal: already in order
-#pragma unroll
-            for (int i = 0; i < ITEMS; ++i) {
-                const uint32_t e = tid + i * THREADS;
-                if (e < n) {
-                    kout[base + e] = key[i] ^ flip_out;
-                    if (PAY) pout[base + e] = pin[base + e];
-                }
-            }
-            __syncthreads();
-            continue;
-        }
-        const uint64_t range = kmax - kmin;
-        const uint64_t mult = interp_mult(range, (uint32_t)kChipRadix);
-        uint32_t dp[ITEMS];  // digit in bits 0..11, group slot from bit 12
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            const uint32_t e = tid + i * THREADS;
-            dp[i] = 0;
-            if (e < n) {
-                const uint64_t off = key[i] - kmin;
-                const uint32_t d = mult ? min((uint32_t)__umul64hi(off, mult), (uint32_t)kChipRadix - 1) : (uint32_t)off;
-                dp[i] = d;
-                atomicAdd(&s_start[d], 1u);
-            }
-        }
-        __syncthreads();
-        uint32_t mx = 0;
-        for (int d = tid; d < kChipRadix; d += THREADS) mx = max(mx, s_start[d]);
-        mx = __reduce_max_sync(0xffffffffu, mx);
-        scan_smem_inplace<THREADS, kChipRadix>(s_start, s_warp);
-        if (lane == 0) s_warp[w] = mx;
-        for (int d = tid; d < kChipRadix; d += THREADS) s_run[d] = s_start[d];
-        if (tid == 0) s_start[kChipRadix] = n;
-        __syncthreads();
-        mx = 0;
-        for (int i = 0; i < WARPS; ++i) mx = max(mx, s_warp[i]);
-        if (mx > (uint32_t)kTinyGroup) {  // skewed: the shared-memory kernel takes this segment
-            if (tid == 0) slow_list[atomicAdd(slow_count, 1u)] = (uint32_t)s;
-            __syncthreads();
-            continue;
-        }
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            const uint32_t e = tid + i * THREADS;
-            if (e < n) {
-                const uint32_t slot = atomicAdd(&s_run[dp[i]], 1u);
-                s_key[slot] = key[i];
-                s_idx[slot] = (uint16_t)e;
-                dp[i] |= slot << 12;
-            }
-        }
-        __syncthreads();
-        // Final position: the group start plus the keys of the group below
-        // this one in (key, input position) order; a singleton keeps its slot.
-        uint32_t fin[ITEMS];
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            const uint32_t e = tid + i * THREADS;
-            fin[i] = dp[i] >> 12;
-            if (e < n) {
-                const uint32_t d = dp[i] & 4095u;
-                const uint32_t a = s_start[d], b = s_start[d + 1];
-                if (b - a > 1u) {
-                    uint32_t r = 0;
-                    for (uint32_t g = a; g < b; ++g) {
-                        const uint64_t ky = s_key[g];
-                        r += (ky < key[i] || (ky == key[i] && s_idx[g] < e)) ? 1u : 0u;
-                    }
-                    fin[i] = a + r;
-                }
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            const uint32_t e = tid + i * THREADS;
-            if (e < n && fin[i] != (dp[i] >> 12)) {
-                s_key[fin[i]] = key[i];
-                if (PAY) s_idx[fin[i]] = (uint16_t)e;
-            }
-        }
-        __syncthreads();
-        if (PAY) {  // the output may be the input: gather every payload first
-            uint32_t pv[ITEMS];
-#pragma unroll
-            for (int i = 0; i < ITEMS; ++i) {
-                const uint32_t j = tid + i * THREADS;
-                pv[i] = j < n ? pin[base + s_idx[j]] : 0u;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < ITEMS; ++i) {
-                const uint32_t j = tid + i * THREADS;
-                if (j < n) pout[base + j] = pv[i];
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            const uint32_t j = tid + i * THREADS;
-            if (j < n) kout[base + j] = s_key[j] ^ flip_out;
-        }
-        __syncthreads();
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Keys alone, on chip, segments of up to CAP = THREADS * ITEMS keys held in
-// registers.  Equal keys are indistinguishable, so no input order has to be
-// kept.  A counting pass on a digit interpolating the segment's key range (R
-// groups, monotone in the key) hands every key a slot in its group through
-// one shared counter, and the keys are scattered into group order; since the
-// groups come in key order, what is left is the order inside each group:
-// a key of a small group counts the group's keys below it (the keys stay in
-// registers, so the only shared-memory traffic is the group's few keys), and
-// a large group holding distinct keys is sorted by the CTA (a segment with
-// more than kKeysMixedMax of them goes to slow_list for the shared-memory
-// kernel).  The digit has about as many values as the segment has keys, so
-// most groups hold one key.
-// With PREFETCH the segments move between HBM and shared memory by bulk
-// asynchronous copies (the TMA engine): one thread copies the next segment of
-// the list into a staging buffer while the current one is sorted, and copies
-// each sorted segment out of shared memory, so the threads issue no load or
-// store per key.  A bulk copy needs 16-byte aligned addresses, so a segment's
-// first key (when its address is 8 mod 16) and its last key (when one is left
-// over) travel by 8-byte copies, and the keys sit in shared memory one slot
-// further on in that case (key j at buffer[j + head]).
-// ---------------------------------------------------------------------------
 __device__ __forceinline__ void cp_async8(void* sdst, const void* gsrc) {
     const uint32_t sa = (uint32_t)__cvta_generic_to_shared(sdst);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gsrc) : "memory");
@@ -895,28 +701,6 @@ __device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t
                  "l"(gsrc), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
 }
-__device__ __forceinline__ void bulk_store(void* gdst, const void* ssrc, uint32_t bytes) {
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(gdst), "r"(smem_u32(ssrc)),
-                 "r"(bytes)
-                 : "memory");
-    asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
-}
-// The issuing thread's bulk stores have read their shared-memory source.
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
-// Shared-memory writes of this thread become visible to bulk copies.
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
-
-template <int CAP, int R, bool PREFETCH>
-constexpr size_t keys_sort_smem() {
-    return (size_t)(CAP + 2) * 8 * (PREFETCH ? 2 : 1) + (size_t)(R + 1) * 4 + 32 * 4 + 2 * 32 * 8 + 64 + (size_t)R +
-           16;
-}
-
-// Mixed large groups sorted in place by the CTA per segment (more go to the
-// shared-memory kernel).
-constexpr int kKeysMixedMax = 8;
-
 // In-place ascending sort of base[SI(a + i)], i in [0, m), by the whole CTA
 // (SI: the caller's index map): a bitonic network over
 // the next power of two P >= m in the form whose comparators all put the
@@ -950,60 +734,191 @@ __device__ __forceinline__ void cta_bitonic_sort(uint64_t* base, uint32_t a, uin
     }
 }
 
-// CTAs per SM the register budget must allow: the small classes live on
-// many buckets in flight per SM (their keys are prefetched while the
-// previous bucket is sorted).
-template <int THREADS>
-constexpr int keys_min_blocks() { return THREADS <= 128 ? 8 : (THREADS <= 256 ? 3 : 1); }
+// CTAs per SM the register budget must allow: what their shared memory lets
+// an SM hold.
+template <bool PAY, int THREADS>
+constexpr int chip_min_blocks() { return THREADS <= 128 ? (PAY ? 6 : 8) : (THREADS <= 256 ? 3 : 1); }
 
-// A digit monotone in off that spreads keys over many binary orders of
-// magnitude: the position e of off's leading one, counted from e_lo (32
-// positions e_lo .. e_lo + 31), followed by the M = log2(R) - 5 bits below
-// the leading one; offsets below 2^e_lo (zero included) take digit 0.
-template <int R>
-__device__ __forceinline__ uint32_t log_digit(uint64_t off, int e_lo) {
-    constexpr int M = (R >= 4096) ? 7 : (R >= 2048 ? 6 : (R >= 1024 ? 5 : 4));
-    static_assert(32 * (1 << M) <= R, "log digit width");
-    if (off == 0ull) return 0u;
-    const int e = 63 - __clzll((long long)off);
-    if (e < e_lo) return 0u;
-    const uint32_t mant = e >= M ? (uint32_t)(off >> (e - M)) & ((1u << M) - 1u)
-                                 : (uint32_t)(off << (M - e)) & ((1u << M) - 1u);
-    return ((uint32_t)(e - e_lo) << M) | mant;
+// ---------------------------------------------------------------------------
+// On chip, segments of min_n < n <= max_n keys (n <= CAP), with or without a
+// payload: the stable sort by (key, position).
+//
+// One bulk copy brings the keys (and the payload) into shared memory, where
+// they stay until they are written in order; what is sorted is one 32-bit
+// word per key.
+//  * x, the 32 key bits below the segment's common prefix (key - min,
+//    normalised), is multiplied by R / range: the high word of the product is
+//    the key's group, the low word its place inside the group.  One shared
+//    counter per group (16 bits, two to a word) hands out slots.
+//  * A segment whose keys crowd (a group above kChipRefine keys) counts again
+//    with one group per key: group g's range is cut into as many parts as it
+//    holds keys, so the groups follow the keys' distribution (a piecewise
+//    linear estimate of it), up to three times.
+//  * The words (group start mod 64 | place in the group | position) are
+//    scattered into group order, and ordered inside the groups by windows of
+//    eight in registers, two instructions per comparator: each window is
+//    sorted, then windows shifted by four merge the upper half of one with the
+//    lower half of the next, back and forth (an odd-even transposition of
+//    sorted blocks of four).  A group of g words spans at most
+//    ceil((g-1)/4) + 1 blocks and is in order after that many rounds.
+//  * Neighbours that agree in group and place (equal keys, or rarely distinct
+//    ones closer than the place resolves) are in position order, which is the
+//    stable order of equal keys; where their keys are found out of order the
+//    run is sorted by (key, position).
+// A segment that still holds a group above kChipMaxGroup words goes to
+// slow_list, unless the group holds a single key value: then nothing is left
+// to order (keys alone), or its positions refine it once more (payload).
+//
+// Bound by shared-memory wavefronts and issue slots together (67% and 66% of
+// their peaks; about 34 wavefronts and 146 instructions per key of a warp): the
+// counting atomics, the group-start and key gathers and the word scatter each
+// meet random banks.  Words of 32 bits instead of the keys themselves halve
+// the scatter's wavefronts and make a comparator two instructions (six for 64
+// bits: a variant that ordered the keys in registers spilled and took 3.9 ms).
+// 2^28 uniform keys in buckets of about 1024: 2.28 ms with an insertion sort
+// per thread over 64-bit keys (60 wavefronts, 204 instructions), 1.5 ms here;
+// 2^28 Morton keys with a payload in segments of 2^14, whose groups crowd:
+// 57.9 ms (most of it in the LSD kernel), 6.6 ms.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void cp_async4(void* sdst, const void* gsrc) {
+    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(sdst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gsrc) : "memory");
 }
 
-template <int THREADS, int CAP, int R, bool PREFETCH>
-__global__ __launch_bounds__(THREADS, keys_min_blocks<THREADS>()) void k_small_keys(
-    const uint64_t* kin, uint64_t* kout, const uint64_t* __restrict__ seg_lo, const uint64_t* __restrict__ seg_hi,
-    const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist, uint64_t nseg, uint32_t min_n,
-    uint32_t max_n, uint64_t flip_in, uint64_t flip_out, uint32_t* __restrict__ slow_list,
-    uint32_t* __restrict__ slow_count, uint32_t* __restrict__ err) {
+// Exclusive scan in place of 2 NW 16-bit counters packed in NW shared words
+// (counter 2i in the low half of word i) by a CTA of T threads, and the
+// largest counter.  The counters add up to less than 2^16.  Ends with a
+// barrier.
+template <int T, int NW>
+__device__ __forceinline__ uint32_t scan_pairs_inplace(uint32_t* v, uint32_t* s_warp /* 64 */) {
+    constexpr int K = NW / T;
+    constexpr int W = T / 32;
+    static_assert(NW % T == 0 && K % 4 == 0 && W <= 32, "packed scan size");
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    uint32_t loc[K];
+    uint32_t sum = 0, m2 = 0;
+#pragma unroll
+    for (int k = 0; k < K; k += 4) {
+        const uint4 q = ((const uint4*)v)[(tid * K + k) / 4];
+        loc[k] = q.x; loc[k + 1] = q.y; loc[k + 2] = q.z; loc[k + 3] = q.w;
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        sum += (loc[k] & 0xffffu) + (loc[k] >> 16);
+        m2 = __vmaxu2(m2, loc[k]);
+    }
+    uint32_t mx = __reduce_max_sync(0xffffffffu, max(m2 & 0xffffu, m2 >> 16));
+    uint32_t x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) { s_warp[w] = x; s_warp[32 + w] = mx; }
+    __syncthreads();
+    uint32_t run = x - sum;
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+        if (i < w) run += s_warp[i];
+        mx = max(mx, s_warp[32 + i]);
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const uint32_t lo = loc[k] & 0xffffu, hi = loc[k] >> 16;
+        loc[k] = run | ((run + lo) << 16);
+        run += lo + hi;
+    }
+#pragma unroll
+    for (int k = 0; k < K; k += 4)
+        ((uint4*)v)[(tid * K + k) / 4] = make_uint4(loc[k], loc[k + 1], loc[k + 2], loc[k + 3]);
+    __syncthreads();
+    return mx;
+}
+
+__device__ __forceinline__ void cmp_swap(uint32_t& x, uint32_t& y) {
+    const uint32_t lo = min(x, y), hi = max(x, y);
+    x = lo;
+    y = hi;
+}
+// Batcher's odd-even merge of the sorted halves k[0..3] and k[4..7], and his
+// sort of eight built on it (9 and 19 comparators).
+__device__ __forceinline__ void merge_4_4(uint32_t (&k)[8]) {
+    cmp_swap(k[0], k[4]); cmp_swap(k[1], k[5]); cmp_swap(k[2], k[6]); cmp_swap(k[3], k[7]);
+    cmp_swap(k[2], k[4]); cmp_swap(k[3], k[5]);
+    cmp_swap(k[1], k[2]); cmp_swap(k[3], k[4]); cmp_swap(k[5], k[6]);
+}
+__device__ __forceinline__ void sort_8(uint32_t (&k)[8]) {
+    cmp_swap(k[0], k[1]); cmp_swap(k[2], k[3]); cmp_swap(k[4], k[5]); cmp_swap(k[6], k[7]);
+    cmp_swap(k[0], k[2]); cmp_swap(k[1], k[3]); cmp_swap(k[4], k[6]); cmp_swap(k[5], k[7]);
+    cmp_swap(k[1], k[2]); cmp_swap(k[5], k[6]);
+    merge_4_4(k);
+}
+
+constexpr uint32_t kChipRefine = 24;    // a larger group: count again on the refined groups
+constexpr uint32_t kChipMaxGroup = 56;  // the largest group the window rounds order (start mod 64 is unambiguous)
+constexpr int kChipRefines = 3;
+constexpr uint32_t kChipRounds = (kChipMaxGroup + 2) / 4 + 3;  // rounds that order the largest group, and the one that finds it so
+constexpr int kStartBits = 6;
+
+// Position bits of a word (a segment of at most CAP keys).
+template <int CAP>
+constexpr int chip_pos_bits() { return CAP <= 2048 ? 11 : (CAP <= 4096 ? 12 : 14); }
+// Counters: R groups of the first pass, one group per key of a refined one.
+template <int THREADS, int CAP, int R>
+constexpr int chip_counters() {
+    constexpr int unit = 8 * THREADS;  // whole 16-byte vectors per thread
+    return ((CAP > R ? CAP : R) + unit - 1) / unit * unit;
+}
+template <int THREADS, int CAP>
+constexpr int chip_windows() { return (CAP / 8 + THREADS - 1) / THREADS; }
+// The payload is staged on chip beside the keys, but for the largest class
+// (its keys and words leave no room: gathered from its place in the input).
+template <bool PAY, int CAP>
+constexpr bool chip_stage_pay() { return PAY && CAP <= 4096; }
+
+template <bool PAY, int THREADS, int CAP, int R>
+constexpr size_t chip_smem() {
+    return (size_t)(CAP + 2) * 8 + (size_t)(CAP + 16) * 4 + (chip_stage_pay<PAY, CAP>() ? (size_t)(CAP + 8) * 4 : 0) +
+           (size_t)(chip_counters<THREADS, CAP, R>() / 2 + 4 + 32) * 4 + 64 * 4 +
+           2 * (size_t)chip_windows<THREADS, CAP>() * (THREADS / 32) * 4 * 4 + 4 * 4 + 8 + 16;
+}
+
+template <bool PAY, int THREADS, int CAP, int R>
+__global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_chip(
+    const uint64_t* kin, uint64_t* kout, const uint32_t* pin, uint32_t* pout, const uint64_t* __restrict__ seg_lo,
+    const uint64_t* __restrict__ seg_hi, const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist,
+    uint64_t nseg, uint32_t min_n, uint32_t max_n, uint64_t flip_in, uint64_t flip_out,
+    uint32_t* __restrict__ slow_list, uint32_t* __restrict__ slow_count, uint32_t* __restrict__ err) {
     constexpr int ITEMS = CAP / THREADS;
     constexpr int WARPS = THREADS / 32;
-    static_assert(CAP % THREADS == 0 && R % THREADS == 0 && R <= 4096 && CAP <= 16384 && WARPS <= 16 &&
-                      THREADS >= 64,
-                  "keys sort shape");
-    // dp[i]: digit in bits 0..11, slot in its group from bit 12
-    constexpr uint32_t kDigitMask = 4095u, kSlotShift = 12, kSlotMask = 16383u;
+    constexpr int WIN = chip_windows<THREADS, CAP>();
+    constexpr int IDX = chip_pos_bits<CAP>();
+    constexpr int FR = 32 - IDX - kStartBits;  // bits of the place inside the group
+    constexpr int SH = FR + IDX;
+    constexpr int NC = chip_counters<THREADS, CAP, R>();
+    constexpr bool SPAY = chip_stage_pay<PAY, CAP>();
+    constexpr uint32_t kPosMask = (1u << IDX) - 1u;
+    constexpr uint32_t kSlotShift = 15, kGroupMask = (1u << kSlotShift) - 1u;
+    static_assert(CAP % THREADS == 0 && CAP <= (1 << IDX) && NC + 66 < (1 << kSlotShift) && R % (8 * THREADS) == 0 &&
+                      CAP < 16384 + 1,
+                  "on-chip sort shape");
     extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t* s_key = (uint64_t*)smem;                                              // CAP + 2
-    uint64_t* s_stage = s_key + (CAP + 2);                                          // CAP + 2 (PREFETCH)
-    uint32_t* s_start = (uint32_t*)(s_stage + (PREFETCH ? CAP + 2 : 0));            // R + 1
-    uint32_t* s_warp = s_start + (R + 1);                                           // 32
-    uint64_t* s_red = (uint64_t*)(((uintptr_t)(s_warp + 32) + 7) & ~(uintptr_t)7);  // 2 * 32
-    uint32_t* s_flag = (uint32_t*)(s_red + 64);  // [0] mixed large groups, [1..kKeysMixedMax] their digits
-    uint8_t* s_mark = (uint8_t*)(s_flag + 16);   // R: the group is large and holds distinct keys
-    uint64_t* s_bar = (uint64_t*)(((uintptr_t)(s_mark + R) + 7) & ~(uintptr_t)7);  // staging buffer full
+    uint64_t* s_key = (uint64_t*)smem;                                  // CAP + 2: the keys as read, key j at [j + sh]
+    uint32_t* s_w = (uint32_t*)(s_key + (CAP + 2));                     // CAP + 16
+    uint32_t* s_pay = s_w + (CAP + 16);                                 // CAP + 8 (SPAY)
+    uint32_t* s_cnt = s_pay + (SPAY ? CAP + 8 : 0);                     // NC/2 words, the end, 32 words for empty items
+    const uint16_t* s_start = (const uint16_t*)s_cnt;                   // after the scan: group starts, [groups] = n
+    uint32_t* s_warp = s_cnt + (NC / 2 + 4 + 32);                       // 64
+    uint32_t* s_edge = s_warp + 64;                                     // 2 x WIN * WARPS * 4
+    uint32_t* s_first = s_edge + 2 * WIN * WARPS * 4;                   // 4
+    uint64_t* s_bar = (uint64_t*)(((uintptr_t)(s_first + 4) + 7) & ~(uintptr_t)7);  // the keys have landed
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const uint64_t count = list ? (uint64_t)*nlist : nseg;
-    for (int d = tid; d < R; d += THREADS) s_mark[d] = 0;
-    if (PREFETCH && tid == 0) mbar_init(s_bar, 1u);
+    const uint32_t hflip = (uint32_t)(flip_in >> 32);  // the sign bit, or nothing
+    const uint64_t flip = flip_in ^ flip_out;          // from the input's key bits to the output's
+    if (tid == 0) mbar_init(s_bar, 1u);
     __syncthreads();
-    // Segment descriptors travel one iteration ahead in registers: the loads
-    // of the next segment's list entry and bounds are issued at the top of an
-    // iteration and first used after its first barrier, so their latency
-    // hides behind the current segment's work.
     struct Desc {
         uint64_t base;
         uint32_t n;
@@ -1020,321 +935,384 @@ __global__ __launch_bounds__(THREADS, keys_min_blocks<THREADS>()) void k_small_k
         }
         return d;
     };
-    // 1 when the segment's first key sits at an address that is 8 mod 16.
-    auto head_of = [](const uint64_t* p) -> uint32_t { return (uint32_t)(((uintptr_t)p >> 3) & 1u); };
-    uint32_t phase = 0;  // parity of the staging buffer's next completion
-    auto prefetch = [&](const Desc& d) {  // copy a segment into the staging buffer
-        if (!d.ok) return;  // uniform
+    // A bulk copy needs 16-byte aligned addresses: the elements in front of
+    // the first boundary and behind the last one travel by small copies, and
+    // everything sits in shared memory at the same offset mod 16 bytes.
+    auto fetch = [&](const Desc& d) {
         const uint64_t* g = kin + d.base;
-        const uint32_t hd = head_of(g), m = ((d.n - hd) >> 1) << 1;
-        if (tid == 0) {
-            mbar_arrive_expect_tx(s_bar, m * 8u);
-            if (m) bulk_load(s_stage + 2 * hd, g + hd, m * 8u, s_bar);
+        const uint32_t hd = (uint32_t)(((uintptr_t)g >> 3) & 1u), m = ((d.n - hd) >> 1) << 1;
+        uint32_t ph = 0, pm = 0, po = 0;
+        const uint32_t* gp = nullptr;
+        if (SPAY) {
+            gp = pin + d.base;
+            po = (uint32_t)(((uintptr_t)gp >> 2) & 3u);
+            ph = min(d.n, (4u - po) & 3u);
+            pm = ((d.n - ph) >> 2) << 2;
         }
-        if (hd && tid == 1) cp_async8(&s_stage[1], g);
-        if (hd + m < d.n && tid == 2) cp_async8(&s_stage[d.n - 1 + hd], g + d.n - 1);
+        if (tid == 0) {
+            mbar_arrive_expect_tx(s_bar, m * 8u + pm * 4u);
+            if (m) bulk_load(s_key + 2 * hd, g + hd, m * 8u, s_bar);
+            if (SPAY && pm) bulk_load(s_pay + po + ph, gp + ph, pm * 4u, s_bar);
+        }
+        if (hd && tid == 32) cp_async8(&s_key[1], g);
+        if (hd + m < d.n && tid == 33) cp_async8(&s_key[d.n - 1 + hd], g + d.n - 1);
+        if (SPAY) {
+            if (tid >= 40 && (uint32_t)(tid - 40) < ph) cp_async4(&s_pay[po + tid - 40], gp + tid - 40);
+            if (tid >= 44 && tid < 48 && ph + pm + (uint32_t)(tid - 44) < d.n)
+                cp_async4(&s_pay[po + ph + pm + tid - 44], gp + ph + pm + tid - 44);
+        }
         cp_async_commit();
     };
-    Desc nxt = load_desc(blockIdx.x);
-    if (PREFETCH) prefetch(nxt);
+    // Slot of a key among the keys of group d counted so far.
+    auto take_slot = [&](uint32_t d) -> uint32_t {
+        const uint32_t sft = (d & 1u) * 16u;
+        return (atomicAdd(&s_cnt[d >> 1], 1u << sft) >> sft) & 0xffffu;
+    };
+    uint32_t phase = 0;
+    Desc cur = load_desc(blockIdx.x);
+    if (cur.ok) fetch(cur);
     for (uint64_t k = blockIdx.x; k < count; k += gridDim.x) {
-        const Desc cur = nxt;
-        nxt = load_desc(k + gridDim.x);
-        if (!cur.ok) {  // uniform per CTA; such a segment was never prefetched
-            if (PREFETCH) prefetch(nxt);
+        const Desc nxt = load_desc(k + gridDim.x);
+        if (!cur.ok) {  // uniform per CTA; such a segment was never fetched
+            cur = nxt;
+            if (cur.ok) fetch(cur);
             continue;
         }
-        const uint64_t s = list ? (uint64_t)list[k] : k;
         const uint64_t base = cur.base;
         const uint32_t n = cur.n;
-        uint32_t sh = 0;  // key j of the segment at src[j + sh]
-        if (PREFETCH) {
-            cp_async_wait_all();
-            const bool late = !mbar_wait(s_bar, phase);
-            phase ^= 1u;
-            if (__syncthreads_or(late)) {  // uniform; not expected: a bulk copy that never landed
-                if (tid == 0) atomicOr(err, kDevErrTimeout);
-                break;
-            }
-            sh = head_of(kin + base);
+        const uint32_t sh = (uint32_t)(((uintptr_t)(kin + base) >> 3) & 1u);
+        const uint64_t* key = s_key + sh;
+        cp_async_wait_all();
+        const bool late = !mbar_wait(s_bar, phase);
+        phase ^= 1u;
+        if (__syncthreads_or(late)) {  // uniform; not expected: a bulk copy that never landed
+            if (tid == 0) atomicOr(err, kDevErrTimeout);
+            cur.ok = false;
+            break;
         }
-        const uint64_t* src = PREFETCH ? s_stage : kin + base;
-        // The sorted keys: key j at s_key[j + ho], so that the part written
-        // back by a bulk copy starts on a 16-byte boundary.
-        const uint32_t ho = PREFETCH ? head_of(kout + base) : 0u;
-        uint64_t* sk = s_key + ho;
-        // Items past the segment are skipped by a uniform break (n is the
-        // same for the whole CTA), so a short segment costs no predicated work.
-        uint64_t key[ITEMS];
-        uint32_t hmin = ~0u, hmax = 0u;
+        // Range of the high words (of the low words when those are all equal).
+        uint32_t vmin = ~0u, vmax = 0u;
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
             if ((uint32_t)(i * THREADS) >= n) break;
-            const uint32_t e = tid + i * THREADS;
-            key[i] = e < n ? src[e + sh] ^ flip_in : 0ull;
-            const uint32_t h = (uint32_t)(key[i] >> 32);
-            if (e < n) { hmin = min(hmin, h); hmax = max(hmax, h); }
+            const uint32_t e = min((uint32_t)(tid + i * THREADS), n - 1);
+            const uint32_t h = (uint32_t)(key[e] >> 32) ^ hflip;
+            vmin = min(vmin, h);
+            vmax = max(vmax, h);
         }
-        hmin = __reduce_min_sync(0xffffffffu, hmin);
-        hmax = __reduce_max_sync(0xffffffffu, hmax);
-        if (lane == 0) { s_warp[w] = hmin; s_warp[WARPS + w] = hmax; }
-        for (int d = tid; d < R; d += THREADS) s_start[d] = 0;
-        if (tid == 0) s_flag[0] = 0;
+        vmin = __reduce_min_sync(0xffffffffu, vmin);
+        vmax = __reduce_max_sync(0xffffffffu, vmax);
+        if (lane == 0) { s_warp[w] = vmin; s_warp[32 + w] = vmax; }
+        for (int d = tid; d < R / 8; d += THREADS) ((uint4*)s_cnt)[d] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
-        if (PREFETCH) prefetch(nxt);  // the staging buffer has been read
-        hmin = ~0u; hmax = 0u;
 #pragma unroll
-        for (int i = 0; i < WARPS; ++i) { hmin = min(hmin, s_warp[i]); hmax = max(hmax, s_warp[WARPS + i]); }
-        // Digit: the high 32 key bits interpolated onto R groups when they
-        // spread over at least 8 R values (the common case, 32-bit work);
-        // else the whole 64-bit key range.  Either is monotone in the key.
-        const bool hi_mode = hmax - hmin >= 8u * (uint32_t)R;
-        uint64_t kmin = 0, mult64 = 0;
-        uint32_t mult32 = 0;
-        if (hi_mode) {
-            mult32 = interp_mult32(hmax - hmin, (uint32_t)R);
-        } else {
-            uint64_t lo = ~0ull, hi = 0ull;
+        for (int i = 0; i < WARPS; ++i) { vmin = min(vmin, s_warp[i]); vmax = max(vmax, s_warp[32 + i]); }
+        const bool by_hi = vmin != vmax;  // uniform
+        if (!by_hi) {
+            __syncthreads();  // s_warp is written again
+            vmin = ~0u; vmax = 0u;
+            for (uint32_t e = tid; e < n; e += THREADS) {
+                const uint32_t l = (uint32_t)key[e];
+                vmin = min(vmin, l);
+                vmax = max(vmax, l);
+            }
+            vmin = __reduce_min_sync(0xffffffffu, vmin);
+            vmax = __reduce_max_sync(0xffffffffu, vmax);
+            if (lane == 0) { s_warp[w] = vmin; s_warp[32 + w] = vmax; }
+            __syncthreads();
+            for (int i = 0; i < WARPS; ++i) { vmin = min(vmin, s_warp[i]); vmax = max(vmax, s_warp[32 + i]); }
+        }
+        uint64_t* dst = kout + base;
+        const uint32_t po = SPAY ? (uint32_t)(((uintptr_t)(pin + base) >> 2) & 3u) : 0u;
+        bool done = false;
+        if (vmin == vmax) {  // all keys equal: already in order
+            for (uint32_t j = tid; j < n; j += THREADS) {
+                dst[j] = key[j] ^ flip;
+                if (PAY) pout[base + j] = SPAY ? s_pay[po + j] : pin[base + j];
+            }
+            done = true;
+        }
+        if (!done) {
+            // x: the 32 bits below the common prefix of key - min; the largest
+            // one, top, has its high bit set, and the multiplier stays a
+            // little below R 2^32 / top so that no group number reaches R.
+            const int norm = __clz((int)(vmax - vmin));
+            const uint32_t top = (vmax - vmin) << norm | (norm ? (by_hi ? ~0u >> (32 - norm) : 0u) : 0u);
+            const uint32_t mult = __float2uint_rz(__fdividef((float)R * 4294967296.0f, (float)top) * (1.0f - 0x1p-20f));
+            uint32_t fr[ITEMS], dp[ITEMS];  // place in the group; group and slot
 #pragma unroll
             for (int i = 0; i < ITEMS; ++i) {
                 if ((uint32_t)(i * THREADS) >= n) break;
-                if (tid + i * THREADS < n) { lo = min(lo, key[i]); hi = max(hi, key[i]); }
+                const uint32_t e = tid + i * THREADS;
+                const uint64_t kk = key[min(e, n - 1)];
+                const uint32_t lo = (uint32_t)kk, hi = (uint32_t)(kk >> 32) ^ hflip;
+                const uint32_t x = by_hi ? __funnelshift_l(lo, hi - vmin, norm) : (lo - vmin) << norm;
+                const uint64_t prod = (uint64_t)x * mult;
+                const uint32_t d = e < n ? (uint32_t)(prod >> 32) : (uint32_t)(NC + 8 + 2 * lane);
+                fr[i] = (uint32_t)prod;
+                dp[i] = d | take_slot(d) << kSlotShift;
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                lo = min(lo, (uint64_t)__shfl_xor_sync(0xffffffffu, lo, o));
-                hi = max(hi, (uint64_t)__shfl_xor_sync(0xffffffffu, hi, o));
-            }
-            if (lane == 0) { s_red[w] = lo; s_red[32 + w] = hi; }
+            if (tid == 0) s_cnt[R / 2] = n;  // the end of the last group
             __syncthreads();
-            lo = ~0ull; hi = 0ull;
-            for (int i = 0; i < WARPS; ++i) { lo = min(lo, s_red[i]); hi = max(hi, s_red[32 + i]); }
-            if (lo == hi) {  // all keys equal
-#pragma unroll
-                for (int i = 0; i < ITEMS; ++i) {
-                    if ((uint32_t)(i * THREADS) >= n) break;
-                    const uint32_t e = tid + i * THREADS;
-                    if (e < n) kout[base + e] = key[i] ^ flip_out;
-                }
-                __syncthreads();
-                continue;
-            }
-            kmin = lo;
-            mult64 = interp_mult(hi - lo, (uint32_t)R);
-        }
-        uint32_t dp[ITEMS];
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            if ((uint32_t)(i * THREADS) >= n) break;
-            const uint32_t e = tid + i * THREADS;
-            uint32_t d = (uint32_t)R;  // past the segment
-            if (e < n) {
-                if (hi_mode) {
-                    d = min(__umulhi((uint32_t)(key[i] >> 32) - hmin, mult32), (uint32_t)R - 1);
-                } else {
-                    const uint64_t off = key[i] - kmin;
-                    d = mult64 ? min((uint32_t)__umul64hi(off, mult64), (uint32_t)R - 1) : (uint32_t)off;
-                }
-            }
-            if (d < (uint32_t)R) {
-                dp[i] = d | (atomicAdd(&s_start[d], 1u) << kSlotShift);
-            }
-        }
-        // The previous segment's bulk store has read s_key before the
-        // scatter below overwrites it (ordered by the scan's barriers).
-        if (PREFETCH && tid == 0) bulk_wait_read();
-        __syncthreads();
-        uint32_t mx = 0;
-        for (int d = tid; d < R; d += THREADS) mx = max(mx, s_start[d]);
-        mx = __reduce_max_sync(0xffffffffu, mx);
-        scan_smem_inplace<THREADS, R>(s_start, s_warp);
-        if (lane == 0) s_warp[w] = mx;
-        if (tid == 0) s_start[R] = n;
-        __syncthreads();
-        mx = 0;
-#pragma unroll
-        for (int i = 0; i < WARPS; ++i) mx = max(mx, s_warp[i]);
-        // scatter into group order
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            if ((uint32_t)(i * THREADS) >= n) break;
-            const uint32_t e = tid + i * THREADS;
-            if (e < n) sk[s_start[dp[i] & kDigitMask] + (dp[i] >> kSlotShift)] = key[i];
-        }
-        __syncthreads();
-        if (mx >= (uint32_t)kTinyGroup) {
-            // A large group is fine as it is if it holds a single value;
-            // the few that hold distinct keys are sorted in place by the CTA
-            // (a segment with more goes to the shared-memory kernel).
-#pragma unroll
-            for (int i = 0; i < ITEMS; ++i) {
-                if ((uint32_t)(i * THREADS) >= n) break;
-                if (tid + i * THREADS >= n) continue;
-                const uint32_t d = dp[i] & kDigitMask;
-                const uint32_t a = s_start[d];
-                if (s_start[d + 1] - a >= (uint32_t)kTinyGroup && sk[a] != sk[a + ((dp[i] >> kSlotShift) & kSlotMask)])
-                    s_mark[d] = 1u;
-            }
-            __syncthreads();
-            for (int d = tid; d < R; d += THREADS) {
-                if (s_mark[d]) {
-                    s_mark[d] = 0;
-                    const uint32_t q = atomicAdd(&s_flag[0], 1u);
-                    if (q < (uint32_t)kKeysMixedMax) s_flag[1 + q] = (uint32_t)d;
-                }
-            }
-            __syncthreads();
-            uint32_t nmixed = s_flag[0];
-            if (nmixed > (uint32_t)kKeysMixedMax) {  // uniform
-                // Keys spread over many binary orders of magnitude (lognormal
-                // ones, say) crowd the lowest groups of the linear digit: count
-                // and scatter once more on the logarithmic digit (log_digit of
-                // key - min, also monotone in the key), the keys re-read from
-                // the input, which is untouched until this segment is written.
-                const uint64_t* g = kin + base;
-                uint64_t lo = ~0ull, hi = 0ull;
-                for (uint32_t j = tid; j < n; j += THREADS) {
-                    const uint64_t k = g[j] ^ flip_in;
-                    lo = min(lo, k);
-                    hi = max(hi, k);
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    lo = min(lo, (uint64_t)__shfl_xor_sync(0xffffffffu, lo, o));
-                    hi = max(hi, (uint64_t)__shfl_xor_sync(0xffffffffu, hi, o));
-                }
-                if (lane == 0) { s_red[w] = lo; s_red[32 + w] = hi; }
-                for (int d = tid; d < R; d += THREADS) s_start[d] = 0;
-                __syncthreads();
-                lo = ~0ull;
-                hi = 0ull;
-                for (int i = 0; i < WARPS; ++i) { lo = min(lo, s_red[i]); hi = max(hi, s_red[32 + i]); }
-                // the 32 binary orders of magnitude below the range's top
-                const int e_lo = max(0, (63 - __clzll((long long)(hi - lo))) - 31);
-#pragma unroll
-                for (int i = 0; i < ITEMS; ++i) {
-                    if ((uint32_t)(i * THREADS) >= n) break;
-                    const uint32_t e = tid + i * THREADS;
-                    if (e < n) {
-                        const uint32_t d = log_digit<R>((g[e] ^ flip_in) - lo, e_lo);
-                        dp[i] = d | (atomicAdd(&s_start[d], 1u) << kSlotShift);
-                    }
-                }
-                __syncthreads();
-                uint32_t m2 = 0;
-                for (int d = tid; d < R; d += THREADS) m2 = max(m2, s_start[d]);
-                m2 = __reduce_max_sync(0xffffffffu, m2);
-                scan_smem_inplace<THREADS, R>(s_start, s_warp);
-                if (lane == 0) s_warp[w] = m2;
-                if (tid == 0) { s_start[R] = n; s_flag[0] = 0; }
-                __syncthreads();
-                mx = 0;
-#pragma unroll
-                for (int i = 0; i < WARPS; ++i) mx = max(mx, s_warp[i]);
-#pragma unroll
-                for (int i = 0; i < ITEMS; ++i) {
-                    if ((uint32_t)(i * THREADS) >= n) break;
-                    const uint32_t e = tid + i * THREADS;
-                    if (e < n) sk[s_start[dp[i] & kDigitMask] + (dp[i] >> kSlotShift)] = g[e] ^ flip_in;
-                }
-                __syncthreads();
-                if (mx >= (uint32_t)kTinyGroup) {
+            uint32_t mx = scan_pairs_inplace<THREADS, R / 2>(s_cnt, s_warp);
+            // Crowded groups: group d cut into as many parts as it holds keys,
+            // and counted again.  Where that no longer helps, a group above
+            // kChipMaxGroup has to hold one key value (else the segment is
+            // left to the shared-memory kernel); with a payload its keys want
+            // position order, so their position takes the place in the group
+            // for one more count.
+            bool slow = false;
+            if (mx > kChipRefine) {  // uniform
+                auto each_key = [&](auto body) {
 #pragma unroll
                     for (int i = 0; i < ITEMS; ++i) {
                         if ((uint32_t)(i * THREADS) >= n) break;
-                        if (tid + i * THREADS >= n) continue;
-                        const uint32_t d = dp[i] & kDigitMask;
-                        const uint32_t a = s_start[d];
-                        if (s_start[d + 1] - a >= (uint32_t)kTinyGroup &&
-                            sk[a] != sk[a + ((dp[i] >> kSlotShift) & kSlotMask)])
-                            s_mark[d] = 1u;
+                        if (tid + i * THREADS < n) body(i, (uint32_t)(tid + i * THREADS));
                     }
-                    __syncthreads();
-                    for (int d = tid; d < R; d += THREADS) {
-                        if (s_mark[d]) {
-                            s_mark[d] = 0;
-                            const uint32_t q = atomicAdd(&s_flag[0], 1u);
-                            if (q < (uint32_t)kKeysMixedMax) s_flag[1 + q] = (uint32_t)d;
-                        }
+                };
+                bool stuck = false, by_pos = false;
+                for (int it = 0;; ++it) {
+                    if (stuck || it >= kChipRefines) {
+                        if (mx <= kChipMaxGroup) break;
+                        if (by_pos) { slow = true; break; }
+                        each_key([&](int i, uint32_t e) {
+                            const uint32_t d = dp[i] & kGroupMask;
+                            s_w[s_start[d] + (dp[i] >> kSlotShift)] = e;
+                        });
+                        __syncthreads();
+                        bool mixed = false;
+                        const uint32_t unit = 0xffffffffu / n;
+                        each_key([&](int i, uint32_t e) {
+                            const uint32_t d = dp[i] & kGroupMask, a = s_start[d];
+                            if (s_start[d + 1] - a > kChipMaxGroup) {
+                                mixed = mixed || key[s_w[a]] != key[e];
+                                if (PAY) fr[i] = e * unit;
+                            }
+                        });
+                        slow = __syncthreads_or(mixed) != 0;
+                        if (slow || !PAY) break;
+                        by_pos = true;
                     }
+                    each_key([&](int i, uint32_t) {
+                        const uint32_t d = dp[i] & kGroupMask, a = s_start[d];
+                        const uint64_t prod = (uint64_t)fr[i] * (s_start[d + 1] - a);
+                        dp[i] = a + (uint32_t)(prod >> 32);
+                        fr[i] = (uint32_t)prod;
+                    });
                     __syncthreads();
-                }
-                nmixed = s_flag[0];
-                if (nmixed > (uint32_t)kKeysMixedMax) {  // the log digit crowds too
-                    if (tid == 0) slow_list[atomicAdd(slow_count, 1u)] = (uint32_t)s;
+                    for (int d = tid; d < NC / 8; d += THREADS) ((uint4*)s_cnt)[d] = make_uint4(0u, 0u, 0u, 0u);
                     __syncthreads();
-                    continue;
+                    each_key([&](int i, uint32_t) { dp[i] |= take_slot(dp[i]) << kSlotShift; });
+                    if (tid == 0) s_cnt[NC / 2] = n;
+                    __syncthreads();
+                    const uint32_t m2 = scan_pairs_inplace<THREADS, NC / 2>(s_cnt, s_warp);
+                    stuck = m2 >= mx || by_pos;
+                    mx = m2;
+                    if (mx <= kChipRefine) break;
                 }
             }
-            for (uint32_t q = 0; q < nmixed; ++q) {
-                const uint32_t d = s_flag[1 + q];
-                const uint32_t a = s_start[d];
-                cta_bitonic_sort<THREADS>(sk, a, s_start[d + 1] - a, [](uint32_t i) { return i; });
-            }
-        }
-        if (mx > 1u) {
-            // Every group of 2..kTinyGroup-1 keys is sorted in place by the
-            // thread owning it (each thread owns G consecutive groups; the
-            // groups hold a few keys, nearly in order); a large group holding
-            // one value needs nothing.  The groups come in key order, so when
-            // a thread's groups hold few keys in all, one insertion sort over
-            // their whole range does it.
-            constexpr int G = R / THREADS;
-            const uint32_t ga = s_start[tid * G], gb = s_start[tid * G + G];
-            if (gb - ga < (uint32_t)kTinyGroup) {
-                for (uint32_t j = ga + 1; j < gb; ++j) {
-                    const uint64_t x = sk[j];
-                    uint32_t i = j;
-                    while (i > ga) {
-                        const uint64_t y = sk[i - 1];
-                        if (y <= x) break;
-                        sk[i] = y;
-                        --i;
-                    }
-                    sk[i] = x;
-                }
+            if (slow) {  // uniform: left to the shared-memory kernel
+                if (tid == 0) slow_list[atomicAdd(slow_count, 1u)] = (uint32_t)(list ? (uint64_t)list[k] : k);
             } else {
-                for (int g = tid * G; g < tid * G + G; ++g) {
-                    const uint32_t a = s_start[g], b = s_start[g + 1];
-                    if (b - a < 2u || b - a >= (uint32_t)kTinyGroup) continue;
-                    for (uint32_t j = a + 1; j < b; ++j) {
-                        const uint64_t x = sk[j];
-                        uint32_t i = j;
-                        while (i > a) {
-                            const uint64_t y = sk[i - 1];
-                            if (y <= x) break;
-                            sk[i] = y;
-                            --i;
+                const uint32_t W = (n + 7) / 8;  // windows of eight words
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i) {
+                    if ((uint32_t)(i * THREADS) >= n) break;
+                    const uint32_t e = tid + i * THREADS;
+                    const uint32_t a = s_start[dp[i] & kGroupMask];
+                    const uint32_t word = a << SH | (fr[i] >> (32 - FR)) << IDX | e;
+                    if (e < n) s_w[a + (dp[i] >> kSlotShift)] = word;
+                }
+                if (tid < 8 && n + tid < 8 * W) s_w[n + tid] = (n + tid) << SH | ((1u << SH) - 1u);
+                if (!PAY && mx > kChipMaxGroup) {
+                    // keys alone: the words of a large group (one key value)
+                    // stay where they are, their own index as group start
+#pragma unroll
+                    for (int i = 0; i < ITEMS; ++i) {
+                        if ((uint32_t)(i * THREADS) >= n) break;
+                        const uint32_t e = tid + i * THREADS, d = dp[i] & kGroupMask;
+                        const uint32_t a = s_start[d], at = a + (dp[i] >> kSlotShift);
+                        if (e < n && s_start[d + 1] - a > kChipMaxGroup) s_w[at] = at << SH | e;
+                    }
+                }
+                __syncthreads();
+                {
+                    // Words relative to their window: start - window + 56 in the top bits.
+                    uint32_t q[WIN][8];
+#pragma unroll
+                    for (int v = 0; v < WIN; ++v) {
+                        const uint32_t b = tid + v * THREADS;
+                        if (b < W) {
+                            const uint4* src4 = (const uint4*)(s_w + 8 * b);
+                            const uint4 x = src4[(tid >> 2) & 1], y = src4[((tid >> 2) & 1) ^ 1];  // no bank met twice
+                            const uint32_t rel = (8 * b + 8) << SH;  // 8 b - 56 mod 64
+                            q[v][0] = x.x - rel; q[v][1] = x.y - rel; q[v][2] = x.z - rel; q[v][3] = x.w - rel;
+                            q[v][4] = y.x - rel; q[v][5] = y.y - rel; q[v][6] = y.z - rel; q[v][7] = y.w - rel;
+                            sort_8(q[v]);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) q[v][i] = ~0u;
                         }
-                        sk[i] = x;
+                    }
+                    if (tid == 0) *(uint4*)s_first = make_uint4(q[0][0], q[0][1], q[0][2], q[0][3]);
+                    constexpr uint32_t kStep = 4u << SH;
+                    // Round 2 and every even one: window b takes the lower half
+                    // of window b + 1; odd rounds: back.  s_first: the lower
+                    // half of window 0 meanwhile.
+                    auto round_up = [&](uint32_t* edge, bool moved_before) -> int {
+#pragma unroll
+                        for (int v = 0; v < WIN; ++v)
+                            if (lane == 0)
+                                *(uint4*)(edge + (v * WARPS + w) * 4) = make_uint4(q[v][0], q[v][1], q[v][2], q[v][3]);
+                        return __syncthreads_or(moved_before);
+                    };
+                    auto merge_up = [&](const uint32_t* edge) -> bool {
+                        bool moved = false;
+#pragma unroll
+                        for (int v = 0; v < WIN; ++v) {
+                            if ((uint32_t)(v * THREADS + w * 32) >= W) break;  // uniform per warp
+                            uint32_t o[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) o[i] = __shfl_down_sync(0xffffffffu, q[v][i], 1);
+                            const uint32_t b = tid + v * THREADS;
+                            if (lane == 31) {
+                                const uint4 x = b + 1 < W ? *(const uint4*)(edge + (v * WARPS + w + 1) * 4)
+                                                          : make_uint4(~0u, ~0u, ~0u, ~0u);
+                                o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w;
+                            }
+                            const bool last = b + 1 >= W;
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                q[v][i] = q[v][4 + i] - kStep;
+                                q[v][4 + i] = last ? ~0u : o[i] + kStep;
+                            }
+                            moved = moved || (b < W && q[v][4] < q[v][3]);
+                            merge_4_4(q[v]);
+                        }
+                        return moved;
+                    };
+                    round_up(s_edge, false);
+                    merge_up(s_edge);
+                    uint32_t off = 4;
+                    if (mx > 5u) {  // uniform
+                        bool moved = false;
+                        for (uint32_t round = 3; round <= kChipRounds; ++round) {
+                            uint32_t* edge = s_edge + (round & 1u) * (WIN * WARPS * 4);
+                            if (off) {
+#pragma unroll
+                                for (int v = 0; v < WIN; ++v)
+                                    if (lane == 31)
+                                        *(uint4*)(edge + (v * WARPS + w) * 4) =
+                                            make_uint4(q[v][4], q[v][5], q[v][6], q[v][7]);
+                                if (!__syncthreads_or(moved) && round > 3) break;  // the last round changed nothing
+                                moved = false;
+#pragma unroll
+                                for (int v = 0; v < WIN; ++v) {
+                                    if ((uint32_t)(v * THREADS + w * 32) >= W) break;
+                                    uint32_t o[4];
+#pragma unroll
+                                    for (int i = 0; i < 4; ++i) o[i] = __shfl_up_sync(0xffffffffu, q[v][4 + i], 1);
+                                    const uint32_t b = tid + v * THREADS;
+                                    if (lane == 0) {
+                                        const uint4 x = b > 0 ? *(const uint4*)(edge + (v * WARPS + w - 1) * 4)
+                                                              : *(const uint4*)s_first;
+                                        o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w;
+                                    }
+#pragma unroll
+                                    for (int i = 0; i < 4; ++i) {
+                                        q[v][4 + i] = q[v][i] + kStep;
+                                        q[v][i] = b > 0 ? o[i] - kStep : o[i];
+                                    }
+                                    moved = moved || (b < W && q[v][4] < q[v][3]);
+                                    merge_4_4(q[v]);
+                                }
+                                if (tid == 0) *(uint4*)s_first = make_uint4(q[0][0], q[0][1], q[0][2], q[0][3]);
+                            } else {
+                                if (!round_up(edge, moved)) break;
+                                moved = merge_up(edge);
+                            }
+                            off ^= 4u;
+                            if (mx <= 9u) break;  // three rounds order groups of nine
+                        }
+                    }
+                    // The words in order, as they were scattered.
+                    if (off && tid == 0) {
+                        const uint4 x = *(const uint4*)s_first;
+                        constexpr uint32_t rel = 8u << SH;
+                        *(uint4*)s_w = make_uint4(x.x + rel, x.y + rel, x.z + rel, x.w + rel);
+                    }
+#pragma unroll
+                    for (int v = 0; v < WIN; ++v) {
+                        const uint32_t b = tid + v * THREADS;
+                        if (b < W) {
+                            const uint32_t rel = (8 * b + off + 8) << SH;
+                            uint4* o = (uint4*)(s_w + 8 * b + off);
+                            o[0] = make_uint4(q[v][0] + rel, q[v][1] + rel, q[v][2] + rel, q[v][3] + rel);
+                            o[1] = make_uint4(q[v][4] + rel, q[v][5] + rel, q[v][6] + rel, q[v][7] + rel);
+                        }
+                    }
+                    __syncthreads();
+                    bool wrong = false;
+                    auto put = [&](uint32_t j, uint32_t wj) {
+                        const uint32_t e = wj & kPosMask;
+                        dst[j] = key[e] ^ flip;
+                        if (SPAY) pout[base + j] = s_pay[po + e];
+                    };
+#pragma unroll 4
+                    for (uint32_t j = tid; j < n; j += THREADS) {
+                        const uint32_t wj = s_w[j], w1 = s_w[j + 1];
+                        if (((wj ^ w1) >> IDX) == 0u && j + 1 < n) {
+                            const uint64_t f = (uint64_t)hflip << 32;
+                            wrong = wrong || (key[wj & kPosMask] ^ f) > (key[w1 & kPosMask] ^ f);
+                        }
+                        put(j, wj);
+                    }
+                    if (__syncthreads_or(wrong)) {
+                        // Distinct keys that the words do not tell apart: each
+                        // run of equal (group, place) by (key, position).
+                        const uint64_t f = (uint64_t)hflip << 32;
+                        for (uint32_t j = tid; j + 1 < n; j += THREADS) {
+                            if (j > 0 && ((s_w[j - 1] ^ s_w[j]) >> IDX) == 0u) continue;  // not the start of a run
+                            const uint32_t head = s_w[j] >> IDX;
+                            uint32_t z = j + 1;
+                            for (; z < n && s_w[z] >> IDX == head; ++z) {
+                                const uint32_t wz = s_w[z], ez = wz & kPosMask;
+                                const uint64_t kz = key[ez] ^ f;
+                                uint32_t i = z;
+                                for (; i > j; --i) {
+                                    const uint32_t wy = s_w[i - 1], ey = wy & kPosMask;
+                                    const uint64_t ky = key[ey] ^ f;
+                                    if (ky < kz || (ky == kz && ey < ez)) break;
+                                    s_w[i] = wy;
+                                }
+                                s_w[i] = wz;
+                            }
+                        }
+                        __syncthreads();
+                        for (uint32_t j = tid; j < n; j += THREADS) put(j, s_w[j]);
+                    }
+                    if (PAY && !SPAY) {  // the output may be the input: gather every payload first
+                        uint32_t pv[ITEMS];
+#pragma unroll
+                        for (int i = 0; i < ITEMS; ++i) {
+                            const uint32_t j = tid + i * THREADS;
+                            pv[i] = j < n ? pin[base + (s_w[j] & kPosMask)] : 0u;
+                        }
+                        __syncthreads();
+#pragma unroll
+                        for (int i = 0; i < ITEMS; ++i) {
+                            const uint32_t j = tid + i * THREADS;
+                            if (j < n) pout[base + j] = pv[i];
+                        }
                     }
                 }
             }
-            __syncthreads();
         }
-        uint64_t* dst = kout + base;
-        if (PREFETCH) {
-            if (flip_out) {  // uniform: signed keys back from order-preserving bits
-                for (uint32_t j = tid; j < n; j += THREADS) sk[j] ^= flip_out;
-                __syncthreads();
-            }
-            // One bulk copy writes the 16-byte aligned middle; the first and
-            // last key go by plain stores when they fall outside it.
-            const uint32_t m = ((n - ho) >> 1) << 1;
-            if (ho && tid == 1) dst[0] = sk[0];
-            if (ho + m < n && tid == 2) dst[n - 1] = sk[n - 1];
-            fence_async_smem();
-            __syncthreads();
-            if (tid == 0 && m) bulk_store(dst + ho, s_key + 2 * ho, m * 8u);
-        } else {
-            for (uint32_t j = tid; j < n; j += THREADS) dst[j] = sk[j] ^ flip_out;
-            __syncthreads();
-        }
+        __syncthreads();  // the staged keys have been read
+        cur = nxt;
+        if (cur.ok) fetch(cur);
     }
-    if (PREFETCH) {
-        cp_async_wait_all();
-        if (tid == 0) bulk_wait_all();
-    }
+    cp_async_wait_all();
 }
 
 // ---------------------------------------------------------------------------
@@ -1544,8 +1522,7 @@ __global__ __launch_bounds__(1024) void k_plan_scan(uint32_t nblk, uint32_t* __r
             host_counts[7] = (uint32_t)(carry.keys >> 32);
         }
         counters[24] = 0;  // fallback list of this level's on-chip sorts
-        counters[25] = 0;  // segments the register kernels leave to the shared-memory kernel
-        counters[26] = 0;  // ... and the keys-only kernels, per size class
+        counters[26] = 0;  // segments k_chip leaves to the shared-memory kernel, per size class
         counters[27] = 0;
         counters[28] = 0;
     }
@@ -2276,42 +2253,24 @@ static cudaError_t launch_small(const uint64_t* in, uint64_t* out, const uint32_
     return cudaGetLastError();
 }
 
-template <bool PAY, int THREADS, int CAP>
-static cudaError_t launch_small_reg(const uint64_t* in, uint64_t* out, const uint32_t* pin, uint32_t* pout,
-                                    const uint64_t* seg_lo, const uint64_t* seg_hi, const uint32_t* list,
-                                    const uint32_t* nlist, uint64_t count, uint64_t nseg, uint32_t min_n, uint32_t max_n,
-                                    uint64_t fin, uint64_t fout, const SegSortWs& ws, cudaStream_t st) {
-    constexpr size_t smem = reg_sort_smem<CAP>();
-    {
-        const cudaError_t e = ensure_func_attrs((const void*)k_small_reg<PAY, THREADS, CAP>, (int)smem, 100);
-        if (e != cudaSuccess) return e;
-    }
-    const int per_sm = resident_ctas((const void*)k_small_reg<PAY, THREADS, CAP>, THREADS, smem);
-    const uint64_t grid = std::min<uint64_t>(count, (uint64_t)num_sms() * per_sm * 4);
-    if (grid == 0) return cudaSuccess;
-    HSS_LAUNCH((k_small_reg<PAY, THREADS, CAP>), (unsigned)grid, THREADS, smem, st, in, out, pin, pout, seg_lo, seg_hi,
-               list, nlist, nseg, min_n, max_n, fin, fout, ws.slow_list, ws.counters + 25);
-    return cudaGetLastError();
-}
-
-template <int THREADS, int CAP, int R, bool PREFETCH>
-static cudaError_t launch_keys(const uint64_t* in, uint64_t* out, const uint64_t* seg_lo, const uint64_t* seg_hi,
-                               const uint32_t* list, const uint32_t* nlist, uint64_t count, uint64_t nseg,
-                               uint32_t min_n, uint32_t max_n, uint64_t fin, uint64_t fout, uint32_t* slow,
-                               uint32_t* slow_count, uint32_t* err, cudaStream_t st) {
-    constexpr size_t smem = keys_sort_smem<CAP, R, PREFETCH>();
-    const void* fn = (const void*)k_small_keys<THREADS, CAP, R, PREFETCH>;
+template <bool PAY, int THREADS, int CAP, int R>
+static cudaError_t launch_chip(const uint64_t* in, uint64_t* out, const uint32_t* pin, uint32_t* pout,
+                               const uint64_t* seg_lo, const uint64_t* seg_hi, const uint32_t* list,
+                               const uint32_t* nlist, uint64_t count, uint64_t nseg, uint32_t min_n, uint32_t max_n,
+                               uint64_t fin, uint64_t fout, uint32_t* slow, uint32_t* slow_count, uint32_t* err,
+                               cudaStream_t st) {
+    constexpr size_t smem = chip_smem<PAY, THREADS, CAP, R>();
+    const void* fn = (const void*)k_chip<PAY, THREADS, CAP, R>;
     {
         // all of L1 as shared memory: the CTAs per SM are limited by their buffers
         const cudaError_t e = ensure_func_attrs(fn, (int)smem, 100);
         if (e != cudaSuccess) return e;
     }
     const int per_sm = resident_ctas(fn, THREADS, smem);
-    // With prefetching every CTA walks several segments of the list.
-    const uint64_t grid = std::min<uint64_t>(count, (uint64_t)num_sms() * per_sm * (PREFETCH ? 1 : 4));
+    const uint64_t grid = std::min<uint64_t>(count, (uint64_t)num_sms() * per_sm);
     if (grid == 0) return cudaSuccess;
-    HSS_LAUNCH((k_small_keys<THREADS, CAP, R, PREFETCH>), (unsigned)grid, THREADS, smem, st, in, out, seg_lo, seg_hi,
-               list, nlist, nseg, min_n, max_n, fin, fout, slow, slow_count, err);
+    HSS_LAUNCH((k_chip<PAY, THREADS, CAP, R>), (unsigned)grid, THREADS, smem, st, in, out, pin, pout, seg_lo, seg_hi, list,
+               nlist, nseg, min_n, max_n, fin, fout, slow, slow_count, err);
     return cudaGetLastError();
 }
 
@@ -2347,6 +2306,36 @@ struct Level {
     int depth;
     const uint64_t* hint_hi = nullptr;  // largest key of each segment, when known
 };
+
+// The on-chip sort of one size class: its segments, then those it leaves to
+// the shared-memory kernel (whose own leftovers go to the fallback list).
+template <bool PAY>
+static cudaError_t chip_class(int c, const Level& L, uint64_t* dst, uint32_t* pdst, const uint32_t* list,
+                              const uint32_t* nlist, uint64_t count, uint32_t lo_n, uint32_t hi_n, uint64_t fout,
+                              const SegSortWs& ws, cudaStream_t st) {
+    uint32_t* slow = ws.slow_keys[c];
+    uint32_t* slow_n = ws.counters + 26 + c;
+    cudaError_t e;
+    if (c == 0) {
+        e = launch_chip<PAY, kC0Threads, kC0Cap, 1024>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
+                                                       L.nseg, lo_n, hi_n, L.flip_in, fout, slow, slow_n, ws.err, st);
+        if (e != cudaSuccess) return e;
+        return launch_small<PAY, kC0Threads, kC0Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, slow, slow_n, count,
+                                                     L.nseg, lo_n, hi_n, L.flip_in, fout, ws, st);
+    }
+    if (c == 1) {
+        e = launch_chip<PAY, kC1Threads, kC1Cap, 4096>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
+                                                       L.nseg, lo_n, hi_n, L.flip_in, fout, slow, slow_n, ws.err, st);
+        if (e != cudaSuccess) return e;
+        return launch_small<PAY, kC1Threads, kC1Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, slow, slow_n, count,
+                                                     L.nseg, lo_n, hi_n, L.flip_in, fout, ws, st);
+    }
+    e = launch_chip<PAY, 1024, kSmallCap, 8192>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count, L.nseg,
+                                                lo_n, hi_n, L.flip_in, fout, slow, slow_n, ws.err, st);
+    if (e != cudaSuccess) return e;
+    return launch_small<PAY, kC2Threads, kSmallCap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, slow, slow_n, count, L.nseg,
+                                                    lo_n, hi_n, L.flip_in, fout, ws, st);
+}
 
 // This thread's mapped pinned buffer for the planning counts (allocated once
 // per thread; null if the allocation fails, and then the counts are copied).
@@ -2399,25 +2388,16 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
     if (N <= (uint64_t)kSmallCap) {
         // No segment can exceed the on-chip capacity: sort every segment in
         // its class without planning (and without a host round trip).
-        if ((e = cudaMemsetAsync(ws.counters + 24, 0, 8, st)) != cudaSuccess) return e;
-        if ((e = launch_small<PAY, kC0Threads, kC0Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, nullptr, nullptr, nseg,
-                                                       nseg, 0u, (uint32_t)kC0Cap, L.flip_in, fout, ws, st)) !=
-            cudaSuccess)
-            return e;
-        if (N > (uint64_t)kC0Cap &&
-            (e = launch_small_reg<PAY, kC1Threads, kC1Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, nullptr, nullptr,
-                                                           nseg, nseg, (uint32_t)kC0Cap, (uint32_t)kC1Cap, L.flip_in,
-                                                           fout, ws, st)) != cudaSuccess)
-            return e;
-        if ((e = launch_small<PAY, kC1Threads, kC1Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, ws.slow_list,
-                                                       ws.counters + 25, nseg, nseg, 0u, (uint32_t)kC1Cap, L.flip_in,
-                                                       fout, ws, st)) != cudaSuccess)
-            return e;
-        if (N > (uint64_t)kC1Cap &&
-            (e = launch_small<PAY, kC2Threads, kSmallCap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, nullptr, nullptr,
-                                                          nseg, nseg, (uint32_t)kC1Cap, (uint32_t)kSmallCap, L.flip_in,
-                                                          fout, ws, st)) != cudaSuccess)
-            return e;
+        if ((e = cudaMemsetAsync(ws.counters + 24, 0, 20, st)) != cudaSuccess) return e;
+        for (int c = 0; c < 3; ++c) {
+            const uint32_t lo_n = c == 0 || nseg == 1 ? 0u : (c == 1 ? (uint32_t)kC0Cap : (uint32_t)kC1Cap);
+            const uint32_t hi_n = c == 0 ? (uint32_t)kC0Cap : (c == 1 ? (uint32_t)kC1Cap : (uint32_t)kSmallCap);
+            // one segment: the class of the largest it can be takes it whatever its size
+            if (N <= lo_n || (nseg == 1 && c < 2 && N > hi_n)) continue;
+            if ((e = chip_class<PAY>(c, L, dst, pdst, nullptr, nullptr, nseg, lo_n, hi_n, fout, ws, st)) != cudaSuccess)
+                return e;
+            if (nseg == 1) break;
+        }
         return launch_fallback<PAY>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, L.flip_in, fout, ws, st, nseg);
     }
     for (;;) {
@@ -2440,59 +2420,14 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
         const uint32_t n_large = hc[3], tiles = hc[4];
         const uint64_t keys_large = (uint64_t)hc[6] | ((uint64_t)hc[7] << 32);
         // Segments of this level that fit on chip: straight to the output.
-        if (!PAY) {
-            // keys alone: the register kernels first, their leftovers to the
-            // shared-memory kernel of the same class
-            const uint32_t* lists[3] = {ws.list[0], ws.list[1], ws.list[2]};
-            for (int c = 0; c < 3; ++c) {
-                if (!hc[c]) continue;
-                const uint32_t lo_n = c == 0 ? 0u : (c == 1 ? (uint32_t)kC0Cap : (uint32_t)kC1Cap);
-                const uint32_t hi_n = c == 0 ? (uint32_t)kC0Cap : (c == 1 ? (uint32_t)kC1Cap : (uint32_t)kSmallCap);
-                uint32_t* slow = ws.slow_keys[c];
-                uint32_t* slow_n = ws.counters + 26 + c;
-                if (c == 0)
-                    e = launch_keys<kC0Threads, kC0Cap, 512, true>(L.in, dst, L.seg_lo, L.seg_hi, lists[c], ws.counters + 16,
-                                                            hc[c], L.nseg, lo_n, hi_n, L.flip_in, fout, slow, slow_n, ws.err, st);
-                else if (c == 1)
-                    e = launch_keys<kC1Threads, kC1Cap, 2048, true>(L.in, dst, L.seg_lo, L.seg_hi, lists[c], ws.counters + 17,
-                                                            hc[c], L.nseg, lo_n, hi_n, L.flip_in, fout, slow, slow_n, ws.err, st);
-                else
-                    e = launch_keys<kC2Threads, kSmallCap, 4096, false>(L.in, dst, L.seg_lo, L.seg_hi, lists[c],
-                                                               ws.counters + 18, hc[c], L.nseg, lo_n, hi_n, L.flip_in,
-                                                               fout, slow, slow_n, ws.err, st);
-                if (e != cudaSuccess) return e;
-                if (c == 0)
-                    e = launch_small<PAY, kC0Threads, kC0Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, slow, slow_n,
-                                                              hc[c], L.nseg, lo_n, hi_n, L.flip_in, fout, ws, st);
-                else if (c == 1)
-                    e = launch_small<PAY, kC1Threads, kC1Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, slow, slow_n,
-                                                              hc[c], L.nseg, lo_n, hi_n, L.flip_in, fout, ws, st);
-                else
-                    e = launch_small<PAY, kC2Threads, kSmallCap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, slow,
-                                                                 slow_n, hc[c], L.nseg, lo_n, hi_n, L.flip_in, fout,
-                                                                 ws, st);
-                if (e != cudaSuccess) return e;
-            }
+        for (int c = 0; c < 3; ++c) {
+            if (!hc[c]) continue;
+            const uint32_t lo_n = c == 0 ? 0u : (c == 1 ? (uint32_t)kC0Cap : (uint32_t)kC1Cap);
+            const uint32_t hi_n = c == 0 ? (uint32_t)kC0Cap : (c == 1 ? (uint32_t)kC1Cap : (uint32_t)kSmallCap);
+            if ((e = chip_class<PAY>(c, L, dst, pdst, ws.list[c], ws.counters + 16 + c, hc[c], lo_n, hi_n, fout, ws, st)) !=
+                cudaSuccess)
+                return e;
         }
-        if (PAY && hc[0] && (e = launch_small<PAY, kC0Threads, kC0Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, ws.list[0],
-                                                                ws.counters + 16, hc[0], L.nseg, 0u, (uint32_t)kC0Cap,
-                                                                L.flip_in, fout, ws, st)) != cudaSuccess)
-            return e;
-        if (PAY && hc[1] && (e = launch_small_reg<PAY, kC1Threads, kC1Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi,
-                                                                    ws.list[1], ws.counters + 17, hc[1], L.nseg,
-                                                                    (uint32_t)kC0Cap, (uint32_t)kC1Cap, L.flip_in, fout,
-                                                                    ws, st)) != cudaSuccess)
-            return e;
-        if (PAY && hc[1] &&
-            (e = launch_small<PAY, kC1Threads, kC1Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, ws.slow_list,
-                                                       ws.counters + 25, hc[1], L.nseg, 0u, (uint32_t)kC1Cap, L.flip_in,
-                                                       fout, ws, st)) != cudaSuccess)
-            return e;
-        if (PAY && hc[2] && (e = launch_small<PAY, kC2Threads, kSmallCap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi,
-                                                                   ws.list[2], ws.counters + 18, hc[2], L.nseg,
-                                                                   (uint32_t)kC1Cap, (uint32_t)kSmallCap, L.flip_in, fout,
-                                                                   ws, st)) != cudaSuccess)
-            return e;
         if ((hc[0] || hc[1] || hc[2]) &&
             (e = launch_fallback<PAY>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, L.flip_in, fout, ws, st,
                                       (uint64_t)hc[0] + hc[1] + hc[2])) != cudaSuccess)

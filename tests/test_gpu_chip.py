@@ -1,0 +1,64 @@
+"""The on-chip sort at the edges of its classes, windows and groups, against
+numpy's stable sort: sizes around the class limits and the window of eight,
+segment starts that are not 16- or 32-byte aligned, crowded and duplicated
+keys (the refined groups, the run sort of keys the 32-bit words do not tell
+apart, groups of one value) and both key types."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [1, 2, 7, 8, 9, 31, 33, 1023, 1024, 1025, 1033, 1535, 1536, 1537, 2047, 4089, 4095, 4096, 4097, 14335, 14336,
+         14337]
+
+
+def _keys(kind, n, g):
+    r = g.integers(0, 1 << 63, size=n, dtype=np.uint64) * np.uint64(2) + g.integers(0, 2, size=n, dtype=np.uint64)
+    if kind == "uniform":
+        return r
+    if kind == "narrow":  # all high words equal
+        return (np.uint64(0x123456789) << np.uint64(28)) + (r >> np.uint64(45))
+    if kind == "clusters":  # a few narrow clusters: one group holds most of the segment
+        return (r >> np.uint64(40)) + (g.integers(0, 3, size=n).astype(np.uint64) << np.uint64(61))
+    if kind == "orders":  # every binary order of magnitude
+        return r >> g.integers(0, 64, size=n).astype(np.uint64)
+    if kind == "close":  # distinct keys that agree in their upper 40 bits, among spread ones
+        return np.where(g.random(n) < 0.3, (r & np.uint64(0x7)) + np.uint64(1 << 62), r)
+    if kind == "few":  # groups of one value
+        return g.integers(0, 5, size=n).astype(np.uint64) << np.uint64(40)
+    if kind == "pairs":  # every key about twice
+        return r[g.integers(0, max(1, n // 2), size=n)]
+    if kind == "ends":  # the smallest and largest values of both key types
+        return np.array([0, 1, (1 << 63) - 1, 1 << 63, (1 << 64) - 2, (1 << 64) - 1], dtype=np.uint64)[
+            g.integers(0, 6, size=n)]
+    raise ValueError(kind)
+
+
+@pytest.mark.parametrize("payload", [False, True])
+@pytest.mark.parametrize("kind", ["uniform", "narrow", "clusters", "orders", "close", "few", "pairs", "ends"])
+def test_on_chip_sort_edges(kind, payload):
+    import torch
+
+    from paper_1803_01237_gb300 import hss
+
+    g = np.random.Generator(np.random.Philox(key=[17, sum(map(ord, kind))]))
+    for n in SIZES:
+        # 1 segment, and (for the larger sizes) 3 segments of n keys in a larger call
+        for p, shift in ((1, 0), (1, 1), (3, 3), (40, 2)):
+            if p == 40 and n > 4097:
+                continue
+            N = n * p
+            for key_type in ("u64", "i64"):
+                raw = _keys(kind, N + shift, g)
+                kv = raw.view(np.int64) if key_type == "i64" else raw
+                dk = torch.from_numpy(raw.view(np.int64)).cuda()[shift:]
+                pay = np.arange(N + shift, dtype=np.int32)
+                dp = torch.from_numpy(pay).cuda()[shift:] if payload else None
+                out = torch.empty(N + 3, dtype=torch.int64, device="cuda")[shift:shift + N]
+                o = hss.local_sort(dk, p, payload=dp, key_type=key_type, out=out)
+                off = [(s * N) // p for s in range(p + 1)]
+                want = np.concatenate([shift + off[s] + np.argsort(kv[shift + off[s]:shift + off[s + 1]], kind="stable")
+                                       for s in range(p)])
+                assert np.array_equal(out.cpu().numpy(), raw.view(np.int64)[want]), (kind, n, p, shift, key_type)
+                if payload:
+                    assert np.array_equal(o[1].cpu().numpy(), pay[want]), (kind, n, p, shift, key_type)
