@@ -293,7 +293,7 @@ __device__ __forceinline__ void block_rank(DigitOf digit_of, uint32_t count, uin
 }
 
 // ---------------------------------------------------------------------------
-// On-chip sort of the segments k_chip leaves, with min_n < n <= max_n keys
+// On-chip sort of segments that k_chip leaves, with min_n < n <= max_n keys
 // (n <= CAP), taken from `list` (compact ids, count at *nlist).  The keys are read once into shared memory.  One counting
 // pass on a 10-bit digit (the segment's key range interpolated onto 1024
 // groups) splits them into groups that come in key order; inside a group the
