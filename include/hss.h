@@ -516,14 +516,13 @@ typedef struct {
      * up to pack_keys keys (their keys are already in order between them, so
      * sorting the run sorts each).  1 .. 4096; 0 = 1024; 1 packs nothing. */
     uint32_t pack_keys;
-    /* First split of each segment of a local sort: 0 (default) on its top
-     * varying byte; 1 samples the segment first and, when the sample's top
-     * varying byte crowds its keys into few values (Gaussian clusters, heavy
-     * duplicates, spatially clustered Morton codes), splits on 255 splitters
-     * taken from the sorted sample (a binary search per key) and packs those
-     * sub-buckets by at most 256 keys.  Faster on the clustered Morton
-     * payload workload, slower on the Gaussian mixture and Zipf keys: off by
-     * default, left to the autotuner. */
+    /* First split of each segment of a local sort.  A sample of the segment
+     * shows whether its top varying byte would crowd the keys into a few
+     * sub-buckets too large for the chip (Gaussian clusters, spatially
+     * clustered Morton codes): then the segment splits on 255 splitters taken
+     * from the sorted sample (a binary search per key) instead.  0 (default):
+     * calls of 2^22 keys and more in segments of 2^15 keys and more on average
+     * are sampled; 1: every local sort is. */
     uint32_t first_split;
     /* How the split pass writes a tile: 0 stages the tile in shared memory in
      * digit order and writes each digit's run with consecutive stores; 1

@@ -98,7 +98,7 @@ size_t segsort_ws_bytes(uint64_t N, uint64_t nseg) {
     b += align_up(d.ml * 4, 256);                                     // large_seg
     b += align_up(d.tiles * 2 * kRadix * 2, 256);                     // tile_hist
     b += align_up(d.tiles, 256);                                      // tile_skew
-    b += align_up(std::min(nseg, d.ml) * kRadix * 8, 256);           // spl_tab
+    b += align_up(std::min(nseg, d.ml) * kRadix * 4, 256);           // spl_tab
     b += align_up(std::min(nseg, d.ml), 256);                        // spl_mode
     b += 2 * align_up(d.ml * 8, 256);                                 // vor, vand
     b += 4 * align_up(d.ml * 4, 256);                                 // msd_shift x2, spec, direct
@@ -128,7 +128,7 @@ SegSortWs segsort_ws_carve(void* base, uint64_t N, uint64_t nseg, uint32_t* err)
     w.tile_hist = (uint16_t*)take(d.tiles * 2 * kRadix * 2);
     w.tile_skew = (uint8_t*)take(d.tiles);
     w.max_spl = std::min(nseg, d.ml);
-    w.spl_tab = (uint64_t*)take(w.max_spl * kRadix * 8);
+    w.spl_tab = (uint32_t*)take(w.max_spl * kRadix * 4);
     w.spl_mode = (uint8_t*)take(w.max_spl);
     w.vor = (unsigned long long*)take(d.ml * 8);
     w.vand = (unsigned long long*)take(d.ml * 8);
@@ -701,15 +701,13 @@ __device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t
                  "l"(gsrc), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
 }
-// In-place ascending sort of base[SI(a + i)], i in [0, m), by the whole CTA
-// (SI: the caller's index map): a bitonic network over
+// In-place ascending sort of s[0..m) by the whole CTA: a bitonic network over
 // the next power of two P >= m in the form whose comparators all put the
 // smaller key at the lower index (the first step of every merge compares
 // mirrored positions), so that positions past m act as +infinity and are
 // never touched.  Ends with a barrier.
-template <int THREADS, typename Index>
-__device__ __forceinline__ void cta_bitonic_sort(uint64_t* base, uint32_t a, uint32_t m, Index SI) {
-    auto s = [&](uint32_t i) -> uint64_t& { return base[SI(a + i)]; };
+template <int THREADS, typename T>
+__device__ __forceinline__ void cta_bitonic_sort(T* s, uint32_t m) {
     uint32_t P = 1;
     while (P < m) P <<= 1;
     for (uint32_t k = 2; k <= P; k <<= 1) {
@@ -725,8 +723,8 @@ __device__ __forceinline__ void cta_bitonic_sort(uint64_t* base, uint32_t a, uin
                     l = i + j;
                 }
                 if (l < m) {
-                    const uint64_t x = s(i), y = s(l);
-                    if (y < x) { s(i) = y; s(l) = x; }
+                    const T x = s[i], y = s[l];
+                    if (y < x) { s[i] = y; s[l] = x; }
                 }
             }
             __syncthreads();
@@ -753,7 +751,7 @@ constexpr int chip_min_blocks() { return THREADS <= 128 ? (PAY ? 6 : 8) : (THREA
 //  * A segment whose keys crowd (a group above kChipRefine keys) counts again
 //    with one group per key: group g's range is cut into as many parts as it
 //    holds keys, so the groups follow the keys' distribution (a piecewise
-//    linear estimate of it), up to three times.
+//    linear estimate of it), up to kChipRefines times.
 //  * The words (group start mod 64 | place in the group | position) are
 //    scattered into group order, and ordered inside the groups by windows of
 //    eight in registers, two instructions per comparator: each window is
@@ -778,7 +776,9 @@ constexpr int chip_min_blocks() { return THREADS <= 128 ? (PAY ? 6 : 8) : (THREA
 // 2^28 uniform keys in buckets of about 1024: 2.28 ms with an insertion sort
 // per thread over 64-bit keys (60 wavefronts, 204 instructions), 1.5 ms here;
 // 2^28 Morton keys with a payload in segments of 2^14, whose groups crowd:
-// 57.9 ms (most of it in the LSD kernel), 6.6 ms.
+// 57.9 ms (most of it in the LSD kernel), 6.6 ms.  Refining by a group's own
+// ranges leaves the LSD kernel nothing of these inputs (packs that span the gap
+// between two clusters used to end there: 1.3 ms per 2^28 pairs).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cp_async4(void* sdst, const void* gsrc) {
     const uint32_t sa = (uint32_t)__cvta_generic_to_shared(sdst);
@@ -856,7 +856,7 @@ __device__ __forceinline__ void sort_8(uint32_t (&k)[8]) {
 
 constexpr uint32_t kChipRefine = 24;    // a larger group: count again on the refined groups
 constexpr uint32_t kChipMaxGroup = 56;  // the largest group the window rounds order (start mod 64 is unambiguous)
-constexpr int kChipRefines = 3;
+constexpr int kChipRefines = 6;
 constexpr uint32_t kChipRounds = (kChipMaxGroup + 2) / 4 + 3;  // rounds that order the largest group, and the one that finds it so
 constexpr int kStartBits = 6;
 
@@ -898,6 +898,7 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
     constexpr int NC = chip_counters<THREADS, CAP, R>();
     constexpr bool SPAY = chip_stage_pay<PAY, CAP>();
     constexpr uint32_t kPosMask = (1u << IDX) - 1u;
+    constexpr int kVote = PAY ? 0 : IDX;  // keys alone: the order of equal keys is free
     constexpr uint32_t kSlotShift = 15, kGroupMask = (1u << kSlotShift) - 1u;
     static_assert(CAP % THREADS == 0 && CAP <= (1 << IDX) && NC + 66 < (1 << kSlotShift) && R % (8 * THREADS) == 0 &&
                       CAP < 16384 + 1,
@@ -1055,14 +1056,16 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
             if (tid == 0) s_cnt[R / 2] = n;  // the end of the last group
             __syncthreads();
             uint32_t mx = scan_pairs_inplace<THREADS, R / 2>(s_cnt, s_warp);
-            // Crowded groups: group d cut into as many parts as it holds keys,
-            // and counted again.  Where that no longer helps, a group above
-            // kChipMaxGroup has to hold one key value (else the segment is
-            // left to the shared-memory kernel); with a payload its keys want
-            // position order, so their position takes the place in the group
-            // for one more count.
-            bool slow = false;
-            if (mx > kChipRefine) {  // uniform
+            // Crowded groups: every group cut into as many parts as it holds
+            // keys, and counted again.  Where that did not bring the largest
+            // group to a quarter, the place of a key in a group above
+            // kChipRefine keys is first taken again from the group's own key
+            // range (or, with a payload, its range of positions where it holds
+            // one key value), so that clusters inside clusters resolve
+            // whatever their widths.
+            bool slow = false, tried_pos = false;
+            uint32_t before = 0;
+            for (int it = 0; mx > kChipRefine; ++it) {  // uniform
                 auto each_key = [&](auto body) {
 #pragma unroll
                     for (int i = 0; i < ITEMS; ++i) {
@@ -1070,46 +1073,83 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
                         if (tid + i * THREADS < n) body(i, (uint32_t)(tid + i * THREADS));
                     }
                 };
-                bool stuck = false, by_pos = false;
-                for (int it = 0;; ++it) {
-                    if (stuck || it >= kChipRefines) {
-                        if (mx <= kChipMaxGroup) break;
-                        if (by_pos) { slow = true; break; }
-                        each_key([&](int i, uint32_t e) {
-                            const uint32_t d = dp[i] & kGroupMask;
-                            s_w[s_start[d] + (dp[i] >> kSlotShift)] = e;
-                        });
-                        __syncthreads();
-                        bool mixed = false;
-                        const uint32_t unit = 0xffffffffu / n;
-                        each_key([&](int i, uint32_t e) {
-                            const uint32_t d = dp[i] & kGroupMask, a = s_start[d];
-                            if (s_start[d + 1] - a > kChipMaxGroup) {
-                                mixed = mixed || key[s_w[a]] != key[e];
-                                if (PAY) fr[i] = e * unit;
-                            }
-                        });
-                        slow = __syncthreads_or(mixed) != 0;
-                        if (slow || !PAY) break;
-                        by_pos = true;
-                    }
-                    each_key([&](int i, uint32_t) {
+                if (it == kChipRefines) {
+                    slow = mx > kChipMaxGroup;
+                    break;
+                }
+                // body(item, position, the group's part of s_w)
+                auto each_crowded = [&](auto body) {
+                    each_key([&](int i, uint32_t e) {
                         const uint32_t d = dp[i] & kGroupMask, a = s_start[d];
-                        const uint64_t prod = (uint64_t)fr[i] * (s_start[d + 1] - a);
-                        dp[i] = a + (uint32_t)(prod >> 32);
-                        fr[i] = (uint32_t)prod;
+                        if (s_start[d + 1] - a > kChipRefine) body(i, e, s_w + a);
+                    });
+                };
+                if (it > 0 && 4u * mx > before) {
+                    // Crowded groups of one key value each are in order (keys
+                    // alone), or the window rounds put them in order.
+                    each_crowded([&](int i, uint32_t e, uint32_t* r) {
+                        if (dp[i] >> kSlotShift == 0u) r[0] = e;
                     });
                     __syncthreads();
-                    for (int d = tid; d < NC / 8; d += THREADS) ((uint4*)s_cnt)[d] = make_uint4(0u, 0u, 0u, 0u);
-                    __syncthreads();
-                    each_key([&](int i, uint32_t) { dp[i] |= take_slot(dp[i]) << kSlotShift; });
-                    if (tid == 0) s_cnt[NC / 2] = n;
-                    __syncthreads();
-                    const uint32_t m2 = scan_pairs_inplace<THREADS, NC / 2>(s_cnt, s_warp);
-                    stuck = m2 >= mx || by_pos;
-                    mx = m2;
-                    if (mx <= kChipRefine) break;
+                    bool open = false;
+                    each_crowded([&](int, uint32_t e, uint32_t* r) { open = open || key[r[0]] != key[e]; });
+                    open = __syncthreads_or(open) != 0;
+                    if (!open && (!PAY || mx <= kChipMaxGroup)) break;
+                    if (!open && !tried_pos) {
+                        // one value per group: by position over the whole segment
+                        const uint32_t unit = 0xffffffffu / n;
+                        tried_pos = true;
+                        each_crowded([&](int i, uint32_t e, uint32_t*) { fr[i] = e * unit; });
+                    } else {
+                        // the group's ranges: high words, low words, positions
+                        each_crowded([&](int i, uint32_t, uint32_t* r) {
+                            if (dp[i] >> kSlotShift == 0u) {
+                                r[0] = r[2] = r[4] = ~0u;
+                                r[1] = r[3] = r[5] = 0u;
+                            }
+                        });
+                        __syncthreads();
+                        each_crowded([&](int, uint32_t e, uint32_t* r) {
+                            const uint32_t h = (uint32_t)(key[e] >> 32) ^ hflip;
+                            atomicMin(r, h);
+                            atomicMax(r + 1, h);
+                        });
+                        __syncthreads();
+                        each_crowded([&](int, uint32_t e, uint32_t* r) {
+                            if (r[0] == r[1]) {
+                                const uint32_t l = (uint32_t)key[e];
+                                atomicMin(r + 2, l);
+                                atomicMax(r + 3, l);
+                                if (PAY) { atomicMin(r + 4, e); atomicMax(r + 5, e); }
+                            }
+                        });
+                        __syncthreads();
+                        each_crowded([&](int i, uint32_t e, uint32_t* r) {
+                            const uint64_t kk = key[e];
+                            if (r[0] != r[1])
+                                fr[i] = __funnelshift_l((uint32_t)kk, ((uint32_t)(kk >> 32) ^ hflip) - r[0],
+                                                        __clz((int)(r[1] - r[0])));
+                            else if (r[2] != r[3])
+                                fr[i] = ((uint32_t)kk - r[2]) << __clz((int)(r[3] - r[2]));
+                            else if (PAY)
+                                fr[i] = (e - r[4]) << __clz((int)(r[5] - r[4]));
+                        });
+                    }
                 }
+                before = mx;
+                each_key([&](int i, uint32_t) {
+                    const uint32_t d = dp[i] & kGroupMask, a = s_start[d];
+                    const uint64_t prod = (uint64_t)fr[i] * (s_start[d + 1] - a);
+                    dp[i] = a + (uint32_t)(prod >> 32);
+                    fr[i] = (uint32_t)prod;
+                });
+                __syncthreads();
+                for (int d = tid; d < NC / 8; d += THREADS) ((uint4*)s_cnt)[d] = make_uint4(0u, 0u, 0u, 0u);
+                __syncthreads();
+                each_key([&](int i, uint32_t) { dp[i] |= take_slot(dp[i]) << kSlotShift; });
+                if (tid == 0) s_cnt[NC / 2] = n;
+                __syncthreads();
+                mx = scan_pairs_inplace<THREADS, NC / 2>(s_cnt, s_warp);
             }
             if (slow) {  // uniform: left to the shared-memory kernel
                 if (tid == 0) slow_list[atomicAdd(slow_count, 1u)] = (uint32_t)(list ? (uint64_t)list[k] : k);
@@ -1186,7 +1226,7 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
                                 q[v][i] = q[v][4 + i] - kStep;
                                 q[v][4 + i] = last ? ~0u : o[i] + kStep;
                             }
-                            moved = moved || (b < W && q[v][4] < q[v][3]);
+                            moved = moved || (b < W && q[v][4] >> kVote < q[v][3] >> kVote);
                             merge_4_4(q[v]);
                         }
                         return moved;
@@ -1223,7 +1263,7 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
                                         q[v][4 + i] = q[v][i] + kStep;
                                         q[v][i] = b > 0 ? o[i] - kStep : o[i];
                                     }
-                                    moved = moved || (b < W && q[v][4] < q[v][3]);
+                                    moved = moved || (b < W && q[v][4] >> kVote < q[v][3] >> kVote);
                                     merge_4_4(q[v]);
                                 }
                                 if (tid == 0) *(uint4*)s_first = make_uint4(q[0][0], q[0][1], q[0][2], q[0][3]);
@@ -1571,46 +1611,68 @@ constexpr uint32_t kShiftInterp = 0x100u;
 // msd_shift flag: the split's digit is the bucket among 255 sampled splitters.
 constexpr uint32_t kShiftSplit = 0x200u;
 
-// Bucket of key k among the 255 sorted splitters spl[0..254]: the number of
-// splitters <= k (0..255), by eight halvings without branches.  Monotone in
-// the key, so it serves as a digit of the split.
-__device__ __forceinline__ uint32_t splitter_digit(const uint64_t* spl, uint64_t k) {
-    uint32_t i = 0;
+// Bucket of key k among the 255 splitters of its segment: the number of
+// splitters <= x, x the 32 bits of the key from the sample's highest set bit
+// down (saturated above it).  spl[0]: the shift to x; spl[1..255]: the
+// splitters as a search tree in level order (children of i at 2i, 2i + 1), so
+// that the first six of the eight steps meet no bank twice.  Monotone in the
+// key, so it serves as a digit of the split.
+__device__ __forceinline__ uint32_t splitter_digit(const uint32_t* spl, uint64_t k) {
+    const uint64_t y = k >> spl[0];
+    const uint32_t x = (y >> 32) != 0ull ? ~0u : (uint32_t)y;
+    uint32_t i = 1;
 #pragma unroll
-    for (uint32_t step = 128; step > 0; step >>= 1)
-        if (spl[i + step - 1] <= k) i += step;
-    return i;
+    for (int step = 0; step < 8; ++step) i = 2 * i + (spl[i] <= x ? 1u : 0u);
+    return i - 256u;
 }
 
-// Splitters of the first split of a segment with skewed keys (Gaussian
-// clusters, heavy duplicates), where the top varying byte would leave most of
-// the segment in a few buckets and cost another level: one CTA per segment
-// split at this level draws 2048 keys at evenly spaced positions; when the
-// busiest value of the sample's top varying byte holds more than 4x its
-// share (32 of 2048), it sorts the sample and keeps every 8th key as the 255
-// splitters (spl_mode 1), else the byte split stays (spl_mode 0).
+// Splitters of the first split of a segment with clustered keys (Gaussian
+// clusters, Morton codes), whose top varying byte would leave most of it in sub-buckets too
+// large for the chip: one CTA per segment split at this level draws 2048 keys
+// at evenly spaced places (four neighbours each, a sector) and weighs, by the sample, the keys in such
+// sub-buckets of the byte split against those in runs of one value too long
+// for the chip (which no split on splitters divides).  Where a quarter of the
+// keys would be spared a second level, every 8th key of the sorted sample is
+// a splitter (spl_mode 1), else the byte split stays (spl_mode 0).  The
+// search costs each of the two passes over the keys about 0.3 ms per 2^28
+// keys, a second level of keys alone 2.9 ms.  Segments above kSplMax keys
+// take the byte split: 256 sub-buckets of theirs are too large anyway.
 constexpr int kSplSample = 2048;
+constexpr uint64_t kSplMax = 1ull << 19;
+// By default only calls of 4 Mi keys and more, whose segments hold 2^15 keys
+// and more on average, are sampled: below that the sample (11 us, and a
+// sixteenth of a segment's keys) costs more than a uniform input's call can
+// hide, and the 256 byte sub-buckets of a clustered one mostly fit the chip.
+constexpr uint64_t kSplMinKeys = 1ull << 22;
+constexpr uint64_t kSplMinSeg = 1ull << 15;
 __global__ __launch_bounds__(256) void k_seg_sample(const uint64_t* __restrict__ kin, const uint64_t* __restrict__ seg_lo,
                                                     const uint64_t* __restrict__ seg_hi,
                                                     const uint32_t* __restrict__ large_seg,
                                                     const uint32_t* __restrict__ counters, uint64_t flip_in,
-                                                    uint64_t* __restrict__ spl_tab, uint8_t* __restrict__ spl_mode) {
-    __shared__ uint64_t s_k[kSplSample];
+                                                    uint32_t chip_max, uint32_t* __restrict__ spl_tab,
+                                                    uint8_t* __restrict__ spl_mode) {
+    constexpr int kPer = kSplSample / 256;
+    __shared__ uint32_t s_x[kSplSample];
     __shared__ uint32_t s_h[kRadix];
     __shared__ unsigned long long s_or[8], s_and[8];
+    __shared__ uint32_t s_sum[2];
     const uint32_t id = blockIdx.x;
     if (id >= counters[19]) return;  // uniform
     const uint32_t s = large_seg[id];
     const uint64_t lo = seg_lo[s], n = seg_hi[s] - lo;
     const int tid = threadIdx.x;
+    if (tid == 0) spl_mode[id] = 0u;
+    if (n > kSplMax) return;  // uniform
     s_h[tid] = 0;
+    if (tid < 2) s_sum[tid] = 0;
+    uint64_t key[kPer];
     unsigned long long o = 0, an = ~0ull;
-    for (int i = tid; i < kSplSample; i += 256) {
-        const uint64_t pos = (uint64_t)(((unsigned __int128)(2 * i + 1) * n) / (2 * kSplSample));
-        const uint64_t k = kin[lo + pos] ^ flip_in;
-        s_k[i] = k;
-        o |= k;
-        an &= k;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const uint32_t q = (uint32_t)(tid + i * 256);  // runs of four neighbours (n > 4096)
+        key[i] = kin[lo + (uint64_t)(q >> 2) * (n - 3) / (kSplSample / 4) + (q & 3u)] ^ flip_in;
+        o |= key[i];
+        an &= key[i];
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -1619,27 +1681,40 @@ __global__ __launch_bounds__(256) void k_seg_sample(const uint64_t* __restrict__
     }
     if ((tid & 31) == 0) { s_or[tid >> 5] = o; s_and[tid >> 5] = an; }
     __syncthreads();
-    unsigned long long vo = 0, va = ~0ull;
-    for (int i = 0; i < 8; ++i) { vo |= s_or[i]; va &= s_and[i]; }
-    const unsigned long long vary = vo ^ va;
-    if (vary == 0ull) {  // uniform: a single value in the sample
-        if (tid == 0) spl_mode[id] = 0u;
-        return;
-    }
+    o = 0; an = ~0ull;
+    for (int i = 0; i < 8; ++i) { o |= s_or[i]; an &= s_and[i]; }
+    const unsigned long long vary = o ^ an;
+    if (vary == 0ull) return;  // uniform: a single value in the sample
     const int sh = 8 * (int)((uint32_t)(63 - __clzll((long long)vary)) >> 3);
-    for (int i = tid; i < kSplSample; i += 256) atomicAdd(&s_h[(uint32_t)(s_k[i] >> sh) & 255u], 1u);
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) atomicAdd(&s_h[(uint32_t)(key[i] >> sh) & 255u], 1u);
     __syncthreads();
-    const int crowded = __syncthreads_or(s_h[tid] > 4u * (kSplSample / kRadix));
-    if (!crowded) {
-        if (tid == 0) spl_mode[id] = 0u;
-        return;
+    // more sampled keys than this: a sub-bucket above the on-chip size
+    const uint32_t thr = (uint32_t)((uint64_t)kSplSample * chip_max / n);
+    if (s_h[tid] > thr) atomicAdd(&s_sum[0], s_h[tid]);
+    __syncthreads();
+    const uint32_t crowded = s_sum[0];
+    if (crowded < kSplSample / 4) return;  // uniform
+    const int sft = max(0, 32 - __clzll((long long)o));
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) s_x[tid + i * 256] = (uint32_t)(key[i] >> sft);
+    __syncthreads();
+    cta_bitonic_sort<256>(s_x, (uint32_t)kSplSample);
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const uint32_t j = tid + i * 256;
+        if (j + thr < (uint32_t)kSplSample && s_x[j] == s_x[j + thr])  // inside a run longer than thr
+            atomicAdd(&s_sum[1], j == 0 || s_x[j - 1] != s_x[j] ? thr + 1u : 1u);
     }
-    cta_bitonic_sort<256>(s_k, 0u, (uint32_t)kSplSample, [](uint32_t i) { return i; });
-    uint64_t* spl = spl_tab + (uint64_t)id * kRadix;
-    for (int i = tid; i < kRadix - 1; i += 256) spl[i] = s_k[(i + 1) * (kSplSample / kRadix) - 1];
+    __syncthreads();
+    if (crowded < s_sum[1] + kSplSample / 4) return;  // uniform
+    uint32_t* spl = spl_tab + (uint64_t)id * kRadix;
     if (tid == 0) {
-        spl[kRadix - 1] = ~0ull;
+        spl[0] = (uint32_t)sft;
         spl_mode[id] = 1u;
+    } else {
+        const int level = 31 - __clz(tid), j = tid - (1 << level);  // node tid of the search tree
+        spl[tid] = s_x[(((2 * j + 1) << (7 - level))) * (kSplSample / kRadix) - 1];
     }
 }
 
@@ -1672,11 +1747,11 @@ __global__ __launch_bounds__(256) void k_tile_stats(const uint64_t* __restrict__
                                                     const uint64_t* __restrict__ hint_lo, const uint64_t* __restrict__ hint_mult,
                                                     const uint64_t* __restrict__ hint_hi,
                                                     const uint32_t* __restrict__ prev_shift, uint32_t* __restrict__ spec_out,
-                                                    uint64_t flip_in, const uint64_t* __restrict__ spl_tab,
+                                                    uint64_t flip_in, const uint32_t* __restrict__ spl_tab,
                                                     const uint8_t* __restrict__ spl_mode) {
     __shared__ uint32_t s_h[kRadix];
     __shared__ unsigned long long s_or[8], s_and[8];
-    __shared__ uint64_t s_spl[kRadix];
+    __shared__ uint32_t s_spl[kRadix];
     const uint32_t t = blockIdx.x;
     if (t >= tile_start[nseg]) return;  // uniform
     s_h[threadIdx.x] = 0;
@@ -1704,15 +1779,21 @@ __global__ __launch_bounds__(256) void k_tile_stats(const uint64_t* __restrict__
     const uint64_t hm = win ? hint_mult[s] : 0ull;
     const int sh = 8 * spec;
     unsigned long long o = 0, an = ~0ull;
+    auto count = [&](auto digit) {
 #pragma unroll 4
-    for (uint64_t e = a + threadIdx.x; e < b; e += 256) {
-        const uint64_t k = kin[lo + e] ^ flip_in;
-        o |= k;
-        an &= k;
-        const uint32_t d =
-            bysplit ? splitter_digit(s_spl, k) : (win ? split_digit(k, 0, hb, hm) : (uint32_t)(k >> sh) & 255u);
-        atomicAdd(&s_h[d], 1u);
-    }
+        for (uint64_t e = a + threadIdx.x; e < b; e += 256) {
+            const uint64_t k = kin[lo + e] ^ flip_in;
+            o |= k;
+            an &= k;
+            atomicAdd(&s_h[digit(k)], 1u);
+        }
+    };
+    if (SPL && bysplit)
+        count([&](uint64_t k) { return splitter_digit(s_spl, k); });
+    else if (win)
+        count([&](uint64_t k) { return split_digit(k, 0, hb, hm); });
+    else
+        count([&](uint64_t k) { return (uint32_t)(k >> sh) & 255u; });
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         o |= __shfl_xor_sync(0xffffffffu, o, off);
@@ -1928,7 +2009,7 @@ struct SplitArgs {
     const uint32_t* large_id;
     const uint32_t* tile_off;  // [tile][256] destination of the tile's digit-d keys, relative to the segment
     const uint8_t* tile_skew;  // [tile] one digit holds more than an eighth of the tile
-    const uint64_t* spl_tab;   // [large id][256] sampled splitters (segments split with kShiftSplit)
+    const uint32_t* spl_tab;   // [large id][256] sampled splitters (segments split with kShiftSplit)
     const uint32_t* msd_shift;
     const uint64_t* msd_base;
     const uint64_t* msd_mult;
@@ -1963,7 +2044,7 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 2 : 4) void k_split(con
     __shared__ uint64_t s_gbase[kRadix];
     __shared__ uint32_t s_warp[32];
     __shared__ uint64_t s_mn[kRadix], s_mx[kRadix];
-    __shared__ uint64_t s_spl[kRadix];
+    __shared__ uint32_t s_spl[SPL ? kRadix : 1];
     __shared__ uint32_t s_mask[8];
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -1994,12 +2075,13 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 2 : 4) void k_split(con
         if (tid < kRadix) { s_mn[tid] = ~0ull; s_mx[tid] = 0ull; }
         if (tid < 8) s_mask[tid] = A.large_mask[(uint64_t)id * 8 + tid];
     }
-    if (bysplit) {
+    if (SPL && bysplit) {
         if (tid < kRadix) s_spl[tid] = A.spl_tab[(uint64_t)id * kRadix + tid];
         __syncthreads();
     }
     auto dig = [&](uint64_t k) -> uint32_t {
-        return bysplit ? splitter_digit(s_spl, k) : split_digit(k, shift, dbase, dmult);
+        if (SPL && bysplit) return splitter_digit(s_spl, k);
+        return split_digit(k, shift, dbase, dmult);
     };
 
     uint64_t key[kItems];
@@ -2102,12 +2184,18 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 2 : 4) void k_split(con
             }
             return;
         }
+        if (SPL && bysplit) {
+#pragma unroll
+            for (int i = 0; i < kItems; ++i) rank[i] = splitter_digit(s_spl, key[i]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < kItems; ++i) rank[i] = split_digit(key[i], shift, dbase, dmult);
+        }
         if (A.tile_skew[t]) {  // uniform per CTA: see tile_skew_flag
             const uint32_t lt_mask = (1u << lane) - 1u;
 #pragma unroll
             for (int i = 0; i < kItems; ++i) {
-                const uint32_t d =
-                    wbase + i * 32 < count ? dig(key[i]) : (uint32_t)kRadix;
+                const uint32_t d = wbase + i * 32 < count ? rank[i] : (uint32_t)kRadix;
                 const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
                 const uint32_t eq = __ballot_sync(0xffffffffu, d == d0);
                 uint32_t b0 = 0;
@@ -2119,10 +2207,7 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 2 : 4) void k_split(con
         } else {
 #pragma unroll
             for (int i = 0; i < kItems; ++i) {
-                if (wbase + i * 32 < count) {
-                    const uint32_t d = dig(key[i]);
-                    rank[i] = d | (atomicAdd(&s_total[d], 1u) << 8);
-                }
+                if (wbase + i * 32 < count) rank[i] |= atomicAdd(&s_total[rank[i]], 1u) << 8;
             }
         }
         __syncthreads();
@@ -2441,10 +2526,11 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
         const uint32_t* prev_shift = L.depth > 0 ? ws.msd_shift[buf ^ 1] : nullptr;
         // The first split of a level-0 segment may take sampled splitters
         // (skewed keys); later levels and hinted splits keep their digits.
-        const bool bysplit_level = use_splitters && L.depth == 0 && !L.hint_lo && n_large <= ws.max_spl;
+        const bool bysplit_level = L.depth == 0 && !L.hint_lo && n_large <= ws.max_spl &&
+                                   (use_splitters || (keys_large >= kSplMinKeys && keys_large / n_large >= kSplMinSeg));
         if (bysplit_level)
             HSS_LAUNCH(k_seg_sample, n_large, 256, 0, st, L.in, L.seg_lo, L.seg_hi, ws.large_seg, ws.counters, L.flip_in,
-                       ws.spl_tab, ws.spl_mode);
+                       chip_max, ws.spl_tab, ws.spl_mode);
         if (bysplit_level)
             HSS_LAUNCH(k_tile_stats<true>, tiles, 256, 0, st, L.in, L.seg_lo, L.seg_hi, L.nseg, ws.tile_start, ws.tile_seg,
                        ws.large_id, ws.tile_hist, ws.tile_skew, ws.vor, ws.vand, L.hint_lo, L.hint_mult, L.hint_hi,
@@ -2462,8 +2548,7 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
                    ws.vor, ws.vand, L.hint_lo, L.hint_mult, ws.msd_base, ws.msd_mult, ws.msd_shift[buf], ws.spec,
                    ws.direct, ws.sub_lo[buf], ws.sub_hi[buf], ws.tile_off, child_interp ? chip_max : 0xffffffffu,
                    ws.large_mask, ws.any_large, ws.cmin[buf], ws.cmax[buf], chip_max,
-                   // sampled-splitter sub-buckets (about 256 keys, unevenly wide) pack at most 256 keys
-                   std::min(bysplit_level ? std::min(pack_keys, 256u) : pack_keys, chip_max),
+                   std::min(pack_keys, chip_max),
                    bysplit_level ? ws.spl_mode : nullptr);
         // The split pass: level buffers alternate tmp, dst, tmp, ... after src.
         uint64_t* next = (L.depth & 1) ? dst : tmp;

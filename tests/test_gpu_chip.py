@@ -62,3 +62,39 @@ def test_on_chip_sort_edges(kind, payload):
                 assert np.array_equal(out.cpu().numpy(), raw.view(np.int64)[want]), (kind, n, p, shift, key_type)
                 if payload:
                     assert np.array_equal(o[1].cpu().numpy(), pay[want]), (kind, n, p, shift, key_type)
+
+
+@pytest.mark.parametrize("payload", [False, True])
+@pytest.mark.parametrize("kind", ["uniform", "clusters", "orders", "nested", "runs"])
+def test_first_split_of_clustered_segments(kind, payload):
+    """Segments large enough to be sampled, at both ends of the range that
+    takes sampled splitters and ragged in between: clustered keys (split on
+    splitters), keys whose crowding is duplicates (the byte split stays) and
+    uniform ones."""
+    import torch
+
+    from paper_1803_01237_gb300 import hss
+
+    N = (1 << 22) + 3
+    g = np.random.Generator(np.random.Philox(key=[23, sum(map(ord, kind))]))
+    r = g.integers(0, 1 << 63, size=N, dtype=np.uint64) * np.uint64(2) + g.integers(0, 2, size=N, dtype=np.uint64)
+    if kind == "clusters":
+        means = g.integers(0, 1 << 63, size=32, dtype=np.uint64) * np.uint64(2)
+        r = means[g.integers(0, 32, size=N)] + np.rint(g.standard_normal(N) * 2.0**40).astype(np.int64).view(np.uint64)
+    elif kind == "orders":
+        r = r >> g.integers(0, 64, size=N).astype(np.uint64)
+    elif kind == "nested":  # clusters far narrower than a splitter resolves, and one value with a third of the keys
+        r = np.where(g.random(N) < 0.33, np.uint64(77), (r >> np.uint64(44)) + (r % np.uint64(9) << np.uint64(60)))
+    elif kind == "runs":  # long runs of equal keys next to each other in the input
+        r = np.repeat(r[: N // 50 + 1] >> np.uint64(50), 50)[:N]
+    pay = np.arange(N, dtype=np.int32)
+    for p in (8, 9, 127, 128):
+        for key_type in ("u64", "i64"):
+            kv = r.view(np.int64) if key_type == "i64" else r
+            o = hss.local_sort(torch.from_numpy(r.view(np.int64)).cuda(), p, key_type=key_type,
+                               payload=torch.from_numpy(pay).cuda() if payload else None)
+            off = [(s * N) // p for s in range(p + 1)]
+            want = np.concatenate([off[s] + np.argsort(kv[off[s]:off[s + 1]], kind="stable") for s in range(p)])
+            assert np.array_equal((o[0] if payload else o).cpu().numpy(), r.view(np.int64)[want]), (kind, p, key_type)
+            if payload:
+                assert np.array_equal(o[1].cpu().numpy(), pay[want]), (kind, p, key_type)
