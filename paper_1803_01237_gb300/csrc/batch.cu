@@ -125,28 +125,15 @@ __global__ __launch_bounds__(kSampThreads) void kb_sample_mark(
     const uint32_t n_s = (uint32_t)(seg_start(J, s + 1) - seg_start(J, s));
     const uint64_t T = ctl[j].T;
     const bool take_all = ctl[j].take_all != 0;
+    PairDraw pd;
+    pd.init(J.seed, s, round);
     uint32_t cnt = 0;
     for (uint32_t u0 = 0; u0 < nint; u0 += kIntChunk) {
         const uint32_t nu = min((uint32_t)kIntChunk, nint - u0);
         const uint32_t P = load_seg_intervals(s, n_s, S, u0, nu, Lpos + J.lbase, Upos + J.lbase, Lcut + J.ibase,
                                               int_rep + J.ibase, s_a, s_b, s_pre, s_warp);
-        for_each_pair(s_pre, nu, P, [&](uint32_t u, uint32_t f) {
-            const uint32_t a = s_a[u], b = s_b[u];
-            const uint32_t m = (a >> 1) + (f - s_pre[u]);
-            uint64_t w0, w1;
-            sample_words(J.seed, s, round, m, w0, w1);
-            const uint32_t p0 = 2 * m, p1 = 2 * m + 1;
-            if (p0 >= a && p0 < b && (take_all || w0 < T)) {
-                const uint64_t q = base + p0;
-                atomicOr(&bitmap[q >> 5], 1u << (q & 31));
-                ++cnt;
-            }
-            if (p1 >= a && p1 < b && (take_all || w1 < T)) {
-                const uint64_t q = base + p1;
-                atomicOr(&bitmap[q >> 5], 1u << (q & 31));
-                ++cnt;
-            }
-        });
+        auto thr = [&](uint32_t, uint64_t& Tu, bool& all_u) { Tu = T; all_u = take_all; };
+        mark_pairs(pd, s_a, s_b, s_pre, nu, 0u, P, thr, base, bitmap, cnt);
         __syncthreads();
     }
     uint32_t tot;
