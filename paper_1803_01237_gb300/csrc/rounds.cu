@@ -139,11 +139,11 @@ __global__ void k_rounds_init(const uint64_t* __restrict__ seg_off, uint32_t S, 
 // ---------------------------------------------------------------------------
 // schedule THEORY: the next round's threshold comes from the host (T_ovr,
 // all_ovr); EQUAL: per-interval thresholds into int_T / int_all.
-__global__ __launch_bounds__(1024) void k_intervals(uint32_t S, uint64_t N, uint32_t p, uint64_t tol, float oversample,
-                                                    const DCut* __restrict__ Lcut, const DCut* __restrict__ Ucut,
-                                                    uint32_t* __restrict__ res, uint32_t* __restrict__ int_rep,
-                                                    RoundCtl* ctl, uint32_t schedule, uint64_t T_ovr, uint32_t all_ovr,
-                                                    uint64_t* __restrict__ int_T, uint32_t* __restrict__ int_all) {
+__device__ __forceinline__ void intervals_pass(uint32_t S, uint64_t N, uint32_t p, uint64_t tol, float oversample,
+                                               const DCut* Lcut, const DCut* Ucut, uint32_t* __restrict__ res,
+                                               uint32_t* __restrict__ int_rep, RoundCtl* ctl, uint32_t schedule,
+                                               uint64_t T_ovr, uint32_t all_ovr, uint64_t* __restrict__ int_T,
+                                               uint32_t* __restrict__ int_all) {
     IntervalsOut o;
     const bool equal = schedule == HSS_SCHEDULE_EQUAL;
     intervals_body(S, N, p, tol, oversample, Lcut, Ucut, res, int_rep, o, equal ? int_T : nullptr,
@@ -158,9 +158,28 @@ __global__ __launch_bounds__(1024) void k_intervals(uint32_t S, uint64_t N, uint
     }
 }
 
+__global__ __launch_bounds__(1024) void k_intervals(uint32_t S, uint64_t N, uint32_t p, uint64_t tol, float oversample,
+                                                    const DCut* Lcut, const DCut* Ucut, uint32_t* __restrict__ res,
+                                                    uint32_t* __restrict__ int_rep, RoundCtl* ctl, uint32_t schedule,
+                                                    uint64_t T_ovr, uint32_t all_ovr, uint64_t* __restrict__ int_T,
+                                                    uint32_t* __restrict__ int_all) {
+    intervals_pass(S, N, p, tol, oversample, Lcut, Ucut, res, int_rep, ctl, schedule, T_ovr, all_ovr, int_T, int_all);
+}
+
 // ---------------------------------------------------------------------------
 // Sampling.
 // ---------------------------------------------------------------------------
+// Positions in segment s of the cuts that the last histogram moved.
+__device__ __forceinline__ void update_pos_row(uint64_t s, uint32_t S, const int32_t* __restrict__ chgL,
+                                               const int32_t* __restrict__ chgU, const uint32_t* __restrict__ probe_pos,
+                                               uint64_t cap, uint32_t* Lpos, uint32_t* Upos) {
+    for (uint32_t i = threadIdx.x; i < S; i += blockDim.x) {
+        const int32_t cl = chgL[i], cu = chgU[i];
+        if (cl >= 0) Lpos[s * S + i] = probe_pos[s * cap + (uint32_t)cl];
+        if (cu >= 0) Upos[s * S + i] = probe_pos[s * cap + (uint32_t)cu];
+    }
+}
+
 // Round-j Bernoulli marks of segment blockIdx.x (Sec. 4.2.2 step 4, Sec. 6):
 // every key of an unresolved interval draws its Philox word and is kept when
 // the word is below the round's threshold.  gridDim.y CTAs share a segment,
@@ -170,14 +189,18 @@ __global__ __launch_bounds__(1024) void k_intervals(uint32_t S, uint64_t N, uint
 // of the two words alone are drawn, and the rest only where one of them does
 // not exceed the threshold's.  Round 1 over 2^28 keys: 507 -> 296 us.
 __global__ __launch_bounds__(kSampThreads, 4) void k_sample_mark(
-    const uint64_t* __restrict__ seg_off, uint32_t S, const uint32_t* __restrict__ Lpos, const uint32_t* __restrict__ Upos,
-    const DCut* __restrict__ Lcut, const uint32_t* __restrict__ int_rep, const RoundCtl* __restrict__ ctl,
-    uint64_t seed, uint32_t round, uint32_t* __restrict__ bitmap, uint32_t* __restrict__ seg_cnt,
-    const uint64_t* __restrict__ int_T, const uint32_t* __restrict__ int_all) {
+    const uint64_t* __restrict__ seg_off, uint32_t S, uint32_t* Lpos, uint32_t* Upos, const DCut* __restrict__ Lcut,
+    const uint32_t* __restrict__ int_rep, const RoundCtl* __restrict__ ctl, uint64_t seed, uint32_t round, uint32_t* __restrict__ bitmap, uint32_t* __restrict__ seg_cnt,
+    const uint64_t* __restrict__ int_T, const uint32_t* __restrict__ int_all, const int32_t* __restrict__ chgL,
+    const int32_t* __restrict__ chgU, const uint32_t* __restrict__ probe_pos, uint64_t cap) {
     __shared__ uint32_t s_a[kIntChunk], s_b[kIntChunk], s_pre[kIntChunk + 1];
     __shared__ uint32_t s_warp[32];
     const uint32_t s = blockIdx.x;
     const uint64_t base = seg_off[s];
+    if (chgL) {  // the cuts the last histogram moved, in this segment (gridDim.y is 1)
+        update_pos_row(s, S, chgL, chgU, probe_pos, cap, Lpos, Upos);
+        __syncthreads();
+    }
     if (round == 0) {  // device-driven loop: the next round and the seed come from the control record
         round = ctl->round + 1;
         seed = ctl->seed;
@@ -219,38 +242,21 @@ static unsigned mark_chunks(uint64_t N, uint32_t p) {
     return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(8, pairs / 16384));
 }
 
-__global__ __launch_bounds__(1024) void k_count_scan(const uint32_t* __restrict__ seg_cnt, uint32_t p, uint32_t* __restrict__ seg_cnt_off,
-                                                     uint64_t cap, RoundCtl* ctl) {
-    __shared__ uint32_t s_warp[32];
-    uint64_t carry = 0;
-    for (uint32_t base = 0; base < p; base += blockDim.x) {
-        const uint32_t s = base + threadIdx.x;
-        const uint32_t v = s < p ? seg_cnt[s] : 0u;
-        uint32_t tot;
-        const uint32_t incl = block_incl_scan<uint32_t>(v, 0u, AddU32(), s_warp, tot);
-        if (s < p) seg_cnt_off[s] = (uint32_t)(carry + incl - v < 0xffffffffull ? carry + incl - v : 0xffffffffull);
-        carry += tot;
-    }
-    if (threadIdx.x == 0) {
-        seg_cnt_off[p] = (uint32_t)(carry < 0xffffffffull ? carry : 0xffffffffull);
-        ctl->Z = carry;
-        ctl->seg_off_z[0] = 0;
-        ctl->seg_off_z[1] = carry < cap ? carry : cap;
-    }
-}
-
 // Write the kept keys of each segment, in position order, at the segment's
 // offset of the sample buffer.  Kept keys are exactly the set bits of the
 // bitmap inside the segment, so the pass scans the segment's bitmap words and
-// skips empty runs of them.
+// skips empty runs of them.  It leaves the bitmap and the counts zero (two
+// memsets a round otherwise, one of them of N/8 bytes).
 __global__ __launch_bounds__(kSampThreads) void k_sample_write(
-    const uint64_t* __restrict__ skeys, const uint64_t* __restrict__ seg_off, const uint32_t* __restrict__ bitmap,
-    const uint32_t* __restrict__ seg_cnt, const uint32_t* __restrict__ seg_cnt_off, uint64_t cap,
+    const uint64_t* __restrict__ skeys, const uint64_t* __restrict__ seg_off, uint32_t* bitmap, uint32_t* seg_cnt,
+    const uint32_t* __restrict__ seg_cnt_off, uint64_t cap,
     uint64_t* __restrict__ skey, uint32_t* __restrict__ sseg, uint32_t* __restrict__ sspos, uint32_t* __restrict__ siota) {
     __shared__ uint32_t s_warp[32];
     const uint32_t s = blockIdx.x;
     const uint32_t want = seg_cnt[s];
+    __syncthreads();
     if (want == 0) return;
+    if (threadIdx.x == 0) seg_cnt[s] = 0;  // for the next round's marks
     const uint64_t base = seg_off[s], end = seg_off[s + 1];
     const uint64_t w0 = base >> 5, w1 = (end + 31) >> 5;
     uint64_t out = seg_cnt_off[s];
@@ -263,6 +269,12 @@ __global__ __launch_bounds__(kSampThreads) void k_sample_write(
             const uint64_t g0 = wi << 5;
             if (g0 < base) bits &= ~0u << (uint32_t)(base - g0);               // bits of the previous segment
             if (g0 + 32 > end) bits &= (uint32_t)((1ull << (uint32_t)(end - g0)) - 1ull);  // bits of the next
+            // the next round's marks start from an empty bitmap (a word on
+            // the border keeps the neighbour's bits)
+            if (bits) {
+                if (g0 >= base && g0 + 32 <= end) bitmap[wi] = 0u;
+                else atomicAnd(&bitmap[wi], ~bits);
+            }
         }
         if (__syncthreads_count(bits != 0u) == 0) continue;
         const uint32_t c = __popc(bits);
@@ -289,34 +301,55 @@ __global__ __launch_bounds__(kSampThreads) void k_sample_write(
 // ---------------------------------------------------------------------------
 // Probes: gather the sorted sample, find each probe's interval.
 // ---------------------------------------------------------------------------
-__global__ void k_probe_build(uint64_t Z, const uint64_t* __restrict__ skey_sorted, const uint32_t* __restrict__ sperm,
-                              const uint32_t* __restrict__ sseg, const uint32_t* __restrict__ sspos,
-                              const DCut* __restrict__ Ucut, const uint32_t* __restrict__ int_rep, const RoundCtl* __restrict__ ctl,
-                              uint64_t* __restrict__ pkey, int32_t* __restrict__ pseg, uint32_t* __restrict__ pspos,
-                              uint32_t* __restrict__ pint, uint64_t* __restrict__ prank) {
+// The intervals' upper cuts are staged in shared memory where they fit: a
+// search is a chain of loads, two per step from the splitter tables.
+constexpr uint32_t kProbeCuts = 1024;
+__global__ __launch_bounds__(256) void k_probe_build(
+    uint64_t Z, const uint64_t* __restrict__ skey_sorted, const uint32_t* __restrict__ sperm,
+    const uint32_t* __restrict__ sseg, const uint32_t* __restrict__ sspos, const DCut* __restrict__ Ucut,
+    const uint32_t* __restrict__ int_rep, const RoundCtl* __restrict__ ctl, uint64_t* __restrict__ pkey,
+    int32_t* __restrict__ pseg, uint32_t* __restrict__ pspos, uint32_t* __restrict__ pint, uint64_t* __restrict__ prank) {
+    __shared__ DCut s_cut[kProbeCuts];
     const uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (Z == kZFromCtl) Z = ctl->seg_off_z[1];
-    if (k >= Z) return;
-    const uint32_t j = sperm[k];
+    if ((uint64_t)blockIdx.x * blockDim.x >= Z) return;  // uniform
+    const uint32_t nint = ctl->nint;
+    const bool staged = nint <= kProbeCuts;
+    if (staged)
+        for (uint32_t u = threadIdx.x; u < nint; u += blockDim.x) s_cut[u] = Ucut[int_rep[u]];
     DCut c;
-    c.okey = skey_sorted[k]; c.seg = (int32_t)sseg[j]; c.spos = sspos[j]; c.rank = 0; c.kind = kMember; c.pad = 0;
-    pkey[k] = c.okey; pseg[k] = c.seg; pspos[k] = c.spos; prank[k] = 0;
-    uint32_t lo = 0, hi = ctl->nint;  // first interval whose upper cut lies above the probe
+    c.okey = 0; c.seg = 0; c.spos = 0; c.rank = 0; c.kind = kMember; c.pad = 0;
+    if (k < Z) {
+        const uint32_t j = sperm[k];
+        c.okey = skey_sorted[k]; c.seg = (int32_t)sseg[j]; c.spos = sspos[j];
+        pkey[k] = c.okey; pseg[k] = c.seg; pspos[k] = c.spos; prank[k] = 0;
+    }
+    __syncthreads();
+    if (k >= Z) return;
+    uint32_t lo = 0, hi = nint;  // first interval whose upper cut lies above the probe
     while (lo < hi) {
         const uint32_t mid = (lo + hi) >> 1;
-        if (cut_less(c, Ucut[int_rep[mid]])) hi = mid; else lo = mid + 1;
+        if (cut_less(c, staged ? s_cut[mid] : Ucut[int_rep[mid]])) hi = mid; else lo = mid + 1;
     }
     pint[k] = lo;
 }
 
-constexpr int kHistSegPerBlock = 64;
+constexpr int kHistSegPerBlock = 64;  // k_rank_cuts
+
+// Segments each warp of k_histogram walks: eight, or fewer where that would
+// leave the SMs short of warps (a walk is a chain of dependent loads per
+// segment: 1250 probes over 256 segments took 16 us by eights, 7 by ones).
+static uint32_t hist_per_warp(double Z, uint32_t p) {
+    const double warps = std::ceil(Z / 32.0) * (double)p;
+    return (uint32_t)std::max(1.0, std::min(8.0, warps / (64.0 * (double)device_sm_count())));
+}
 
 __global__ __launch_bounds__(256) void k_histogram(
     const uint64_t* __restrict__ skeys, const uint64_t* __restrict__ seg_off, uint32_t p, uint32_t S,
     const uint32_t* __restrict__ Lpos, const uint32_t* __restrict__ Upos, const uint32_t* __restrict__ int_rep,
     const uint64_t* __restrict__ pkey, const int32_t* __restrict__ pseg, const uint32_t* __restrict__ pspos,
     const uint32_t* __restrict__ pint, uint64_t Z, uint64_t* __restrict__ prank, uint32_t* __restrict__ probe_pos,
-    uint64_t cap, uint32_t* __restrict__ err, const RoundCtl* __restrict__ ctl) {
+    uint64_t cap, uint32_t* __restrict__ err, const RoundCtl* __restrict__ ctl, uint32_t per_warp) {
     __shared__ uint64_t s_part[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (Z == kZFromCtl) {  // device-driven loop: this form runs unless the round is staged
@@ -330,8 +363,8 @@ __global__ __launch_bounds__(256) void k_histogram(
     if (valid) { key = pkey[k]; seg = pseg[k]; spos = pspos[k]; rep = int_rep[pint[k]]; }
     uint64_t partial = 0;
 #pragma unroll 2
-    for (int j = 0; j < kHistSegPerBlock / 8; ++j) {
-        const uint32_t s = blockIdx.y * kHistSegPerBlock + j * 8 + w;
+    for (uint32_t j = 0; j < per_warp; ++j) {
+        const uint32_t s = (blockIdx.y * per_warp + j) * 8 + w;
         if (valid && s < p) {
             uint32_t pos;
             if ((int32_t)s == seg) {
@@ -489,20 +522,23 @@ __global__ void k_prop_probes(uint32_t nprop, const uint64_t* __restrict__ okey_
 // Probes of one launch are all input keys (kind kMember, distinct ranks) or
 // all proposed non-member cuts (kind kNonMember), whose ranks may repeat: then
 // the best cut of a rank is the first of its run (the smallest tag).
-__global__ void k_update(uint32_t S, uint64_t N, uint32_t p, const uint64_t* __restrict__ pkey, const int32_t* __restrict__ pseg,
-                         const uint32_t* __restrict__ pspos, const uint64_t* __restrict__ prank, uint64_t Z, int32_t pkind,
-                         DCut* __restrict__ Lcut, DCut* __restrict__ Ucut, int32_t* __restrict__ chgL, int32_t* __restrict__ chgU,
-                         const RoundCtl* __restrict__ ctl) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= S) return;
-    if (Z == kZFromCtl) Z = ctl->seg_off_z[1];
+__device__ __forceinline__ void update_splitter(uint32_t i, uint64_t N, uint32_t p, const uint64_t* __restrict__ pkey,
+                                                const int32_t* __restrict__ pseg, const uint32_t* __restrict__ pspos,
+                                                const uint64_t* __restrict__ prank, uint64_t Z, int32_t pkind, DCut* Lcut,
+                                                DCut* Ucut, int32_t* __restrict__ chgL, int32_t* __restrict__ chgU) {
     const uint64_t t = ideal_rank(i + 1, N, p);
     uint64_t lo = 0, hi = Z;  // first probe with rank > t
     while (lo < hi) { const uint64_t m = (lo + hi) >> 1; if (prank[m] <= t) lo = m + 1; else hi = m; }
     const uint64_t kgt = lo;
-    lo = 0; hi = Z;           // first probe with rank >= t
-    while (lo < hi) { const uint64_t m = (lo + hi) >> 1; if (prank[m] < t) lo = m + 1; else hi = m; }
-    const uint64_t kge = lo;
+    uint64_t kge = kgt;  // first probe with rank >= t
+    if (kgt > 0 && prank[kgt - 1] == t) {
+        kge = kgt - 1;
+        if (pkind != kMember) {
+            lo = 0; hi = kgt - 1;
+            while (lo < hi) { const uint64_t m = (lo + hi) >> 1; if (prank[m] < t) lo = m + 1; else hi = m; }
+            kge = lo;
+        }
+    }
     DCut L = Lcut[i], U = Ucut[i];
     int32_t cl = -1, cu = -1;
     auto probe = [&](uint64_t k) {
@@ -523,15 +559,41 @@ __global__ void k_update(uint32_t S, uint64_t N, uint32_t p, const uint64_t* __r
     Lcut[i] = L; Ucut[i] = U; chgL[i] = cl; chgU[i] = cu;
 }
 
-__global__ void k_update_pos(uint32_t S, const int32_t* __restrict__ chgL, const int32_t* __restrict__ chgU,
-                             const uint32_t* __restrict__ probe_pos, uint64_t cap, uint32_t* __restrict__ Lpos,
-                             uint32_t* __restrict__ Upos) {
-    const uint64_t s = blockIdx.x;
-    const uint32_t i = blockIdx.y * blockDim.x + threadIdx.x;
+__global__ void k_update(uint32_t S, uint64_t N, uint32_t p, const uint64_t* __restrict__ pkey, const int32_t* __restrict__ pseg,
+                         const uint32_t* __restrict__ pspos, const uint64_t* __restrict__ prank, uint64_t Z, int32_t pkind,
+                         DCut* Lcut, DCut* Ucut, int32_t* __restrict__ chgL, int32_t* __restrict__ chgU,
+                         const RoundCtl* __restrict__ ctl) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= S) return;
-    const int32_t cl = chgL[i], cu = chgU[i];
-    if (cl >= 0) Lpos[s * S + i] = probe_pos[s * cap + (uint32_t)cl];
-    if (cu >= 0) Upos[s * S + i] = probe_pos[s * cap + (uint32_t)cu];
+    if (Z == kZFromCtl) Z = ctl->seg_off_z[1];
+    update_splitter(i, N, p, pkey, pseg, pspos, prank, Z, pkind, Lcut, Ucut, chgL, chgU);
+}
+
+// The update and the interval pass in one launch, by one CTA: for up to
+// kFusedSplitters splitters its few searches cost less than another launch.
+constexpr uint32_t kFusedSplitters = 2048;
+constexpr uint64_t kFusedProbes = 16384;  // 128 KB of ranks
+__global__ __launch_bounds__(1024) void k_update_intervals(
+    uint32_t S, uint64_t N, uint32_t p, const uint64_t* __restrict__ pkey, const int32_t* __restrict__ pseg,
+    const uint32_t* __restrict__ pspos, const uint64_t* __restrict__ prank, uint64_t Z, DCut* Lcut, DCut* Ucut,
+    int32_t* __restrict__ chgL, int32_t* __restrict__ chgU, uint64_t tol, float oversample, uint32_t* __restrict__ res,
+    uint32_t* __restrict__ int_rep, RoundCtl* ctl, uint32_t schedule, uint64_t T_ovr, uint32_t all_ovr,
+    uint64_t* __restrict__ int_T, uint32_t* __restrict__ int_all) {
+    extern __shared__ uint64_t s_rank[];  // the probes' ranks: the searches run on chip
+    if (Z == kZFromCtl) Z = ctl->seg_off_z[1];
+    for (uint32_t k = threadIdx.x; k < (uint32_t)Z; k += blockDim.x) s_rank[k] = prank[k];
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < S; i += blockDim.x)
+        update_splitter(i, N, p, pkey, pseg, pspos, s_rank, Z, kMember, Lcut, Ucut, chgL, chgU);
+    __syncthreads();
+    intervals_pass(S, N, p, tol, oversample, Lcut, Ucut, res, int_rep, ctl, schedule, T_ovr, all_ovr, int_T, int_all);
+}
+
+// The positions of proposed cuts (those of a round's probes are taken by the
+// marking pass that follows, see k_sample_mark).
+__global__ void k_update_pos(uint32_t S, const int32_t* __restrict__ chgL, const int32_t* __restrict__ chgU,
+                             const uint32_t* __restrict__ probe_pos, uint64_t cap, uint32_t* Lpos, uint32_t* Upos) {
+    update_pos_row(blockIdx.x, S, chgL, chgU, probe_pos, cap, Lpos, Upos);
 }
 
 // ---------------------------------------------------------------------------
@@ -658,8 +720,8 @@ __global__ void k_ctl_record(RoundCtl* ctl, uint32_t rounds, int32_t status, uin
     }
 }
 
-__global__ void k_round_decide(RoundCtl* ctl, uint64_t cap, uint64_t N, uint32_t p, uint32_t hist_mode,
-                               cudaGraphConditionalHandle loop) {
+__device__ void round_decide(RoundCtl* ctl, uint64_t cap, uint64_t N, uint32_t p, uint32_t hist_mode,
+                             cudaGraphConditionalHandle loop) {
     const uint32_t j = ctl->round;  // rounds done
     ctl->hist_unres[j] = ctl->unresolved;
     uint32_t go = 0;
@@ -684,21 +746,76 @@ __global__ void k_round_decide(RoundCtl* ctl, uint64_t cap, uint64_t N, uint32_t
     cudaGraphSetConditional(loop, go);
 }
 
+__global__ void k_round_decide(RoundCtl* ctl, uint64_t cap, uint64_t N, uint32_t p, uint32_t hist_mode,
+                               cudaGraphConditionalHandle loop) {
+    round_decide(ctl, cap, N, p, hist_mode, loop);
+}
+
+// Offsets of the segments' samples and the round's sample size; in the
+// device-driven loop (DECIDE) also the decision on the next round.
+template <bool DECIDE>
+__global__ __launch_bounds__(1024) void k_count_scan(const uint32_t* __restrict__ seg_cnt, uint32_t p,
+                                                     uint32_t* __restrict__ seg_cnt_off, uint64_t cap, RoundCtl* ctl,
+                                                     uint64_t N, uint32_t hist_mode, cudaGraphConditionalHandle loop) {
+    __shared__ uint32_t s_warp[32];
+    uint64_t carry = 0;
+    for (uint32_t base = 0; base < p; base += blockDim.x) {
+        const uint32_t s = base + threadIdx.x;
+        const uint32_t v = s < p ? seg_cnt[s] : 0u;
+        uint32_t tot;
+        const uint32_t incl = block_incl_scan<uint32_t>(v, 0u, AddU32(), s_warp, tot);
+        if (s < p) seg_cnt_off[s] = (uint32_t)(carry + incl - v < 0xffffffffull ? carry + incl - v : 0xffffffffull);
+        carry += tot;
+    }
+    if (threadIdx.x == 0) {
+        seg_cnt_off[p] = (uint32_t)(carry < 0xffffffffull ? carry : 0xffffffffull);
+        ctl->Z = carry;
+        ctl->seg_off_z[0] = 0;
+        ctl->seg_off_z[1] = carry < cap ? carry : cap;
+        if (DECIDE) round_decide(ctl, cap, N, p, hist_mode, loop);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Host driver of the rounds.
 // ---------------------------------------------------------------------------
 #define HSS_TRY(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return HSS_ERR_CUDA; } while (0)
 
-static void enqueue_sampling(const RoundWs& ws, const uint64_t* d_seg_off, uint64_t N, uint32_t p, uint32_t S,
-                             uint64_t seed, uint32_t round, cudaStream_t st, bool per_interval) {
-    cudaMemsetAsync(ws.bitmap, 0, (N / 32 + 2) * sizeof(uint32_t), st);
-    cudaMemsetAsync(ws.seg_cnt, 0, (size_t)p * sizeof(uint32_t), st);
+// The marks and sample offsets of a round.  Round 1 starts from cleared marks;
+// later ones find them cleared by k_sample_write and take the positions of the
+// cuts that the last histogram moved (moved: there was one).
+static cudaError_t enqueue_sampling(const RoundWs& ws, const uint64_t* d_seg_off, uint64_t N, uint32_t p, uint32_t S,
+                                    uint64_t seed, uint32_t round, cudaStream_t st, bool per_interval, bool moved) {
+    if (round == 1) {
+        cudaError_t e = cudaMemsetAsync(ws.bitmap, 0, (N / 32 + 2) * sizeof(uint32_t), st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(ws.seg_cnt, 0, (size_t)p * sizeof(uint32_t), st);
+        if (e != cudaSuccess) return e;
+    }
     // round 1 samples whole segments: several CTAs share each; later rounds
     // sample narrow intervals, one CTA per segment
     HSS_LAUNCH(k_sample_mark, dim3(p, round == 1 ? mark_chunks(N, p) : 1u), kSampThreads, 0, st, d_seg_off, S, ws.Lpos,
                ws.Upos, ws.Lcut, ws.int_rep, ws.ctl, seed, round, ws.bitmap, ws.seg_cnt,
-               per_interval ? ws.int_T : nullptr, per_interval ? ws.int_all : nullptr);
-    HSS_LAUNCH(k_count_scan, 1, 1024, 0, st, ws.seg_cnt, p, ws.seg_cnt_off, ws.cap, ws.ctl);
+               per_interval ? ws.int_T : nullptr, per_interval ? ws.int_all : nullptr, moved ? ws.chgL : nullptr, ws.chgU,
+               ws.probe_pos, ws.cap);
+    return cudaGetLastError();
+}
+
+// L/U of every splitter from the ranked probes of a round, then the intervals
+// of the next one.
+static void enqueue_update(const RoundWs& ws, uint32_t S, uint64_t N, uint32_t NB, uint64_t Z, uint64_t tol,
+                           float oversample, uint32_t schedule, uint64_t T_ovr, uint32_t all_ovr, cudaStream_t st) {
+    const uint64_t most = Z == kZFromCtl ? ws.cap : Z;
+    if (S <= kFusedSplitters && most <= kFusedProbes &&
+        ensure_func_attrs((const void*)k_update_intervals, (int)(kFusedProbes * 8)) == cudaSuccess) {
+        HSS_LAUNCH(k_update_intervals, 1, 1024, (size_t)most * 8, st, S, N, NB, ws.pkey, ws.pseg, ws.pspos, ws.prank, Z, ws.Lcut, ws.Ucut,
+                   ws.chgL, ws.chgU, tol, oversample, ws.res, ws.int_rep, ws.ctl, schedule, T_ovr, all_ovr, ws.int_T,
+                   ws.int_all);
+        return;
+    }
+    HSS_LAUNCH(k_update, (unsigned)cdiv(S, 256), 256, 0, st, S, N, NB, ws.pkey, ws.pseg, ws.pspos, ws.prank, Z,
+               (int32_t)kMember, ws.Lcut, ws.Ucut, ws.chgL, ws.chgU, ws.ctl);
+    HSS_LAUNCH(k_intervals, 1, 1024, 0, st, S, N, NB, tol, oversample, ws.Lcut, ws.Ucut, ws.res, ws.int_rep, ws.ctl,
+               schedule, T_ovr, all_ovr, ws.int_T, ws.int_all);
 }
 
 bool device_loop_possible(uint64_t cap, uint32_t schedule) {
@@ -719,7 +836,6 @@ cudaError_t enqueue_device_round(const uint64_t* skeys, const uint64_t* d_seg_of
                                  uint64_t tol, float oversample, uint32_t schedule, uint32_t hist_mode, const RoundWs& ws,
                                  cudaGraphConditionalHandle loop, cudaStream_t st) {
     const uint32_t S = NB - 1;
-    const unsigned sblk = (unsigned)cdiv(S, 256);
     const uint64_t cap = ws.cap;
     const bool per_interval = schedule == HSS_SCHEDULE_EQUAL;
     HSS_LAUNCH(k_sample_write, p, kSampThreads, 0, st, skeys, d_seg_off, ws.bitmap, ws.seg_cnt, ws.seg_cnt_off, cap, ws.skey,
@@ -732,21 +848,13 @@ cudaError_t enqueue_device_round(const uint64_t* skeys, const uint64_t* d_seg_of
     HSS_LAUNCH(k_histogram_staged, dim3((unsigned)cdiv(cap, kStgProbes), (unsigned)cdiv(p, kStgSegs)), kStgThreads, 0, st,
                skeys, d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, kZFromCtl, ws.prank,
                ws.probe_pos, cap, ws.sws.err, ws.ctl);
-    HSS_LAUNCH(k_histogram, dim3((unsigned)cdiv(cap, 32), (unsigned)cdiv(p, kHistSegPerBlock)), 256, 0, st, skeys,
-               d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, ws.pint, kZFromCtl, ws.prank,
-               ws.probe_pos, cap, ws.sws.err, ws.ctl);
-    HSS_LAUNCH(k_update, sblk, 256, 0, st, S, N, NB, ws.pkey, ws.pseg, ws.pspos, ws.prank, kZFromCtl, (int32_t)kMember,
-               ws.Lcut, ws.Ucut, ws.chgL, ws.chgU, ws.ctl);
-    HSS_LAUNCH(k_update_pos, dim3(p, sblk), 256, 0, st, S, ws.chgL, ws.chgU, ws.probe_pos, cap, ws.Lpos, ws.Upos);
-    HSS_LAUNCH(k_intervals, 1, 1024, 0, st, S, N, NB, tol, oversample, ws.Lcut, ws.Ucut, ws.res, ws.int_rep, ws.ctl,
-               schedule, 0ull, 0u, ws.int_T, ws.int_all);
-    if ((e = cudaMemsetAsync(ws.bitmap, 0, (N / 32 + 2) * sizeof(uint32_t), st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(ws.seg_cnt, 0, (size_t)p * sizeof(uint32_t), st)) != cudaSuccess) return e;
-    HSS_LAUNCH(k_sample_mark, dim3(p, 1u), kSampThreads, 0, st, d_seg_off, S, ws.Lpos, ws.Upos, ws.Lcut, ws.int_rep,
-               ws.ctl, 0ull, 0u, ws.bitmap, ws.seg_cnt, per_interval ? ws.int_T : nullptr,
-               per_interval ? ws.int_all : nullptr);
-    HSS_LAUNCH(k_count_scan, 1, 1024, 0, st, ws.seg_cnt, p, ws.seg_cnt_off, cap, ws.ctl);
-    HSS_LAUNCH(k_round_decide, 1, 1, 0, st, ws.ctl, cap, N, p, hist_mode, loop);
+    const uint32_t per_warp = hist_per_warp((double)oversample * (double)NB, p);
+    HSS_LAUNCH(k_histogram, dim3((unsigned)cdiv(cap, 32), (unsigned)cdiv(p, 8 * per_warp)), 256, 0, st, skeys, d_seg_off, p,
+               S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, ws.pint, kZFromCtl, ws.prank, ws.probe_pos, cap,
+               ws.sws.err, ws.ctl, per_warp);
+    enqueue_update(ws, S, N, NB, kZFromCtl, tol, oversample, schedule, 0ull, 0u, st);
+    if ((e = enqueue_sampling(ws, d_seg_off, N, p, S, 0ull, 0u, st, per_interval, true)) != cudaSuccess) return e;
+    HSS_LAUNCH(k_count_scan<true>, 1, 1024, 0, st, ws.seg_cnt, p, ws.seg_cnt_off, cap, ws.ctl, N, hist_mode, loop);
     return cudaGetLastError();
 }
 
@@ -899,9 +1007,9 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
     // The interval pass before sampling round r; under the k-round schedule
     // the host supplies round r's threshold: probability p s_r / N,
     // s_r = (2 ln p / eps)^(min(r,k)/k) (Theorem 4.7), in IEEE double.
-    auto intervals = [&](uint32_t r) {
-        uint64_t Tq = 0;
-        uint32_t allq = 0;
+    auto threshold = [&](uint32_t r, uint64_t& Tq, uint32_t& allq) {
+        Tq = 0;
+        allq = 0;
         if (schedule == HSS_SCHEDULE_THEORY) {
             const uint32_t rr = r < schedule_k ? r : schedule_k;
             const double sj = std::pow(2.0 * std::log((double)NB) / eps, (double)rr / (double)schedule_k);
@@ -909,6 +1017,11 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
             if (q >= 1.0) allq = 1u;
             else Tq = (uint64_t)std::floor(std::ldexp(q, 64));
         }
+    };
+    auto intervals = [&](uint32_t r) {
+        uint64_t Tq;
+        uint32_t allq;
+        threshold(r, Tq, allq);
         HSS_LAUNCH(k_intervals, 1, 1024, 0, st, S, N, NB, tol, oversample, ws.Lcut, ws.Ucut, ws.res, ws.int_rep, ws.ctl,
                    schedule, Tq, allq, ws.int_T, ws.int_all);
     };
@@ -924,9 +1037,10 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
                        st, skeys, d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, Z, ws.prank,
                        ws.probe_pos, ws.cap, ws.sws.err, ws.ctl);
         } else {
-            HSS_LAUNCH(k_histogram, dim3((unsigned)cdiv(Z, 32), (unsigned)cdiv(p, kHistSegPerBlock)), 256, 0, st, skeys,
+            const uint32_t per_warp = hist_per_warp((double)Z, p);
+            HSS_LAUNCH(k_histogram, dim3((unsigned)cdiv(Z, 32), (unsigned)cdiv(p, 8 * per_warp)), 256, 0, st, skeys,
                        d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, ws.pint, Z, ws.prank,
-                       ws.probe_pos, ws.cap, ws.sws.err, ws.ctl);
+                       ws.probe_pos, ws.cap, ws.sws.err, ws.ctl, per_warp);
         }
         return cudaGetLastError();
     };
@@ -954,9 +1068,13 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
         HSS_TRY(histogram((uint64_t)nprop, 1u));
         HSS_LAUNCH(k_update, sblk, 256, 0, st, S, N, NB, ws.pkey, ws.pseg, ws.pspos, ws.prank, (uint64_t)nprop,
                    (int32_t)kNonMember, ws.Lcut, ws.Ucut, ws.chgL, ws.chgU, ws.ctl);
-        HSS_LAUNCH(k_update_pos, dim3(p, sblk), 256, 0, st, S, ws.chgL, ws.chgU, ws.probe_pos, ws.cap, ws.Lpos, ws.Upos);
+        HSS_LAUNCH(k_update_pos, p, 256, 0, st, S, ws.chgL, ws.chgU, ws.probe_pos, ws.cap, ws.Lpos, ws.Upos);
         intervals(1);
     }
+    auto count_scan = [&]() {
+        HSS_LAUNCH(k_count_scan<false>, 1, 1024, 0, st, ws.seg_cnt, p, ws.seg_cnt_off, ws.cap, ws.ctl, N, hist_mode,
+                   cudaGraphConditionalHandle{});
+    };
     cudaGraphExec_t exec = nullptr;
     if (loop_mode != kLoopHost && device_loop_possible(ws.cap, schedule)) {
         // Sampling of round 1 on the stream, then the loop's graph: no host
@@ -970,7 +1088,8 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
     }
     if (exec) {
         HSS_LAUNCH(k_ctl_init, 1, 1, 0, st, ws.ctl, seed, max_rounds);
-        enqueue_sampling(ws, d_seg_off, N, p, S, seed, 1, st, per_interval);
+        HSS_TRY(enqueue_sampling(ws, d_seg_off, N, p, S, seed, 1, st, per_interval, false));
+        count_scan();
         HSS_TRY(cudaGetLastError());
         HSS_TRY(cudaGraphLaunch(exec, st));
         HSS_LAUNCH(k_finalize, (unsigned)cdiv(S, 256), 256, 0, st, S, N, NB, key_type, ws.Lcut, ws.Ucut, d_splitters,
@@ -980,7 +1099,8 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
         if (used_device_loop) *used_device_loop = true;
         return HSS_OK;
     }
-    enqueue_sampling(ws, d_seg_off, N, p, S, seed, 1, st, per_interval);
+    HSS_TRY(enqueue_sampling(ws, d_seg_off, N, p, S, seed, 1, st, per_interval, false));
+    count_scan();
     HSS_TRY(cudaGetLastError());
     RoundCtl h;
     HSS_TRY(read_small(&h, ws.ctl, sizeof(h), st));
@@ -1003,12 +1123,15 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
             HSS_LAUNCH(k_probe_build, (unsigned)cdiv(Z, 256), 256, 0, st, Z, ws.skey_sorted, ws.sperm, ws.sseg, ws.sspos,
                        ws.Ucut, ws.int_rep, ws.ctl, ws.pkey, ws.pseg, ws.pspos, ws.pint, ws.prank);
             HSS_TRY(histogram(Z, h.nint));
-            HSS_LAUNCH(k_update, sblk, 256, 0, st, S, N, NB, ws.pkey, ws.pseg, ws.pspos, ws.prank, Z, (int32_t)kMember,
-                       ws.Lcut, ws.Ucut, ws.chgL, ws.chgU, ws.ctl);
-            HSS_LAUNCH(k_update_pos, dim3(p, sblk), 256, 0, st, S, ws.chgL, ws.chgU, ws.probe_pos, ws.cap, ws.Lpos, ws.Upos);
+            uint64_t Tq;
+            uint32_t allq;
+            threshold(j + 1, Tq, allq);
+            enqueue_update(ws, S, N, NB, Z, tol, oversample, schedule, Tq, allq, st);
+        } else {
+            intervals(j + 1);
         }
-        intervals(j + 1);
-        enqueue_sampling(ws, d_seg_off, N, p, S, seed, j + 1, st, per_interval);
+        HSS_TRY(enqueue_sampling(ws, d_seg_off, N, p, S, seed, j + 1, st, per_interval, Z > 0));
+        count_scan();
         HSS_TRY(cudaGetLastError());
         HSS_TRY(read_small(&h, ws.ctl, sizeof(h), st));
         out->unresolved[j] = h.unresolved;

@@ -81,9 +81,8 @@ struct IntervalsOut {
 // With int_T non-null, every distinct interval u also gets the threshold of
 // the equal-per-interval schedule: probability (s p / nint) / its length.
 __device__ __forceinline__ void intervals_body(uint32_t S, uint64_t N, uint32_t p, uint64_t tol, float oversample,
-                                               const DCut* __restrict__ Lcut, const DCut* __restrict__ Ucut,
-                                               uint32_t* __restrict__ res, uint32_t* __restrict__ int_rep,
-                                               IntervalsOut& out, uint64_t* __restrict__ int_T = nullptr,
+                                               const DCut* Lcut, const DCut* Ucut, uint32_t* __restrict__ res,
+                                               uint32_t* int_rep, IntervalsOut& out, uint64_t* __restrict__ int_T = nullptr,
                                                uint32_t* __restrict__ int_all = nullptr) {
     __shared__ uint32_t s_u32[32];
     __shared__ int32_t s_i32[32];
@@ -169,7 +168,7 @@ constexpr int kSampThreads = 256;
 // Fill the interval ranges of segment s for intervals [u0, u0+nu) and the
 // exclusive prefix of their position-pair counts.  Returns the pair total.
 __device__ __forceinline__ uint32_t load_seg_intervals(uint32_t s, uint32_t n_s, uint32_t S, uint32_t u0, uint32_t nu,
-                                       const uint32_t* __restrict__ Lpos, const uint32_t* __restrict__ Upos,
+                                       const uint32_t* Lpos, const uint32_t* Upos,
                                        const DCut* __restrict__ Lcut, const uint32_t* __restrict__ int_rep,
                                        uint32_t* s_a, uint32_t* s_b, uint32_t* s_pre, uint32_t* s_warp) {
     constexpr int kPer = kIntChunk / kSampThreads;

@@ -1531,6 +1531,22 @@ __global__ __launch_bounds__(1024) void k_plan_count(const uint64_t* __restrict_
     if (threadIdx.x == 0) blk_store(blk, blockIdx.x, tot);
 }
 
+// The level's totals into counters (and for the host), its lists' lengths zeroed.
+__device__ __forceinline__ void plan_totals(const PlanV& carry, uint32_t* counters, volatile uint32_t* host_counts) {
+    for (int k = 0; k < 5; ++k) counters[16 + k] = carry.c[k];
+    *(unsigned long long*)(counters + 22) = carry.keys;
+    if (host_counts) {  // the same eight words for the host, in mapped pinned memory
+        for (int k = 0; k < 5; ++k) host_counts[k] = carry.c[k];
+        host_counts[5] = 0;
+        host_counts[6] = (uint32_t)carry.keys;
+        host_counts[7] = (uint32_t)(carry.keys >> 32);
+    }
+    counters[24] = 0;  // fallback list of this level's on-chip sorts
+    counters[26] = 0;  // segments k_chip leaves to the shared-memory kernel, per size class
+    counters[27] = 0;
+    counters[28] = 0;
+}
+
 // Exclusive scan of the chunk totals (one CTA), totals into counters.
 __global__ __launch_bounds__(1024) void k_plan_scan(uint32_t nblk, uint32_t* __restrict__ blk, uint32_t* __restrict__ counters,
                                                     volatile uint32_t* host_counts) {
@@ -1552,50 +1568,73 @@ __global__ __launch_bounds__(1024) void k_plan_scan(uint32_t nblk, uint32_t* __r
         for (int k = 0; k < 5; ++k) carry.c[k] += tot.c[k];
         carry.keys += tot.keys;
     }
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < 5; ++k) counters[16 + k] = carry.c[k];
-        *(unsigned long long*)(counters + 22) = carry.keys;
-        if (host_counts) {  // the same eight words for the host, in mapped pinned memory
-            for (int k = 0; k < 5; ++k) host_counts[k] = carry.c[k];
-            host_counts[5] = 0;
-            host_counts[6] = (uint32_t)carry.keys;
-            host_counts[7] = (uint32_t)(carry.keys >> 32);
-        }
-        counters[24] = 0;  // fallback list of this level's on-chip sorts
-        counters[26] = 0;  // segments k_chip leaves to the shared-memory kernel, per size class
-        counters[27] = 0;
-        counters[28] = 0;
+    if (threadIdx.x == 0) plan_totals(carry, counters, host_counts);
+}
+
+// The entries of segment s, given the totals of the segments before its chunk
+// (off) and its inclusive scan inside the chunk (v).
+struct PlanOut {
+    uint32_t* tile_start;
+    uint32_t* large_id;
+    uint32_t* large_seg;
+    uint32_t* list0;
+    uint32_t* list1;
+    uint32_t* list2;
+    uint32_t* err;
+    uint32_t* tile_seg;
+};
+__device__ __forceinline__ void plan_entries(uint64_t s, const PlanV& item, const PlanV& v, const PlanV& off,
+                                             const PlanOut& P) {
+    P.tile_start[s] = off.c[4] + v.c[4] - item.c[4];
+    P.large_id[s] = 0xffffffffu;
+    if (item.c[0]) P.list0[off.c[0] + v.c[0] - 1] = (uint32_t)s;
+    if (item.c[1]) P.list1[off.c[1] + v.c[1] - 1] = (uint32_t)s;
+    if (item.c[2]) P.list2[off.c[2] + v.c[2] - 1] = (uint32_t)s;
+    if (item.c[3]) {
+        const uint32_t id = off.c[3] + v.c[3] - 1;
+        P.large_id[s] = id;
+        P.large_seg[id] = (uint32_t)s;
+        const uint32_t t0 = off.c[4] + v.c[4] - item.c[4];
+        for (uint32_t u = 0; u < item.c[4]; ++u) P.tile_seg[t0 + u] = (uint32_t)s;
     }
 }
 
 __global__ __launch_bounds__(1024) void k_plan_write(const uint64_t* __restrict__ seg_lo, const uint64_t* __restrict__ seg_hi,
                                                      uint64_t nseg, const uint32_t* __restrict__ blk,
-                                                     const uint32_t* __restrict__ counters, uint32_t* __restrict__ tile_start,
-                                                     uint32_t* __restrict__ large_id, uint32_t* __restrict__ large_seg,
-                                                     uint32_t* __restrict__ list0, uint32_t* __restrict__ list1,
-                                                     uint32_t* __restrict__ list2, uint32_t* __restrict__ err,
-                                                     uint32_t* __restrict__ tile_seg, uint32_t chip_max) {
+                                                     const uint32_t* __restrict__ counters, const PlanOut P,
+                                                     uint32_t chip_max) {
     const uint64_t s = (uint64_t)blockIdx.x * 1024 + threadIdx.x;
     const PlanV item = plan_item(seg_lo, seg_hi, nseg, s, chip_max);
-    if (s < nseg && seg_hi[s] - seg_lo[s] >= kMaxSegKeys) atomicOr(err, kDevErrSize);
+    if (s < nseg && seg_hi[s] - seg_lo[s] >= kMaxSegKeys) atomicOr(P.err, kDevErrSize);
     PlanV v = item, tot;
     plan_scan(v, tot);
-    const PlanV off = blk_load(blk, blockIdx.x);
-    if (s < nseg) {
-        tile_start[s] = off.c[4] + v.c[4] - item.c[4];
-        large_id[s] = 0xffffffffu;
-        if (item.c[0]) list0[off.c[0] + v.c[0] - 1] = (uint32_t)s;
-        if (item.c[1]) list1[off.c[1] + v.c[1] - 1] = (uint32_t)s;
-        if (item.c[2]) list2[off.c[2] + v.c[2] - 1] = (uint32_t)s;
-        if (item.c[3]) {
-            const uint32_t id = off.c[3] + v.c[3] - 1;
-            large_id[s] = id;
-            large_seg[id] = (uint32_t)s;
-            const uint32_t t0 = off.c[4] + v.c[4] - item.c[4];
-            for (uint32_t u = 0; u < item.c[4]; ++u) tile_seg[t0 + u] = (uint32_t)s;
-        }
+    if (s < nseg) plan_entries(s, item, v, blk_load(blk, blockIdx.x), P);
+    if (s == nseg) P.tile_start[nseg] = counters[20];
+}
+
+// The three steps in one launch by one CTA that carries the totals from chunk
+// to chunk: for a few chunks (kPlanOneChunks) that is faster than two more
+// launches (6 us each; about 2 us a chunk).
+constexpr uint32_t kPlanOneChunks = 4;
+__global__ __launch_bounds__(1024) void k_plan_one(const uint64_t* __restrict__ seg_lo, const uint64_t* __restrict__ seg_hi,
+                                                   uint64_t nseg, uint32_t* __restrict__ counters,
+                                                   volatile uint32_t* host_counts, const PlanOut P, uint32_t chip_max) {
+    PlanV carry = {{0, 0, 0, 0, 0}, 0ull};
+    for (uint64_t s0 = 0; s0 < nseg; s0 += 1024) {
+        const uint64_t s = s0 + threadIdx.x;
+        const PlanV item = plan_item(seg_lo, seg_hi, nseg, s, chip_max);
+        if (s < nseg && seg_hi[s] - seg_lo[s] >= kMaxSegKeys) atomicOr(P.err, kDevErrSize);
+        PlanV v = item, tot;
+        plan_scan(v, tot);
+        if (s < nseg) plan_entries(s, item, v, carry, P);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) carry.c[k] += tot.c[k];
+        carry.keys += tot.keys;
     }
-    if (s == nseg) tile_start[nseg] = counters[20];
+    if (threadIdx.x == 0) {
+        P.tile_start[nseg] = carry.c[4];
+        plan_totals(carry, counters, host_counts);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -2398,26 +2437,29 @@ template <bool PAY>
 static cudaError_t chip_class(int c, const Level& L, uint64_t* dst, uint32_t* pdst, const uint32_t* list,
                               const uint32_t* nlist, uint64_t count, uint32_t lo_n, uint32_t hi_n, uint64_t fout,
                               const SegSortWs& ws, cudaStream_t st) {
-    uint32_t* slow = ws.slow_keys[c];
-    uint32_t* slow_n = ws.counters + 26 + c;
+    // one segment without a plan (the probes of a round): what k_chip leaves
+    // goes straight to the LSD kernel, a launch less
+    const bool one = list == nullptr && L.nseg == 1;
+    uint32_t* slow = one ? ws.fb_list : ws.slow_keys[c];
+    uint32_t* slow_n = ws.counters + (one ? 24 : 26 + c);
     cudaError_t e;
     if (c == 0) {
         e = launch_chip<PAY, kC0Threads, kC0Cap, 1024>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
                                                        L.nseg, lo_n, hi_n, L.flip_in, fout, slow, slow_n, ws.err, st);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess || one) return e;
         return launch_small<PAY, kC0Threads, kC0Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, slow, slow_n, count,
                                                      L.nseg, lo_n, hi_n, L.flip_in, fout, ws, st);
     }
     if (c == 1) {
         e = launch_chip<PAY, kC1Threads, kC1Cap, 4096>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
                                                        L.nseg, lo_n, hi_n, L.flip_in, fout, slow, slow_n, ws.err, st);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess || one) return e;
         return launch_small<PAY, kC1Threads, kC1Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, slow, slow_n, count,
                                                      L.nseg, lo_n, hi_n, L.flip_in, fout, ws, st);
     }
     e = launch_chip<PAY, 1024, kSmallCap, 8192>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count, L.nseg,
                                                 lo_n, hi_n, L.flip_in, fout, slow, slow_n, ws.err, st);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || one) return e;
     return launch_small<PAY, kC2Threads, kSmallCap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, slow, slow_n, count, L.nseg,
                                                     lo_n, hi_n, L.flip_in, fout, ws, st);
 }
@@ -2492,10 +2534,14 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
         // (into buckets of about a thousand keys that the small classes sort)
         // rather than sorted by the largest class (tuning.chip_max_keys).
         const uint32_t chip_max = tune_chip_max;
-        HSS_LAUNCH(k_plan_count, nblk, 1024, 0, st, L.seg_lo, L.seg_hi, L.nseg, ws.blk, chip_max);
-        HSS_LAUNCH(k_plan_scan, 1, 1024, 0, st, nblk, ws.blk, ws.counters, mapped_dev);
-        HSS_LAUNCH(k_plan_write, nblk, 1024, 0, st, L.seg_lo, L.seg_hi, L.nseg, ws.blk, ws.counters, ws.tile_start,
-                   ws.large_id, ws.large_seg, ws.list[0], ws.list[1], ws.list[2], ws.err, ws.tile_seg, chip_max);
+        const PlanOut P{ws.tile_start, ws.large_id, ws.large_seg, ws.list[0], ws.list[1], ws.list[2], ws.err, ws.tile_seg};
+        if (nblk <= kPlanOneChunks) {
+            HSS_LAUNCH(k_plan_one, 1, 1024, 0, st, L.seg_lo, L.seg_hi, L.nseg, ws.counters, mapped_dev, P, chip_max);
+        } else {
+            HSS_LAUNCH(k_plan_count, nblk, 1024, 0, st, L.seg_lo, L.seg_hi, L.nseg, ws.blk, chip_max);
+            HSS_LAUNCH(k_plan_scan, 1, 1024, 0, st, nblk, ws.blk, ws.counters, mapped_dev);
+            HSS_LAUNCH(k_plan_write, nblk, 1024, 0, st, L.seg_lo, L.seg_hi, L.nseg, ws.blk, ws.counters, P, chip_max);
+        }
         uint32_t hc[8];
         if (!mapped && (e = cudaMemcpyAsync(hc, ws.counters + 16, sizeof(hc), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
             return e;
