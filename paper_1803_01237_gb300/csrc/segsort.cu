@@ -6,10 +6,7 @@
 //    keys (and payload) are copied from HBM once into shared memory, counted
 //    into groups that follow their distribution, ordered inside the groups as
 //    32-bit words in registers, and written once (16 B of HBM traffic per key).
-//    Three CTA shapes by segment size (128, 256, 1024 threads).  The few
-//    segments it cannot order that way (large groups of distinct keys closer
-//    than its words resolve) go to k_small_msd and from there to a stable LSD
-//    kernel (8-bit digit passes over a 16-bit index permutation).
+//    Three CTA shapes by segment size (128, 256, 1024 threads).
 //  * A larger segment takes one read pass for statistics (digit counts and the
 //    OR/AND of its keys) and one stable scatter on its first-split
 //    digit (its top varying byte, or an interpolation of the key range the
@@ -108,7 +105,7 @@ size_t segsort_ws_bytes(uint64_t N, uint64_t nseg) {
     b += align_up(d.ml * 8 * 4, 256) + align_up(d.ml * 4, 256);       // large_mask, any_large
     b += align_up(d.tiles * kRadix * 4, 256);                         // tile_off
     b += align_up(64 * 4, 256);                                       // counters
-    b += 7 * align_up(d.list * 4, 256);                               // class lists, fallback, slow lists
+    b += 3 * align_up(d.list * 4, 256);                               // class lists
     b += align_up(8 * (d.list / 1024 + 2) * 4, 256);                  // blk
     return b;
 }
@@ -150,8 +147,6 @@ SegSortWs segsort_ws_carve(void* base, uint64_t N, uint64_t nseg, uint32_t* err)
     w.tile_off = (uint32_t*)take(d.tiles * kRadix * 4);
     w.counters = (uint32_t*)take(64 * 4);
     for (int i = 0; i < 3; ++i) w.list[i] = (uint32_t*)take(d.list * 4);
-    w.fb_list = (uint32_t*)take(d.list * 4);
-    for (int i = 0; i < 3; ++i) w.slow_keys[i] = (uint32_t*)take(d.list * 4);
     w.blk = (uint32_t*)take(8 * (d.list / 1024 + 2) * 4);
     w.err = err;
     return w;
@@ -212,455 +207,75 @@ __device__ __forceinline__ void scan256_smem(const uint32_t* in, uint32_t* out, 
 
 // ---------------------------------------------------------------------------
 // Peer mask of an 8-bit digit inside a warp, from eight ballots: the lanes
-// whose digit equals this lane's.  Lanes with valid == false match nobody and
-// are matched by nobody.
+// whose digit equals this lane's.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t warp_peers8(uint32_t d, bool valid) {
-    uint32_t peers = __ballot_sync(0xffffffffu, valid);
+__device__ __forceinline__ uint32_t warp_peers8(uint32_t d) {
+    uint32_t peers = 0xffffffffu;
 #pragma unroll
     for (int b = 0; b < kRadixBits; ++b) {
         const bool bit = (d >> b) & 1u;
         const uint32_t m = __ballot_sync(0xffffffffu, bit);
         peers &= bit ? m : ~m;
     }
-    return valid ? peers : 0u;
+    return peers;
 }
 
 // ---------------------------------------------------------------------------
-// Stable block ranking of 8-bit digits, in three steps:
+// Stable block ranking of 8-bit digits (digit_of(i): the thread's item i), in
+// three steps:
 //   1. counts: every warp counts its digits into its own 256 shared counters
 //      (fire-and-forget shared atomics, no dependency chain);
 //   2. offsets: the counts become absolute bases start[d] + (earlier warps'
-//      counts of d), plus the tile totals;
+//      counts of d);
 //   3. ranks: per item, the lanes holding the same digit (ballot peer mask)
-//      take consecutive slots: the highest such lane adds their number to the
-//      warp's base for that digit and broadcasts the old value.
+//      take consecutive slots from the warp's base for that digit, which the
+//      lowest of them moves on.
 // Items are warp-striped: item i of lane l in warp w is element
 // w*32*ITEMS + i*32 + l, so (w, i, l) order is element order and the ranks are
-// stable.  Shared atomics issued by one warp in program order are applied in
-// that order, which the running bases of step 3 rely on.  `between` runs after
-// step 2.
+// stable.  Every item takes part; empty ones carry the last digit and, being
+// last in element order, rank behind all others, so nothing tests for them
+// (with such tests and an atomic for the base the split of pairs took 6% more).
 // ---------------------------------------------------------------------------
-struct NoOp { __device__ void operator()() const {} };
-
-template <int WARPS, int ITEMS, typename DigitOf, typename Between>
-__device__ __forceinline__ void block_rank(DigitOf digit_of, uint32_t count, uint32_t (&rank)[ITEMS],
-                                           uint32_t* s_cnt /*[WARPS*256]*/, uint32_t* s_total, uint32_t* s_start,
-                                           uint32_t* s_warp, Between between) {
+template <int WARPS, int ITEMS, typename DigitOf>
+__device__ __forceinline__ void block_rank(DigitOf digit_of, uint32_t (&rank)[ITEMS], uint32_t* s_cnt /*[WARPS*256]*/,
+                                           uint32_t* s_total, uint32_t* s_start, uint32_t* s_warp) {
     constexpr int T = WARPS * 32;
+    static_assert(T >= kRadix, "a thread per digit");
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const uint32_t wfirst = (uint32_t)w * 32 * ITEMS;  // element of the warp's first item slot
-    for (int i = tid; i < WARPS * kRadix; i += T) s_cnt[i] = 0;
-    __syncthreads();
     uint32_t* c = s_cnt + w * kRadix;
+    for (int i = lane; i < kRadix; i += 32) c[i] = 0;
+    __syncwarp();
 #pragma unroll
-    for (int i = 0; i < ITEMS; ++i) {
-        if (wfirst + i * 32 >= count) break;  // the rest of this warp's slots are empty
-        const uint32_t d = digit_of(i);
-        if (d < kRadix) atomicAdd(&c[d], 1u);
-    }
+    for (int i = 0; i < ITEMS; ++i) atomicAdd(&c[digit_of(i)], 1u);
     __syncthreads();
-    for (int d = tid; d < kRadix; d += T) {
+    if (tid < kRadix) {
         uint32_t run = 0;
-        for (int ww = 0; ww < WARPS; ++ww) {
-            const uint32_t x = s_cnt[ww * kRadix + d];
-            s_cnt[ww * kRadix + d] = run;
-            run += x;
-        }
-        s_total[d] = run;
+#pragma unroll
+        for (int ww = 0; ww < WARPS; ++ww) run += s_cnt[ww * kRadix + tid];
+        s_total[tid] = run;
     }
     __syncthreads();
     scan256_smem<T>(s_total, s_start, s_warp);
-    for (int d = tid; d < kRadix; d += T) {
-        const uint32_t st = s_start[d];
-        for (int ww = 0; ww < WARPS; ++ww) s_cnt[ww * kRadix + d] += st;
+    if (tid < kRadix) {
+        uint32_t run = s_start[tid];
+#pragma unroll
+        for (int ww = 0; ww < WARPS; ++ww) {
+            const uint32_t x = s_cnt[ww * kRadix + tid];
+            s_cnt[ww * kRadix + tid] = run;
+            run += x;
+        }
     }
     __syncthreads();
-    between();
     const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
-        if (wfirst + i * 32 >= count) break;
         const uint32_t d = digit_of(i);
-        const bool valid = d < kRadix;
-        const uint32_t peers = warp_peers8(d & 255u, valid);
-        const int leader = valid ? 31 - __clz(peers) : lane;
-        uint32_t base = 0;
-        if (valid && lane == leader) base = atomicAdd(&c[d], (uint32_t)__popc(peers));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        rank[i] = base + __popc(peers & lt);
-    }
-}
-
-// ---------------------------------------------------------------------------
-// On-chip sort of segments that k_chip leaves, with min_n < n <= max_n keys
-// (n <= CAP), taken from `list` (compact ids, count at *nlist).  The keys are read once into shared memory.  One counting
-// pass on a 10-bit digit (the segment's key range interpolated onto 1024
-// groups) splits them into groups that come in key order; inside a group the
-// atomics leave an arbitrary order, and each key's final slot is its group's
-// start plus the number of keys of the group below it in (key, input
-// position) order -- a total order, so the result is the stable sort.
-// Groups larger than kTinyGroup are not ranked that way: when every such
-// group holds one key value (heavy duplicates), its members only need input
-// order, which two ordered warp passes over the positions give; a segment
-// with a larger group of distinct keys is left to the stable LSD kernel below
-// (appended to the fallback list).
-// ---------------------------------------------------------------------------
-constexpr int kChipRadix = 1024;  // groups of the on-chip counting pass
-constexpr int kMaxBig = 64;       // groups above kTinyGroup keys that one segment may hold
-constexpr uint32_t kMixedMax = 256;  // a big group of distinct keys up to this size is ranked on chip
-
-// Exclusive scan of NV shared values in place by a CTA of T threads.
-template <int T, int NV>
-__device__ __forceinline__ void scan_smem_inplace(uint32_t* v, uint32_t* s_warp) {
-    constexpr int K = NV / T;
-    static_assert(NV % T == 0, "scan size");
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    uint32_t loc[K];
-    uint32_t sum = 0;
-#pragma unroll
-    for (int k = 0; k < K; ++k) { loc[k] = v[tid * K + k]; sum += loc[k]; }
-    uint32_t x = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) s_warp[w] = x;
-    __syncthreads();
-    uint32_t run = x - sum;
-    for (int i = 0; i < w; ++i) run += s_warp[i];
-#pragma unroll
-    for (int k = 0; k < K; ++k) { v[tid * K + k] = run; run += loc[k]; }
-    __syncthreads();
-}
-
-// Write a sorted segment: keys from shared memory in the order `order`, and
-// the payload gathered from the segment's input payload.  The output may be
-// the input itself (every second level of the recursion sorts its small
-// buckets in place), so every payload value is gathered into registers before
-// the barrier and stored after it, and the on-chip kernels take their key and
-// payload buffers without __restrict__: with it the compiler may move the
-// gathers past the stores.
-template <bool PAY, int THREADS, int CAP>
-__device__ __forceinline__ void write_sorted(uint64_t* kout, uint32_t* pout, const uint32_t* pin, uint64_t base,
-                                             uint32_t n, const uint64_t* s_keys, const uint16_t* order, uint64_t flip_out) {
-    const int tid = threadIdx.x;
-    if (PAY) {
-        constexpr int PER = (CAP + THREADS - 1) / THREADS;
-        uint32_t pv[PER];
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const uint32_t j = tid + i * THREADS;
-            pv[i] = j < n ? pin[base + order[j]] : 0u;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const uint32_t j = tid + i * THREADS;
-            if (j < n) pout[base + j] = pv[i];
-        }
-    }
-    for (uint32_t j = tid; j < n; j += THREADS) kout[base + j] = s_keys[order[j]] ^ flip_out;
-    __syncthreads();
-}
-
-// Groups of the counting pass by size class: about two keys per group for
-// the smallest segments (a smaller scan per segment), 1024 groups above that
-// (clustered keys in larger segments would otherwise crowd one group).
-template <int CAP>
-constexpr int chip_radix() { return CAP <= kC0Cap ? 512 : kChipRadix; }
-
-// The largest class re-splits crowded groups on chip (see k_small_msd).
-template <int CAP>
-constexpr bool chip_resplit() { return CAP > kC1Cap; }
-
-template <int THREADS, int CAP>
-constexpr size_t msd_sort_smem() {
-    return (size_t)CAP * 8 + 3 * (size_t)CAP * 2 + 2 * (chip_radix<CAP>() + 1) * 4 + 32 * 4 + 2 * 32 * 8 +
-           (size_t)(THREADS / 32) * kMaxBig * 4 + kMaxBig * 4 + chip_radix<CAP>() + 64 +
-           (chip_resplit<CAP>() ? (size_t)(chip_radix<CAP>() + 1) * 4 + kMaxBig * 2 : 0);
-}
-
-template <bool PAY, int THREADS, int CAP>
-__global__ __launch_bounds__(THREADS) void k_small_msd(
-    const uint64_t* kin, uint64_t* kout, const uint32_t* pin, uint32_t* pout, const uint64_t* __restrict__ seg_lo,
-    const uint64_t* __restrict__ seg_hi, const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist,
-    uint64_t nseg, uint32_t min_n,
-    uint32_t max_n, uint64_t flip_in, uint64_t flip_out, uint32_t* __restrict__ fb_list, uint32_t* __restrict__ fb_count) {
-    constexpr int WARPS = THREADS / 32;
-    constexpr int R = chip_radix<CAP>();
-    // Mixed big groups are ranked on chip in the two smaller classes (up to
-    // kMixedMax keys).  The largest class, where big groups come from
-    // clustered keys, re-splits each one by a second counting pass that
-    // interpolates the group's own key range; a segment with a sub-group
-    // still above kTinyGroup keys goes to the LSD kernel.
-    constexpr bool kMixed = CAP <= kC1Cap;
-    constexpr bool kResplit = chip_resplit<CAP>();
-    extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t* s_keys = (uint64_t*)smem;                        // CAP u64
-    uint16_t* s_grp = (uint16_t*)(s_keys + CAP);               // CAP u16: positions grouped by digit
-    uint16_t* s_out = s_grp + CAP;                             // CAP u16: positions in sorted order
-    uint16_t* s_dig = s_out + CAP;                             // CAP u16: digit of each position
-    uint32_t* s_start = (uint32_t*)(s_dig + CAP);              // R+1: counts, then group starts
-    uint32_t* s_run = s_start + (R + 1);              // R+1: running write positions
-    uint32_t* s_warp = s_run + (R + 1);               // 32
-    uint64_t* s_red = (uint64_t*)(((uintptr_t)(s_warp + 32) + 7) & ~(uintptr_t)7);  // 2*32
-    uint32_t* s_wcnt = (uint32_t*)(s_red + 64);                 // WARPS*kMaxBig: per-warp counts of the big groups
-    uint32_t* s_misc = s_wcnt + WARPS * kMaxBig;                // [0] big groups, [1] a mixed group above kMixedMax
-    uint32_t* s_mixed = s_misc + 2;                             // kMaxBig: the big group holds distinct keys
-    uint8_t* s_bigid = (uint8_t*)(s_mixed + kMaxBig);           // R: index of a big group, 0xff otherwise
-    uint32_t* s_h2 = (uint32_t*)(s_bigid + R);                  // R+1 (kResplit): sub-group starts
-    uint16_t* s_bigd = (uint16_t*)(s_h2 + R + 1);               // kMaxBig (kResplit): digit of each big group
-
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const uint64_t count = list ? (uint64_t)*nlist : nseg;
-    for (uint64_t k = blockIdx.x; k < count; k += gridDim.x) {
-        const uint64_t s = list ? (uint64_t)list[k] : k;
-        const uint64_t base = seg_lo[s];
-        const uint64_t n64 = seg_hi[s] - base;
-        if (n64 <= min_n || n64 > max_n) continue;  // uniform per CTA
-        const uint32_t n = (uint32_t)n64;
-        uint64_t kmin = ~0ull, kmax = 0;
-        for (uint32_t j = tid; j < n; j += THREADS) {
-            const uint64_t key = kin[base + j] ^ flip_in;
-            s_keys[j] = key;
-            kmin = min(kmin, key);
-            kmax = max(kmax, key);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            kmin = min(kmin, (uint64_t)__shfl_xor_sync(0xffffffffu, kmin, o));
-            kmax = max(kmax, (uint64_t)__shfl_xor_sync(0xffffffffu, kmax, o));
-        }
-        if (lane == 0) { s_red[w] = kmin; s_red[32 + w] = kmax; }
-        for (int d = tid; d < R; d += THREADS) s_start[d] = 0;
-        if (tid == 0) { s_misc[0] = 0; s_misc[1] = 0; }
-        __syncthreads();
-        {
-            uint64_t a = ~0ull, b = 0;
-            for (int i = 0; i < WARPS; ++i) { a = min(a, s_red[i]); b = max(b, s_red[32 + i]); }
-            kmin = a;
-            kmax = b;
-        }
-        if (kmin == kmax) {  // all keys equal: already in order
-            for (uint32_t j = tid; j < n; j += THREADS) {
-                kout[base + j] = s_keys[j] ^ flip_out;
-                if (PAY) pout[base + j] = pin[base + j];
-            }
-            __syncthreads();
-            continue;
-        }
-        // Counting pass on a 10-bit digit: the key range [kmin, kmax]
-        // interpolated onto 0..1023, monotone in the key (a plain offset when
-        // the range is narrower than 1024).  The groups come in key order; the
-        // atomics leave an arbitrary order inside a group, and each key's final
-        // slot is its group's start plus the number of keys of the group below
-        // it in (key, input position) order -- a total order, so the result is
-        // the stable sort.  Any monotone digit gives the same result, so the
-        // multiplier only needs to be about 1023 * 2^64 / range.
-        const uint64_t range = kmax - kmin;
-        const uint64_t mult = interp_mult(range, (uint32_t)R);
-        for (uint32_t e = tid; e < n; e += THREADS) {
-            const uint64_t off = s_keys[e] - kmin;
-            const uint32_t d = mult ? min((uint32_t)__umul64hi(off, mult), (uint32_t)R - 1) : (uint32_t)off;
-            s_dig[e] = (uint16_t)d;
-            atomicAdd(&s_start[d], 1u);
-        }
-        __syncthreads();
-        uint32_t mx = 0;
-        for (int d = tid; d < R; d += THREADS) mx = max(mx, s_start[d]);
-        mx = __reduce_max_sync(0xffffffffu, mx);
-        scan_smem_inplace<THREADS, R>(s_start, s_warp);
-        if (lane == 0) s_warp[w] = mx;
-        for (int d = tid; d < R; d += THREADS) s_run[d] = s_start[d];
-        if (tid == 0) s_start[R] = n;
-        __syncthreads();
-        mx = 0;
-        for (int i = 0; i < WARPS; ++i) mx = max(mx, s_warp[i]);
-        const bool big = mx > (uint32_t)kTinyGroup;  // uniform per CTA
-        if (big) {
-            for (int d = tid; d < R; d += THREADS) {
-                uint8_t id = 0xff;
-                if (s_start[d + 1] - s_start[d] > (uint32_t)kTinyGroup) {
-                    const uint32_t i = atomicAdd(&s_misc[0], 1u);
-                    if (kResplit && i < (uint32_t)kMaxBig) s_bigd[i] = (uint16_t)d;
-                    id = (uint8_t)min(i, 255u);
-                }
-                s_bigid[d] = id;
-            }
-            if (kMixed || kResplit)
-                for (int g = tid; g < kMaxBig; g += THREADS) s_mixed[g] = 0u;
-            __syncthreads();
-            if (s_misc[0] > (uint32_t)kMaxBig) {  // too many big groups: the LSD kernel takes this segment
-                if (tid == 0) fb_list[atomicAdd(fb_count, 1u)] = (uint32_t)s;
-                __syncthreads();
-                continue;
-            }
-        }
-        for (uint32_t e = tid; e < n; e += THREADS) s_grp[atomicAdd(&s_run[s_dig[e]], 1u)] = (uint16_t)e;
-        __syncthreads();
-        for (uint32_t q = tid; q < n; q += THREADS) {
-            const uint16_t x = s_grp[q];
-            const uint64_t kx = s_keys[x];
-            const uint32_t d = s_dig[x];
-            const uint32_t a = s_start[d], b = s_start[d + 1];
-            if (b - a > (uint32_t)kTinyGroup) {  // big group: only check whether it holds one key value
-                if (kx != s_keys[s_grp[a]]) {
-                    if (kResplit) {
-                        s_mixed[s_bigid[d]] = 2u;  // re-split below
-                    } else {
-                        if (kMixed) s_mixed[s_bigid[d]] = 1u;
-                        if (!kMixed || b - a > kMixedMax) s_misc[1] = 1u;
-                    }
-                }
-                continue;
-            }
-            uint32_t r = 0;
-            for (uint32_t g = a; g < b; ++g) {
-                const uint16_t y = s_grp[g];
-                const uint64_t ky = s_keys[y];
-                r += (ky < kx || (ky == kx && y < x)) ? 1u : 0u;
-            }
-            s_out[a + r] = x;
-        }
-        __syncthreads();
-        if (big && kResplit) {
-            // Re-split every big group of distinct keys, one at a time by the
-            // whole CTA: a counting pass on a digit interpolating the group's
-            // own key range (any monotone digit keeps the order), positions
-            // scattered by sub-group into the group's slots of s_out, then
-            // each key ranked inside its sub-group by (key, input position)
-            // into s_grp and copied back to s_out.
-            const uint32_t nbig = s_misc[0];
-            for (uint32_t g = 0; g < nbig; ++g) {
-                if (s_mixed[g] != 2u) continue;  // uniform: read after a barrier
-                const uint32_t dg = s_bigd[g];
-                const uint32_t a = s_start[dg], b = s_start[dg + 1];
-                uint64_t gmin = ~0ull, gmax = 0;
-                for (uint32_t q = a + tid; q < b; q += THREADS) {
-                    const uint64_t kq = s_keys[s_grp[q]];
-                    gmin = min(gmin, kq);
-                    gmax = max(gmax, kq);
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    gmin = min(gmin, (uint64_t)__shfl_xor_sync(0xffffffffu, gmin, o));
-                    gmax = max(gmax, (uint64_t)__shfl_xor_sync(0xffffffffu, gmax, o));
-                }
-                if (lane == 0) { s_red[w] = gmin; s_red[32 + w] = gmax; }
-                for (int i = tid; i < R; i += THREADS) s_h2[i] = 0u;
-                __syncthreads();
-                for (int i = 0; i < WARPS; ++i) { gmin = min(gmin, s_red[i]); gmax = max(gmax, s_red[32 + i]); }
-                const uint64_t r2 = gmax - gmin;
-                const uint64_t m2 = interp_mult(r2, (uint32_t)R);
-                auto dig2 = [&](uint64_t kq) -> uint32_t {
-                    const uint64_t off = kq - gmin;
-                    return m2 ? min((uint32_t)__umul64hi(off, m2), (uint32_t)R - 1) : (uint32_t)off;
-                };
-                for (uint32_t q = a + tid; q < b; q += THREADS) atomicAdd(&s_h2[dig2(s_keys[s_grp[q]])], 1u);
-                __syncthreads();
-                for (int i = tid; i < R; i += THREADS)
-                    if (s_h2[i] > (uint32_t)kTinyGroup) s_misc[1] = 1u;  // still crowded: LSD kernel
-                scan_smem_inplace<THREADS, R>(s_h2, s_warp);        // ends with a barrier
-                if (s_misc[1]) break;                               // uniform
-                for (int i = tid; i < R; i += THREADS) s_run[i] = s_h2[i];
-                if (tid == 0) s_h2[R] = b - a;
-                __syncthreads();
-                for (uint32_t q = a + tid; q < b; q += THREADS) {
-                    const uint16_t x = s_grp[q];
-                    s_out[a + atomicAdd(&s_run[dig2(s_keys[x])], 1u)] = x;
-                }
-                __syncthreads();
-                for (uint32_t q = a + tid; q < b; q += THREADS) {
-                    const uint16_t x = s_out[q];
-                    const uint64_t kx = s_keys[x];
-                    const uint32_t d2 = dig2(kx);
-                    const uint32_t lo2 = a + s_h2[d2], hi2 = a + s_h2[d2 + 1];
-                    uint32_t r = 0;
-                    for (uint32_t q2 = lo2; q2 < hi2; ++q2) {
-                        const uint16_t y = s_out[q2];
-                        const uint64_t ky = s_keys[y];
-                        r += (ky < kx || (ky == kx && y < x)) ? 1u : 0u;
-                    }
-                    s_grp[lo2 + r] = x;
-                }
-                __syncthreads();
-                for (uint32_t q = a + tid; q < b; q += THREADS) s_out[q] = s_grp[q];
-                __syncthreads();
-            }
-        }
-        if (big) {
-            if (s_misc[1]) {  // a large group of distinct keys: the LSD kernel takes this segment
-                if (tid == 0) fb_list[atomicAdd(fb_count, 1u)] = (uint32_t)s;
-                __syncthreads();
-                continue;
-            }
-            // Big groups of distinct keys (at most kMixedMax): the same rank by
-            // (key, input position), quadratic in the group size.
-            for (uint32_t q = tid; kMixed && q < n; q += THREADS) {
-                const uint16_t x = s_grp[q];
-                const uint32_t d = s_dig[x];
-                const uint32_t a = s_start[d], b = s_start[d + 1];
-                if (b - a <= (uint32_t)kTinyGroup || !s_mixed[s_bigid[d]]) continue;
-                const uint64_t kx = s_keys[x];
-                uint32_t r = 0;
-                for (uint32_t g = a; g < b; ++g) {
-                    const uint16_t y = s_grp[g];
-                    const uint64_t ky = s_keys[y];
-                    r += (ky < kx || (ky == kx && y < x)) ? 1u : 0u;
-                }
-                s_out[a + r] = x;
-            }
-            // Members of each big group in input order: warp w walks the
-            // positions [w*C, (w+1)*C) in order; pass A counts the members of
-            // every big group per warp, a scan over the warps turns the counts
-            // into starts, and pass B places each member at its group's start
-            // plus the members before it.
-            const uint32_t nbig = s_misc[0];
-            const uint32_t C = ((n + WARPS - 1) / WARPS + 31) / 32 * 32;
-            const uint32_t lo = min(n, (uint32_t)w * C), hi = min(n, lo + C);
-            const uint32_t lt = (1u << lane) - 1u;
-            uint32_t* wc = s_wcnt + w * kMaxBig;
-            for (uint32_t b = lane; b < nbig; b += 32) wc[b] = 0;
-            __syncwarp();
-            for (uint32_t p0 = lo; p0 < hi; p0 += 32) {
-                const uint32_t e = p0 + lane;
-                uint32_t g = e < hi ? (uint32_t)s_bigid[s_dig[e]] : 0xffu;
-                if ((kMixed || kResplit) && g != 0xffu && s_mixed[g]) g = 0xffu;  // ranked above
-                const bool valid = g != 0xffu;
-                const uint32_t peers = __match_any_sync(0xffffffffu, valid ? g : 0x100u + lane);
-                if (valid && (peers & lt) == 0u) wc[g] += (uint32_t)__popc(peers);
-                __syncwarp();
-            }
-            __syncthreads();
-            for (uint32_t b = tid; b < nbig; b += THREADS) {
-                uint32_t run = 0;
-                for (int v = 0; v < WARPS; ++v) {
-                    const uint32_t c = s_wcnt[v * kMaxBig + b];
-                    s_wcnt[v * kMaxBig + b] = run;
-                    run += c;
-                }
-            }
-            __syncthreads();
-            for (uint32_t p0 = lo; p0 < hi; p0 += 32) {
-                const uint32_t e = p0 + lane;
-                const uint32_t d = e < hi ? (uint32_t)s_dig[e] : 0u;
-                uint32_t g = e < hi ? (uint32_t)s_bigid[d] : 0xffu;
-                if ((kMixed || kResplit) && g != 0xffu && s_mixed[g]) g = 0xffu;  // ranked above
-                const bool valid = g != 0xffu;
-                const uint32_t peers = __match_any_sync(0xffffffffu, valid ? g : 0x100u + lane);
-                const uint32_t before = valid ? wc[g] : 0u;
-                __syncwarp();
-                if (valid) {
-                    s_out[s_start[d] + before + (uint32_t)__popc(peers & lt)] = (uint16_t)e;
-                    if ((peers & lt) == 0u) wc[g] = before + (uint32_t)__popc(peers);
-                }
-                __syncwarp();
-            }
-            __syncthreads();
-        }
-        write_sorted<PAY, THREADS, CAP>(kout, pout, pin, base, n, s_keys, s_out, flip_out);
+        const uint32_t peers = warp_peers8(d);
+        const uint32_t base = c[d], below = __popc(peers & lt);
+        __syncwarp();
+        if (below == 0) c[d] = base + (uint32_t)__popc(peers);
+        __syncwarp();
+        rank[i] = base + below;
     }
 }
 
@@ -738,8 +353,9 @@ template <bool PAY, int THREADS>
 constexpr int chip_min_blocks() { return THREADS <= 128 ? (PAY ? 6 : 8) : (THREADS <= 256 ? 3 : 1); }
 
 // ---------------------------------------------------------------------------
-// On chip, segments of min_n < n <= max_n keys (n <= CAP), with or without a
-// payload: the stable sort by (key, position).
+// On-chip sort of segments with min_n < n <= max_n keys (n <= CAP), with or
+// without a payload, taken from `list` (compact ids, count at *nlist) or, when
+// list is null, from all nseg segments: the stable sort by (key, position).
 //
 // One bulk copy brings the keys (and the payload) into shared memory, where
 // they stay until they are written in order; what is sorted is one 32-bit
@@ -763,9 +379,12 @@ constexpr int chip_min_blocks() { return THREADS <= 128 ? (PAY ? 6 : 8) : (THREA
 //    ones closer than the place resolves) are in position order, which is the
 //    stable order of equal keys; where their keys are found out of order the
 //    run is sorted by (key, position).
-// A segment that still holds a group above kChipMaxGroup words goes to
-// slow_list, unless the group holds a single key value: then nothing is left
-// to order (keys alone), or its positions refine it once more (payload).
+// A group above kChipMaxGroup words that is left holds one key value (keys
+// alone): its order is free.  The refining ends: a count that takes a crowded
+// group's places from its own range leaves no part wider than 2/57 of it, so
+// thirteen of them use up 64 bits (one more order of magnitude covers the
+// positions of a payload's equal keys), and a count without that follows only
+// where the largest group shrank to a quarter, at most seven times.
 //
 // Bound by shared-memory wavefronts and issue slots together (67% and 66% of
 // their peaks; about 34 wavefronts and 146 instructions per key of a warp): the
@@ -856,7 +475,7 @@ __device__ __forceinline__ void sort_8(uint32_t (&k)[8]) {
 
 constexpr uint32_t kChipRefine = 24;    // a larger group: count again on the refined groups
 constexpr uint32_t kChipMaxGroup = 56;  // the largest group the window rounds order (start mod 64 is unambiguous)
-constexpr int kChipRefines = 6;
+constexpr int kChipRefines = 32;  // never reached (see above)
 constexpr uint32_t kChipRounds = (kChipMaxGroup + 2) / 4 + 3;  // rounds that order the largest group, and the one that finds it so
 constexpr int kStartBits = 6;
 
@@ -888,7 +507,7 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
     const uint64_t* kin, uint64_t* kout, const uint32_t* pin, uint32_t* pout, const uint64_t* __restrict__ seg_lo,
     const uint64_t* __restrict__ seg_hi, const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist,
     uint64_t nseg, uint32_t min_n, uint32_t max_n, uint64_t flip_in, uint64_t flip_out,
-    uint32_t* __restrict__ slow_list, uint32_t* __restrict__ slow_count, uint32_t* __restrict__ err) {
+    uint32_t* __restrict__ err) {
     constexpr int ITEMS = CAP / THREADS;
     constexpr int WARPS = THREADS / 32;
     constexpr int WIN = chip_windows<THREADS, CAP>();
@@ -1063,7 +682,7 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
             // range (or, with a payload, its range of positions where it holds
             // one key value), so that clusters inside clusters resolve
             // whatever their widths.
-            bool slow = false, tried_pos = false;
+            bool tried_pos = false;
             uint32_t before = 0;
             for (int it = 0; mx > kChipRefine; ++it) {  // uniform
                 auto each_key = [&](auto body) {
@@ -1074,7 +693,7 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
                     }
                 };
                 if (it == kChipRefines) {
-                    slow = mx > kChipMaxGroup;
+                    if (tid == 0) atomicOr(err, kDevErrBounds);
                     break;
                 }
                 // body(item, position, the group's part of s_w)
@@ -1101,7 +720,8 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
                         tried_pos = true;
                         each_crowded([&](int i, uint32_t e, uint32_t*) { fr[i] = e * unit; });
                     } else {
-                        // the group's ranges: high words, low words, positions
+                        // the group's key range (high words, then the low
+                        // words at its ends) and positions
                         each_crowded([&](int i, uint32_t, uint32_t* r) {
                             if (dp[i] >> kSlotShift == 0u) {
                                 r[0] = r[2] = r[4] = ~0u;
@@ -1116,21 +736,18 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
                         });
                         __syncthreads();
                         each_crowded([&](int, uint32_t e, uint32_t* r) {
-                            if (r[0] == r[1]) {
-                                const uint32_t l = (uint32_t)key[e];
-                                atomicMin(r + 2, l);
-                                atomicMax(r + 3, l);
-                                if (PAY) { atomicMin(r + 4, e); atomicMax(r + 5, e); }
-                            }
+                            const uint64_t kk = key[e];
+                            const uint32_t h = (uint32_t)(kk >> 32) ^ hflip, l = (uint32_t)kk;
+                            if (h == r[0]) atomicMin(r + 2, l);
+                            if (h == r[1]) atomicMax(r + 3, l);
+                            if (PAY && r[0] == r[1]) { atomicMin(r + 4, e); atomicMax(r + 5, e); }
                         });
                         __syncthreads();
                         each_crowded([&](int i, uint32_t e, uint32_t* r) {
-                            const uint64_t kk = key[e];
-                            if (r[0] != r[1])
-                                fr[i] = __funnelshift_l((uint32_t)kk, ((uint32_t)(kk >> 32) ^ hflip) - r[0],
-                                                        __clz((int)(r[1] - r[0])));
-                            else if (r[2] != r[3])
-                                fr[i] = ((uint32_t)kk - r[2]) << __clz((int)(r[3] - r[2]));
+                            const uint64_t lo = (uint64_t)r[0] << 32 | r[2], range = ((uint64_t)r[1] << 32 | r[3]) - lo;
+                            const uint64_t kk = key[e] ^ ((uint64_t)hflip << 32);
+                            if (range != 0ull)
+                                fr[i] = (uint32_t)(((kk - lo) << __clzll((long long)range)) >> 32);
                             else if (PAY)
                                 fr[i] = (e - r[4]) << __clz((int)(r[5] - r[4]));
                         });
@@ -1151,9 +768,7 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
                 __syncthreads();
                 mx = scan_pairs_inplace<THREADS, NC / 2>(s_cnt, s_warp);
             }
-            if (slow) {  // uniform: left to the shared-memory kernel
-                if (tid == 0) slow_list[atomicAdd(slow_count, 1u)] = (uint32_t)(list ? (uint64_t)list[k] : k);
-            } else {
+            {
                 const uint32_t W = (n + 7) / 8;  // windows of eight words
 #pragma unroll
                 for (int i = 0; i < ITEMS; ++i) {
@@ -1356,89 +971,6 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
 }
 
 // ---------------------------------------------------------------------------
-// Stable LSD sort on chip of the segments in the fallback list (at most
-// kSmallCap keys each): 8-bit digit passes over a 16-bit index permutation,
-// skipping digits that are constant over the segment.
-// ---------------------------------------------------------------------------
-template <int THREADS, int ITEMS>
-constexpr size_t lsd_sort_smem() {
-    return (size_t)THREADS * ITEMS * 8 + 2 * (size_t)THREADS * ITEMS * 2 + (size_t)(THREADS / 32) * kRadix * 4 +
-           2 * kRadix * 4 + 32 * 4 + 2 * 32 * 8;
-}
-
-template <bool PAY, int THREADS, int ITEMS>
-__global__ __launch_bounds__(THREADS, 1) void k_small_lsd(
-    const uint64_t* kin, uint64_t* kout, const uint32_t* pin, uint32_t* pout, const uint64_t* __restrict__ seg_lo,
-    const uint64_t* __restrict__ seg_hi, const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist,
-    uint64_t flip_in, uint64_t flip_out) {
-    constexpr int WARPS = THREADS / 32;
-    constexpr int CAP = THREADS * ITEMS;
-    extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t* s_keys = (uint64_t*)smem;                        // CAP u64
-    uint16_t* s_idx0 = (uint16_t*)(s_keys + CAP);              // CAP u16
-    uint16_t* s_idx1 = s_idx0 + CAP;                           // CAP u16
-    uint32_t* s_cnt = (uint32_t*)(s_idx1 + CAP);               // WARPS*256
-    uint32_t* s_total = s_cnt + WARPS * kRadix;                // 256
-    uint32_t* s_start = s_total + kRadix;                      // 256
-    uint32_t* s_warp = s_start + kRadix;                       // 32
-    uint64_t* s_red = (uint64_t*)(s_warp + 32);                // 2*32
-
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const uint64_t count = *nlist;
-    const uint32_t wbase = w * 32 * ITEMS + lane;
-    const uint32_t wfirst = (uint32_t)w * 32 * ITEMS;
-    for (uint64_t k = blockIdx.x; k < count; k += gridDim.x) {
-        const uint64_t s = list[k];
-        const uint64_t base = seg_lo[s];
-        const uint64_t n64 = seg_hi[s] - base;
-        if (n64 == 0 || n64 > (uint64_t)CAP) continue;
-        const uint32_t n = (uint32_t)n64;
-        uint64_t vor = 0, vand = ~0ull;
-        for (uint32_t j = tid; j < n; j += THREADS) {
-            const uint64_t key = kin[base + j] ^ flip_in;
-            s_keys[j] = key;
-            s_idx0[j] = (uint16_t)j;
-            vor |= key;
-            vand &= key;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            vor |= __shfl_xor_sync(0xffffffffu, vor, o);
-            vand &= __shfl_xor_sync(0xffffffffu, vand, o);
-        }
-        if (lane == 0) { s_red[w] = vor; s_red[32 + w] = vand; }
-        __syncthreads();
-        uint64_t vary;
-        {
-            uint64_t a = 0, b = ~0ull;
-            for (int i = 0; i < WARPS; ++i) { a |= s_red[i]; b &= s_red[32 + i]; }
-            vary = a ^ b;
-        }
-        uint16_t* cur = s_idx0;
-        uint16_t* nxt = s_idx1;
-        for (int pass = 0; pass < 8; ++pass) {
-            const int shift = 8 * pass;
-            if (((vary >> shift) & 255u) == 0u) continue;  // digit constant: identity pass
-            uint32_t idx[ITEMS], rank[ITEMS];
-#pragma unroll
-            for (int i = 0; i < ITEMS; ++i) idx[i] = (wbase + i * 32 < n) ? cur[wbase + i * 32] : 0u;
-            auto digit_of = [&](int i) -> uint32_t {
-                return (wbase + i * 32 < n) ? ((uint32_t)(s_keys[idx[i]] >> shift) & 255u) : (uint32_t)kRadix;
-            };
-            block_rank<WARPS, ITEMS>(digit_of, n, rank, s_cnt, s_total, s_start, s_warp, NoOp());
-#pragma unroll
-            for (int i = 0; i < ITEMS; ++i) {
-                if (wfirst + i * 32 >= n) break;
-                if (wbase + i * 32 < n && rank[i] < n) nxt[rank[i]] = (uint16_t)idx[i];
-            }
-            __syncthreads();
-            uint16_t* t = cur; cur = nxt; nxt = t;
-        }
-        write_sorted<PAY, THREADS, CAP>(kout, pout, pin, base, n, s_keys, cur, flip_out);
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Planning of one level, as a three-step scan over chunks of 1024 segments:
 // compact lists of the segments of each on-chip size class, compact ids and
 // tiles of the segments above the on-chip capacity.
@@ -1531,7 +1063,7 @@ __global__ __launch_bounds__(1024) void k_plan_count(const uint64_t* __restrict_
     if (threadIdx.x == 0) blk_store(blk, blockIdx.x, tot);
 }
 
-// The level's totals into counters (and for the host), its lists' lengths zeroed.
+// The level's totals into counters (and for the host).
 __device__ __forceinline__ void plan_totals(const PlanV& carry, uint32_t* counters, volatile uint32_t* host_counts) {
     for (int k = 0; k < 5; ++k) counters[16 + k] = carry.c[k];
     *(unsigned long long*)(counters + 22) = carry.keys;
@@ -1541,10 +1073,6 @@ __device__ __forceinline__ void plan_totals(const PlanV& carry, uint32_t* counte
         host_counts[6] = (uint32_t)carry.keys;
         host_counts[7] = (uint32_t)(carry.keys >> 32);
     }
-    counters[24] = 0;  // fallback list of this level's on-chip sorts
-    counters[26] = 0;  // segments k_chip leaves to the shared-memory kernel, per size class
-    counters[27] = 0;
-    counters[28] = 0;
 }
 
 // Exclusive scan of the chunk totals (one CTA), totals into counters.
@@ -2139,17 +1667,15 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 2 : 4) void k_split(con
         }
     }
     if constexpr (PAY) {
-        // Each key's digit once, byte-packed in four registers.
+        // Each key's digit once, byte-packed (past the segment the last one).
         uint32_t dpk[kItems / 4];
 #pragma unroll
         for (int i = 0; i < kItems / 4; ++i) dpk[i] = 0;
 #pragma unroll
         for (int i = 0; i < kItems; ++i)
-            dpk[i >> 2] |= dig(key[i]) << (8 * (i & 3));
-        auto digit_of = [&](int i) -> uint32_t {
-            return (wbase + i * 32 < count) ? (dpk[i >> 2] >> (8 * (i & 3))) & 255u : (uint32_t)kRadix;
-        };
-        block_rank<kWarps, kItems>(digit_of, count, rank, s_hist, s_total, s_start, s_warp, NoOp());
+            dpk[i >> 2] |= (wbase + i * 32 < count ? dig(key[i]) : (uint32_t)kRadix - 1u) << (8 * (i & 3));
+        auto digit_of = [&](int i) -> uint32_t { return (dpk[i >> 2] >> (8 * (i & 3))) & 255u; };
+        block_rank<kWarps, kItems>(digit_of, rank, s_hist, s_total, s_start, s_warp);
         if (A.scatter && !gather) {  // uniform per CTA
             // The stable tile rank less the digit's tile start is the key's
             // place in its digit's run: write it there.
@@ -2159,7 +1685,7 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 2 : 4) void k_split(con
 #pragma unroll
             for (int i = 0; i < kItems; ++i) {
                 if (wbase + i * 32 < count) {
-                    const uint64_t dst = s_gbase[(dpk[i >> 2] >> (8 * (i & 3))) & 255u] + rank[i];
+                    const uint64_t dst = s_gbase[digit_of(i)] + rank[i];
                     if (dst - seg_base >= seg_n) {  // never taken when the digit offsets are consistent
                         atomicOr(A.err, kDevErrBounds);
                         continue;
@@ -2172,11 +1698,9 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 2 : 4) void k_split(con
         }
 #pragma unroll
         for (int i = 0; i < kItems; ++i) {
-            if (wbase + i * 32 < count) {
-                s_keys[rank[i]] = key[i];
-                s_dg[rank[i]] = (uint8_t)((dpk[i >> 2] >> (8 * (i & 3))) & 255u);
-                s_pay[rank[i]] = pay[i];
-            }
+            s_keys[rank[i]] = key[i];
+            s_dg[rank[i]] = (uint8_t)digit_of(i);
+            s_pay[rank[i]] = pay[i];
         }
     } else {
         // Keys alone: equal keys are indistinguishable, so the order of a
@@ -2359,30 +1883,11 @@ cudaError_t fill_even_offsets(uint64_t* d_seg_off, uint64_t N, uint64_t p, cudaS
 // ---------------------------------------------------------------------------
 static int num_sms() { return device_sm_count(); }
 
-template <bool PAY, int THREADS, int CAP>
-static cudaError_t launch_small(const uint64_t* in, uint64_t* out, const uint32_t* pin, uint32_t* pout,
-                                const uint64_t* seg_lo, const uint64_t* seg_hi, const uint32_t* list,
-                                const uint32_t* nlist, uint64_t count, uint64_t nseg, uint32_t min_n, uint32_t max_n,
-                                uint64_t fin, uint64_t fout, const SegSortWs& ws, cudaStream_t st) {
-    constexpr size_t smem = msd_sort_smem<THREADS, CAP>();
-    {
-        const cudaError_t e = ensure_func_attrs((const void*)k_small_msd<PAY, THREADS, CAP>, (int)smem, 100);
-        if (e != cudaSuccess) return e;
-    }
-    const int per_sm = resident_ctas((const void*)k_small_msd<PAY, THREADS, CAP>, THREADS, smem);
-    const uint64_t grid = std::min<uint64_t>(count, (uint64_t)num_sms() * per_sm * 4);
-    if (grid == 0) return cudaSuccess;
-    HSS_LAUNCH((k_small_msd<PAY, THREADS, CAP>), (unsigned)grid, THREADS, smem, st, in, out, pin, pout, seg_lo, seg_hi,
-               list, nlist, nseg, min_n, max_n, fin, fout, ws.fb_list, ws.counters + 24);
-    return cudaGetLastError();
-}
-
 template <bool PAY, int THREADS, int CAP, int R>
 static cudaError_t launch_chip(const uint64_t* in, uint64_t* out, const uint32_t* pin, uint32_t* pout,
                                const uint64_t* seg_lo, const uint64_t* seg_hi, const uint32_t* list,
                                const uint32_t* nlist, uint64_t count, uint64_t nseg, uint32_t min_n, uint32_t max_n,
-                               uint64_t fin, uint64_t fout, uint32_t* slow, uint32_t* slow_count, uint32_t* err,
-                               cudaStream_t st) {
+                               uint64_t fin, uint64_t fout, uint32_t* err, cudaStream_t st) {
     constexpr size_t smem = chip_smem<PAY, THREADS, CAP, R>();
     const void* fn = (const void*)k_chip<PAY, THREADS, CAP, R>;
     {
@@ -2394,27 +1899,7 @@ static cudaError_t launch_chip(const uint64_t* in, uint64_t* out, const uint32_t
     const uint64_t grid = std::min<uint64_t>(count, (uint64_t)num_sms() * per_sm);
     if (grid == 0) return cudaSuccess;
     HSS_LAUNCH((k_chip<PAY, THREADS, CAP, R>), (unsigned)grid, THREADS, smem, st, in, out, pin, pout, seg_lo, seg_hi, list,
-               nlist, nseg, min_n, max_n, fin, fout, slow, slow_count, err);
-    return cudaGetLastError();
-}
-
-// The stable LSD kernel over this level's fallback list (length on the device).
-template <bool PAY>
-// max_entries bounds the list on the host (the segments that could have
-// been appended): a CTA per entry at most, since each launch of this kernel
-// reconfigures the SMs for its large shared-memory tile.
-static cudaError_t launch_fallback(const uint64_t* in, uint64_t* out, const uint32_t* pin, uint32_t* pout,
-                                   const uint64_t* seg_lo, const uint64_t* seg_hi, uint64_t fin, uint64_t fout,
-                                   const SegSortWs& ws, cudaStream_t st, uint64_t max_entries) {
-    constexpr size_t smem = lsd_sort_smem<kC2Threads, kC2Items>();
-    {
-        const cudaError_t e = ensure_func_attrs((const void*)k_small_lsd<PAY, kC2Threads, kC2Items>, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    const uint64_t grid = std::min<uint64_t>((uint64_t)num_sms(), max_entries);
-    if (grid == 0) return cudaSuccess;
-    HSS_LAUNCH((k_small_lsd<PAY, kC2Threads, kC2Items>), (unsigned)grid, kC2Threads, smem, st, in, out, pin, pout,
-               seg_lo, seg_hi, ws.fb_list, ws.counters + 24, fin, fout);
+               nlist, nseg, min_n, max_n, fin, fout, err);
     return cudaGetLastError();
 }
 
@@ -2431,37 +1916,19 @@ struct Level {
     const uint64_t* hint_hi = nullptr;  // largest key of each segment, when known
 };
 
-// The on-chip sort of one size class: its segments, then those it leaves to
-// the shared-memory kernel (whose own leftovers go to the fallback list).
+// The on-chip sort of the segments of one size class.
 template <bool PAY>
 static cudaError_t chip_class(int c, const Level& L, uint64_t* dst, uint32_t* pdst, const uint32_t* list,
                               const uint32_t* nlist, uint64_t count, uint32_t lo_n, uint32_t hi_n, uint64_t fout,
                               const SegSortWs& ws, cudaStream_t st) {
-    // one segment without a plan (the probes of a round): what k_chip leaves
-    // goes straight to the LSD kernel, a launch less
-    const bool one = list == nullptr && L.nseg == 1;
-    uint32_t* slow = one ? ws.fb_list : ws.slow_keys[c];
-    uint32_t* slow_n = ws.counters + (one ? 24 : 26 + c);
-    cudaError_t e;
-    if (c == 0) {
-        e = launch_chip<PAY, kC0Threads, kC0Cap, 1024>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
-                                                       L.nseg, lo_n, hi_n, L.flip_in, fout, slow, slow_n, ws.err, st);
-        if (e != cudaSuccess || one) return e;
-        return launch_small<PAY, kC0Threads, kC0Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, slow, slow_n, count,
-                                                     L.nseg, lo_n, hi_n, L.flip_in, fout, ws, st);
-    }
-    if (c == 1) {
-        e = launch_chip<PAY, kC1Threads, kC1Cap, 4096>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
-                                                       L.nseg, lo_n, hi_n, L.flip_in, fout, slow, slow_n, ws.err, st);
-        if (e != cudaSuccess || one) return e;
-        return launch_small<PAY, kC1Threads, kC1Cap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, slow, slow_n, count,
-                                                     L.nseg, lo_n, hi_n, L.flip_in, fout, ws, st);
-    }
-    e = launch_chip<PAY, 1024, kSmallCap, 8192>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count, L.nseg,
-                                                lo_n, hi_n, L.flip_in, fout, slow, slow_n, ws.err, st);
-    if (e != cudaSuccess || one) return e;
-    return launch_small<PAY, kC2Threads, kSmallCap>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, slow, slow_n, count, L.nseg,
-                                                    lo_n, hi_n, L.flip_in, fout, ws, st);
+    if (c == 0)
+        return launch_chip<PAY, kC0Threads, kC0Cap, 1024>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
+                                                          L.nseg, lo_n, hi_n, L.flip_in, fout, ws.err, st);
+    if (c == 1)
+        return launch_chip<PAY, kC1Threads, kC1Cap, 4096>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
+                                                          L.nseg, lo_n, hi_n, L.flip_in, fout, ws.err, st);
+    return launch_chip<PAY, kC2Threads, kSmallCap, 8192>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
+                                                         L.nseg, lo_n, hi_n, L.flip_in, fout, ws.err, st);
 }
 
 // This thread's mapped pinned buffer for the planning counts (allocated once
@@ -2515,7 +1982,6 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
     if (N <= (uint64_t)kSmallCap) {
         // No segment can exceed the on-chip capacity: sort every segment in
         // its class without planning (and without a host round trip).
-        if ((e = cudaMemsetAsync(ws.counters + 24, 0, 20, st)) != cudaSuccess) return e;
         for (int c = 0; c < 3; ++c) {
             const uint32_t lo_n = c == 0 || nseg == 1 ? 0u : (c == 1 ? (uint32_t)kC0Cap : (uint32_t)kC1Cap);
             const uint32_t hi_n = c == 0 ? (uint32_t)kC0Cap : (c == 1 ? (uint32_t)kC1Cap : (uint32_t)kSmallCap);
@@ -2525,7 +1991,7 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
                 return e;
             if (nseg == 1) break;
         }
-        return launch_fallback<PAY>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, L.flip_in, fout, ws, st, nseg);
+        return cudaSuccess;
     }
     for (;;) {
         if (L.nseg > ws.max_list) return cudaErrorInvalidValue;
@@ -2559,10 +2025,6 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
                 cudaSuccess)
                 return e;
         }
-        if ((hc[0] || hc[1] || hc[2]) &&
-            (e = launch_fallback<PAY>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, L.flip_in, fout, ws, st,
-                                      (uint64_t)hc[0] + hc[1] + hc[2])) != cudaSuccess)
-            return e;
         if (n_large == 0) return cudaSuccess;
         if (n_large > ws.max_large || tiles > ws.max_tiles || L.depth >= kMaxDepth) return cudaErrorInvalidValue;
         // Statistics per tile, the split window and every tile's offsets.

@@ -28,11 +28,10 @@ constexpr int kOsTile = kOsThreads * kOsItems;  // 4096 keys per split tile
 // On-chip sort: three CTA shapes by segment size (threads x items per thread).
 constexpr int kC0Threads = 128, kC0Items = 12;  // up to 1536 keys
 constexpr int kC1Threads = 256, kC1Items = 16;  // up to 4096 keys
-constexpr int kC2Threads = 512, kC2Items = 28;  // up to 14336 keys
+constexpr int kC2Threads = 1024, kC2Items = 14; // up to 14336 keys
 constexpr int kC0Cap = kC0Threads * kC0Items;
 constexpr int kC1Cap = kC1Threads * kC1Items;
 constexpr int kSmallCap = kC2Threads * kC2Items;
-constexpr int kTinyGroup = 64;  // on chip: rank inside the groups of one MSD pass when none is larger
 
 struct SegSortWs {
     uint64_t max_large;    // bound on segments larger than kSmallCap at any depth
@@ -67,8 +66,6 @@ struct SegSortWs {
     uint32_t* tile_off;    // [max_tiles][256] destination of each tile's digit-d keys, relative to its segment
     uint32_t* counters;    // [64]
     uint32_t* list[3];     // [max_list] segments of each on-chip size class
-    uint32_t* fb_list;     // [max_list] segments left to the stable LSD kernel (count in counters[24])
-    uint32_t* slow_keys[3];  // [max_list] per size class: segments k_chip leaves to the shared-memory kernel (counters[26..28])
     uint32_t* blk;         // [8 * (max_list / 1024 + 2)] per-chunk counts of the planning scan
     uint32_t* err;         // device error word (kDevErr*)
     // false: the planning counts come back by a copy into pageable host

@@ -31,11 +31,16 @@ def _keys(kind, n, g):
     if kind == "ends":  # the smallest and largest values of both key types
         return np.array([0, 1, (1 << 63) - 1, 1 << 63, (1 << 64) - 2, (1 << 64) - 1], dtype=np.uint64)[
             g.integers(0, 6, size=n)]
+    if kind == "border":  # small values of both signs: narrow around a border of the high words
+        return (r.view(np.int64) >> g.integers(30, 64, size=n)).view(np.uint64) + (r & np.uint64(1) << np.uint64(32))
+    if kind == "ladder":  # 60 close keys under outliers at every order of magnitude: each count peels off one
+        return np.where(np.arange(n) % 97 < 60, r & np.uint64(0xffff),
+                        np.uint64(1) << (np.uint64(16) + r % np.uint64(48)))
     raise ValueError(kind)
 
 
 @pytest.mark.parametrize("payload", [False, True])
-@pytest.mark.parametrize("kind", ["uniform", "narrow", "clusters", "orders", "close", "few", "pairs", "ends"])
+@pytest.mark.parametrize("kind", ["uniform", "narrow", "clusters", "orders", "close", "few", "pairs", "ends", "ladder", "border"])
 def test_on_chip_sort_edges(kind, payload):
     import torch
 
