@@ -476,7 +476,7 @@ int hss_cdf_grad(const hss_cdf_model* d_model, const void* d_keys, const uint64_
                  float* d_grad, float* d_loss, void* d_work, size_t work_bytes, void* stream);
 
 /* `steps` full-batch Adam steps of learning rate lr on the n points; the loss
- * before the last step into d_loss (nullable).  Two kernels per step. */
+ * before the last step into d_loss (nullable).  One kernel per step. */
 int hss_cdf_train(hss_cdf_model* d_model, const void* d_keys, const uint64_t* d_ranks, uint32_t n, uint64_t N,
                   uint32_t steps, float lr, float* d_loss, void* d_work, size_t work_bytes, void* stream);
 

@@ -27,10 +27,11 @@ namespace {
 constexpr int kH = HSS_CDF_HIDDEN;
 constexpr int kP = HSS_CDF_NPARAM;
 constexpr int kOffB1 = kH, kOffW2 = 2 * kH, kOffB2 = 2 * kH + kH * kH, kOffW3 = kOffB2 + kH, kOffB3 = kOffW3 + kH;
-constexpr int kGradThreads = 256;
+constexpr int kGradThreads = 128;   // a point each; four warps, one per scheduler
 constexpr int kMaxGradBlocks = 32;  // training shares the GPU with the sorts it serves: a few SMs
-constexpr int kPartStride = kP + 3;  // gradient, loss partial, padding
-constexpr int kStage = kH + 1;       // padded row of a staged activation vector
+constexpr int kPartStride = kP + 3;  // gradient, loss partial, padding (a multiple of four floats)
+constexpr int kStage = kH + 4;       // row of a staged activation vector: 16-byte aligned, rows start four banks apart
+constexpr int kRowGroups = kGradThreads / 64;  // 64 threads hold the 4 x 4 tiles of dW2, each group sums a share of the rows
 constexpr uint32_t kInitTag = 0x43444621u;
 constexpr float kBeta1 = 0.9f, kBeta2 = 0.999f, kAdamEps = 1e-8f;
 
@@ -49,8 +50,41 @@ __device__ __forceinline__ float weight_of(const hss_cdf_model* M, int k) {
     return M->weights == HSS_CDF_W_BF16 ? __bfloat162float(__float2bfloat16_rn(w)) : w;
 }
 
-// y(x) with the parameters in shared memory (every thread reads the same
-// weight at the same time: broadcasts).
+// Hidden layers of one point with the parameters in shared memory (every
+// thread reads the same weights at the same time: broadcasts, four at once).
+// Four rows of W2 advance together, so four chains of multiply-adds hide each
+// other's latency.  Returns y(x).
+__device__ __forceinline__ float layers(const float* th, float x, float (&h1)[kH], float (&h2)[kH]) {
+#pragma unroll
+    for (int i = 0; i < kH; ++i) h1[i] = fmaxf(fmaf(th[i], x, th[kOffB1 + i]), 0.f);
+    float y = th[kOffB3];
+#pragma unroll
+    for (int i = 0; i < kH; i += 4) {
+        float a[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) a[r] = th[kOffB2 + i + r];
+#pragma unroll
+        for (int j = 0; j < kH; j += 4) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float4 w = *(const float4*)(th + kOffW2 + (i + r) * kH + j);
+                a[r] = fmaf(w.x, h1[j], a[r]);
+                a[r] = fmaf(w.y, h1[j + 1], a[r]);
+                a[r] = fmaf(w.z, h1[j + 2], a[r]);
+                a[r] = fmaf(w.w, h1[j + 3], a[r]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            h2[i + r] = fmaxf(a[r], 0.f);
+            y = fmaf(th[kOffW3 + i + r], h2[i + r], y);
+        }
+    }
+    return y;
+}
+// y(x) alone, the same operations in the same order, a few rows unrolled: a
+// loop around it (the bisection) would have the compiler keep every weight of
+// `layers` in registers, and spill them.
 __device__ __forceinline__ float net(const float* th, float x) {
     float h1[kH];
 #pragma unroll
@@ -98,153 +132,230 @@ __global__ void k_cdf_init(hss_cdf_model* M, uint64_t seed, int feature, int key
     M->v[k] = 0.f;
 }
 
-// Partial gradient of the mean squared error over a grid-stride share of the
-// n points.  Each thread runs the forward and backward pass of one point;
-// the activations and their gradients are staged in shared memory and every
-// thread then sums its own gradient entries over the 256 staged points, so
-// each CTA writes one deterministic partial.
-__global__ __launch_bounds__(kGradThreads) void k_cdf_grad(const hss_cdf_model* __restrict__ M,
-                                                           const uint64_t* __restrict__ keys,
-                                                           const uint64_t* __restrict__ ranks, uint32_t n, double invN,
-                                                           float inv_n, float* __restrict__ part) {
+// Features and targets of the training points, once per call: the feature map
+// is double precision (log2), which the steps would otherwise repeat.
+__global__ __launch_bounds__(kGradThreads) void k_cdf_points(const hss_cdf_model* __restrict__ M,
+                                                             const uint64_t* __restrict__ keys,
+                                                             const uint64_t* __restrict__ ranks, uint32_t n, double invN,
+                                                             float2* __restrict__ pts, uint32_t* __restrict__ arrived) {
+    const uint32_t b = blockIdx.x * kGradThreads + threadIdx.x;
+    if (b == 0) *arrived = 0u;
+    if (b >= n) return;
+    const uint64_t flip = M->key_type == HSS_KEY_I64 ? kSignBit : 0ull;
+    pts[b] = make_float2(feature_of(keys[b], M, flip), (float)((double)ranks[b] * invN));
+}
+
+// One step: the gradient of the mean squared error, and Adam.  Each CTA takes
+// a grid-stride share of the points, a thread running the forward and backward
+// pass of one; the activations and their gradients are staged in shared memory,
+// where dW2 = DZ2^T H1 is summed as 4 x 4 tiles (two 16-byte reads per 16
+// multiply-adds) and the other entries column by column, and the CTA writes
+// one partial.  The last CTA to arrive sums the partials in block order
+// (deterministic) and applies the update: one launch per step.
+// Bound by the latency of its dependent chains (four warps on an SM, a few
+// SMs).  4096 points: 78 us per step as two kernels that walked the 256 staged
+// rows one load at a time, here 19 us.
+__global__ __launch_bounds__(kGradThreads) void k_cdf_step(hss_cdf_model* M, const float2* __restrict__ pts, uint32_t n,
+                                                           float inv_n, float* __restrict__ part,
+                                                           uint32_t* __restrict__ arrived, float lr, int apply,
+                                                           float* __restrict__ grad_out, float* __restrict__ loss_out) {
     extern __shared__ __align__(16) float sm[];
     float* th = sm;                                 // kP (+3)
-    float* H1s = th + kP + 3;                       // 256 x 33
+    float* H1s = th + kP + 3;                       // rows of kStage
     float* H2s = H1s + kGradThreads * kStage;
     float* DZ2s = H2s + kGradThreads * kStage;
     float* DZ1s = DZ2s + kGradThreads * kStage;
-    float* Xs = DZ1s + kGradThreads * kStage;       // 256
-    float* Ds = Xs + kGradThreads;                  // 256
-    float* Ls = Ds + kGradThreads;                  // 256
-    const int tid = threadIdx.x;
-    for (int k = tid; k < kP; k += kGradThreads) th[k] = weight_of(M, k);
-    const uint64_t flip = M->key_type == HSS_KEY_I64 ? kSignBit : 0ull;
+    float* Xs = DZ1s + kGradThreads * kStage;       // kGradThreads
+    float* Ds = Xs + kGradThreads;                  // kGradThreads
+    __shared__ float s_sum[2 * kGradThreads / 32];
+    __shared__ uint32_t s_last;
+    __shared__ float s_c[2];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    {
+        const bool half = M->weights == HSS_CDF_W_BF16;
+#pragma unroll
+        for (int u = 0; u < (kP + kGradThreads - 1) / kGradThreads; ++u) {
+            const int k = tid + u * kGradThreads;
+            if (k < kP) {
+                const float x = M->theta[k];
+                th[k] = half ? __bfloat162float(__float2bfloat16_rn(x)) : x;
+            }
+        }
+    }
     __syncthreads();
 
-    float accW2[4] = {0.f, 0.f, 0.f, 0.f};
-    float accS = 0.f;  // small entry owned by threads 0..128, loss by thread 129
+    const int tile = tid & 63, i0 = (tile >> 3) * 4, j0 = (tile & 7) * 4, grp = tid >> 6;
+    float acc[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
+    float accS = 0.f;              // warp 0: dw1, 1: db1, 2: db2, 3: dw3, a column per lane
+    float accD = 0.f, accL = 0.f;  // db3 and the squared errors of this thread's points
     for (uint64_t base = (uint64_t)blockIdx.x * kGradThreads; base < n; base += (uint64_t)gridDim.x * kGradThreads) {
         const uint64_t b = base + tid;
-        float x = 0.f, d = 0.f, l = 0.f;
-        float h1[kH], h2[kH], dz2[kH];
+        float x = 0.f, d = 0.f;
+        float h1[kH], h2[kH], dz1[kH];
         if (b < n) {
-            x = feature_of(keys[b], M, flip);
-            const float t = (float)((double)ranks[b] * invN);
-#pragma unroll
-            for (int i = 0; i < kH; ++i) h1[i] = fmaxf(fmaf(th[i], x, th[kOffB1 + i]), 0.f);
-            float y = th[kOffB3];
-#pragma unroll
-            for (int i = 0; i < kH; ++i) {
-                float a = th[kOffB2 + i];
-#pragma unroll
-                for (int j = 0; j < kH; ++j) a = fmaf(th[kOffW2 + i * kH + j], h1[j], a);
-                h2[i] = fmaxf(a, 0.f);
-                y = fmaf(th[kOffW3 + i], h2[i], y);
-            }
-            const float e = y - t;
+            const float2 pt = pts[b];
+            x = pt.x;
+            const float e = layers(th, x, h1, h2) - pt.y;
             d = 2.f * e * inv_n;
-            l = e * e;
-#pragma unroll
-            for (int i = 0; i < kH; ++i) dz2[i] = h2[i] > 0.f ? d * th[kOffW3 + i] : 0.f;
+            accL = fmaf(e, e, accL);
         } else {
 #pragma unroll
-            for (int i = 0; i < kH; ++i) { h1[i] = 0.f; h2[i] = 0.f; dz2[i] = 0.f; }
+            for (int i = 0; i < kH; ++i) { h1[i] = 0.f; h2[i] = 0.f; }
         }
+        accD += d;
+#pragma unroll
+        for (int j = 0; j < kH; ++j) dz1[j] = 0.f;
 #pragma unroll
         for (int i = 0; i < kH; ++i) {
-            H1s[tid * kStage + i] = h1[i];
-            H2s[tid * kStage + i] = h2[i];
-            DZ2s[tid * kStage + i] = dz2[i];
-        }
-#pragma unroll 4
-        for (int j = 0; j < kH; ++j) {
-            float a = 0.f;
+            const float dz2 = h2[i] > 0.f ? d * th[kOffW3 + i] : 0.f;
+            DZ2s[tid * kStage + i] = dz2;
 #pragma unroll
-            for (int i = 0; i < kH; ++i) a = fmaf(th[kOffW2 + i * kH + j], dz2[i], a);
-            DZ1s[tid * kStage + j] = h1[j] > 0.f ? a : 0.f;
+            for (int j = 0; j < kH; j += 4) {
+                const float4 wv = *(const float4*)(th + kOffW2 + i * kH + j);
+                dz1[j] = fmaf(wv.x, dz2, dz1[j]);
+                dz1[j + 1] = fmaf(wv.y, dz2, dz1[j + 1]);
+                dz1[j + 2] = fmaf(wv.z, dz2, dz1[j + 2]);
+                dz1[j + 3] = fmaf(wv.w, dz2, dz1[j + 3]);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kH; ++j) {
+            H1s[tid * kStage + j] = h1[j];
+            H2s[tid * kStage + j] = h2[j];
+            DZ1s[tid * kStage + j] = h1[j] > 0.f ? dz1[j] : 0.f;
         }
         Xs[tid] = x;
         Ds[tid] = d;
-        Ls[tid] = l;
         __syncthreads();
-        // dW2[i][j] = sum_b dz2[b][i] h1[b][j]: thread owns entries tid + 256 q.
+        // dW2[i][j] = sum_b dz2[b][i] h1[b][j]
+        constexpr int kRows = kGradThreads / kRowGroups;
+#pragma unroll 8
+        for (int r = grp * kRows; r < (grp + 1) * kRows; ++r) {
+            const float4 a = *(const float4*)(DZ2s + r * kStage + i0), h = *(const float4*)(H1s + r * kStage + j0);
+            const float av[4] = {a.x, a.y, a.z, a.w}, hv[4] = {h.x, h.y, h.z, h.w};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int e = tid + q * kGradThreads, i = e >> 5, j = e & 31;
-            float a = accW2[q];
-            for (int r = 0; r < kGradThreads; ++r) a = fmaf(DZ2s[r * kStage + i], H1s[r * kStage + j], a);
-            accW2[q] = a;
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(av[p], hv[q], acc[p][q]);
         }
-        if (tid < 130) {
-            float a = accS;
-            if (tid < 32) {              // dw1[j] = sum_b dz1[b][j] x_b
-                for (int r = 0; r < kGradThreads; ++r) a = fmaf(DZ1s[r * kStage + tid], Xs[r], a);
-            } else if (tid < 64) {       // db1[j]
-                for (int r = 0; r < kGradThreads; ++r) a += DZ1s[r * kStage + tid - 32];
-            } else if (tid < 96) {       // db2[i]
-                for (int r = 0; r < kGradThreads; ++r) a += DZ2s[r * kStage + tid - 64];
-            } else if (tid < 128) {      // dw3[i] = sum_b d_b h2[b][i]
-                for (int r = 0; r < kGradThreads; ++r) a = fmaf(Ds[r], H2s[r * kStage + tid - 96], a);
-            } else if (tid == 128) {     // db3
-                for (int r = 0; r < kGradThreads; ++r) a += Ds[r];
-            } else {                     // sum of squared errors
-                for (int r = 0; r < kGradThreads; ++r) a += Ls[r];
-            }
-            accS = a;
+        // dw1[j] = sum_b dz1[b][j] x_b, db1, db2, dw3[i] = sum_b d_b h2[b][i]
+        {
+            const float* col = (w < 2 ? DZ1s : (w == 2 ? DZ2s : H2s)) + lane;
+            const float* f = w == 0 ? Xs : Ds;
+            const bool plain = w == 1 || w == 2;
+            float t[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+            for (int r = 0; r < kGradThreads; r += 4)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) t[u] = fmaf(col[(r + u) * kStage], plain ? 1.f : f[r + u], t[u]);
+            accS += (t[0] + t[1]) + (t[2] + t[3]);
         }
         __syncthreads();
     }
+    // the row groups of dW2 together, through the staging area
+    if (grp > 0) {
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+            *(float4*)(H1s + (grp - 1) * 1024 + (i0 + p) * kH + j0) = make_float4(acc[p][0], acc[p][1], acc[p][2], acc[p][3]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        accD += __shfl_xor_sync(0xffffffffu, accD, o);
+        accL += __shfl_xor_sync(0xffffffffu, accL, o);
+    }
+    if (lane == 0) { s_sum[w] = accD; s_sum[kGradThreads / 32 + w] = accL; }
+    __syncthreads();
     float* out = part + (uint64_t)blockIdx.x * kPartStride;
+    if (grp == 0) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) out[kOffW2 + tid + q * kGradThreads] = accW2[q];
-    if (tid < 32) out[tid] = accS;
-    else if (tid < 64) out[kOffB1 + tid - 32] = accS;
-    else if (tid < 96) out[kOffB2 + tid - 64] = accS;
-    else if (tid < 128) out[kOffW3 + tid - 96] = accS;
-    else if (tid == 128) out[kOffB3] = accS;
-    else if (tid == 129) out[kP] = accS;
-}
-
-// Sum of the partials (in block order: deterministic), optional gradient and
-// loss outputs, optional Adam step.
-__global__ __launch_bounds__(1024) void k_cdf_adam(hss_cdf_model* M, const float* __restrict__ part, int G, float lr,
-                                                   float inv_n, int apply, float* __restrict__ grad_out,
-                                                   float* __restrict__ loss_out) {
-    const uint32_t t = M->step + 1;
-    const float c1 = (float)(1.0 - pow((double)kBeta1, (double)t));
-    const float c2 = (float)(1.0 - pow((double)kBeta2, (double)t));
-    for (int k = threadIdx.x; k < kP; k += blockDim.x) {
-        float g = 0.f;
-        for (int c = 0; c < G; ++c) g += part[(uint64_t)c * kPartStride + k];
-        if (grad_out) grad_out[k] = g;
-        if (apply) {
-            const float m = kBeta1 * M->m[k] + (1.f - kBeta1) * g;
-            const float v = kBeta2 * M->v[k] + (1.f - kBeta2) * g * g;
-            M->m[k] = m;
-            M->v[k] = v;
-            M->theta[k] -= lr * (m / c1) / (sqrtf(v / c2) + kAdamEps);
+        for (int p = 0; p < 4; ++p) {
+            float4 v = make_float4(acc[p][0], acc[p][1], acc[p][2], acc[p][3]);
+#pragma unroll
+            for (int g = 1; g < kRowGroups; ++g) {
+                const float4 o = *(const float4*)(H1s + (g - 1) * 1024 + (i0 + p) * kH + j0);
+                v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+            }
+            *(float4*)(out + kOffW2 + (i0 + p) * kH + j0) = v;
         }
     }
-    if (threadIdx.x == 0) {
-        float l = 0.f;
-        for (int c = 0; c < G; ++c) l += part[(uint64_t)c * kPartStride + kP];
-        if (loss_out) *loss_out = l * inv_n;
+    out[(w == 0 ? 0 : (w == 1 ? kOffB1 : (w == 2 ? kOffB2 : kOffW3))) + lane] = accS;
+    if (tid == 0) {
+        float sd = 0.f, sl = 0.f;
+        for (int i = 0; i < kGradThreads / 32; ++i) { sd += s_sum[i]; sl += s_sum[kGradThreads / 32 + i]; }
+        out[kOffB3] = sd;
+        out[kP] = sl;
+    }
+    // the last CTA sums the partials
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicInc(arrived, gridDim.x - 1) == gridDim.x - 1 ? 1u : 0u;  // back to 0 for the next step
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const uint32_t t = M->step + 1;
+    if (apply && tid < 2) {  // 1 - beta^t by squaring (pow takes microseconds in double precision)
+        double f = (double)(tid ? kBeta2 : kBeta1), q = 1.0;
+        for (uint32_t e = t; e > 0; e >>= 1) {
+            if (e & 1u) q *= f;
+            f *= f;
+        }
+        s_c[tid] = (float)(1.0 - q);
+    }
+    const int G = (int)gridDim.x;
+    for (int k4 = tid; k4 < kPartStride / 4; k4 += kGradThreads) {
+        float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 16
+        for (int c = 0; c < G; ++c) {
+            const float4 v = __ldcg((const float4*)(part + (uint64_t)c * kPartStride) + k4);
+            g4.x += v.x; g4.y += v.y; g4.z += v.z; g4.w += v.w;
+        }
+        ((float4*)H1s)[k4] = g4;
     }
     __syncthreads();
-    if (apply && threadIdx.x == 0) M->step = t;
+    if (tid == 0 && loss_out) *loss_out = H1s[kP] * inv_n;
+    constexpr int kPer = (kP + kGradThreads - 1) / kGradThreads;
+    if (grad_out) {
+        for (int k = tid; k < kP; k += kGradThreads) grad_out[k] = H1s[k];
+    }
+    if (apply) {  // all loads first: the stores go to the same struct
+        float m[kPer], v[kPer], x[kPer];
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            const int k = tid + u * kGradThreads;
+            if (k < kP) { m[u] = M->m[k]; v[u] = M->v[k]; x[u] = M->theta[k]; }
+        }
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            const int k = tid + u * kGradThreads;
+            if (k >= kP) continue;
+            const float g = H1s[k];
+            m[u] = kBeta1 * m[u] + (1.f - kBeta1) * g;
+            v[u] = kBeta2 * v[u] + (1.f - kBeta2) * g * g;
+            M->m[k] = m[u];
+            M->v[k] = v[u];
+            M->theta[k] = x[u] - lr * (m[u] / s_c[0]) / (sqrtf(v[u] / s_c[1]) + kAdamEps);
+        }
+    }
+    __syncthreads();
+    if (apply && tid == 0) M->step = t;
 }
 
 __global__ void k_cdf_set_weights(hss_cdf_model* M, int weights) { M->weights = weights; }
 
 __global__ void k_cdf_eval(const hss_cdf_model* __restrict__ M, const uint64_t* __restrict__ keys, uint32_t n,
                            float* __restrict__ y) {
-    __shared__ float th[kP];
+    __shared__ __align__(16) float th[kP + 3];
     for (int k = threadIdx.x; k < kP; k += blockDim.x) th[k] = weight_of(M, k);
     __syncthreads();
     const uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= n) return;
     const uint64_t flip = M->key_type == HSS_KEY_I64 ? kSignBit : 0ull;
-    y[b] = net(th, feature_of(keys[b], M, flip));
+    float h1[kH], h2[kH];
+    y[b] = layers(th, feature_of(keys[b], M, flip), h1, h2);
 }
 
 // Cut q = (i-1) per + k of splitter i (1..p-1): target tau = i/p + delta
@@ -253,7 +364,7 @@ __global__ void k_cdf_eval(const hss_cdf_model* __restrict__ M, const uint64_t* 
 // clamped to the key range.
 __global__ void k_cdf_propose(const hss_cdf_model* __restrict__ M, uint32_t p, uint32_t per, double delta, int iters,
                               uint64_t* __restrict__ out) {
-    __shared__ float th[kP];
+    __shared__ __align__(16) float th[kP + 3];
     for (int k = threadIdx.x; k < kP; k += blockDim.x) th[k] = weight_of(M, k);
     __syncthreads();
     const uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -278,15 +389,33 @@ __global__ void k_cdf_propose(const hss_cdf_model* __restrict__ M, uint32_t p, u
     out[q] = bits ^ flip;
 }
 
-int grad_blocks(uint32_t n) { return (int)std::max<uint32_t>(1, std::min<uint32_t>(kMaxGradBlocks, (n + 255) / 256)); }
+int grad_blocks(uint32_t n) {
+    return (int)std::max<uint32_t>(1, std::min<uint64_t>(kMaxGradBlocks, ((uint64_t)n + kGradThreads - 1) / kGradThreads));
+}
 
-size_t grad_smem() { return (size_t)(kP + 3 + 4 * kGradThreads * kStage + 3 * kGradThreads) * sizeof(float); }
+size_t grad_smem() { return (size_t)(kP + 3 + 4 * kGradThreads * kStage + 2 * kGradThreads) * sizeof(float); }
 
-int launch_grad(const hss_cdf_model* M, const uint64_t* keys, const uint64_t* ranks, uint32_t n, uint64_t N,
-                float* part, cudaStream_t st) {
-    if (ensure_func_attrs((const void*)k_cdf_grad, (int)grad_smem()) != cudaSuccess) return HSS_ERR_CUDA;
-    HSS_LAUNCH(k_cdf_grad, grad_blocks(n), kGradThreads, grad_smem(), st, M, keys, ranks, n, 1.0 / (double)N,
-               (float)(1.0 / (double)n), part);
+// Scratch: the CTAs' partials, the arrival counter, the points.
+struct Work {
+    float* part;
+    uint32_t* arrived;
+    float2* pts;
+    size_t bytes;
+    Work(void* base, uint32_t n) {
+        const size_t p = (size_t)grad_blocks(n) * kPartStride * sizeof(float);  // a multiple of 16
+        char* q = (char*)(((uintptr_t)base + 15) & ~(uintptr_t)15);
+        part = (float*)q;
+        arrived = (uint32_t*)(q + p);
+        pts = (float2*)(q + p + 16);
+        bytes = 16 + p + 16 + (size_t)n * sizeof(float2);
+    }
+};
+
+int launch_points(const hss_cdf_model* M, const uint64_t* keys, const uint64_t* ranks, uint32_t n, uint64_t N,
+                  const Work& wk, cudaStream_t st) {
+    if (ensure_func_attrs((const void*)k_cdf_step, (int)grad_smem()) != cudaSuccess) return HSS_ERR_CUDA;
+    HSS_LAUNCH(k_cdf_points, (unsigned)(((uint64_t)n + kGradThreads - 1) / kGradThreads), kGradThreads, 0, st, M, keys, ranks,
+               n, 1.0 / (double)N, wk.pts, wk.arrived);
     return cudaGetLastError() == cudaSuccess ? HSS_OK : HSS_ERR_CUDA;
 }
 
@@ -311,7 +440,7 @@ int hss_cdf_set_weights(hss_cdf_model* d_model, int weights, void* stream) {
     return cudaGetLastError() == cudaSuccess ? HSS_OK : HSS_ERR_CUDA;
 }
 
-size_t hss_cdf_work_bytes(uint32_t n) { return (size_t)grad_blocks(n) * kPartStride * sizeof(float); }
+size_t hss_cdf_work_bytes(uint32_t n) { return Work(nullptr, n).bytes; }
 
 int hss_cdf_init(hss_cdf_model* d_model, uint64_t seed, int feature, int key_type, uint64_t lo_key, uint64_t hi_key,
                  void* stream) {
@@ -329,11 +458,11 @@ int hss_cdf_grad(const hss_cdf_model* d_model, const void* d_keys, const uint64_
     if (!d_model || n == 0 || N == 0 || !d_keys || !d_ranks || !d_work) return HSS_ERR_INVALID;
     if (work_bytes < hss_cdf_work_bytes(n)) return HSS_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
-    float* part = (float*)d_work;
-    const int rc = launch_grad(d_model, (const uint64_t*)d_keys, d_ranks, n, N, part, st);
+    const Work wk(d_work, n);
+    const int rc = launch_points(d_model, (const uint64_t*)d_keys, d_ranks, n, N, wk, st);
     if (rc != HSS_OK) return rc;
-    HSS_LAUNCH(k_cdf_adam, 1, 1024, 0, st, const_cast<hss_cdf_model*>(d_model), part, grad_blocks(n), 0.f,
-               (float)(1.0 / (double)n), 0, d_grad, d_loss);
+    HSS_LAUNCH(k_cdf_step, grad_blocks(n), kGradThreads, grad_smem(), st, const_cast<hss_cdf_model*>(d_model), wk.pts, n,
+               (float)(1.0 / (double)n), wk.part, wk.arrived, 0.f, 0, d_grad, d_loss);
     return cudaGetLastError() == cudaSuccess ? HSS_OK : HSS_ERR_CUDA;
 }
 
@@ -342,13 +471,13 @@ int hss_cdf_train(hss_cdf_model* d_model, const void* d_keys, const uint64_t* d_
     if (!d_model || n == 0 || N == 0 || !d_keys || !d_ranks || !d_work || !(lr > 0.f)) return HSS_ERR_INVALID;
     if (work_bytes < hss_cdf_work_bytes(n)) return HSS_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
-    float* part = (float*)d_work;
-    for (uint32_t s = 0; s < steps; ++s) {
-        const int rc = launch_grad(d_model, (const uint64_t*)d_keys, d_ranks, n, N, part, st);
-        if (rc != HSS_OK) return rc;
-        HSS_LAUNCH(k_cdf_adam, 1, 1024, 0, st, d_model, part, grad_blocks(n), lr, (float)(1.0 / (double)n), 1, nullptr,
-                   s + 1 == steps ? d_loss : nullptr);
-    }
+    if (steps == 0) return HSS_OK;
+    const Work wk(d_work, n);
+    const int rc = launch_points(d_model, (const uint64_t*)d_keys, d_ranks, n, N, wk, st);
+    if (rc != HSS_OK) return rc;
+    for (uint32_t s = 0; s < steps; ++s)
+        HSS_LAUNCH(k_cdf_step, grad_blocks(n), kGradThreads, grad_smem(), st, d_model, wk.pts, n, (float)(1.0 / (double)n),
+                   wk.part, wk.arrived, lr, 1, nullptr, s + 1 == steps ? d_loss : nullptr);
     return cudaGetLastError() == cudaSuccess ? HSS_OK : HSS_ERR_CUDA;
 }
 
