@@ -81,6 +81,20 @@ __global__ void kb_init(const BJob* __restrict__ jobs, BCtl* __restrict__ ctl, h
     }
 }
 
+// The tables over the segments and splitters of all jobs (segment bounds, the
+// job of each), one CTA per job.
+__global__ void kb_tables(uint32_t njobs, const BJob* __restrict__ jobs, uint64_t* __restrict__ seg_off,
+                          uint32_t* __restrict__ job_of_seg, uint32_t* __restrict__ job_of_spl) {
+    const uint32_t j = blockIdx.x;
+    const BJob J = jobs[j];
+    for (uint32_t s = threadIdx.x; s < J.p; s += blockDim.x) {
+        seg_off[J.sbase + s] = J.koff + seg_start(J, s);
+        job_of_seg[J.sbase + s] = j;
+        if (s + 1 < J.p) job_of_spl[J.ibase + s] = j;
+    }
+    if (j + 1 == njobs && threadIdx.x == 0) seg_off[J.sbase + J.p] = J.koff + J.n;
+}
+
 // One CTA per job: resolved flags, distinct unresolved intervals, |gamma|,
 // next threshold.  A failed job keeps its state.
 __global__ __launch_bounds__(1024) void kb_intervals(const BJob* __restrict__ jobs, BCtl* __restrict__ ctl,
@@ -648,8 +662,6 @@ __global__ void kb_bucket_hint(uint32_t P_tot, const BJob* __restrict__ jobs, co
 // ---------------------------------------------------------------------------
 struct Tables {
     std::vector<BJob> jobs;
-    std::vector<uint32_t> job_of_seg, job_of_spl;
-    std::vector<uint64_t> seg_off;
     uint64_t N_tot = 0, L_tot = 0, D_tot = 0, C_tot = 0, PP_tot = 0, O_tot = 0;
     uint32_t P_tot = 0, S_tot = 0, max_p = 0, max_seg = 0;
 };
@@ -674,18 +686,11 @@ int build_tables(const uint64_t* sizes, const uint32_t* ps, uint32_t njobs, cons
         J.tol = (uint64_t)std::floor(((double)n * prm->eps) / (2.0 * (double)p));
         J.seed = seeds ? seeds[j] : prm->seed + j;
         J.obase = ob;
-        for (uint32_t s = 0; s < p; ++s) {
-            T.seg_off.push_back(koff + (uint64_t)(((unsigned __int128)s * n) / p));
-            T.job_of_seg.push_back(j);
-            const uint64_t len = (uint64_t)(((unsigned __int128)(s + 1) * n) / p) - (uint64_t)(((unsigned __int128)s * n) / p);
-            T.max_seg = std::max<uint32_t>(T.max_seg, (uint32_t)len);
-        }
-        for (uint32_t i = 0; i + 1 < p; ++i) T.job_of_spl.push_back(j);
+        T.max_seg = std::max<uint32_t>(T.max_seg, (uint32_t)((n + p - 1) / p));
         koff += n; sb += p; ib += p - 1;
         lb += (uint64_t)p * (p - 1); db += (uint64_t)p * p; cb += J.cap; pp += (uint64_t)p * J.cap; ob += p + 1;
         T.max_p = std::max(T.max_p, p);
     }
-    T.seg_off.push_back(koff);
     T.N_tot = koff; T.P_tot = sb; T.S_tot = ib; T.L_tot = lb; T.D_tot = db; T.C_tot = cb; T.PP_tot = pp; T.O_tot = ob;
     return HSS_OK;
 }
@@ -806,13 +811,12 @@ int run_batch(const void* d_keys, const uint32_t* d_payload, int key_type, const
     SegSortWs sws = segsort_ws_carve(at<void>(d_work, L.sws), std::max<uint64_t>(T.N_tot, 1), T.P_tot, err);
     SegSortWs sws_s = segsort_ws_carve(at<void>(d_work, L.sws_s), std::max<uint64_t>(T.C_tot, 1), njobs, err);
 
-    // Tables to the device (the host vectors stay alive until the copies end).
+    // The jobs to the device (the host vector stays alive until the copy ends).
     HSS_BTRY(cudaMemsetAsync(err, 0, 256, st));
     HSS_BTRY(cudaMemsetAsync(jst, 0, njobs * sizeof(hss_job_stats), st));
     HSS_BTRY(cudaMemcpyAsync(jobs, T.jobs.data(), njobs * sizeof(BJob), cudaMemcpyHostToDevice, st));
-    HSS_BTRY(cudaMemcpyAsync(jseg, T.job_of_seg.data(), (size_t)T.P_tot * 4, cudaMemcpyHostToDevice, st));
-    if (T.S_tot) HSS_BTRY(cudaMemcpyAsync(jspl, T.job_of_spl.data(), (size_t)T.S_tot * 4, cudaMemcpyHostToDevice, st));
-    HSS_BTRY(cudaMemcpyAsync(seg_off, T.seg_off.data(), ((size_t)T.P_tot + 1) * 8, cudaMemcpyHostToDevice, st));
+    HSS_LAUNCH(kb_tables, njobs, 256, 0, st, njobs, jobs, seg_off, jseg, jspl);
+    HSS_BTRY(cudaGetLastError());
 
     float ms[4] = {0, 0, 0, 0};
     TimingEvents<5> tev;
@@ -900,8 +904,9 @@ int run_batch(const void* d_keys, const uint32_t* d_payload, int key_type, const
 
     uint32_t h_err = 0;
     HSS_BTRY(cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, st));
-    std::vector<hss_job_stats> js(njobs);
-    HSS_BTRY(cudaMemcpyAsync(js.data(), jst, njobs * sizeof(hss_job_stats), cudaMemcpyDeviceToHost, st));
+    std::vector<hss_job_stats> own(h_job_stats ? 0 : njobs);
+    hss_job_stats* js = h_job_stats ? h_job_stats : own.data();
+    HSS_BTRY(cudaMemcpyAsync(js, jst, njobs * sizeof(hss_job_stats), cudaMemcpyDeviceToHost, st));
     HSS_BTRY(cudaStreamSynchronize(st));
     int status = HSS_OK;
     if (h_err & kDevErrTimeout) status = HSS_ERR_TIMEOUT;
@@ -914,7 +919,6 @@ int run_batch(const void* d_keys, const uint32_t* d_payload, int key_type, const
         for (uint32_t r = 0; r < js[j].rounds && r < HSS_MAX_ROUNDS; ++r) samples += js[j].sample_size[r];
         if (status == HSS_OK && js[j].status != HSS_OK) status = js[j].status;
     }
-    if (h_job_stats) std::memcpy(h_job_stats, js.data(), njobs * sizeof(hss_job_stats));
     if (h_stats) {
         h_stats->njobs = njobs;
         h_stats->max_rounds = maxr;

@@ -615,6 +615,20 @@ class BatchStats(ctypes.Structure):
                 ("ms_phase", ctypes.c_float * NUM_PHASES)]
 
 
+def _job_lists(js, n: int) -> dict:
+    """The per-job statistics of n JobStats records as the lists a result
+    carries (read as one numpy record array: thousands of jobs)."""
+    a = np.frombuffer(js, dtype=np.dtype(JobStats), count=n)
+    rounds = a["rounds"].tolist()
+    most = min(max(rounds, default=0), MAX_ROUNDS)
+
+    def rows(name, extra=0):
+        return [row[:r + extra] for row, r in zip(a[name][:, :most + extra].tolist(), rounds)]
+
+    return {"rounds": rounds, "status": a["status"].tolist(), "tol": a["tol"].tolist(), "sample_size": rows("sample_size"),
+            "gamma": rows("gamma"), "unresolved": rows("unresolved", 1)}
+
+
 @dataclass
 class BatchResult:
     keys: torch.Tensor | None
@@ -707,14 +721,11 @@ def _batch(keys, sizes, ps, eps, seed, payload, oversample, max_rounds, key_type
                                             ctypes.byref(st), js, _stream(stream))
     if rc in (ERR_INVALID, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT):
         raise HSSError(rc, "hss_sort_batch" if sort else "hss_partition_batch")
+    jl = _job_lists(js, nj)
     return BatchResult(
         keys=out if sort else None, payload=out_payload if sort else None, splitters=spl[:S_tot], offsets=off,
-        sizes=[int(x) for x in sizes], ps=[int(x) for x in ps], status=rc,
-        job_rounds=[int(x.rounds) for x in js], job_status=[int(x.status) for x in js],
-        job_tol=[int(x.tol) for x in js],
-        job_sample_size=[[int(v) for v in x.sample_size[:x.rounds]] for x in js],
-        job_gamma=[[int(v) for v in x.gamma[:x.rounds]] for x in js],
-        job_unresolved=[[int(v) for v in x.unresolved[:x.rounds + 1]] for x in js],
+        sizes=sizes.tolist(), ps=ps.tolist(), status=rc, job_rounds=jl["rounds"], job_status=jl["status"],
+        job_tol=jl["tol"], job_sample_size=jl["sample_size"], job_gamma=jl["gamma"], job_unresolved=jl["unresolved"],
         lockstep_rounds=int(st.lockstep_rounds), total_samples=int(st.total_samples),
         kernel_launches=int(st.kernel_launches),
         ms_phase={PHASES[i]: float(st.ms_phase[i]) for i in range(NUM_PHASES)})
@@ -832,12 +843,10 @@ def sort_two_stage(keys, p: int, groups: int, eps: float, seed: int, payload=Non
     s1 = _result(None, None, gspl[:r - 1], goff, st.stage1)
     ms = {f"stage1_{PHASES[i]}": float(st.stage1.ms_phase[i]) for i in range(3)}
     ms.update({f"stage2_{PHASES[i]}": float(st.stage2.ms_phase[i]) for i in range(NUM_PHASES)})
+    jl = _job_lists(js, r)
     return TwoStageResult(
         keys=out, payload=out_payload, offsets=off, group_splitters=gspl[:r - 1], splitters=spl[:r * (pg - 1)],
         groups=r, status=rc, stage1=s1,
-        group_rounds=[int(x.rounds) for x in js], group_status=[int(x.status) for x in js],
-        group_tol=[int(x.tol) for x in js],
-        group_sample_size=[[int(v) for v in x.sample_size[:x.rounds]] for x in js],
-        group_gamma=[[int(v) for v in x.gamma[:x.rounds]] for x in js],
-        group_unresolved=[[int(v) for v in x.unresolved[:x.rounds + 1]] for x in js],
+        group_rounds=jl["rounds"], group_status=jl["status"], group_tol=jl["tol"],
+        group_sample_size=jl["sample_size"], group_gamma=jl["gamma"], group_unresolved=jl["unresolved"],
         lockstep_rounds=int(st.stage2.lockstep_rounds), kernel_launches=int(st.kernel_launches), ms_phase=ms)
