@@ -224,29 +224,32 @@ __device__ __forceinline__ uint32_t warp_peers8(uint32_t d) {
 // Stable block ranking of 8-bit digits (digit_of(i): the thread's item i), in
 // three steps:
 //   1. counts: every warp counts its digits into its own 256 shared counters
-//      (fire-and-forget shared atomics, no dependency chain);
+//      (16 bits, two to a word; fire-and-forget shared atomics);
 //   2. offsets: the counts become absolute bases start[d] + (earlier warps'
-//      counts of d);
+//      counts of d); `between` runs before the barrier that ends the step;
 //   3. ranks: per item, the lanes holding the same digit (ballot peer mask)
 //      take consecutive slots from the warp's base for that digit, which the
-//      lowest of them moves on.
+//      lowest of them moves on; body(i, rank) takes each.
 // Items are warp-striped: item i of lane l in warp w is element
 // w*32*ITEMS + i*32 + l, so (w, i, l) order is element order and the ranks are
 // stable.  Every item takes part; empty ones carry the last digit and, being
 // last in element order, rank behind all others, so nothing tests for them
 // (with such tests and an atomic for the base the split of pairs took 6% more).
 // ---------------------------------------------------------------------------
-template <int WARPS, int ITEMS, typename DigitOf>
-__device__ __forceinline__ void block_rank(DigitOf digit_of, uint32_t (&rank)[ITEMS], uint32_t* s_cnt /*[WARPS*256]*/,
-                                           uint32_t* s_total, uint32_t* s_start, uint32_t* s_warp) {
+template <int WARPS, int ITEMS, typename DigitOf, typename Between, typename Body>
+__device__ __forceinline__ void block_rank(DigitOf digit_of, uint16_t* s_cnt /*[WARPS*256]*/, uint32_t* s_total,
+                                           uint32_t* s_start, uint32_t* s_warp, Between between, Body body) {
     constexpr int T = WARPS * 32;
-    static_assert(T >= kRadix, "a thread per digit");
+    static_assert(T >= kRadix && T * ITEMS < 65536, "a thread per digit, 16-bit counters");
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    uint32_t* c = s_cnt + w * kRadix;
-    for (int i = lane; i < kRadix; i += 32) c[i] = 0;
+    uint16_t* c = s_cnt + w * kRadix;
+    *(uint4*)(c + lane * 8) = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
 #pragma unroll
-    for (int i = 0; i < ITEMS; ++i) atomicAdd(&c[digit_of(i)], 1u);
+    for (int i = 0; i < ITEMS; ++i) {
+        const uint32_t d = digit_of(i);
+        atomicAdd((uint32_t*)c + (d >> 1), 1u << ((d & 1u) * 16u));
+    }
     __syncthreads();
     if (tid < kRadix) {
         uint32_t run = 0;
@@ -261,10 +264,11 @@ __device__ __forceinline__ void block_rank(DigitOf digit_of, uint32_t (&rank)[IT
 #pragma unroll
         for (int ww = 0; ww < WARPS; ++ww) {
             const uint32_t x = s_cnt[ww * kRadix + tid];
-            s_cnt[ww * kRadix + tid] = run;
+            s_cnt[ww * kRadix + tid] = (uint16_t)run;
             run += x;
         }
     }
+    between();
     __syncthreads();
     const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll
@@ -273,15 +277,19 @@ __device__ __forceinline__ void block_rank(DigitOf digit_of, uint32_t (&rank)[IT
         const uint32_t peers = warp_peers8(d);
         const uint32_t base = c[d], below = __popc(peers & lt);
         __syncwarp();
-        if (below == 0) c[d] = base + (uint32_t)__popc(peers);
+        if (below == 0) c[d] = (uint16_t)(base + (uint32_t)__popc(peers));
         __syncwarp();
-        rank[i] = base + below;
+        body(i, base + below);
     }
 }
 
 __device__ __forceinline__ void cp_async8(void* sdst, const void* gsrc) {
     const uint32_t sa = (uint32_t)__cvta_generic_to_shared(sdst);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* sdst, const void* gsrc) {
+    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(sdst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gsrc) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
@@ -399,11 +407,6 @@ constexpr int chip_min_blocks() { return THREADS <= 128 ? (PAY ? 6 : 8) : (THREA
 // ranges leaves the LSD kernel nothing of these inputs (packs that span the gap
 // between two clusters used to end there: 1.3 ms per 2^28 pairs).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void cp_async4(void* sdst, const void* gsrc) {
-    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(sdst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gsrc) : "memory");
-}
-
 // Exclusive scan in place of 2 NW 16-bit counters packed in NW shared words
 // (counter 2i in the low half of word i) by a CTA of T threads, and the
 // largest counter.  The counters add up to less than 2^16.  Ends with a
@@ -1591,28 +1594,45 @@ struct SplitArgs {
     uint32_t scatter;  // 1: tiles that gather no key ranges write each key straight to its run
 };
 
-// The tile's shape: keys alone 256 threads x 16 keys (four CTAs per SM);
-// with a payload 512 threads x 8 (two per SM), whose stable ranking then
-// fits 64 registers without spilling.
+// The tile's shape: keys alone 256 threads x 16 keys, with a payload 512 x 8.
 template <bool PAY>
 constexpr int split_threads() { return PAY ? 512 : 256; }
 
 template <bool PAY, bool SPL>
-__global__ __launch_bounds__(split_threads<PAY>(), PAY ? 2 : 4) void k_split(const SplitArgs A) {
+constexpr size_t split_smem(bool gather) {
+    return (size_t)(kOsTile + 2) * 8 + (PAY ? (size_t)(kOsTile + 8) * 4 : 0) + (size_t)kOsTile * 2 +
+           (SPL ? (size_t)kOsTile : 0) + (PAY ? (size_t)(split_threads<PAY>() / 32) * kRadix * 2 : 0) +
+           (gather ? 2 * (size_t)kRadix * 8 : 0);
+}
+
+// One bulk copy brings the tile's keys (and payload) into shared memory, where
+// they stay; what is put into digit order is a 16-bit index per key, and the
+// tile is then written run by run through it.  So no thread holds its keys in
+// registers across the ranking (64 registers and half the warps of an SM
+// before), and shared memory sees 2 bytes per key scattered instead of 9 (13).
+// Bound by shared-memory wavefronts (80% of their peak keys alone, 74% with a
+// payload: the counting atomics, the index scatter and the key gather meet
+// random banks).  2^28 keys, 256-way: keys alone 1.10 -> 0.90 ms, with a
+// payload 2.50 -> 1.95 ms.  Keys alone with 512 threads: 6% slower.
+template <bool PAY, bool SPL>
+__global__ __launch_bounds__(split_threads<PAY>(), PAY ? 3 : 5) void k_split(const SplitArgs A) {
     constexpr int kThreads = split_threads<PAY>();
     constexpr int kWarps = kThreads / 32;
     constexpr int kItems = kOsTile / kThreads;
     extern __shared__ __align__(16) unsigned char os_smem[];
-    uint64_t* s_keys = (uint64_t*)os_smem;             // kOsTile keys
-    uint32_t* s_pay = (uint32_t*)(s_keys + kOsTile);   // kOsTile payloads (PAY)
-    uint8_t* s_dg = (uint8_t*)(s_pay + (PAY ? kOsTile : 0));  // kOsTile digits of the staged keys
-    __shared__ uint32_t s_hist[PAY ? kWarps * kRadix : 1];
+    uint64_t* s_keys = (uint64_t*)os_smem;                         // kOsTile + 2: key e at [e + hd]
+    uint32_t* s_pay = (uint32_t*)(s_keys + kOsTile + 2);           // kOsTile + 8 (PAY): payload e at [e + po]
+    uint16_t* s_hist = (uint16_t*)(s_pay + (PAY ? kOsTile + 8 : 0));  // kWarps * 256 (PAY)
+    uint16_t* s_idx = s_hist + (PAY ? kWarps * kRadix : 0);        // kOsTile: the keys in digit order
+    uint8_t* s_dg = (uint8_t*)(s_idx + kOsTile);                   // kOsTile (SPL): their digits
+    uint64_t* s_mn = (uint64_t*)(s_dg + (SPL ? kOsTile : 0));      // 2 x 256 (gather): key ranges of sub-buckets
+    uint64_t* s_mx = s_mn + kRadix;
     __shared__ uint32_t s_total[kRadix], s_start[kRadix];
-    __shared__ uint64_t s_gbase[kRadix];
+    __shared__ uint32_t s_gbase[kRadix];  // start of the digit's run in the segment, less its start in the tile
     __shared__ uint32_t s_warp[32];
-    __shared__ uint64_t s_mn[kRadix], s_mx[kRadix];
     __shared__ uint32_t s_spl[SPL ? kRadix : 1];
     __shared__ uint32_t s_mask[8];
+    __shared__ uint64_t s_bar;
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const uint32_t total_tiles = A.tile_start[A.nseg];
@@ -1621,87 +1641,99 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 2 : 4) void k_split(con
     const uint32_t s = A.tile_seg[t];
     const uint32_t id = A.large_id[s];
     const uint64_t seg_base = A.seg_lo[s];
-    const uint64_t seg_n = A.seg_hi[s] - seg_base;
-    const uint32_t ti = t - A.tile_start[s];
-    const uint64_t tile_lo = (uint64_t)ti * kOsTile;
-    const uint32_t count = (uint32_t)min((uint64_t)kOsTile, seg_n - tile_lo);
+    const uint32_t seg_n = (uint32_t)(A.seg_hi[s] - seg_base);  // below 2^30
+    const uint32_t tile_lo = (t - A.tile_start[s]) * (uint32_t)kOsTile;
+    const uint32_t count = min((uint32_t)kOsTile, seg_n - tile_lo);
     const int shift = (int)(A.msd_shift[id] & 0xffu);
     const uint64_t dbase = A.msd_base[id];
     const uint64_t dmult = A.msd_mult[id];
     // SPL: this level's segments may split on sampled splitters (uniform per CTA)
     const bool bysplit = SPL && (A.msd_shift[id] & kShiftSplit) != 0u;
     const bool dir = A.direct[id] != 0u;
-    uint64_t* kout = dir ? A.kfinal : A.kout;
-    uint32_t* pout = dir ? A.pfinal : A.pout;
     const uint64_t flip_out = dir ? A.flip_out : 0ull;
     // A segment of one key value already in place in the output (every
     // second level reads the output buffer) needs no copy at all.
     if (dir && A.kin == A.kfinal && flip_out == 0ull && (!PAY || A.pin == A.pfinal)) return;
+    uint64_t* kout = (dir ? A.kfinal : A.kout) + seg_base;
+    uint32_t* pout = PAY ? (dir ? A.pfinal : A.pout) + seg_base : nullptr;
+    // The tile: 16-byte aligned middle by a bulk copy, the ends by small ones.
+    const uint64_t* g = A.kin + seg_base + tile_lo;
+    const uint32_t* gp = PAY ? A.pin + seg_base + tile_lo : nullptr;
+    const uint32_t hd = (uint32_t)(((uintptr_t)g >> 3) & 1u), m = ((count - hd) >> 1) << 1;
+    const uint32_t po = PAY ? (uint32_t)(((uintptr_t)gp >> 2) & 3u) : 0u;
+    const uint32_t ph = PAY ? min(count, (4u - po) & 3u) : 0u, pm = PAY ? ((count - ph) >> 2) << 2 : 0u;
+    if (tid == 0) {
+        mbar_init(&s_bar, 1u);
+        mbar_arrive_expect_tx(&s_bar, m * 8u + pm * 4u);
+        if (m) bulk_load(s_keys + 2 * hd, g + hd, m * 8u, &s_bar);
+        if (PAY && pm) bulk_load(s_pay + po + ph, gp + ph, pm * 4u, &s_bar);
+    }
+    if (hd && tid == 32) cp_async8(&s_keys[1], g);
+    if (hd + m < count && tid == 33) cp_async8(&s_keys[count - 1 + hd], g + count - 1);
+    if (PAY) {
+        if (tid >= 40 && (uint32_t)(tid - 40) < ph) cp_async4(&s_pay[po + tid - 40], gp + tid - 40);
+        if (tid >= 44 && tid < 48 && ph + pm + (uint32_t)(tid - 44) < count)
+            cp_async4(&s_pay[po + ph + pm + tid - 44], gp + ph + pm + tid - 44);
+    }
+    cp_async_commit();
     const bool gather = A.any_large[id] != 0u;  // some sub-bucket is split again: note its key range
     if (gather) {
         if (tid < kRadix) { s_mn[tid] = ~0ull; s_mx[tid] = 0ull; }
         if (tid < 8) s_mask[tid] = A.large_mask[(uint64_t)id * 8 + tid];
     }
-    if (SPL && bysplit) {
-        if (tid < kRadix) s_spl[tid] = A.spl_tab[(uint64_t)id * kRadix + tid];
-        __syncthreads();
+    if (SPL && bysplit && tid < kRadix) s_spl[tid] = A.spl_tab[(uint64_t)id * kRadix + tid];
+    if (!PAY && tid < kRadix) s_total[tid] = 0;
+    cp_async_wait_all();
+    __syncthreads();  // the barrier is initialised, the small copies have landed
+    if (__syncthreads_or(!mbar_wait(&s_bar, 0u))) {  // uniform; not expected: a bulk copy that never landed
+        if (tid == 0) atomicOr(A.err, kDevErrTimeout);
+        return;
     }
-    auto dig = [&](uint64_t k) -> uint32_t {
+    const uint64_t* keys = s_keys + hd;
+    const uint32_t* pays = s_pay + po;
+    auto digit = [&](uint64_t k) -> uint32_t {  // of a key as read
+        k ^= A.flip_in;
         if (SPL && bysplit) return splitter_digit(s_spl, k);
         return split_digit(k, shift, dbase, dmult);
     };
-
-    uint64_t key[kItems];
-    uint32_t pay[kItems];
-    uint32_t rank[kItems];
-    const uint32_t wbase = w * 32 * kItems + lane;
-#pragma unroll
-    for (int i = 0; i < kItems; ++i) {
-        const uint32_t e = wbase + i * 32;
-        if (e < count) {
-            key[i] = A.kin[seg_base + tile_lo + e] ^ A.flip_in;
-            if (PAY) pay[i] = A.pin[seg_base + tile_lo + e];
-        } else {
-            key[i] = 0;
-            if (PAY) pay[i] = 0;
+    const bool direct = A.scatter && !gather;  // uniform per CTA: each key straight to its run
+    const uint64_t flip = A.flip_in ^ flip_out;
+    const uint32_t off_d = tid < kRadix ? A.tile_off[(uint64_t)t * kRadix + tid] : 0u;
+    auto put = [&](uint32_t dst, uint32_t e) {
+        if (dst >= seg_n) {  // never taken when the digit offsets are consistent
+            atomicOr(A.err, kDevErrBounds);
+            return;
         }
-    }
+        kout[dst] = keys[e] ^ flip;
+        if (PAY) pout[dst] = pays[e];
+    };
     if constexpr (PAY) {
         // Each key's digit once, byte-packed (past the segment the last one).
+        const uint32_t wbase = w * 32 * kItems + lane;
         uint32_t dpk[kItems / 4];
 #pragma unroll
         for (int i = 0; i < kItems / 4; ++i) dpk[i] = 0;
 #pragma unroll
-        for (int i = 0; i < kItems; ++i)
-            dpk[i >> 2] |= (wbase + i * 32 < count ? dig(key[i]) : (uint32_t)kRadix - 1u) << (8 * (i & 3));
-        auto digit_of = [&](int i) -> uint32_t { return (dpk[i >> 2] >> (8 * (i & 3))) & 255u; };
-        block_rank<kWarps, kItems>(digit_of, rank, s_hist, s_total, s_start, s_warp);
-        if (A.scatter && !gather) {  // uniform per CTA
-            // The stable tile rank less the digit's tile start is the key's
-            // place in its digit's run: write it there.
-            if (tid < kRadix)
-                s_gbase[tid] = seg_base + (uint64_t)A.tile_off[(uint64_t)t * kRadix + tid] - (uint64_t)s_start[tid];
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < kItems; ++i) {
-                if (wbase + i * 32 < count) {
-                    const uint64_t dst = s_gbase[digit_of(i)] + rank[i];
-                    if (dst - seg_base >= seg_n) {  // never taken when the digit offsets are consistent
-                        atomicOr(A.err, kDevErrBounds);
-                        continue;
-                    }
-                    kout[dst] = key[i] ^ flip_out;
-                    pout[dst] = pay[i];
-                }
-            }
-            return;
-        }
-#pragma unroll
         for (int i = 0; i < kItems; ++i) {
-            s_keys[rank[i]] = key[i];
-            s_dg[rank[i]] = (uint8_t)digit_of(i);
-            s_pay[rank[i]] = pay[i];
+            const uint32_t e = wbase + i * 32;
+            dpk[i >> 2] |= (e < count ? digit(keys[e]) : (uint32_t)kRadix - 1u) << (8 * (i & 3));
         }
+        auto digit_of = [&](int i) -> uint32_t { return (dpk[i >> 2] >> (8 * (i & 3))) & 255u; };
+        block_rank<kWarps, kItems>(
+            digit_of, s_hist, s_total, s_start, s_warp,
+            [&]() {
+                if (tid < kRadix) s_gbase[tid] = off_d - s_start[tid];
+            },
+            [&](int i, uint32_t rank) {
+                const uint32_t e = wbase + i * 32;
+                if (direct) {
+                    if (e < count) put(s_gbase[digit_of(i)] + rank, e);
+                } else {
+                    s_idx[rank] = (uint16_t)e;
+                    if (SPL && bysplit) s_dg[rank] = (uint8_t)digit_of(i);
+                }
+            });
+        if (direct) return;
     } else {
         // Keys alone: equal keys are indistinguishable, so the order of a
         // digit's keys inside the tile is free and one shared counter per
@@ -1710,55 +1742,26 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 2 : 4) void k_split(con
         // holds the digit and, from bit 8, the key's slot.  (Aggregating the
         // lanes of a warp that share a digit with a match instruction costs
         // more than it saves, even on heavily duplicated keys.)
-        const bool direct = A.scatter && !gather;  // uniform per CTA
-        for (int d = tid; d < kRadix; d += kThreads) {
-            s_total[d] = 0;
-            // direct: digit d's keys of this tile start here in the output
-            if (direct) s_gbase[d] = seg_base + (uint64_t)A.tile_off[(uint64_t)t * kRadix + d];
-        }
-        __syncthreads();
-        if (direct) {
-            // Each key goes straight to the slot its digit's counter hands
-            // out; nothing is staged, so no further barrier.
-            const bool skew = A.tile_skew[t] != 0;
-            const uint32_t lt_mask = (1u << lane) - 1u;
-#pragma unroll
-            for (int i = 0; i < kItems; ++i) {
-                const uint32_t d = wbase + i * 32 < count ? dig(key[i]) : (uint32_t)kRadix;
-                uint32_t slot = 0;
-                if (skew) {
-                    const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
-                    const uint32_t eq = __ballot_sync(0xffffffffu, d == d0);
-                    uint32_t b0 = 0;
-                    if (lane == 0 && d0 < (uint32_t)kRadix) b0 = atomicAdd(&s_total[d0], (uint32_t)__popc(eq));
-                    b0 = __shfl_sync(0xffffffffu, b0, 0);
-                    if (d < (uint32_t)kRadix) slot = d == d0 ? b0 + (uint32_t)__popc(eq & lt_mask) : atomicAdd(&s_total[d], 1u);
-                } else if (d < (uint32_t)kRadix) {
-                    slot = atomicAdd(&s_total[d], 1u);
-                }
-                if (d < (uint32_t)kRadix) {
-                    const uint64_t dst = s_gbase[d] + slot;
-                    if (dst - seg_base >= seg_n) {  // never taken when the digit offsets are consistent
-                        atomicOr(A.err, kDevErrBounds);
-                        continue;
-                    }
-                    kout[dst] = key[i] ^ flip_out;
-                }
-            }
-            return;
-        }
+        if (direct && tid < kRadix) s_gbase[tid] = off_d;  // digit d's keys of this tile start here
+        uint32_t rank[kItems];
         if (SPL && bysplit) {
 #pragma unroll
-            for (int i = 0; i < kItems; ++i) rank[i] = splitter_digit(s_spl, key[i]);
+            for (int i = 0; i < kItems; ++i) {
+                const uint32_t e = tid + i * kThreads;
+                rank[i] = e < count ? splitter_digit(s_spl, keys[e] ^ A.flip_in) : (uint32_t)kRadix;
+            }
         } else {
 #pragma unroll
-            for (int i = 0; i < kItems; ++i) rank[i] = split_digit(key[i], shift, dbase, dmult);
+            for (int i = 0; i < kItems; ++i) {
+                const uint32_t e = tid + i * kThreads;
+                rank[i] = e < count ? split_digit(keys[e] ^ A.flip_in, shift, dbase, dmult) : (uint32_t)kRadix;
+            }
         }
         if (A.tile_skew[t]) {  // uniform per CTA: see tile_skew_flag
             const uint32_t lt_mask = (1u << lane) - 1u;
 #pragma unroll
             for (int i = 0; i < kItems; ++i) {
-                const uint32_t d = wbase + i * 32 < count ? rank[i] : (uint32_t)kRadix;
+                const uint32_t d = rank[i];
                 const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
                 const uint32_t eq = __ballot_sync(0xffffffffu, d == d0);
                 uint32_t b0 = 0;
@@ -1769,48 +1772,51 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 2 : 4) void k_split(con
             }
         } else {
 #pragma unroll
-            for (int i = 0; i < kItems; ++i) {
-                if (wbase + i * 32 < count) rank[i] |= atomicAdd(&s_total[rank[i]], 1u) << 8;
-            }
+            for (int i = 0; i < kItems; ++i)
+                if (rank[i] < (uint32_t)kRadix) rank[i] |= atomicAdd(&s_total[rank[i]], 1u) << 8;
         }
         __syncthreads();
+        if (direct) {
+#pragma unroll
+            for (int i = 0; i < kItems; ++i) {
+                const uint32_t e = tid + i * kThreads;
+                if (e < count) put(s_gbase[rank[i] & 255u] + (rank[i] >> 8), e);
+            }
+            return;
+        }
         scan256_smem<kThreads>(s_total, s_start, s_warp);
+        if (tid < kRadix) s_gbase[tid] = off_d - s_start[tid];
 #pragma unroll
         for (int i = 0; i < kItems; ++i) {
-            if (wbase + i * 32 < count) {
-                const uint32_t d = rank[i] & 255u;
-                const uint32_t pos = s_start[d] + (rank[i] >> 8);
-                s_keys[pos] = key[i];
-                s_dg[pos] = (uint8_t)d;
+            const uint32_t e = tid + i * kThreads;
+            if (e < count) {
+                const uint32_t at = s_start[rank[i] & 255u] + (rank[i] >> 8);
+                s_idx[at] = (uint16_t)e;
+                if (SPL && bysplit) s_dg[at] = (uint8_t)rank[i];
             }
         }
     }
-
     // The tile's digit-d keys go to the offsets the statistics scan assigned
     // to this tile (digit offset plus the earlier tiles' digit-d keys).
-    if (tid < kRadix)
-        s_gbase[tid] = seg_base + (uint64_t)A.tile_off[(uint64_t)t * kRadix + tid] - (uint64_t)s_start[tid];
     __syncthreads();
+    auto digit_at = [&](uint32_t j, uint64_t k) -> uint32_t {
+        if (SPL && bysplit) return s_dg[j];
+        return split_digit(k ^ A.flip_in, shift, dbase, dmult);
+    };
+#pragma unroll 4
     for (uint32_t j = tid; j < count; j += kThreads) {
-        const uint64_t k = s_keys[j];
-        const uint32_t d = s_dg[j];
-        const uint64_t dst = s_gbase[d] + j;
-        if (dst - seg_base >= seg_n) {  // never taken when the digit offsets are consistent
-            atomicOr(A.err, kDevErrBounds);
-            continue;
-        }
-        kout[dst] = k ^ flip_out;
-        if (PAY) pout[dst] = s_pay[j];
+        const uint32_t e = s_idx[j];
+        put(s_gbase[digit_at(j, keys[e])] + j, e);
     }
     if (gather) {  // uniform per CTA
         // Smallest and largest key of every sub-bucket the next level splits
-        // again (its digit range there).  The staged keys come in digit runs,
-        // so a warp usually reduces one run and issues one atomic pair.
+        // again (its digit range there).  The keys come in digit runs, so a
+        // warp usually reduces one run and issues one atomic pair.
         for (uint32_t j0 = (uint32_t)w * 32; j0 < count; j0 += kThreads) {
             const uint32_t j = j0 + lane;
             const bool v = j < count;
-            const uint64_t k = v ? s_keys[j] : 0ull;
-            const uint32_t d = v ? (uint32_t)s_dg[j] : 0x1ffu;
+            const uint64_t raw = v ? keys[s_idx[j]] : 0ull, k = raw ^ A.flip_in;
+            const uint32_t d = v ? digit_at(j, raw) : 0x1ffu;
             const bool flagged = v && ((s_mask[d >> 5] >> (d & 31)) & 1u);
             const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
             if (__all_sync(0xffffffffu, d == d0)) {
@@ -2072,10 +2078,11 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
         A.err = ws.err;
         A.scatter = scatter;
         A.flip_in = L.flip_in; A.flip_out = fout;
-        const size_t smem = (size_t)kOsTile * 9 + (PAY ? (size_t)kOsTile * 4 : 0);
+        const size_t smem = bysplit_level ? split_smem<PAY, true>(child_interp) : split_smem<PAY, false>(child_interp);
+        const size_t smem_max = bysplit_level ? split_smem<PAY, true>(true) : split_smem<PAY, false>(true);
         // all of L1 as shared memory: the CTAs per SM are limited by their tiles
         const void* split_fn = bysplit_level ? (const void*)k_split<PAY, true> : (const void*)k_split<PAY, false>;
-        if ((e = ensure_func_attrs(split_fn, (int)smem, 100)) != cudaSuccess) return e;
+        if ((e = ensure_func_attrs(split_fn, (int)smem_max, 100)) != cudaSuccess) return e;
         const bool timed = timing && timing->enabled && timing->n < 16;
         if (timed) {
             cudaEventCreate(&timing->ev[timing->n][0]);
