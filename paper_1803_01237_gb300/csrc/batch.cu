@@ -223,8 +223,8 @@ __global__ __launch_bounds__(1024) void kb_count_scan(uint32_t P_tot, const uint
 // the compact sample buffer.
 __global__ __launch_bounds__(kSampThreads) void kb_sample_write(
     const uint64_t* __restrict__ skeys, const BJob* __restrict__ jobs, const uint32_t* __restrict__ job_of_seg,
-    const BCtl* __restrict__ ctl, const uint32_t* __restrict__ bitmap, const uint32_t* __restrict__ seg_cnt,
-    const uint64_t* __restrict__ G, const uint64_t* __restrict__ zoff, uint64_t* __restrict__ skey,
+    const BCtl* __restrict__ ctl, uint32_t* bitmap, const uint32_t* __restrict__ seg_cnt, const uint64_t* __restrict__ G,
+    const uint64_t* __restrict__ zoff, uint64_t* __restrict__ skey,
     uint32_t* __restrict__ sseg, uint32_t* __restrict__ sspos, uint32_t* __restrict__ siota) {
     __shared__ uint32_t s_warp[32];
     const uint32_t g = blockIdx.x;
@@ -234,39 +234,16 @@ __global__ __launch_bounds__(kSampThreads) void kb_sample_write(
     const BJob J = jobs[j];
     const uint32_t s = g - J.sbase;
     const uint64_t base = J.koff + seg_start(J, s), end = J.koff + seg_start(J, s + 1);
-    const uint64_t w0 = base >> 5, w1 = (end + 31) >> 5;
-    uint64_t out = zoff[j] + (G[g] - G[J.sbase]);
-    const uint64_t lim = zoff[j + 1];
-    uint32_t found = 0;
-    for (uint64_t wb = w0; wb < w1 && found < want; wb += kSampThreads) {
-        const uint64_t wi = wb + threadIdx.x;
-        uint32_t bits = 0;
-        if (wi < w1) {
-            bits = bitmap[wi];
-            const uint64_t g0 = wi << 5;
-            if (g0 < base) bits &= ~0u << (uint32_t)(base - g0);
-            if (g0 + 32 > end) bits &= (uint32_t)((1ull << (uint32_t)(end - g0)) - 1ull);
+    const uint64_t out = zoff[j] + (G[g] - G[J.sbase]), lim = zoff[j + 1];
+    take_marks(bitmap, base, end, want, s_warp, [&](uint64_t q, uint32_t at) {
+        const uint64_t o = out + at;
+        if (o < lim) {
+            skey[o] = skeys[q];
+            sseg[o] = s;
+            sspos[o] = (uint32_t)(q - base);
+            siota[o] = (uint32_t)o;
         }
-        if (__syncthreads_count(bits != 0u) == 0) continue;
-        const uint32_t c = __popc(bits);
-        uint32_t t;
-        const uint32_t incl = block_incl_scan<uint32_t>(c, 0u, AddU32(), s_warp, t);
-        uint64_t o = out + incl - c;
-        while (bits) {
-            const uint32_t b = __ffs(bits) - 1;
-            bits &= bits - 1;
-            const uint64_t q = (wi << 5) + b;
-            if (o < lim) {
-                skey[o] = skeys[q];
-                sseg[o] = s;
-                sspos[o] = (uint32_t)(q - base);
-                siota[o] = (uint32_t)o;
-            }
-            ++o;
-        }
-        out += t;
-        found += t;
-    }
+    });
 }
 
 __device__ __forceinline__ uint32_t job_of_slot(const uint64_t* __restrict__ zoff, uint32_t njobs, uint64_t k) {
@@ -631,7 +608,7 @@ __global__ __launch_bounds__(256) void kb_key_range(const uint64_t* __restrict__
 
 // Window of every bucket for the first split of the merge: its keys lie
 // between the job's final cuts b and b + 1 (tag order), clipped to the job's
-// key range; mulhi(key - lo, mult) maps that interval onto 0..255.
+// key range.
 __global__ void kb_bucket_hint(uint32_t P_tot, const BJob* __restrict__ jobs, const uint32_t* __restrict__ job_of_seg,
                                const DCut* __restrict__ Lcut, const DCut* __restrict__ Ucut,
                                const uint32_t* __restrict__ choose_u, const uint64_t* __restrict__ range,
@@ -654,7 +631,7 @@ __global__ void kb_bucket_hint(uint32_t P_tot, const BJob* __restrict__ jobs, co
     if (hi < lo) hi = lo;  // empty bucket
     const uint64_t r = hi - lo;
     lo_out[g] = lo;
-    mult_out[g] = r < 256 ? 0ull : (uint64_t)(((unsigned __int128)255 << 64) / r);
+    mult_out[g] = interp_hint(r, 256u);
 }
 
 // ---------------------------------------------------------------------------
@@ -838,7 +815,9 @@ int run_batch(const void* d_keys, const uint32_t* d_payload, int key_type, const
     HSS_LAUNCH(kb_init, njobs, 256, 0, st, jobs, ctl, jst, Lcut, Ucut, Lpos, Upos);
     HSS_LAUNCH(kb_intervals, njobs, 1024, 0, st, jobs, ctl, jst, Lcut, Ucut, res, int_rep, s);
     auto sampling = [&](uint32_t round) {
-        cudaMemsetAsync(bitmap, 0, (T.N_tot / 32 + 2) * 4, st);
+        // later rounds find the marks cleared by kb_sample_write (a failed job's
+        // stay, and are not looked at again)
+        if (round == 1) cudaMemsetAsync(bitmap, 0, (T.N_tot / 32 + 2) * 4, st);
         HSS_LAUNCH(kb_sample_mark, T.P_tot, kSampThreads, 0, st, jobs, jseg, ctl, jst, Lpos, Upos, Lcut, int_rep, round,
                    bitmap, seg_cnt);
         HSS_LAUNCH(kb_count_scan, 1, 1024, 0, st, T.P_tot, seg_cnt, G, njobs, jobs, ctl, jst, max_rounds, zoff, tot);

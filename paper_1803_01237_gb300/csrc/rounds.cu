@@ -263,44 +263,16 @@ __global__ __launch_bounds__(kSampThreads) void k_sample_write(
     if (want == 0) return;
     if (threadIdx.x == 0) seg_cnt[s] = 0;  // for the next round's marks
     const uint64_t base = seg_off[s], end = seg_off[s + 1];
-    const uint64_t w0 = base >> 5, w1 = (end + 31) >> 5;
     uint64_t out = seg_cnt_off[s];
-    uint32_t found = 0;
-    for (uint64_t wb = w0; wb < w1 && found < want; wb += kSampThreads) {
-        const uint64_t wi = wb + threadIdx.x;
-        uint32_t bits = 0;
-        if (wi < w1) {
-            bits = bitmap[wi];
-            const uint64_t g0 = wi << 5;
-            if (g0 < base) bits &= ~0u << (uint32_t)(base - g0);               // bits of the previous segment
-            if (g0 + 32 > end) bits &= (uint32_t)((1ull << (uint32_t)(end - g0)) - 1ull);  // bits of the next
-            // the next round's marks start from an empty bitmap (a word on
-            // the border keeps the neighbour's bits)
-            if (bits) {
-                if (g0 >= base && g0 + 32 <= end) bitmap[wi] = 0u;
-                else atomicAnd(&bitmap[wi], ~bits);
-            }
+    take_marks(bitmap, base, end, want, s_warp, [&](uint64_t g, uint32_t at) {
+        const uint64_t o = out + at;
+        if (o < cap) {
+            skey[o] = skeys[g];
+            sseg[o] = s;
+            sspos[o] = (uint32_t)(g - base);
+            siota[o] = (uint32_t)o;
         }
-        if (__syncthreads_count(bits != 0u) == 0) continue;
-        const uint32_t c = __popc(bits);
-        uint32_t tot;
-        const uint32_t incl = block_incl_scan<uint32_t>(c, 0u, AddU32(), s_warp, tot);
-        uint64_t o = out + incl - c;
-        while (bits) {
-            const uint32_t b = __ffs(bits) - 1;
-            bits &= bits - 1;
-            const uint64_t g = (wi << 5) + b;
-            if (o < cap) {
-                skey[o] = skeys[g];
-                sseg[o] = s;
-                sspos[o] = (uint32_t)(g - base);
-                siota[o] = (uint32_t)o;
-            }
-            ++o;
-        }
-        out += tot;
-        found += tot;
-    }
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -629,9 +601,8 @@ __global__ void k_finalize(uint32_t S, uint64_t N, uint32_t p, int key_type, con
 }
 
 // Bucket b holds keys between splitters b and b+1 (sentinels: the ends of the
-// key range).  Its first split interpolates that range onto 256 sub-buckets:
-// digit = mulhi(key - lo, floor(255 * 2^64 / (hi - lo))), monotone in the key
-// and at most 255; a range narrower than 256 uses key - lo itself.
+// key range).  Its first split interpolates that range onto 256 sub-buckets
+// (interp_hint).
 // Smallest and largest key of the whole input: the first and the last key of
 // the locally sorted segments.  One block.
 __global__ void __launch_bounds__(1024) k_key_range(const uint64_t* __restrict__ skeys,
@@ -662,7 +633,7 @@ __global__ void __launch_bounds__(1024) k_key_range(const uint64_t* __restrict__
 
 // Interpolation hint of each bucket for the first digit split of the merge:
 // the bucket's keys lie between splitters b and b+1, clipped to the input's
-// key range, and mulhi(key - lo, mult) maps that interval onto 0..255.
+// key range.
 __global__ void k_bucket_hint(uint32_t p, const uint64_t* __restrict__ fin_okey, const uint32_t* __restrict__ fin_kind,
                               const uint64_t* __restrict__ range, uint64_t* __restrict__ lo_out,
                               uint64_t* __restrict__ mult_out) {
@@ -680,10 +651,8 @@ __global__ void k_bucket_hint(uint32_t p, const uint64_t* __restrict__ fin_okey,
     uint64_t hi = min(bound(b + 1, ~0ull), kmax);
     if (hi < lo) hi = lo;  // empty bucket
     const uint64_t r = hi - lo;
-    // mult = 0 selects the plain form ((key >> 0) - lo) & 255 = key - lo
-    const uint64_t mult = r < 256 ? 0ull : (uint64_t)(((unsigned __int128)255 << 64) / r);
     lo_out[b] = lo;
-    mult_out[b] = mult;
+    mult_out[b] = interp_hint(r, 256u);
 }
 
 cudaError_t bucket_hints(const RoundWs& ws, const uint64_t* skeys, const uint64_t* d_seg_off, uint32_t p,

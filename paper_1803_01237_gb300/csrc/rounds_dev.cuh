@@ -368,4 +368,53 @@ __device__ __forceinline__ void mark_pairs(const PairDraw& pd, const uint32_t* s
     }
 }
 
+// The marked positions g in [base, end) of the bitmap, in order, by the CTA
+// (kSampThreads): body(g, number of marks before it).  want: how many there
+// are.  The marks are cleared on the way, for the next round (a word on the
+// border keeps the neighbour's bits).  Marks are rare, so the pass is bound by
+// its steps over empty words: a thread reads four words a step (2^28 positions
+// in 4096 segments: 35 us a round by single words, 22 by four).
+template <class Body>
+__device__ __forceinline__ void take_marks(uint32_t* bitmap, uint64_t base, uint64_t end, uint32_t want, uint32_t* s_warp,
+                                           Body body) {
+    const uint64_t v0 = base >> 7, v1 = (end + 127) >> 7;  // vectors of 128 positions
+    uint32_t found = 0;
+    for (uint64_t vb = v0; vb < v1 && found < want; vb += kSampThreads) {
+        const uint64_t vi = vb + threadIdx.x;
+        uint32_t bits[4] = {0u, 0u, 0u, 0u};
+        if (vi < v1) {
+            uint4 x;
+            if (((uintptr_t)bitmap & 15u) == 0) x = ((const uint4*)bitmap)[vi];
+            else x = make_uint4(bitmap[4 * vi], bitmap[4 * vi + 1], bitmap[4 * vi + 2], bitmap[4 * vi + 3]);  // a workspace off 16 bytes
+            bits[0] = x.x; bits[1] = x.y; bits[2] = x.z; bits[3] = x.w;
+            if (x.x | x.y | x.z | x.w) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const uint64_t g0 = (vi << 7) + 32 * k;
+                    if (g0 + 32 <= base || g0 >= end) { bits[k] = 0u; continue; }
+                    const bool whole = g0 >= base && g0 + 32 <= end;
+                    if (g0 < base) bits[k] &= ~0u << (uint32_t)(base - g0);                               // the previous segment's
+                    if (g0 + 32 > end) bits[k] &= (uint32_t)((1ull << (uint32_t)(end - g0)) - 1ull);      // the next one's
+                    if (bits[k]) {
+                        if (whole) bitmap[4 * vi + k] = 0u;
+                        else atomicAnd(&bitmap[4 * vi + k], ~bits[k]);
+                    }
+                }
+            }
+        }
+        const uint32_t c = __popc(bits[0]) + __popc(bits[1]) + __popc(bits[2]) + __popc(bits[3]);
+        if (__syncthreads_or(c) == 0) continue;
+        uint32_t tot;
+        uint32_t at = found + block_incl_scan<uint32_t>(c, 0u, AddU32(), s_warp, tot) - c;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            while (bits[k]) {
+                const uint32_t b = __ffs(bits[k]) - 1;
+                bits[k] &= bits[k] - 1;
+                body((vi << 7) + 32 * k + b, at++);
+            }
+        found += tot;
+    }
+}
+
 }  // namespace hss

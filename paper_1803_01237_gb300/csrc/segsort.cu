@@ -153,25 +153,10 @@ SegSortWs segsort_ws_carve(void* base, uint64_t N, uint64_t nseg, uint32_t* err)
 }
 
 // Digit of the first split of a segment: an 8-bit window of the key, or (mult
-// != 0) a linear interpolation of the segment's key range onto 0..255.
+// != 0) an interpolation of the segment's key range onto 0..255 (interp_digit).
 __device__ __forceinline__ uint32_t split_digit(uint64_t key, int shift, uint64_t base, uint64_t mult) {
-    if (mult) return min((uint32_t)__umul64hi(key - base, mult), 255u);
+    if (mult) return interp_digit(key - base, mult);
     return (uint32_t)((key >> shift) - base) & 255u;
-}
-
-// Multiplier m of an interpolating digit mulhi(x - lo, m) of a key range of
-// width `range` onto 0..R-1: about (R-1) 2^64 / range, in single precision.
-// Any m keeps the digit monotone in the key (callers clamp it to R-1); this
-// one spreads the range evenly.  (Double precision is far slower here and
-// buys nothing.)
-__device__ __forceinline__ uint64_t interp_mult(uint64_t range, uint32_t R) {
-    if (range < (uint64_t)R) return 0ull;
-    return __float2ull_rz((float)(R - 1) * 18446744073709551616.0f / (float)range);
-}
-// The same for 32-bit offsets: mulhi(x - lo, m) onto 0..R-1.
-__device__ __forceinline__ uint32_t interp_mult32(uint32_t range, uint32_t R) {
-    if (range < R) return 0u;
-    return __float2uint_rz((float)(R - 1) * 4294967296.0f / (float)range);
 }
 
 // ---------------------------------------------------------------------------
@@ -1125,8 +1110,22 @@ __device__ __forceinline__ void plan_entries(uint64_t s, const PlanV& item, cons
         const uint32_t id = off.c[3] + v.c[3] - 1;
         P.large_id[s] = id;
         P.large_seg[id] = (uint32_t)s;
-        const uint32_t t0 = off.c[4] + v.c[4] - item.c[4];
-        for (uint32_t u = 0; u < item.c[4]; ++u) P.tile_seg[t0 + u] = (uint32_t)s;
+    }
+}
+// The tiles of the warp's segments (t0: the first tile of the lane's, c: their
+// number).  Long rows by the whole warp, one after the other: a lane writing
+// its own row alone took 39 us for 1024 segments of 64 tiles.
+__device__ __forceinline__ void plan_tiles(uint32_t s, uint32_t t0, uint32_t c, uint32_t* __restrict__ tile_seg) {
+    if (__reduce_max_sync(0xffffffffu, c) <= 4u) {
+        for (uint32_t u = 0; u < c; ++u) tile_seg[t0 + u] = s;
+        return;
+    }
+    const uint32_t lane = threadIdx.x & 31;
+    for (uint32_t left = __ballot_sync(0xffffffffu, c > 0u); left; left &= left - 1) {
+        const int from = __ffs(left) - 1;
+        const uint32_t cs = __shfl_sync(0xffffffffu, s, from), ct = __shfl_sync(0xffffffffu, t0, from),
+                       cc = __shfl_sync(0xffffffffu, c, from);
+        for (uint32_t u = lane; u < cc; u += 32) tile_seg[ct + u] = cs;
     }
 }
 
@@ -1139,7 +1138,9 @@ __global__ __launch_bounds__(1024) void k_plan_write(const uint64_t* __restrict_
     if (s < nseg && seg_hi[s] - seg_lo[s] >= kMaxSegKeys) atomicOr(P.err, kDevErrSize);
     PlanV v = item, tot;
     plan_scan(v, tot);
-    if (s < nseg) plan_entries(s, item, v, blk_load(blk, blockIdx.x), P);
+    const PlanV off = blk_load(blk, blockIdx.x);
+    if (s < nseg) plan_entries(s, item, v, off, P);
+    plan_tiles((uint32_t)s, off.c[4] + v.c[4] - item.c[4], item.c[4], P.tile_seg);
     if (s == nseg) P.tile_start[nseg] = counters[20];
 }
 
@@ -1158,6 +1159,7 @@ __global__ __launch_bounds__(1024) void k_plan_one(const uint64_t* __restrict__ 
         PlanV v = item, tot;
         plan_scan(v, tot);
         if (s < nseg) plan_entries(s, item, v, carry, P);
+        plan_tiles((uint32_t)s, carry.c[4] + v.c[4] - item.c[4], item.c[4], P.tile_seg);
 #pragma unroll
         for (int k = 0; k < 5; ++k) carry.c[k] += tot.c[k];
         carry.keys += tot.keys;
@@ -1383,39 +1385,39 @@ __global__ __launch_bounds__(256) void k_tile_stats(const uint64_t* __restrict__
 
 // Recount of the tiles of segments whose top varying byte (from the OR/AND of
 // the statistics pass) is not the speculative one: the histogram of that byte
-// into the tile's second row.  Other CTAs return at once.
-__global__ __launch_bounds__(256) void k_tile_recount(const uint64_t* __restrict__ kin, const uint64_t* __restrict__ seg_lo,
-                                                      const uint64_t* __restrict__ seg_hi, uint64_t nseg,
-                                                      const uint32_t* __restrict__ tile_start,
-                                                      const uint32_t* __restrict__ tile_seg,
-                                                      const uint32_t* __restrict__ large_id, uint16_t* __restrict__ tile_hist,
-                                                      uint8_t* __restrict__ tile_skew, const uint8_t* __restrict__ spl_mode,
-                                                      const unsigned long long* __restrict__ vor,
-                                                      const unsigned long long* __restrict__ vand,
-                                                      const uint32_t* __restrict__ spec, uint64_t flip_in) {
-    // A grid of a few CTAs per SM walks the tiles: most levels recount few
-    // or none, and a CTA per tile would cost a launch of tens of thousands of
-    // CTAs that all return at once.
+// into the tile's second row.  A unit of work is every kRecountUnits-th tile
+// of a segment, so the segments that need none (most) cost a check per unit
+// and not one per tile (2^28 keys in 1024 segments, none to do: 63 -> 11 us).
+constexpr uint32_t kRecountUnits = 8;
+__global__ __launch_bounds__(256) void k_tile_recount(
+    const uint64_t* __restrict__ kin, const uint64_t* __restrict__ seg_lo, const uint64_t* __restrict__ seg_hi,
+    const uint32_t* __restrict__ counters, const uint32_t* __restrict__ large_seg, const uint32_t* __restrict__ tile_start,
+    uint16_t* __restrict__ tile_hist, uint8_t* __restrict__ tile_skew, const uint8_t* __restrict__ spl_mode,
+    const unsigned long long* __restrict__ vor, const unsigned long long* __restrict__ vand,
+    const uint32_t* __restrict__ spec, uint64_t flip_in) {
     __shared__ uint32_t s_h[kRadix];
-    const uint32_t total = tile_start[nseg];
-    for (uint32_t t = blockIdx.x; t < total; t += gridDim.x) {  // uniform per CTA
-        const uint32_t s = tile_seg[t], id = large_id[s];
+    const uint64_t units = (uint64_t)counters[19] * kRecountUnits;
+    for (uint64_t unit = blockIdx.x; unit < units; unit += gridDim.x) {  // uniform per CTA
+        const uint32_t id = (uint32_t)(unit / kRecountUnits);
         if (spl_mode && spl_mode[id]) continue;  // the statistics pass counted the splitter buckets
         const unsigned long long vary = vor[id] ^ vand[id];
         if (vary == 0ull) continue;
         const uint32_t w = (uint32_t)(63 - __clzll((long long)vary)) >> 3;
         if (w == spec[id]) continue;
-        s_h[threadIdx.x] = 0;
-        __syncthreads();
+        const uint32_t s = large_seg[id], t0 = tile_start[s], t1 = tile_start[s + 1];
         const uint64_t lo = seg_lo[s], n = seg_hi[s] - lo;
-        const uint64_t a = (uint64_t)(t - tile_start[s]) * kOsTile, b = min(n, a + kOsTile);
         const int sh = 8 * (int)w;
+        for (uint32_t t = t0 + (uint32_t)(unit % kRecountUnits); t < t1; t += kRecountUnits) {
+            s_h[threadIdx.x] = 0;
+            __syncthreads();
+            const uint64_t a = (uint64_t)(t - t0) * kOsTile, b = min(n, a + kOsTile);
 #pragma unroll 4
-        for (uint64_t e = a + threadIdx.x; e < b; e += 256)
-            atomicAdd(&s_h[(uint32_t)((kin[lo + e] ^ flip_in) >> sh) & 255u], 1u);
-        __syncthreads();
-        tile_hist[(uint64_t)t * (2 * kRadix) + kRadix + threadIdx.x] = (uint16_t)s_h[threadIdx.x];
-        tile_skew_flag(s_h[threadIdx.x], tile_skew, t);  // ends with a barrier
+            for (uint64_t e = a + threadIdx.x; e < b; e += 256)
+                atomicAdd(&s_h[(uint32_t)((kin[lo + e] ^ flip_in) >> sh) & 255u], 1u);
+            __syncthreads();
+            tile_hist[(uint64_t)t * (2 * kRadix) + kRadix + threadIdx.x] = (uint16_t)s_h[threadIdx.x];
+            tile_skew_flag(s_h[threadIdx.x], tile_skew, t);  // ends with a barrier
+        }
     }
 }
 
@@ -1849,7 +1851,8 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 3 : 5) void k_split(con
 // its own key range [min, max] interpolated onto 2^b sub-buckets, b chosen so
 // that they hold about `target` keys on average; a sub-bucket of one key
 // value keeps multiplier 0.  An interpolated split into 2^b sub-buckets
-// narrows the key range by a factor 2^b - 1 >= 2^(b-1) whatever the keys, so
+// narrows the key range by a factor of about 2^b - 1, and (rounding of short
+// ranges included) of at least 2^(b-1) for b >= 2, whatever the keys, so
 // b is at least ceil(B / levels) + 1 for a range of B bits and `levels`
 // levels left before the depth limit (one kept for the copy of single-valued
 // sub-buckets): clustered keys with a few outliers then still end within the
@@ -1870,7 +1873,7 @@ __global__ void k_child_hints(uint32_t n_children, const uint64_t* __restrict__ 
     const uint32_t B = hi > lo ? 64u - (uint32_t)__clzll((long long)(hi - lo)) : 0u;
     const uint32_t b_min = levels >= 1 ? min(8u, (B + (uint32_t)levels - 1u) / (uint32_t)levels + 1u) : 8u;
     b = max(b, b_min);
-    cmult[c] = interp_mult(hi - lo, 1u << b);
+    cmult[c] = interp_hint(hi - lo, 1u << b);
 }
 
 __global__ void k_even_offsets(uint64_t* __restrict__ seg_off, uint64_t N, uint64_t p) {
@@ -2054,10 +2057,9 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
                        ws.large_id, ws.tile_hist, ws.tile_skew, ws.vor, ws.vand, L.hint_lo, L.hint_mult, L.hint_hi,
                        prev_shift, ws.spec, L.flip_in, nullptr, nullptr);
         if (!L.hint_lo)
-            HSS_LAUNCH(k_tile_recount, (unsigned)std::min<uint64_t>(tiles, (uint64_t)num_sms() * 8), 256, 0, st, L.in,
-                       L.seg_lo, L.seg_hi, L.nseg, ws.tile_start, ws.tile_seg, ws.large_id,
-                       ws.tile_hist, ws.tile_skew, bysplit_level ? ws.spl_mode : nullptr, ws.vor, ws.vand, ws.spec,
-                       L.flip_in);
+            HSS_LAUNCH(k_tile_recount, (unsigned)std::min<uint64_t>((uint64_t)n_large * kRecountUnits, (uint64_t)num_sms() * 8),
+                       256, 0, st, L.in, L.seg_lo, L.seg_hi, ws.counters, ws.large_seg, ws.tile_start, ws.tile_hist,
+                       ws.tile_skew, bysplit_level ? ws.spl_mode : nullptr, ws.vor, ws.vand, ws.spec, L.flip_in);
         HSS_LAUNCH(k_msd_prep, n_large, 256, 0, st, L.seg_lo, ws.large_seg, ws.counters, ws.tile_start, ws.tile_hist,
                    ws.vor, ws.vand, L.hint_lo, L.hint_mult, ws.msd_base, ws.msd_mult, ws.msd_shift[buf], ws.spec,
                    ws.direct, ws.sub_lo[buf], ws.sub_hi[buf], ws.tile_off, child_interp ? chip_max : 0xffffffffu,

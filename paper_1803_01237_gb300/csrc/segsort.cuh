@@ -111,9 +111,9 @@ struct SegSortTiming {
 // sign bit into keys as they are read (signed keys), flip_out as they are
 // written.  psrc/pdst/ptmp are all null or all non-null.  hint_lo and
 // hint_mult (both null or both per segment) promise that every key k of
-// segment s satisfies hint_lo[s] <= k and mulhi(k - hint_lo[s], hint_mult[s])
-// <= 255; the first split of s then uses that value, which is monotone in k,
-// as its digit (an interpolation of the key range over 256 sub-buckets).
+// segment s satisfies hint_lo[s] <= k <= hint_lo[s] + range, hint_mult[s] being
+// interp_hint(range, 256); the first split of s then interpolates that range
+// over 256 sub-buckets.
 cudaError_t segsort(const uint64_t* src, uint64_t* dst, uint64_t* tmp,
                     const uint32_t* psrc, uint32_t* pdst, uint32_t* ptmp,
                     uint64_t N, uint64_t nseg, const uint64_t* d_seg_off,
@@ -124,6 +124,24 @@ cudaError_t segsort(const uint64_t* src, uint64_t* dst, uint64_t* tmp,
 // Process-wide tuning of the sort (hss_set_tuning / hss_get_tuning).
 int set_tuning(const hss_tuning* t);
 void get_tuning(hss_tuning* t);
+
+// The interpolating digit of a key range [lo, lo + range] onto 0..R-1: x, the
+// upper 24 bits of key - lo below the range's highest bit, times (R-1) 2^32 /
+// (the range's x), upper half.  Monotone in the key.  interp_hint packs the
+// shift (one more, so that the hint is never 0) and the multiplier; 0 for a
+// range narrower than R, whose digit is key - lo itself.  One 32-bit product
+// per key (statistics pass of a merge of 2^28 keys: 413 us with a 64-bit
+// multiplier, 401 with this).  24 bits of each factor leave the sub-buckets
+// even to 2^-15; digits above 255 (keys outside the range) are cut.
+__device__ __forceinline__ uint64_t interp_hint(uint64_t range, uint32_t R) {
+    if (range < (uint64_t)R) return 0ull;
+    const uint32_t shift = (uint32_t)max(0, 40 - __clzll((long long)range));
+    const uint32_t mult = (uint32_t)(((uint64_t)(R - 1) << 32) / (range >> shift));  // range >> shift >= R
+    return (uint64_t)(shift + 1) << 32 | mult;
+}
+__device__ __forceinline__ uint32_t interp_digit(uint64_t off, uint64_t hint) {
+    return min(__umulhi((uint32_t)(off >> ((uint32_t)(hint >> 32) - 1u)), (uint32_t)hint), 255u);
+}
 
 // seg_off[s] = floor(s * N / p) for s = 0..p.
 cudaError_t fill_even_offsets(uint64_t* d_seg_off, uint64_t N, uint64_t p, cudaStream_t st);
