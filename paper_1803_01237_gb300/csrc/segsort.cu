@@ -1600,10 +1600,11 @@ struct SplitArgs {
 template <bool PAY>
 constexpr int split_threads() { return PAY ? 512 : 256; }
 
+constexpr int kCellShift = 4;  // splitter digits, keys alone: a cell of the digit order is 16 keys
 template <bool PAY, bool SPL>
 constexpr size_t split_smem(bool gather) {
     return (size_t)(kOsTile + 2) * 8 + (PAY ? (size_t)(kOsTile + 8) * 4 : 0) + (size_t)kOsTile * 2 +
-           (SPL ? (size_t)kOsTile : 0) + (PAY ? (size_t)(split_threads<PAY>() / 32) * kRadix * 2 : 0) +
+           (SPL && PAY ? (size_t)kOsTile : 0) + (PAY ? (size_t)(split_threads<PAY>() / 32) * kRadix * 2 : 0) +
            (gather ? 2 * (size_t)kRadix * 8 : 0);
 }
 
@@ -1626,13 +1627,15 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 3 : 5) void k_split(con
     uint32_t* s_pay = (uint32_t*)(s_keys + kOsTile + 2);           // kOsTile + 8 (PAY): payload e at [e + po]
     uint16_t* s_hist = (uint16_t*)(s_pay + (PAY ? kOsTile + 8 : 0));  // kWarps * 256 (PAY)
     uint16_t* s_idx = s_hist + (PAY ? kWarps * kRadix : 0);        // kOsTile: the keys in digit order
-    uint8_t* s_dg = (uint8_t*)(s_idx + kOsTile);                   // kOsTile (SPL): their digits
-    uint64_t* s_mn = (uint64_t*)(s_dg + (SPL ? kOsTile : 0));      // 2 x 256 (gather): key ranges of sub-buckets
+    uint8_t* s_dg = (uint8_t*)(s_idx + kOsTile);                   // kOsTile (SPL, PAY): their digits
+    uint64_t* s_mn = (uint64_t*)(s_dg + (SPL && PAY ? kOsTile : 0));  // 2 x 256 (gather): key ranges of sub-buckets
     uint64_t* s_mx = s_mn + kRadix;
     __shared__ uint32_t s_total[kRadix], s_start[kRadix];
     __shared__ uint32_t s_gbase[kRadix];  // start of the digit's run in the segment, less its start in the tile
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_spl[SPL ? kRadix : 1];
+    __shared__ uint8_t s_cell[SPL && !PAY ? kRadix : 1];  // digit of the cell's first key in digit order
+    static_assert((kOsTile >> kCellShift) == kRadix, "a cell per thread");
     __shared__ uint32_t s_mask[8];
     __shared__ uint64_t s_bar;
 
@@ -1708,6 +1711,20 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 3 : 5) void k_split(con
         }
         kout[dst] = keys[e] ^ flip;
         if (PAY) pout[dst] = pays[e];
+    };
+    // SPL, keys alone: the digit of place j in digit order, the last of [lo, hi]
+    // that starts at or before j.  Two neighbouring cells bound it: a cell per
+    // 16 keys and a step or two of search take 256 bytes, where a digit per key
+    // takes 4 KB and with it one of five CTAs of an SM (2^28 uniform keys, a
+    // level that may split on splitters: 1090 us with those, 975 with cells).
+    // With a payload three CTAs fit either way and the digits are cheaper (2.12
+    // against 2.24 ms).
+    auto last_start = [&](uint32_t lo, uint32_t hi, uint32_t j) -> uint32_t {
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi + 1) >> 1;
+            if (s_start[mid] <= j) lo = mid; else hi = mid - 1;
+        }
+        return lo;
     };
     if constexpr (PAY) {
         // Each key's digit once, byte-packed (past the segment the last one).
@@ -1788,21 +1805,23 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 3 : 5) void k_split(con
         }
         scan256_smem<kThreads>(s_total, s_start, s_warp);
         if (tid < kRadix) s_gbase[tid] = off_d - s_start[tid];
+        if (SPL && bysplit && tid < kRadix)
+            s_cell[tid] = (uint8_t)last_start(0u, kRadix - 1u, (uint32_t)tid << kCellShift);
 #pragma unroll
         for (int i = 0; i < kItems; ++i) {
             const uint32_t e = tid + i * kThreads;
-            if (e < count) {
-                const uint32_t at = s_start[rank[i] & 255u] + (rank[i] >> 8);
-                s_idx[at] = (uint16_t)e;
-                if (SPL && bysplit) s_dg[at] = (uint8_t)rank[i];
-            }
+            if (e < count) s_idx[s_start[rank[i] & 255u] + (rank[i] >> 8)] = (uint16_t)e;
         }
     }
     // The tile's digit-d keys go to the offsets the statistics scan assigned
     // to this tile (digit offset plus the earlier tiles' digit-d keys).
     __syncthreads();
     auto digit_at = [&](uint32_t j, uint64_t k) -> uint32_t {
-        if (SPL && bysplit) return s_dg[j];
+        if (SPL && PAY && bysplit) return s_dg[j];
+        if (SPL && bysplit) {
+            const uint32_t c = j >> kCellShift;
+            return last_start(s_cell[c], c + 1 < (uint32_t)kRadix ? s_cell[c + 1] : (uint32_t)kRadix - 1u, j);
+        }
         return split_digit(k ^ A.flip_in, shift, dbase, dmult);
     };
 #pragma unroll 4
