@@ -69,13 +69,15 @@ extern "C" {
 #define HSS_FLAG_SYNC 1u     /* synchronize `stream` before returning */
 #define HSS_FLAG_TIMING 2u   /* record per-phase device times into hss_stats (implies SYNC) */
 /* Histogram form of the splitter rounds (Sec. 3.3 step 2; the result is the
- * same either way).  By default each round chooses: when all its probes
- * share one interval (round 1) and searching every segment for every probe
+ * same either way).  By default each round chooses: with few keys of a
+ * segment between two probes (one per probe and segment at most in round 1, an
+ * eighth later; 2^24 positions at least) each segment is walked along the
+ * sorted probes; when all its probes share one interval (round 1) and searching every segment for every probe
  * (Z p log2(N/p) dependent loads) would cost more than eight reads of the
  * keys, a staged form ranks blocks of sorted probes against the keys between
  * the block's first and last probe, staged in shared memory; else every
- * probe is searched in every segment.  These flags force one form (at most
- * one may be set, else HSS_ERR_INVALID). */
+ * probe is searched in every segment.  These flags force the last form, or the
+ * staged one where it applies (at most one may be set, else HSS_ERR_INVALID). */
 #define HSS_FLAG_HIST_PROBE 4u
 #define HSS_FLAG_HIST_STAGED 8u
 /* Drivers of the splitter rounds.  A call whose round sample fits one

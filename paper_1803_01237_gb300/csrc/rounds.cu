@@ -313,6 +313,29 @@ __global__ __launch_bounds__(256) void k_probe_build(
 
 constexpr int kHistSegPerBlock = 64;  // k_rank_cuts
 
+// The form of a round's histogram (Z probes in nint intervals of gamma keys).
+// Walks need few keys of a segment between two probes, and enough work to fill
+// the chip.  One interval, p = 4096, round 1 (keys per probe and segment:
+// staged, walk): 0.4: 685, 373 us; 0.8: 777, 680; 1.6: 880, 1650.  Many
+// intervals, each begun by loads of its own (search, walk): 0.04: 298, 271;
+// 0.08: 344, 313; 0.15: 367, 370; 0.3: 413, 461.  The staged form pays when the
+// searches (Z p log2(N/p) dependent loads) would cost several reads of the keys.
+constexpr uint32_t kFormSearch = 0, kFormStaged = 1, kFormWalk = 2;
+constexpr double kWalkMin = (double)(1ull << 24);   // positions per round, at least
+constexpr double kWalkKeysOne = 1.0, kWalkKeysMany = 0.125;  // keys per position, at most
+__host__ __device__ __forceinline__ bool staged_pays(double Z, uint64_t N, uint32_t p) {
+    return Z * (double)p * log2((double)N / (double)p + 2.0) >= 8.0 * (double)N;
+}
+__host__ __device__ __forceinline__ uint32_t hist_form(double Z, uint64_t N, uint32_t p, uint32_t nint, double gamma,
+                                                       uint32_t hist_mode) {
+    const double positions = Z * (double)p;
+    if (hist_mode == kHistAuto && positions >= kWalkMin &&
+        gamma <= (nint == 1 ? kWalkKeysOne : kWalkKeysMany) * positions)
+        return kFormWalk;
+    const bool staged = nint == 1 && hist_mode != kHistProbe && (hist_mode == kHistStaged || staged_pays(Z, N, p));
+    return staged ? kFormStaged : kFormSearch;
+}
+
 // Segments each warp of k_histogram walks: eight, or fewer where that would
 // leave the SMs short of warps (a walk is a chain of dependent loads per
 // segment: 1250 probes over 256 segments took 16 us by eights, 7 by ones).
@@ -329,8 +352,8 @@ __global__ __launch_bounds__(256) void k_histogram(
     uint64_t cap, uint32_t* __restrict__ err, const RoundCtl* __restrict__ ctl, uint32_t per_warp) {
     __shared__ uint64_t s_part[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (Z == kZFromCtl) {  // device-driven loop: this form runs unless the round is staged
-        if (ctl->staged) return;
+    if (Z == kZFromCtl) {  // device-driven loop: this form runs when the round searches
+        if (ctl->form != kFormSearch) return;
         Z = ctl->seg_off_z[1];
         if ((uint64_t)blockIdx.x * 32 >= Z) return;
     }
@@ -394,7 +417,7 @@ __global__ __launch_bounds__(kStgThreads) void k_histogram_staged(
     __shared__ uint64_t s_keys[kStgCap];
     __shared__ uint32_t s_lo[kStgSegs], s_a[kStgSegs], s_b[kStgSegs], s_ok[kStgSegs];
     if (Z == kZFromCtl) {  // device-driven loop: this form runs only when the round is staged
-        if (!ctl->staged) return;
+        if (ctl->form != kFormStaged) return;
         Z = ctl->seg_off_z[1];
     }
     const uint64_t k0 = (uint64_t)blockIdx.x * kStgProbes;
@@ -465,6 +488,129 @@ __global__ __launch_bounds__(kStgThreads) void k_histogram_staged(
     for (int u = 0; u < kStgPer; ++u) {
         const uint64_t k = k0 + threadIdx.x + (uint64_t)u * kStgThreads;
         if (k < k1) atomicAdd((unsigned long long*)&prank[k], (unsigned long long)part[u]);
+    }
+}
+
+// The histogram of many probes in short segments (a few keys of a segment
+// between two probes, or fewer): a lane owns a segment and walks through its
+// keys along a chunk of the sorted probes, from the position of the first one;
+// a cut's position is where the walk stands.  The positions of 32 segments and
+// kWalkTile probes are turned in shared memory, so that rows are written whole
+// and a probe's positions are added up by one lane.  Same positions as
+// k_histogram, without a chain of loads per position.  A probe that is
+// kWalkSteps keys further on is searched.  Bound by issue (70 instructions per
+// probe and warp) and by the sectors of each lane's own keys and bounds.
+constexpr int kWalkThreads = 256;
+constexpr uint32_t kWalkChunk = 256;  // probes per CTA at most
+constexpr int kWalkTile = 16;
+constexpr int kWalkPerSm = 6;         // CTAs per SM
+constexpr uint32_t kWalkSteps = 6;
+// Probes per CTA: long walks (each begins with a search) in full waves of CTAs.
+static uint32_t walk_chunk(double Z, uint32_t p) {
+    const double rows = (double)cdiv(p, kWalkThreads), wave = (double)(kWalkPerSm * device_sm_count());
+    for (double waves = 1.0;; waves += 1.0) {
+        const double chunks = std::max(1.0, std::floor(waves * wave / rows));
+        const double c = std::ceil(Z / chunks / kWalkTile) * kWalkTile;
+        if (c <= (double)kWalkChunk) return (uint32_t)std::max(32.0, c);
+    }
+}
+
+__global__ __launch_bounds__(kWalkThreads, kWalkPerSm) void k_histogram_walk(
+    const uint64_t* __restrict__ skeys, const uint64_t* __restrict__ seg_off, uint32_t p, uint32_t S,
+    const uint32_t* __restrict__ Lpos, const uint32_t* __restrict__ Upos, const uint32_t* __restrict__ int_rep,
+    const uint64_t* __restrict__ pkey, const int32_t* __restrict__ pseg, const uint32_t* __restrict__ pspos,
+    const uint32_t* __restrict__ pint, uint64_t Z, uint64_t* __restrict__ prank, uint32_t* __restrict__ probe_pos,
+    uint64_t cap, uint32_t* __restrict__ err, const RoundCtl* __restrict__ ctl, uint32_t chunk) {
+    constexpr int kRow = kWalkTile + 1;
+    __shared__ __align__(16) uint4 s_probe[kWalkChunk];  // key, segment, interval
+    __shared__ uint32_t s_spos[kWalkChunk];
+    __shared__ uint32_t s_tile[kWalkThreads / 32][32 * kRow];
+    if (Z == kZFromCtl) {  // device-driven loop: this form runs only when the round walks
+        if (ctl->form != kFormWalk) return;
+        Z = ctl->seg_off_z[1];
+    }
+    const uint64_t k0 = (uint64_t)blockIdx.x * chunk;
+    if (k0 >= Z) return;
+    const uint32_t cnt = (uint32_t)min((uint64_t)chunk, Z - k0);
+    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x < cnt) {
+        const uint64_t k = k0 + threadIdx.x;
+        const uint64_t key = pkey[k];
+        s_probe[threadIdx.x] = make_uint4((uint32_t)key, (uint32_t)(key >> 32), (uint32_t)pseg[k], int_rep[pint[k]]);
+        s_spos[threadIdx.x] = pspos[k];
+    }
+    __syncthreads();
+    const uint32_t sw = blockIdx.y * kWalkThreads + 32 * w;  // the warp's first segment
+    if (sw >= p) return;
+    const uint32_t s = sw + lane;
+    const uint64_t off = s < p ? seg_off[s] : 0ull;
+    const uint32_t n = s < p ? (uint32_t)(seg_off[s + 1] - off) : 0u;
+    const uint64_t* K = skeys + off;
+    uint32_t* tile = s_tile[w];
+    uint32_t cur = 0, hi = 0, rep = ~0u;
+    uint64_t kc = 0, kn = 0;  // the keys at cur and after it
+    auto fetch = [&]() {
+        if (cur < hi) kc = K[cur];
+        if (cur + 1 < hi) kn = K[cur + 1];
+    };
+    auto walk = [&](auto passes, uint64_t key, bool strict) {
+        uint32_t left = kWalkSteps;
+        while (cur < hi && passes(kc)) {
+            ++cur;
+            if (--left == 0) {
+                cur += count_below(K + cur, hi - cur, key, strict);
+                fetch();
+                break;
+            }
+            kc = kn;
+            if (cur + 1 < hi) kn = K[cur + 1];
+        }
+    };
+    for (uint32_t i0 = 0; i0 < cnt; i0 += kWalkTile) {
+        const uint32_t m = min((uint32_t)kWalkTile, cnt - i0);
+        for (uint32_t i = 0; i < m; ++i) {
+            const uint4 q = s_probe[i0 + i];
+            const uint64_t key = (uint64_t)q.y << 32 | q.x;
+            const int32_t seg = (int32_t)q.z;
+            if (q.w != rep) {  // the next interval (uniform)
+                rep = q.w;
+                cur = s < p ? Lpos[(uint64_t)s * S + rep] : 0u;
+                hi = s < p ? Upos[(uint64_t)s * S + rep] : 0u;
+                if (cur > hi || hi > n) {  // inconsistent interval state: record, do not read out of range
+                    atomicOr(err, kDevErrBounds);
+                    hi = cur;
+                }
+                if (i0 + i == 0) cur += count_below(K + cur, hi - cur, key, (int32_t)s > seg);
+                fetch();
+            }
+            // Keys equal to the probe's come before it in the segments up to
+            // its own, after it in later ones: for most warps one rule holds
+            // for all lanes and the keys to pass are those up to `last`.
+            const bool after = seg < (int32_t)sw, mixed = !after && seg < (int32_t)sw + 32;
+            if (!mixed) {
+                const uint64_t last = key - (after ? 1ull : 0ull);
+                if (!(after && key == 0ull)) walk([&](uint64_t x) { return x <= last; }, key, after);
+                tile[lane * kRow + i] = cur;
+            } else {
+                const bool strict = (int32_t)s > seg;
+                walk([&](uint64_t x) { return strict ? x < key : x <= key; }, key, strict);
+                tile[lane * kRow + i] = (int32_t)s == seg ? s_spos[i0 + i] : cur;
+            }
+        }
+        __syncwarp();
+        const uint32_t l = lane & (kWalkTile - 1), h = lane / kWalkTile;
+        uint64_t sum = 0;
+        if (l < m)
+#pragma unroll
+            for (uint32_t r = 0; r < 32; r += 32 / kWalkTile)
+                if (sw + r + h < p) {
+                    const uint32_t pos = tile[(r + h) * kRow + l];
+                    probe_pos[(uint64_t)(sw + r + h) * cap + k0 + i0 + l] = pos;
+                    sum += pos;
+                }
+        sum += __shfl_xor_sync(0xffffffffu, sum, kWalkTile);
+        if (h == 0 && l < m) atomicAdd((unsigned long long*)&prank[k0 + i0 + l], (unsigned long long)sum);
+        __syncwarp();
     }
 }
 
@@ -683,7 +829,7 @@ __global__ void k_ctl_init(RoundCtl* ctl, uint64_t seed, uint32_t max_rounds) {
     ctl->max_rounds = max_rounds;
     ctl->round = 0;
     ctl->status = HSS_OK;
-    ctl->staged = 0;
+    ctl->form = kFormSearch;
 }
 
 __global__ void k_ctl_record(RoundCtl* ctl, uint32_t rounds, int32_t status, uint64_t last_z) {
@@ -711,9 +857,7 @@ __device__ void round_decide(RoundCtl* ctl, uint64_t cap, uint64_t N, uint32_t p
             ctl->status = HSS_ERR_CAPACITY;
         } else {
             // the histogram form of this round, as the host loop chooses it
-            const double searches = (double)Z * (double)p * log2((double)N / (double)p + 2.0);
-            ctl->staged = (ctl->nint == 1 && hist_mode != kHistProbe &&
-                           (hist_mode == kHistStaged || searches >= 8.0 * (double)N)) ? 1u : 0u;
+            ctl->form = hist_form((double)Z, N, p, ctl->nint, (double)ctl->gamma, hist_mode);
             go = 1;
         }
     }
@@ -819,10 +963,19 @@ cudaError_t enqueue_device_round(const uint64_t* skeys, const uint64_t* d_seg_of
     if (e != cudaSuccess) return e;
     HSS_LAUNCH(k_probe_build, (unsigned)cdiv(cap, 256), 256, 0, st, kZFromCtl, ws.skey_sorted, ws.sperm, ws.sseg,
                ws.sspos, ws.Ucut, ws.int_rep, ws.ctl, ws.pkey, ws.pseg, ws.pspos, ws.pint, ws.prank);
-    HSS_LAUNCH(k_histogram_staged, dim3((unsigned)cdiv(cap, kStgProbes), (unsigned)cdiv(p, kStgSegs)), kStgThreads, 0, st,
-               skeys, d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, kZFromCtl, ws.prank,
-               ws.probe_pos, cap, ws.sws.err, ws.ctl);
-    const uint32_t per_warp = hist_per_warp((double)oversample * (double)NB, p);
+    // the forms that a round of at most cap probes can take
+    if (hist_mode == kHistStaged || (hist_mode == kHistAuto && staged_pays((double)cap, N, p)))
+        HSS_LAUNCH(k_histogram_staged, dim3((unsigned)cdiv(cap, kStgProbes), (unsigned)cdiv(p, kStgSegs)), kStgThreads, 0,
+                   st, skeys, d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, kZFromCtl,
+                   ws.prank, ws.probe_pos, cap, ws.sws.err, ws.ctl);
+    const double Ze = (double)oversample * (double)NB;  // probes expected
+    if (hist_mode == kHistAuto && (double)cap * (double)p >= kWalkMin) {
+        const uint32_t chunk = walk_chunk(Ze, p);
+        HSS_LAUNCH(k_histogram_walk, dim3((unsigned)cdiv(cap, chunk), (unsigned)cdiv(p, kWalkThreads)), kWalkThreads, 0,
+                   st, skeys, d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, ws.pint,
+                   kZFromCtl, ws.prank, ws.probe_pos, cap, ws.sws.err, ws.ctl, chunk);
+    }
+    const uint32_t per_warp = hist_per_warp(Ze, p);
     HSS_LAUNCH(k_histogram, dim3((unsigned)cdiv(cap, 32), (unsigned)cdiv(p, 8 * per_warp)), 256, 0, st, skeys, d_seg_off, p,
                S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, ws.pint, kZFromCtl, ws.prank, ws.probe_pos, cap,
                ws.sws.err, ws.ctl, per_warp);
@@ -999,17 +1152,18 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
         HSS_LAUNCH(k_intervals, 1, 1024, 0, st, S, N, NB, tol, oversample, ws.Lcut, ws.Ucut, ws.res, ws.int_rep, ws.ctl,
                    schedule, Tq, allq, ws.int_T, ws.int_all);
     };
-    // The histogram of Z probes: staged when they share one interval and
-    // searching every segment for every probe (Z p log2(N/p) dependent loads)
-    // would cost several reads of the keys (the probe-side form otherwise).
-    auto histogram = [&](uint64_t Z, uint32_t nint) -> cudaError_t {
-        const double searches = (double)Z * (double)p * std::log2((double)N / (double)p + 2.0);
-        const bool staged = nint == 1 && hist_mode != kHistProbe &&
-                            (hist_mode == kHistStaged || searches >= 8.0 * (double)N);
-        if (staged) {
+    // The histogram of Z probes in nint intervals of gamma keys.
+    auto histogram = [&](uint64_t Z, uint32_t nint, uint64_t gamma) -> cudaError_t {
+        const uint32_t form = hist_form((double)Z, N, p, nint, (double)gamma, hist_mode);
+        if (form == kFormStaged) {
             HSS_LAUNCH(k_histogram_staged, dim3((unsigned)cdiv(Z, kStgProbes), (unsigned)cdiv(p, kStgSegs)), kStgThreads, 0,
                        st, skeys, d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, Z, ws.prank,
                        ws.probe_pos, ws.cap, ws.sws.err, ws.ctl);
+        } else if (form == kFormWalk) {
+            const uint32_t chunk = walk_chunk((double)Z, p);
+            HSS_LAUNCH(k_histogram_walk, dim3((unsigned)cdiv(Z, chunk), (unsigned)cdiv(p, kWalkThreads)), kWalkThreads, 0,
+                       st, skeys, d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, ws.pint, Z,
+                       ws.prank, ws.probe_pos, ws.cap, ws.sws.err, ws.ctl, chunk);
         } else {
             const uint32_t per_warp = hist_per_warp((double)Z, p);
             HSS_LAUNCH(k_histogram, dim3((unsigned)cdiv(Z, 32), (unsigned)cdiv(p, 8 * per_warp)), 256, 0, st, skeys,
@@ -1039,7 +1193,7 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
                         false, ws.sws, st, nullptr));
         HSS_LAUNCH(k_prop_probes, (unsigned)cdiv(nprop, 256), 256, 0, st, nprop, ws.skey_sorted, ws.pkey, ws.pseg,
                    ws.pspos, ws.pint, ws.prank);
-        HSS_TRY(histogram((uint64_t)nprop, 1u));
+        HSS_TRY(histogram((uint64_t)nprop, 1u, N));
         HSS_LAUNCH(k_update, sblk, 256, 0, st, S, N, NB, ws.pkey, ws.pseg, ws.pspos, ws.prank, (uint64_t)nprop,
                    (int32_t)kNonMember, ws.Lcut, ws.Ucut, ws.chgL, ws.chgU, ws.ctl);
         HSS_LAUNCH(k_update_pos, p, 256, 0, st, S, ws.chgL, ws.chgU, ws.probe_pos, ws.cap, ws.Lpos, ws.Upos);
@@ -1096,7 +1250,7 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
                             false, ws.sws, st, nullptr));
             HSS_LAUNCH(k_probe_build, (unsigned)cdiv(Z, 256), 256, 0, st, Z, ws.skey_sorted, ws.sperm, ws.sseg, ws.sspos,
                        ws.Ucut, ws.int_rep, ws.ctl, ws.pkey, ws.pseg, ws.pspos, ws.pint, ws.prank);
-            HSS_TRY(histogram(Z, h.nint));
+            HSS_TRY(histogram(Z, h.nint, h.gamma));
             uint64_t Tq;
             uint32_t allq;
             threshold(j + 1, Tq, allq);

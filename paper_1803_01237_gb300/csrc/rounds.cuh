@@ -20,7 +20,7 @@ struct RoundCtl {
     // round statistics here, and reads the call's parameters from here (so one
     // captured graph serves every call on the same workspace).
     int32_t status;        // HSS_OK, HSS_ERR_ROUND_LIMIT or HSS_ERR_CAPACITY
-    uint32_t staged;       // the next histogram takes the staged form
+    uint32_t form;         // form of the next histogram
     uint64_t seed;         // Philox key of the sampling
     uint32_t max_rounds;
     uint32_t pad;
