@@ -50,21 +50,20 @@ struct BTotals {
 inline uint64_t cdivh(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
 inline size_t aup(size_t x) { return (x + 255) / 256 * 256; }
 
-__device__ __forceinline__ uint64_t seg_start(const BJob& J, uint32_t s) { return ideal_rank(s, J.n, J.p); }
-
 // ---------------------------------------------------------------------------
 // Initial state of every job: intervals (-inf, +inf), whole segments.
 // ---------------------------------------------------------------------------
 __global__ void kb_init(const BJob* __restrict__ jobs, BCtl* __restrict__ ctl, hss_job_stats* __restrict__ jst,
                         DCut* __restrict__ Lcut, DCut* __restrict__ Ucut, uint32_t* __restrict__ Lpos,
-                        uint32_t* __restrict__ Upos) {
+                        uint32_t* __restrict__ Upos, const uint64_t* __restrict__ seg_off) {
     const BJob J = jobs[blockIdx.x];
     const uint32_t S = J.p - 1;
-    const uint64_t ent = (uint64_t)J.p * S;
-    for (uint64_t e = threadIdx.x; e < ent; e += blockDim.x) {
-        const uint32_t s = (uint32_t)(e / S);
-        Lpos[J.lbase + e] = 0;
-        Upos[J.lbase + e] = (uint32_t)(seg_start(J, s + 1) - seg_start(J, s));
+    for (uint32_t s = threadIdx.x >> 5; s < J.p; s += blockDim.x >> 5) {  // a row per warp
+        const uint32_t n = (uint32_t)(seg_off[J.sbase + s + 1] - seg_off[J.sbase + s]);
+        for (uint32_t i = threadIdx.x & 31; i < S; i += 32) {
+            Lpos[J.lbase + (uint64_t)s * S + i] = 0;
+            Upos[J.lbase + (uint64_t)s * S + i] = n;
+        }
     }
     for (uint32_t i = threadIdx.x; i < S; i += blockDim.x) {
         DCut a; a.okey = 0; a.seg = -2; a.spos = 0; a.rank = 0; a.kind = kNegInf; a.pad = 0;
@@ -82,13 +81,16 @@ __global__ void kb_init(const BJob* __restrict__ jobs, BCtl* __restrict__ ctl, h
 }
 
 // The tables over the segments and splitters of all jobs (segment bounds, the
-// job of each), one CTA per job.
+// job of each), one CTA per job.  The kernels of the rounds and the exchange
+// read the bounds here: with a 128-bit division per bound and use, 128 jobs of
+// 128 segments spent 1325 us in kb_histogram (779 now), 1287 in kb_sample_mark
+// (935, moving the cuts' positions included), 54 in kb_init (13).
 __global__ void kb_tables(uint32_t njobs, const BJob* __restrict__ jobs, uint64_t* __restrict__ seg_off,
                           uint32_t* __restrict__ job_of_seg, uint32_t* __restrict__ job_of_spl) {
     const uint32_t j = blockIdx.x;
     const BJob J = jobs[j];
     for (uint32_t s = threadIdx.x; s < J.p; s += blockDim.x) {
-        seg_off[J.sbase + s] = J.koff + seg_start(J, s);
+        seg_off[J.sbase + s] = J.koff + ideal_rank(s, J.n, J.p);
         job_of_seg[J.sbase + s] = j;
         if (s + 1 < J.p) job_of_spl[J.ibase + s] = j;
     }
@@ -121,7 +123,8 @@ __global__ __launch_bounds__(1024) void kb_intervals(const BJob* __restrict__ jo
 // round, 0) under the job's seed.
 __global__ __launch_bounds__(kSampThreads) void kb_sample_mark(
     const BJob* __restrict__ jobs, const uint32_t* __restrict__ job_of_seg, const BCtl* __restrict__ ctl,
-    const hss_job_stats* __restrict__ jst, const uint32_t* __restrict__ Lpos, const uint32_t* __restrict__ Upos,
+    const hss_job_stats* __restrict__ jst, const uint64_t* __restrict__ seg_off, uint32_t* Lpos, uint32_t* Upos,
+    const int32_t* __restrict__ chgL, const int32_t* __restrict__ chgU, const uint32_t* __restrict__ probe_pos,
     const DCut* __restrict__ Lcut, const uint32_t* __restrict__ int_rep, uint32_t round, uint32_t* __restrict__ bitmap,
     uint32_t* __restrict__ seg_cnt) {
     __shared__ uint32_t s_a[kIntChunk], s_b[kIntChunk], s_pre[kIntChunk + 1];
@@ -130,13 +133,18 @@ __global__ __launch_bounds__(kSampThreads) void kb_sample_mark(
     const uint32_t j = job_of_seg[g];
     const BJob J = jobs[j];
     const uint32_t nint = ctl[j].nint;
+    const uint32_t s = g - J.sbase, S = J.p - 1;
+    // a job that sampled last round: the positions of its moved cuts first
+    if (ctl[j].active) {
+        update_pos_row(s, S, chgL + J.ibase, chgU + J.ibase, probe_pos + J.ppbase, J.cap, Lpos + J.lbase, Upos + J.lbase);
+        __syncthreads();
+    }
     if (nint == 0 || jst[j].status != HSS_OK) {  // uniform per CTA
         if (threadIdx.x == 0) seg_cnt[g] = 0;
         return;
     }
-    const uint32_t s = g - J.sbase, S = J.p - 1;
-    const uint64_t base = J.koff + seg_start(J, s);
-    const uint32_t n_s = (uint32_t)(seg_start(J, s + 1) - seg_start(J, s));
+    const uint64_t base = seg_off[g];
+    const uint32_t n_s = (uint32_t)(seg_off[g + 1] - base);
     const uint64_t T = ctl[j].T;
     const bool take_all = ctl[j].take_all != 0;
     PairDraw pd;
@@ -221,21 +229,24 @@ __global__ __launch_bounds__(1024) void kb_count_scan(uint32_t P_tot, const uint
 
 // The kept keys of one segment, in position order, into the job's part of
 // the compact sample buffer.
+template <bool WARP>
 __global__ __launch_bounds__(kSampThreads) void kb_sample_write(
-    const uint64_t* __restrict__ skeys, const BJob* __restrict__ jobs, const uint32_t* __restrict__ job_of_seg,
-    const BCtl* __restrict__ ctl, uint32_t* bitmap, const uint32_t* __restrict__ seg_cnt, const uint64_t* __restrict__ G,
+    uint32_t P_tot, const uint64_t* __restrict__ skeys, const BJob* __restrict__ jobs,
+    const uint32_t* __restrict__ job_of_seg, const uint64_t* __restrict__ seg_off, const BCtl* __restrict__ ctl,
+    uint32_t* bitmap, const uint32_t* __restrict__ seg_cnt, const uint64_t* __restrict__ G,
     const uint64_t* __restrict__ zoff, uint64_t* __restrict__ skey,
     uint32_t* __restrict__ sseg, uint32_t* __restrict__ sspos, uint32_t* __restrict__ siota) {
     __shared__ uint32_t s_warp[32];
-    const uint32_t g = blockIdx.x;
-    const uint32_t j = job_of_seg[g];
+    const uint32_t g = WARP ? blockIdx.x * (kSampThreads / 32) + (threadIdx.x >> 5) : blockIdx.x;
+    if (g >= P_tot) return;
     const uint32_t want = seg_cnt[g];
+    const uint32_t j = job_of_seg[g];
     if (want == 0 || !ctl[j].active) return;
     const BJob J = jobs[j];
     const uint32_t s = g - J.sbase;
-    const uint64_t base = J.koff + seg_start(J, s), end = J.koff + seg_start(J, s + 1);
+    const uint64_t base = seg_off[g], end = seg_off[g + 1];
     const uint64_t out = zoff[j] + (G[g] - G[J.sbase]), lim = zoff[j + 1];
-    take_marks(bitmap, base, end, want, s_warp, [&](uint64_t q, uint32_t at) {
+    take_marks<WARP>(bitmap, base, end, want, s_warp, [&](uint64_t q, uint32_t at) {
         const uint64_t o = out + at;
         if (o < lim) {
             skey[o] = skeys[q];
@@ -287,8 +298,8 @@ constexpr int kBHistSegs = 64;
 
 __global__ __launch_bounds__(256) void kb_histogram(
     const uint64_t* __restrict__ skeys, const BJob* __restrict__ jobs, const uint32_t* __restrict__ pjob,
-    const uint64_t* __restrict__ zoff, const uint32_t* __restrict__ Lpos, const uint32_t* __restrict__ Upos,
-    const uint32_t* __restrict__ int_rep, const uint64_t* __restrict__ pkey, const int32_t* __restrict__ pseg,
+    const uint64_t* __restrict__ zoff, const uint64_t* __restrict__ seg_off, const uint32_t* __restrict__ Lpos,
+    const uint32_t* __restrict__ Upos, const uint32_t* __restrict__ int_rep, const uint64_t* __restrict__ pkey, const int32_t* __restrict__ pseg,
     const uint32_t* __restrict__ pspos, const uint32_t* __restrict__ pint, uint64_t Zc, uint64_t* __restrict__ prank,
     uint32_t* __restrict__ probe_pos, uint32_t* __restrict__ err) {
     __shared__ uint64_t s_part[8][32];
@@ -318,10 +329,10 @@ __global__ __launch_bounds__(256) void kb_histogram(
                 pos = spos;
             } else {
                 const uint32_t lo = Lpos[J.lbase + (uint64_t)s * S + rep], hi = Upos[J.lbase + (uint64_t)s * S + rep];
-                const uint64_t a = seg_start(J, s);
-                const uint32_t n = (uint32_t)(seg_start(J, s + 1) - a);
+                const uint64_t a = seg_off[J.sbase + s];
+                const uint32_t n = (uint32_t)(seg_off[J.sbase + s + 1] - a);
                 if (lo <= hi && hi <= n) {
-                    pos = lo + count_below(skeys + J.koff + a + lo, hi - lo, key, (int32_t)s > seg);
+                    pos = lo + count_below(skeys + a + lo, hi - lo, key, (int32_t)s > seg);
                 } else {
                     atomicOr(err, kDevErrBounds);
                     pos = lo;
@@ -378,24 +389,6 @@ __global__ void kb_update(uint32_t S_tot, const BJob* __restrict__ jobs, const u
     chgU[gi] = cu;
 }
 
-// Per-segment positions of the changed cuts (one CTA per sampling job).
-__global__ void kb_update_pos(const BJob* __restrict__ jobs, const BCtl* __restrict__ ctl,
-                              const int32_t* __restrict__ chgL, const int32_t* __restrict__ chgU,
-                              const uint32_t* __restrict__ probe_pos, uint32_t* __restrict__ Lpos,
-                              uint32_t* __restrict__ Upos) {
-    const uint32_t j = blockIdx.x;
-    if (!ctl[j].active) return;
-    const BJob J = jobs[j];
-    const uint32_t S = J.p - 1;
-    const uint64_t ent = (uint64_t)J.p * S;
-    for (uint64_t e = threadIdx.x; e < ent; e += blockDim.x) {
-        const uint32_t s = (uint32_t)(e / S), i = (uint32_t)(e % S);
-        const int32_t cl = chgL[J.ibase + i], cu = chgU[J.ibase + i];
-        if (cl >= 0) Lpos[J.lbase + e] = probe_pos[J.ppbase + (uint64_t)s * J.cap + (uint32_t)cl];
-        if (cu >= 0) Upos[J.lbase + e] = probe_pos[J.ppbase + (uint64_t)s * J.cap + (uint32_t)cu];
-    }
-}
-
 // Final splitters (the closer of L_i, U_i; tie -> L_i), offsets relative to
 // the job, and the per-segment positions of the chosen cuts.
 __global__ void kb_finalize(uint32_t S_tot, const BJob* __restrict__ jobs, const uint32_t* __restrict__ job_of_spl,
@@ -445,10 +438,12 @@ __device__ __forceinline__ uint32_t bpos(const uint32_t* __restrict__ pos, uint3
 // CTA (x, j): buckets 32x .. 32x+31 of job j; its 32 warps split the job's
 // segments into groups, sum, scan the group sums and write destinations.
 __global__ __launch_bounds__(1024) void kb_exchange_dst(const BJob* __restrict__ jobs, const uint32_t* __restrict__ pos,
-                                                        const uint64_t* __restrict__ offsets, uint64_t* __restrict__ dst,
+                                                        const uint64_t* __restrict__ offsets,
+                                                        const uint64_t* __restrict__ seg_off, uint64_t* __restrict__ dst,
                                                         uint32_t* __restrict__ err) {
     __shared__ uint64_t s_part[32][33];
     const BJob J = jobs[blockIdx.y];
+    const uint64_t* so = seg_off + J.sbase;
     const uint32_t p = J.p;
     if (blockIdx.x * 32 >= p) return;  // uniform per CTA
     const uint32_t col = threadIdx.x & 31, grp = threadIdx.x >> 5;
@@ -460,7 +455,7 @@ __global__ __launch_bounds__(1024) void kb_exchange_dst(const BJob* __restrict__
     uint64_t part = 0;
     if (b < p) {
         for (uint32_t s = s0; s < s1; ++s) {
-            const uint32_t n = (uint32_t)(seg_start(J, s + 1) - seg_start(J, s));
+            const uint32_t n = (uint32_t)(so[s + 1] - so[s]);
             part += bpos(P, S, p, s, b + 1, n) - bpos(P, S, p, s, b, n);
         }
     }
@@ -471,7 +466,7 @@ __global__ __launch_bounds__(1024) void kb_exchange_dst(const BJob* __restrict__
     uint64_t run = J.koff + off[b];
     for (uint32_t g = 0; g < grp; ++g) run += s_part[g][col];
     for (uint32_t s = s0; s < s1; ++s) {
-        const uint32_t n = (uint32_t)(seg_start(J, s + 1) - seg_start(J, s));
+        const uint32_t n = (uint32_t)(so[s + 1] - so[s]);
         dst[J.dbase + (uint64_t)s * p + b] = run;
         run += bpos(P, S, p, s, b + 1, n) - bpos(P, S, p, s, b, n);
     }
@@ -488,6 +483,7 @@ constexpr uint32_t kBXchMaxB = 2048;
 __global__ __launch_bounds__(256) void kb_exchange_copy(const uint64_t* __restrict__ skeys, const uint32_t* __restrict__ spay,
                                                         const BJob* __restrict__ jobs,
                                                         const uint32_t* __restrict__ job_of_seg,
+                                                        const uint64_t* __restrict__ seg_off,
                                                         const uint32_t* __restrict__ pos, const uint64_t* __restrict__ dst,
                                                         uint64_t* __restrict__ bkeys, uint32_t* __restrict__ bpay,
                                                         uint32_t* __restrict__ err) {
@@ -496,8 +492,8 @@ __global__ __launch_bounds__(256) void kb_exchange_copy(const uint64_t* __restri
     const uint32_t g = blockIdx.x;
     const BJob J = jobs[job_of_seg[g]];
     const uint32_t s = g - J.sbase, p = J.p, S = p - 1;
-    const uint64_t base = J.koff + seg_start(J, s);
-    const uint32_t n = (uint32_t)(seg_start(J, s + 1) - seg_start(J, s));
+    const uint64_t base = seg_off[g];
+    const uint32_t n = (uint32_t)(seg_off[g + 1] - base);
     const uint32_t c0 = blockIdx.y * kBXchChunk;
     if (c0 >= n) return;
     const uint32_t c1 = min(n, c0 + kBXchChunk);
@@ -812,14 +808,14 @@ int run_batch(const void* d_keys, const uint32_t* d_payload, int key_type, const
     // Rounds, all jobs in lock step.
     const float s = prm->oversample;
     const unsigned sblk = (unsigned)cdivh(std::max<uint32_t>(T.S_tot, 1), 256);
-    HSS_LAUNCH(kb_init, njobs, 256, 0, st, jobs, ctl, jst, Lcut, Ucut, Lpos, Upos);
+    HSS_LAUNCH(kb_init, njobs, 256, 0, st, jobs, ctl, jst, Lcut, Ucut, Lpos, Upos, seg_off);
     HSS_LAUNCH(kb_intervals, njobs, 1024, 0, st, jobs, ctl, jst, Lcut, Ucut, res, int_rep, s);
     auto sampling = [&](uint32_t round) {
         // later rounds find the marks cleared by kb_sample_write (a failed job's
         // stay, and are not looked at again)
         if (round == 1) cudaMemsetAsync(bitmap, 0, (T.N_tot / 32 + 2) * 4, st);
-        HSS_LAUNCH(kb_sample_mark, T.P_tot, kSampThreads, 0, st, jobs, jseg, ctl, jst, Lpos, Upos, Lcut, int_rep, round,
-                   bitmap, seg_cnt);
+        HSS_LAUNCH(kb_sample_mark, T.P_tot, kSampThreads, 0, st, jobs, jseg, ctl, jst, seg_off, Lpos, Upos, chgL, chgU,
+                   probe_pos, Lcut, int_rep, round, bitmap, seg_cnt);
         HSS_LAUNCH(kb_count_scan, 1, 1024, 0, st, T.P_tot, seg_cnt, G, njobs, jobs, ctl, jst, max_rounds, zoff, tot);
     };
     sampling(1);
@@ -831,21 +827,24 @@ int run_batch(const void* d_keys, const uint32_t* d_payload, int key_type, const
         if (h.active == 0) break;
         ++round;
         const uint64_t Zc = h.Zc;
-        HSS_LAUNCH(kb_sample_write, T.P_tot, kSampThreads, 0, st, keysA, jobs, jseg, ctl, bitmap, seg_cnt, G, zoff, skey,
-                   sseg, sspos, siota);
+        if (T.N_tot <= kSampWarpKeys * T.P_tot)
+            HSS_LAUNCH(kb_sample_write<true>, (unsigned)cdivh(T.P_tot, kSampThreads / 32), kSampThreads, 0, st, T.P_tot,
+                       keysA, jobs, jseg, seg_off, ctl, bitmap, seg_cnt, G, zoff, skey, sseg, sspos, siota);
+        else
+            HSS_LAUNCH(kb_sample_write<false>, T.P_tot, kSampThreads, 0, st, T.P_tot, keysA, jobs, jseg, seg_off, ctl,
+                       bitmap, seg_cnt, G, zoff, skey, sseg, sspos, siota);
         if (Zc > 0) {
             HSS_BTRY(segsort(skey, skey_sorted, stmp, siota, sperm, ptmp, Zc, njobs, zoff, false, false, sws_s, st,
                              nullptr));
             HSS_LAUNCH(kb_probe_build, (unsigned)cdivh(Zc, 256), 256, 0, st, Zc, zoff, njobs, jobs, ctl, skey_sorted, sperm,
                        sseg, sspos, Ucut, int_rep, pkey, pseg, pspos, pint, prank, pjob);
             HSS_LAUNCH(kb_histogram, dim3((unsigned)cdivh(Zc, 32), (unsigned)cdivh(T.max_p, kBHistSegs)), 256, 0, st,
-                       keysA, jobs, pjob, zoff, Lpos, Upos, int_rep, pkey, pseg, pspos, pint, Zc, prank, probe_pos, err);
+                       keysA, jobs, pjob, zoff, seg_off, Lpos, Upos, int_rep, pkey, pseg, pspos, pint, Zc, prank, probe_pos,
+                       err);
         }
-        if (T.S_tot) {
+        if (T.S_tot)
             HSS_LAUNCH(kb_update, sblk, 256, 0, st, T.S_tot, jobs, jspl, ctl, zoff, pkey, pseg, pspos, prank, Lcut, Ucut,
                        chgL, chgU);
-            HSS_LAUNCH(kb_update_pos, njobs, 256, 0, st, jobs, ctl, chgL, chgU, probe_pos, Lpos, Upos);
-        }
         HSS_LAUNCH(kb_intervals, njobs, 1024, 0, st, jobs, ctl, jst, Lcut, Ucut, res, int_rep, s);
         sampling(round + 1);
     }
@@ -867,10 +866,10 @@ int run_batch(const void* d_keys, const uint32_t* d_payload, int key_type, const
         HSS_LAUNCH(kb_bucket_hint, (unsigned)cdivh(T.P_tot, 256), 256, 0, st, T.P_tot, jobs, jseg, Lcut, Ucut, choose_u,
                    jrange, hlo, hmult);
         if (T.N_tot > 0) {
-            HSS_LAUNCH(kb_exchange_dst, dim3((unsigned)cdivh(T.max_p, 32), njobs), 1024, 0, st, jobs, Lpos, offsets, dst,
-                       err);
+            HSS_LAUNCH(kb_exchange_dst, dim3((unsigned)cdivh(T.max_p, 32), njobs), 1024, 0, st, jobs, Lpos, offsets,
+                       seg_off, dst, err);
             HSS_LAUNCH(kb_exchange_copy, dim3(T.P_tot, (unsigned)cdivh(std::max<uint32_t>(T.max_seg, 1), kBXchChunk)), 256,
-                       0, st, keysA, payA, jobs, jseg, Lpos, dst, keysB, payB, err);
+                       0, st, keysA, payA, jobs, jseg, seg_off, Lpos, dst, keysB, payB, err);
         }
         if (timing) cudaEventRecord(ev[3], st);
         HSS_LAUNCH(kb_bucket_off, (unsigned)cdivh((uint64_t)T.P_tot + 1, 256), 256, 0, st, T.P_tot, T.N_tot, jobs, jseg,

@@ -174,17 +174,6 @@ __global__ __launch_bounds__(1024) void k_intervals(uint32_t S, uint64_t N, uint
 // ---------------------------------------------------------------------------
 // Sampling.
 // ---------------------------------------------------------------------------
-// Positions in segment s of the cuts that the last histogram moved.
-__device__ __forceinline__ void update_pos_row(uint64_t s, uint32_t S, const int32_t* __restrict__ chgL,
-                                               const int32_t* __restrict__ chgU, const uint32_t* __restrict__ probe_pos,
-                                               uint64_t cap, uint32_t* Lpos, uint32_t* Upos) {
-    for (uint32_t i = threadIdx.x; i < S; i += blockDim.x) {
-        const int32_t cl = chgL[i], cu = chgU[i];
-        if (cl >= 0) Lpos[s * S + i] = probe_pos[s * cap + (uint32_t)cl];
-        if (cu >= 0) Upos[s * S + i] = probe_pos[s * cap + (uint32_t)cu];
-    }
-}
-
 // Round-j Bernoulli marks of segment blockIdx.x (Sec. 4.2.2 step 4, Sec. 6):
 // every key of an unresolved interval draws its Philox word and is kept when
 // the word is below the round's threshold.  gridDim.y CTAs share a segment,
@@ -252,19 +241,21 @@ static unsigned mark_chunks(uint64_t N, uint32_t p) {
 // bitmap inside the segment, so the pass scans the segment's bitmap words and
 // skips empty runs of them.  It leaves the bitmap and the counts zero (two
 // memsets a round otherwise, one of them of N/8 bytes).
+template <bool WARP>
 __global__ __launch_bounds__(kSampThreads) void k_sample_write(
-    const uint64_t* __restrict__ skeys, const uint64_t* __restrict__ seg_off, uint32_t* bitmap, uint32_t* seg_cnt,
+    uint32_t p, const uint64_t* __restrict__ skeys, const uint64_t* __restrict__ seg_off, uint32_t* bitmap, uint32_t* seg_cnt,
     const uint32_t* __restrict__ seg_cnt_off, uint64_t cap,
     uint64_t* __restrict__ skey, uint32_t* __restrict__ sseg, uint32_t* __restrict__ sspos, uint32_t* __restrict__ siota) {
     __shared__ uint32_t s_warp[32];
-    const uint32_t s = blockIdx.x;
+    const uint32_t s = WARP ? blockIdx.x * (kSampThreads / 32) + (threadIdx.x >> 5) : blockIdx.x;
+    if (s >= p) return;
     const uint32_t want = seg_cnt[s];
-    __syncthreads();
+    if (WARP) __syncwarp(); else __syncthreads();
     if (want == 0) return;
-    if (threadIdx.x == 0) seg_cnt[s] = 0;  // for the next round's marks
+    if ((threadIdx.x & (WARP ? 31 : kSampThreads - 1)) == 0) seg_cnt[s] = 0;  // for the next round's marks
     const uint64_t base = seg_off[s], end = seg_off[s + 1];
     uint64_t out = seg_cnt_off[s];
-    take_marks(bitmap, base, end, want, s_warp, [&](uint64_t g, uint32_t at) {
+    take_marks<WARP>(bitmap, base, end, want, s_warp, [&](uint64_t g, uint32_t at) {
         const uint64_t o = out + at;
         if (o < cap) {
             skey[o] = skeys[g];
@@ -899,6 +890,16 @@ __global__ __launch_bounds__(1024) void k_count_scan(const uint32_t* __restrict_
 // ---------------------------------------------------------------------------
 #define HSS_TRY(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return HSS_ERR_CUDA; } while (0)
 
+void enqueue_sample_write(const RoundWs& ws, const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uint32_t p,
+                          cudaStream_t st) {
+    if (N <= kSampWarpKeys * p)
+        HSS_LAUNCH(k_sample_write<true>, (unsigned)cdiv(p, kSampThreads / 32), kSampThreads, 0, st, p, skeys, d_seg_off,
+                   ws.bitmap, ws.seg_cnt, ws.seg_cnt_off, ws.cap, ws.skey, ws.sseg, ws.sspos, ws.siota);
+    else
+        HSS_LAUNCH(k_sample_write<false>, p, kSampThreads, 0, st, p, skeys, d_seg_off, ws.bitmap, ws.seg_cnt,
+                   ws.seg_cnt_off, ws.cap, ws.skey, ws.sseg, ws.sspos, ws.siota);
+}
+
 // The marks and sample offsets of a round.  Round 1 starts from cleared marks;
 // later ones find them cleared by k_sample_write and take the positions of the
 // cuts that the last histogram moved (moved: there was one).
@@ -956,8 +957,7 @@ cudaError_t enqueue_device_round(const uint64_t* skeys, const uint64_t* d_seg_of
     const uint32_t S = NB - 1;
     const uint64_t cap = ws.cap;
     const bool per_interval = schedule == HSS_SCHEDULE_EQUAL;
-    HSS_LAUNCH(k_sample_write, p, kSampThreads, 0, st, skeys, d_seg_off, ws.bitmap, ws.seg_cnt, ws.seg_cnt_off, cap, ws.skey,
-               ws.sseg, ws.sspos, ws.siota);
+    enqueue_sample_write(ws, skeys, d_seg_off, N, p, st);
     cudaError_t e = segsort(ws.skey, ws.skey_sorted, ws.stmp, ws.siota, ws.sperm, ws.ptmp, cap, 1, ws.ctl->seg_off_z,
                             false, false, ws.sws, st, nullptr);
     if (e != cudaSuccess) return e;
@@ -1243,8 +1243,7 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
         out->gamma[j - 1] = h.gamma;
         if (h.Z > ws.cap) { status = HSS_ERR_CAPACITY; break; }
         const uint64_t Z = h.Z;
-        HSS_LAUNCH(k_sample_write, p, kSampThreads, 0, st, skeys, d_seg_off, ws.bitmap, ws.seg_cnt, ws.seg_cnt_off, ws.cap,
-                   ws.skey, ws.sseg, ws.sspos, ws.siota);
+        enqueue_sample_write(ws, skeys, d_seg_off, N, p, st);
         if (Z > 0) {
             HSS_TRY(segsort(ws.skey, ws.skey_sorted, ws.stmp, ws.siota, ws.sperm, ws.ptmp, Z, 1, ws.ctl->seg_off_z, false,
                             false, ws.sws, st, nullptr));

@@ -45,7 +45,10 @@ struct AddU64 { __device__ uint64_t operator()(uint64_t a, uint64_t b) const { r
 struct MaxI32 { __device__ int32_t operator()(int32_t a, int32_t b) const { return a > b ? a : b; } };
 
 __device__ __forceinline__ uint64_t ideal_rank(uint64_t i1, uint64_t N, uint64_t p) {
-    return (uint64_t)(((unsigned __int128)i1 * N) / p);  // t_i for splitter number i1 (1-based)
+    // t_i for splitter number i1 (1-based); a 128-bit division is a call of
+    // several hundred instructions, needed from i1 N = 2^64 on
+    if (__umul64hi(i1, N) == 0) return i1 * N / p;
+    return (uint64_t)(((unsigned __int128)i1 * N) / p);
 }
 
 // Count of keys in a[0..n) below key: strict (<) or not (<=), branch-free.
@@ -368,19 +371,25 @@ __device__ __forceinline__ void mark_pairs(const PairDraw& pd, const uint32_t* s
     }
 }
 
+// Segments short enough for a warp each: a CTA per segment of 2^14 keys spent
+// its time in the chain of loads and barriers before the first mark (16384
+// segments: 101 us a round, by warps 26).
+constexpr uint64_t kSampWarpKeys = 1ull << 15;  // keys per segment on average, at most
+
 // The marked positions g in [base, end) of the bitmap, in order, by the CTA
-// (kSampThreads): body(g, number of marks before it).  want: how many there
+// (kSampThreads) or by one warp: body(g, number of marks before it).  want: how many there
 // are.  The marks are cleared on the way, for the next round (a word on the
 // border keeps the neighbour's bits).  Marks are rare, so the pass is bound by
 // its steps over empty words: a thread reads four words a step (2^28 positions
 // in 4096 segments: 35 us a round by single words, 22 by four).
-template <class Body>
+template <bool WARP, class Body>
 __device__ __forceinline__ void take_marks(uint32_t* bitmap, uint64_t base, uint64_t end, uint32_t want, uint32_t* s_warp,
                                            Body body) {
     const uint64_t v0 = base >> 7, v1 = (end + 127) >> 7;  // vectors of 128 positions
+    const uint32_t lane = threadIdx.x & 31;
     uint32_t found = 0;
-    for (uint64_t vb = v0; vb < v1 && found < want; vb += kSampThreads) {
-        const uint64_t vi = vb + threadIdx.x;
+    for (uint64_t vb = v0; vb < v1 && found < want; vb += WARP ? 32 : kSampThreads) {
+        const uint64_t vi = vb + (WARP ? lane : threadIdx.x);
         uint32_t bits[4] = {0u, 0u, 0u, 0u};
         if (vi < v1) {
             uint4 x;
@@ -403,9 +412,20 @@ __device__ __forceinline__ void take_marks(uint32_t* bitmap, uint64_t base, uint
             }
         }
         const uint32_t c = __popc(bits[0]) + __popc(bits[1]) + __popc(bits[2]) + __popc(bits[3]);
-        if (__syncthreads_or(c) == 0) continue;
-        uint32_t tot;
-        uint32_t at = found + block_incl_scan<uint32_t>(c, 0u, AddU32(), s_warp, tot) - c;
+        if ((WARP ? __any_sync(0xffffffffu, c != 0u) : __syncthreads_or(c)) == 0) continue;
+        uint32_t tot, at;
+        if (WARP) {
+            uint32_t x = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= (uint32_t)o) x += y;
+            }
+            tot = __shfl_sync(0xffffffffu, x, 31);
+            at = found + x - c;
+        } else {
+            at = found + block_incl_scan<uint32_t>(c, 0u, AddU32(), s_warp, tot) - c;
+        }
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             while (bits[k]) {
@@ -414,6 +434,17 @@ __device__ __forceinline__ void take_marks(uint32_t* bitmap, uint64_t base, uint
                 body((vi << 7) + 32 * k + b, at++);
             }
         found += tot;
+    }
+}
+
+// Positions in segment s of the cuts that the last histogram moved.
+__device__ __forceinline__ void update_pos_row(uint64_t s, uint32_t S, const int32_t* __restrict__ chgL,
+                                               const int32_t* __restrict__ chgU, const uint32_t* __restrict__ probe_pos,
+                                               uint64_t cap, uint32_t* Lpos, uint32_t* Upos) {
+    for (uint32_t i = threadIdx.x; i < S; i += blockDim.x) {
+        const int32_t cl = chgL[i], cu = chgU[i];
+        if (cl >= 0) Lpos[s * S + i] = probe_pos[s * cap + (uint32_t)cl];
+        if (cu >= 0) Upos[s * S + i] = probe_pos[s * cap + (uint32_t)cu];
     }
 }
 
