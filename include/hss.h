@@ -74,7 +74,7 @@ extern "C" {
  * eighth later; 2^24 positions at least) each segment is walked along the
  * sorted probes; when all its probes share one interval (round 1) and searching every segment for every probe
  * (Z p log2(N/p) dependent loads) would cost more than eight reads of the
- * keys, a staged form ranks blocks of sorted probes against the keys between
+ * keys (four from 2^26 positions on), a staged form ranks blocks of sorted probes against the keys between
  * the block's first and last probe, staged in shared memory; else every
  * probe is searched in every segment.  These flags force the last form, or the
  * staged one where it applies (at most one may be set, else HSS_ERR_INVALID). */

@@ -310,12 +310,17 @@ constexpr int kHistSegPerBlock = 64;  // k_rank_cuts
 // staged, walk): 0.4: 685, 373 us; 0.8: 777, 680; 1.6: 880, 1650.  Many
 // intervals, each begun by loads of its own (search, walk): 0.04: 298, 271;
 // 0.08: 344, 313; 0.15: 367, 370; 0.3: 413, 461.  The staged form pays when the
-// searches (Z p log2(N/p) dependent loads) would cost several reads of the keys.
+// searches (Z p log2(N/p) dependent loads) would cost several reads of the keys:
+// eight, or four where its CTAs (one per 2^15 positions) come in several waves
+// (2^28 keys, p = 4096, five reads: 1564 us searched, 1088 staged; 2^26 keys,
+// p = 2048, five reads: 396 and 407; 2^24 keys, p = 1024: 121 and 203).
 constexpr uint32_t kFormSearch = 0, kFormStaged = 1, kFormWalk = 2;
 constexpr double kWalkMin = (double)(1ull << 24);   // positions per round, at least
+constexpr double kStagedWaves = (double)(1ull << 26);  // positions
 constexpr double kWalkKeysOne = 1.0, kWalkKeysMany = 0.125;  // keys per position, at most
 __host__ __device__ __forceinline__ bool staged_pays(double Z, uint64_t N, uint32_t p) {
-    return Z * (double)p * log2((double)N / (double)p + 2.0) >= 8.0 * (double)N;
+    const double reads = Z * (double)p * log2((double)N / (double)p + 2.0) / (double)N;
+    return reads >= 8.0 || (reads >= 4.0 && Z * (double)p >= kStagedWaves);
 }
 __host__ __device__ __forceinline__ uint32_t hist_form(double Z, uint64_t N, uint32_t p, uint32_t nint, double gamma,
                                                        uint32_t hist_mode) {

@@ -1214,8 +1214,8 @@ __device__ __forceinline__ uint32_t splitter_digit(const uint32_t* spl, uint64_t
 // for the chip (which no split on splitters divides).  Where a quarter of the
 // keys would be spared a second level, every 8th key of the sorted sample is
 // a splitter (spl_mode 1), else the byte split stays (spl_mode 0).  The
-// search costs each of the two passes over the keys about 0.3 ms per 2^28
-// keys, a second level of keys alone 2.9 ms.  Segments above kSplMax keys
+// search costs the statistics pass about 0.4 ms per 2^28 keys (its digits are
+// kept for the split), a second level of keys alone 2.3 ms.  Segments above kSplMax keys
 // take the byte split: 256 sub-buckets of theirs are too large anyway.
 constexpr int kSplSample = 2048;
 constexpr uint64_t kSplMax = 1ull << 19;
@@ -1328,7 +1328,8 @@ __global__ __launch_bounds__(256) void k_tile_stats(const uint64_t* __restrict__
                                                     const uint64_t* __restrict__ hint_hi,
                                                     const uint32_t* __restrict__ prev_shift, uint32_t* __restrict__ spec_out,
                                                     uint64_t flip_in, const uint32_t* __restrict__ spl_tab,
-                                                    const uint8_t* __restrict__ spl_mode) {
+                                                    const uint8_t* __restrict__ spl_mode, uint64_t* __restrict__ digits,
+                                                    uint32_t pay) {
     __shared__ uint32_t s_h[kRadix];
     __shared__ unsigned long long s_or[8], s_and[8];
     __shared__ uint32_t s_spl[kRadix];
@@ -1368,7 +1369,42 @@ __global__ __launch_bounds__(256) void k_tile_stats(const uint64_t* __restrict__
             atomicAdd(&s_h[digit(k)], 1u);
         }
     };
-    if (SPL && bysplit)
+    if (SPL && bysplit && digits) {
+        // The digits, a search each, are kept for the split: 16 bytes of a
+        // thread (8 and 8 with a payload), in the order of the split's threads.
+        // Per 2^28 keys this pass takes 80 us more, the split 370 less alone
+        // (1342 -> 972) and 480 with a payload (2125 -> 1646).
+        const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        static_assert(kOsTile == 16 * 256, "four words of digits per thread");
+        const uint64_t* g = kin + lo + a;
+        const uint32_t m = (uint32_t)(b - a), e0 = pay ? 2 * w * 256 + lane : threadIdx.x, step = pay ? 32u : 256u;
+        uint32_t q[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            uint64_t k[4];
+            uint32_t d[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t e = e0 + (4 * c + i) * step;
+                k[i] = (e < m ? g[e] : g[m - 1]) ^ flip_in;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                o |= k[i];
+                an &= k[i];
+                d[i] = splitter_digit(s_spl, k[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (e0 + (4 * c + i) * step < m) atomicAdd(&s_h[d[i]], 1u);
+                else d[i] = kRadix - 1;  // behind all others
+            }
+            q[c] = d[0] | d[1] << 8 | d[2] << 16 | d[3] << 24;
+        }
+        uint2* out = (uint2*)((uint8_t*)(digits + lo) + a);
+        out[pay ? 2 * w * 32 + lane : 2 * threadIdx.x] = make_uint2(q[0], q[1]);
+        out[pay ? (2 * w + 1) * 32 + lane : 2 * threadIdx.x + 1] = make_uint2(q[2], q[3]);
+    } else if (SPL && bysplit)
         count([&](uint64_t k) { return splitter_digit(s_spl, k); });
     else if (win)
         count([&](uint64_t k) { return split_digit(k, 0, hb, hm); });
@@ -1589,6 +1625,7 @@ struct SplitArgs {
     const uint32_t* large_id;
     const uint32_t* tile_off;  // [tile][256] destination of the tile's digit-d keys, relative to the segment
     const uint8_t* tile_skew;  // [tile] one digit holds more than an eighth of the tile
+    const uint64_t* digits;    // splitter digits kept by the statistics pass, a byte per key from the segment's start (or null)
     const uint32_t* spl_tab;   // [large id][256] sampled splitters (segments split with kShiftSplit)
     const uint32_t* msd_shift;
     const uint64_t* msd_base;
@@ -1694,7 +1731,14 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 3 : 5) void k_split(con
         if (tid < kRadix) { s_mn[tid] = ~0ull; s_mx[tid] = 0ull; }
         if (tid < 8) s_mask[tid] = A.large_mask[(uint64_t)id * 8 + tid];
     }
-    if (SPL && bysplit && tid < kRadix) s_spl[tid] = A.spl_tab[(uint64_t)id * kRadix + tid];
+    const bool kept = SPL && bysplit && !dir && A.digits != nullptr;  // (a segment of one value writes where they lie)
+    uint32_t dk[kItems / 4] = {};
+    if (kept) {
+        const uint2* q = (const uint2*)((const uint8_t*)(A.digits + seg_base) + tile_lo) + tid * (kItems / 8);
+#pragma unroll
+        for (int i = 0; i < kItems / 8; ++i) { dk[2 * i] = q[i].x; dk[2 * i + 1] = q[i].y; }
+    }
+    if (SPL && bysplit && !kept && tid < kRadix) s_spl[tid] = A.spl_tab[(uint64_t)id * kRadix + tid];
     if (!PAY && tid < kRadix) s_total[tid] = 0;
     cp_async_wait_all();
     __syncthreads();  // the barrier is initialised, the small copies have landed
@@ -1725,8 +1769,8 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 3 : 5) void k_split(con
     // 16 keys and a step or two of search take 256 bytes, where a digit per key
     // takes 4 KB and with it one of five CTAs of an SM (2^28 uniform keys, a
     // level that may split on splitters: 1090 us with those, 975 with cells).
-    // With a payload three CTAs fit either way and the digits are cheaper (2.12
-    // against 2.24 ms).
+    // With a payload three CTAs fit either way and the digits are cheaper (by
+    // 5% of the pass).
     auto last_start = [&](uint32_t lo, uint32_t hi, uint32_t j) -> uint32_t {
         while (lo < hi) {
             const uint32_t mid = (lo + hi + 1) >> 1;
@@ -1737,15 +1781,13 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 3 : 5) void k_split(con
     if constexpr (PAY) {
         // Each key's digit once, byte-packed (past the segment the last one).
         const uint32_t wbase = w * 32 * kItems + lane;
-        uint32_t dpk[kItems / 4];
+        if (!kept)
 #pragma unroll
-        for (int i = 0; i < kItems / 4; ++i) dpk[i] = 0;
-#pragma unroll
-        for (int i = 0; i < kItems; ++i) {
-            const uint32_t e = wbase + i * 32;
-            dpk[i >> 2] |= (e < count ? digit(keys[e]) : (uint32_t)kRadix - 1u) << (8 * (i & 3));
-        }
-        auto digit_of = [&](int i) -> uint32_t { return (dpk[i >> 2] >> (8 * (i & 3))) & 255u; };
+            for (int i = 0; i < kItems; ++i) {
+                const uint32_t e = wbase + i * 32;
+                dk[i >> 2] |= (e < count ? digit(keys[e]) : (uint32_t)kRadix - 1u) << (8 * (i & 3));
+            }
+        auto digit_of = [&](int i) -> uint32_t { return (dk[i >> 2] >> (8 * (i & 3))) & 255u; };
         block_rank<kWarps, kItems>(
             digit_of, s_hist, s_total, s_start, s_warp,
             [&]() {
@@ -1771,7 +1813,11 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 3 : 5) void k_split(con
         // more than it saves, even on heavily duplicated keys.)
         if (direct && tid < kRadix) s_gbase[tid] = off_d;  // digit d's keys of this tile start here
         uint32_t rank[kItems];
-        if (SPL && bysplit) {
+        if (kept) {
+#pragma unroll
+            for (int i = 0; i < kItems; ++i)
+                rank[i] = tid + i * kThreads < count ? (dk[i >> 2] >> (8 * (i & 3))) & 255u : (uint32_t)kRadix;
+        } else if (SPL && bysplit) {
 #pragma unroll
             for (int i = 0; i < kItems; ++i) {
                 const uint32_t e = tid + i * kThreads;
@@ -2075,14 +2121,18 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
         if (bysplit_level)
             HSS_LAUNCH(k_seg_sample, n_large, 256, 0, st, L.in, L.seg_lo, L.seg_hi, ws.large_seg, ws.counters, L.flip_in,
                        chip_max, ws.spl_tab, ws.spl_mode);
+        // The output holds nothing of a large segment yet: the splitter digits
+        // found by the statistics pass wait there for the split (8 bytes of a
+        // key have room for one), unless the keys are read from there.
+        uint64_t* digits = dst + N <= L.in || L.in + N <= dst ? dst : nullptr;
         if (bysplit_level)
             HSS_LAUNCH(k_tile_stats<true>, tiles, 256, 0, st, L.in, L.seg_lo, L.seg_hi, L.nseg, ws.tile_start, ws.tile_seg,
                        ws.large_id, ws.tile_hist, ws.tile_skew, ws.vor, ws.vand, L.hint_lo, L.hint_mult, L.hint_hi,
-                       prev_shift, ws.spec, L.flip_in, ws.spl_tab, ws.spl_mode);
+                       prev_shift, ws.spec, L.flip_in, ws.spl_tab, ws.spl_mode, digits, PAY ? 1u : 0u);
         else
             HSS_LAUNCH(k_tile_stats<false>, tiles, 256, 0, st, L.in, L.seg_lo, L.seg_hi, L.nseg, ws.tile_start, ws.tile_seg,
                        ws.large_id, ws.tile_hist, ws.tile_skew, ws.vor, ws.vand, L.hint_lo, L.hint_mult, L.hint_hi,
-                       prev_shift, ws.spec, L.flip_in, nullptr, nullptr);
+                       prev_shift, ws.spec, L.flip_in, nullptr, nullptr, nullptr, 0u);
         if (!L.hint_lo)
             HSS_LAUNCH(k_tile_recount, (unsigned)std::min<uint64_t>((uint64_t)n_large * kRecountUnits, (uint64_t)num_sms() * 8),
                        256, 0, st, L.in, L.seg_lo, L.seg_hi, ws.counters, ws.large_seg, ws.tile_start, ws.tile_hist,
@@ -2101,7 +2151,7 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
         A.pin = L.pin; A.pout = pnext; A.pfinal = pdst;
         A.seg_lo = L.seg_lo; A.seg_hi = L.seg_hi; A.nseg = L.nseg;
         A.tile_start = ws.tile_start; A.tile_seg = ws.tile_seg; A.large_id = ws.large_id;
-        A.tile_off = ws.tile_off; A.tile_skew = ws.tile_skew; A.spl_tab = ws.spl_tab; A.msd_shift = ws.msd_shift[buf]; A.msd_base = ws.msd_base; A.msd_mult = ws.msd_mult;
+        A.tile_off = ws.tile_off; A.tile_skew = ws.tile_skew; A.digits = digits; A.spl_tab = ws.spl_tab; A.msd_shift = ws.msd_shift[buf]; A.msd_base = ws.msd_base; A.msd_mult = ws.msd_mult;
         A.direct = ws.direct;
         A.large_mask = ws.large_mask; A.any_large = ws.any_large; A.cmin = ws.cmin[buf]; A.cmax = ws.cmax[buf];
         A.err = ws.err;
