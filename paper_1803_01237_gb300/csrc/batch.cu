@@ -127,7 +127,8 @@ __global__ __launch_bounds__(kSampThreads) void kb_sample_mark(
     const int32_t* __restrict__ chgL, const int32_t* __restrict__ chgU, const uint32_t* __restrict__ probe_pos,
     const DCut* __restrict__ Lcut, const uint32_t* __restrict__ int_rep, uint32_t round, uint32_t* __restrict__ bitmap,
     uint32_t* __restrict__ seg_cnt) {
-    __shared__ uint32_t s_a[kIntChunk], s_b[kIntChunk], s_pre[kIntChunk + 1];
+    __shared__ uint32_t s_a[kIntChunk], s_b[kIntChunk];
+    __shared__ __align__(16) uint32_t s_pre[kIntChunk + 1];
     __shared__ uint32_t s_warp[32];
     const uint32_t g = blockIdx.x;
     const uint32_t j = job_of_seg[g];
@@ -153,7 +154,7 @@ __global__ __launch_bounds__(kSampThreads) void kb_sample_mark(
     for (uint32_t u0 = 0; u0 < nint; u0 += kIntChunk) {
         const uint32_t nu = min((uint32_t)kIntChunk, nint - u0);
         const uint32_t P = load_seg_intervals(s, n_s, S, u0, nu, Lpos + J.lbase, Upos + J.lbase, Lcut + J.ibase,
-                                              int_rep + J.ibase, s_a, s_b, s_pre, s_warp);
+                                              int_rep + J.ibase, nullptr, s_a, s_b, s_pre, s_warp);
         auto thr = [&](uint32_t, uint64_t& Tu, bool& all_u) { Tu = T; all_u = take_all; };
         mark_pairs(pd, s_a, s_b, s_pre, nu, 0u, P, thr, base, bitmap, cnt);
         __syncthreads();

@@ -91,7 +91,7 @@ RoundWs rounds_ws_carve(void* base, uint64_t N, uint64_t p, uint64_t cap, uint32
     w.int_rep = (uint32_t*)take(S1 * sizeof(uint32_t));
     w.int_T = (uint64_t*)take(S1 * sizeof(uint64_t));
     w.int_all = (uint32_t*)take(S1 * sizeof(uint32_t));
-    take(S1 * sizeof(uint32_t));
+    w.int_seg = (uint32_t*)take(S1 * sizeof(uint32_t));
     w.bitmap = (uint32_t*)take((N / 32 + 2) * sizeof(uint32_t));
     w.seg_cnt = (uint32_t*)take(p * sizeof(uint32_t));
     w.seg_cnt_off = (uint32_t*)take((p + 1) * sizeof(uint32_t));
@@ -148,11 +148,11 @@ __device__ __forceinline__ void intervals_pass(uint32_t S, uint64_t N, uint32_t 
                                                const DCut* Lcut, const DCut* Ucut, uint32_t* __restrict__ res,
                                                uint32_t* __restrict__ int_rep, RoundCtl* ctl, uint32_t schedule,
                                                uint64_t T_ovr, uint32_t all_ovr, uint64_t* __restrict__ int_T,
-                                               uint32_t* __restrict__ int_all) {
+                                               uint32_t* __restrict__ int_all, uint32_t* __restrict__ int_seg) {
     IntervalsOut o;
     const bool equal = schedule == HSS_SCHEDULE_EQUAL;
     intervals_body(S, N, p, tol, oversample, Lcut, Ucut, res, int_rep, o, equal ? int_T : nullptr,
-                   equal ? int_all : nullptr);
+                   equal ? int_all : nullptr, int_seg);
     if (threadIdx.x == 0) {
         ctl->gamma = o.gamma;
         ctl->nint = o.nint;
@@ -167,8 +167,8 @@ __global__ __launch_bounds__(1024) void k_intervals(uint32_t S, uint64_t N, uint
                                                     const DCut* Lcut, const DCut* Ucut, uint32_t* __restrict__ res,
                                                     uint32_t* __restrict__ int_rep, RoundCtl* ctl, uint32_t schedule,
                                                     uint64_t T_ovr, uint32_t all_ovr, uint64_t* __restrict__ int_T,
-                                                    uint32_t* __restrict__ int_all) {
-    intervals_pass(S, N, p, tol, oversample, Lcut, Ucut, res, int_rep, ctl, schedule, T_ovr, all_ovr, int_T, int_all);
+                                                    uint32_t* __restrict__ int_all, uint32_t* __restrict__ int_seg) {
+    intervals_pass(S, N, p, tol, oversample, Lcut, Ucut, res, int_rep, ctl, schedule, T_ovr, all_ovr, int_T, int_all, int_seg);
 }
 
 // ---------------------------------------------------------------------------
@@ -184,10 +184,12 @@ __global__ __launch_bounds__(1024) void k_intervals(uint32_t S, uint64_t N, uint
 // not exceed the threshold's.  Round 1 over 2^28 keys: 507 -> 296 us.
 __global__ __launch_bounds__(kSampThreads, 4) void k_sample_mark(
     const uint64_t* __restrict__ seg_off, uint32_t S, uint32_t* Lpos, uint32_t* Upos, const DCut* __restrict__ Lcut,
-    const uint32_t* __restrict__ int_rep, const RoundCtl* __restrict__ ctl, uint64_t seed, uint32_t round, uint32_t* __restrict__ bitmap, uint32_t* __restrict__ seg_cnt,
+    const uint32_t* __restrict__ int_rep, const uint32_t* __restrict__ int_seg, const RoundCtl* __restrict__ ctl,
+    uint64_t seed, uint32_t round, uint32_t* __restrict__ bitmap, uint32_t* __restrict__ seg_cnt,
     const uint64_t* __restrict__ int_T, const uint32_t* __restrict__ int_all, const int32_t* __restrict__ chgL,
     const int32_t* __restrict__ chgU, const uint32_t* __restrict__ probe_pos, uint64_t cap) {
-    __shared__ uint32_t s_a[kIntChunk], s_b[kIntChunk], s_pre[kIntChunk + 1];
+    __shared__ uint32_t s_a[kIntChunk], s_b[kIntChunk];
+    __shared__ __align__(16) uint32_t s_pre[kIntChunk + 1];
     __shared__ uint32_t s_warp[32];
     const uint32_t s = blockIdx.x;
     const uint64_t base = seg_off[s];
@@ -208,7 +210,7 @@ __global__ __launch_bounds__(kSampThreads, 4) void k_sample_mark(
     for (uint32_t u0 = 0; u0 < nint; u0 += kIntChunk) {
         const uint32_t nu = min((uint32_t)kIntChunk, nint - u0);
         const uint32_t P = load_seg_intervals(s, (uint32_t)(seg_off[s + 1] - base), S, u0, nu, Lpos, Upos, Lcut, int_rep,
-                                              s_a, s_b, s_pre, s_warp);
+                                              int_seg, s_a, s_b, s_pre, s_warp);
         // this CTA's share of the pairs, then each thread's run of it
         const uint32_t F0 = (uint32_t)(((uint64_t)P * blockIdx.y) / gridDim.y);
         const uint32_t F1 = (uint32_t)(((uint64_t)P * (blockIdx.y + 1)) / gridDim.y);
@@ -697,7 +699,7 @@ __global__ __launch_bounds__(1024) void k_update_intervals(
     const uint32_t* __restrict__ pspos, const uint64_t* __restrict__ prank, uint64_t Z, DCut* Lcut, DCut* Ucut,
     int32_t* __restrict__ chgL, int32_t* __restrict__ chgU, uint64_t tol, float oversample, uint32_t* __restrict__ res,
     uint32_t* __restrict__ int_rep, RoundCtl* ctl, uint32_t schedule, uint64_t T_ovr, uint32_t all_ovr,
-    uint64_t* __restrict__ int_T, uint32_t* __restrict__ int_all) {
+    uint64_t* __restrict__ int_T, uint32_t* __restrict__ int_all, uint32_t* __restrict__ int_seg) {
     extern __shared__ uint64_t s_rank[];  // the probes' ranks: the searches run on chip
     if (Z == kZFromCtl) Z = ctl->seg_off_z[1];
     for (uint32_t k = threadIdx.x; k < (uint32_t)Z; k += blockDim.x) s_rank[k] = prank[k];
@@ -705,7 +707,7 @@ __global__ __launch_bounds__(1024) void k_update_intervals(
     for (uint32_t i = threadIdx.x; i < S; i += blockDim.x)
         update_splitter(i, N, p, pkey, pseg, pspos, s_rank, Z, kMember, Lcut, Ucut, chgL, chgU);
     __syncthreads();
-    intervals_pass(S, N, p, tol, oversample, Lcut, Ucut, res, int_rep, ctl, schedule, T_ovr, all_ovr, int_T, int_all);
+    intervals_pass(S, N, p, tol, oversample, Lcut, Ucut, res, int_rep, ctl, schedule, T_ovr, all_ovr, int_T, int_all, int_seg);
 }
 
 // The positions of proposed cuts (those of a round's probes are taken by the
@@ -918,7 +920,7 @@ static cudaError_t enqueue_sampling(const RoundWs& ws, const uint64_t* d_seg_off
     // round 1 samples whole segments: several CTAs share each; later rounds
     // sample narrow intervals, one CTA per segment
     HSS_LAUNCH(k_sample_mark, dim3(p, round == 1 ? mark_chunks(N, p) : 1u), kSampThreads, 0, st, d_seg_off, S, ws.Lpos,
-               ws.Upos, ws.Lcut, ws.int_rep, ws.ctl, seed, round, ws.bitmap, ws.seg_cnt,
+               ws.Upos, ws.Lcut, ws.int_rep, ws.int_seg, ws.ctl, seed, round, ws.bitmap, ws.seg_cnt,
                per_interval ? ws.int_T : nullptr, per_interval ? ws.int_all : nullptr, moved ? ws.chgL : nullptr, ws.chgU,
                ws.probe_pos, ws.cap);
     return cudaGetLastError();
@@ -933,13 +935,13 @@ static void enqueue_update(const RoundWs& ws, uint32_t S, uint64_t N, uint32_t N
         ensure_func_attrs((const void*)k_update_intervals, (int)(kFusedProbes * 8)) == cudaSuccess) {
         HSS_LAUNCH(k_update_intervals, 1, 1024, (size_t)most * 8, st, S, N, NB, ws.pkey, ws.pseg, ws.pspos, ws.prank, Z, ws.Lcut, ws.Ucut,
                    ws.chgL, ws.chgU, tol, oversample, ws.res, ws.int_rep, ws.ctl, schedule, T_ovr, all_ovr, ws.int_T,
-                   ws.int_all);
+                   ws.int_all, ws.int_seg);
         return;
     }
     HSS_LAUNCH(k_update, (unsigned)cdiv(S, 256), 256, 0, st, S, N, NB, ws.pkey, ws.pseg, ws.pspos, ws.prank, Z,
                (int32_t)kMember, ws.Lcut, ws.Ucut, ws.chgL, ws.chgU, ws.ctl);
     HSS_LAUNCH(k_intervals, 1, 1024, 0, st, S, N, NB, tol, oversample, ws.Lcut, ws.Ucut, ws.res, ws.int_rep, ws.ctl,
-               schedule, T_ovr, all_ovr, ws.int_T, ws.int_all);
+               schedule, T_ovr, all_ovr, ws.int_T, ws.int_all, ws.int_seg);
 }
 
 bool device_loop_possible(uint64_t cap, uint32_t schedule) {
@@ -1155,7 +1157,7 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
         uint32_t allq;
         threshold(r, Tq, allq);
         HSS_LAUNCH(k_intervals, 1, 1024, 0, st, S, N, NB, tol, oversample, ws.Lcut, ws.Ucut, ws.res, ws.int_rep, ws.ctl,
-                   schedule, Tq, allq, ws.int_T, ws.int_all);
+                   schedule, Tq, allq, ws.int_T, ws.int_all, ws.int_seg);
     };
     // The histogram of Z probes in nint intervals of gamma keys.
     auto histogram = [&](uint64_t Z, uint32_t nint, uint64_t gamma) -> cudaError_t {

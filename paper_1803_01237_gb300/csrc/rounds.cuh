@@ -43,6 +43,7 @@ struct RoundWs {
     uint32_t* int_rep;   // [S] representative splitter of each distinct unresolved interval
     uint64_t* int_T;     // [S] per-interval threshold (equal-per-interval schedule)
     uint32_t* int_all;   // [S] per-interval take-all flag
+    uint32_t* int_seg;   // [S] segment of the interval's lower cut (~0: not a member)
     uint32_t* bitmap;    // [N/32 + 2]
     uint32_t* seg_cnt;   // [p]
     uint32_t* seg_cnt_off;  // [p + 1]

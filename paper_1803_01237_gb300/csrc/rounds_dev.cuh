@@ -83,10 +83,12 @@ struct IntervalsOut {
 // valid in thread 0.
 // With int_T non-null, every distinct interval u also gets the threshold of
 // the equal-per-interval schedule: probability (s p / nint) / its length.
+// With int_seg non-null, also the segment of its lower cut (~0: not a member).
 __device__ __forceinline__ void intervals_body(uint32_t S, uint64_t N, uint32_t p, uint64_t tol, float oversample,
                                                const DCut* Lcut, const DCut* Ucut, uint32_t* __restrict__ res,
                                                uint32_t* int_rep, IntervalsOut& out, uint64_t* __restrict__ int_T = nullptr,
-                                               uint32_t* __restrict__ int_all = nullptr) {
+                                               uint32_t* __restrict__ int_all = nullptr,
+                                               uint32_t* __restrict__ int_seg = nullptr) {
     __shared__ uint32_t s_u32[32];
     __shared__ int32_t s_i32[32];
     __shared__ uint64_t s_u64[32];
@@ -96,7 +98,7 @@ __device__ __forceinline__ void intervals_body(uint32_t S, uint64_t N, uint32_t 
     for (uint32_t base = 0; base < S; base += blockDim.x) {
         const uint32_t i = base + threadIdx.x;
         const bool valid = i < S;
-        uint32_t head = 0, unres = 0;
+        uint32_t head = 0, unres = 0, member = ~0u;
         uint64_t glen = 0;
         if (valid) {
             const DCut L = Lcut[i], U = Ucut[i];
@@ -106,6 +108,7 @@ __device__ __forceinline__ void intervals_body(uint32_t S, uint64_t N, uint32_t 
             unres = r ? 0u : 1u;
             head = (i == 0) || !(cut_equal(L, Lcut[i - 1]) && cut_equal(U, Ucut[i - 1]));
             glen = U.rank - L.rank - (L.kind == kMember ? 1u : 0u);
+            if (L.kind == kMember) member = (uint32_t)L.seg;
         }
         uint32_t tot;
         const uint32_t heads_incl = block_incl_scan<uint32_t>(head, 0u, AddU32(), s_u32, tot) + carry_heads;
@@ -126,7 +129,10 @@ __device__ __forceinline__ void intervals_body(uint32_t S, uint64_t N, uint32_t 
         const uint32_t f = (valid && unres && mexcl != rid) ? 1u : 0u;
         uint32_t ftot;
         const uint32_t fincl = block_incl_scan<uint32_t>(f, 0u, AddU32(), s_u32, ftot);
-        if (f) int_rep[carry_f + fincl - 1] = i;
+        if (f) {
+            int_rep[carry_f + fincl - 1] = i;
+            if (int_seg) int_seg[carry_f + fincl - 1] = member;
+        }
         carry_f += ftot;
         uint32_t utot;
         block_incl_scan<uint32_t>(unres, 0u, AddU32(), s_u32, utot);
@@ -169,41 +175,61 @@ constexpr int kIntChunk = 2048;
 constexpr int kSampThreads = 256;
 
 // Fill the interval ranges of segment s for intervals [u0, u0+nu) and the
-// exclusive prefix of their position-pair counts.  Returns the pair total.
+// exclusive prefix of their position-pair counts (s_pre, 16-byte aligned).
+// Returns the pair total.  Neighbouring threads read neighbouring intervals,
+// and (int_seg) the segments of the lower cuts from an array of their own: with
+// eight intervals in a row per thread and the cuts' records, 4095 intervals in
+// 4096 segments cost a round 30 to 50 us more.
 __device__ __forceinline__ uint32_t load_seg_intervals(uint32_t s, uint32_t n_s, uint32_t S, uint32_t u0, uint32_t nu,
                                        const uint32_t* Lpos, const uint32_t* Upos,
                                        const DCut* __restrict__ Lcut, const uint32_t* __restrict__ int_rep,
+                                       const uint32_t* __restrict__ int_seg,
                                        uint32_t* s_a, uint32_t* s_b, uint32_t* s_pre, uint32_t* s_warp) {
     constexpr int kPer = kIntChunk / kSampThreads;
-    uint32_t loc[kPer];
-    uint32_t sum = 0;
+    static_assert(kPer == 8, "two vectors of counts per thread");
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
-        const uint32_t u = threadIdx.x * kPer + k;
+        if ((uint32_t)(k * kSampThreads) >= nu) break;
+        const uint32_t u = threadIdx.x + k * kSampThreads;
         uint32_t np = 0;
         if (u < nu) {
             const uint32_t rep = int_rep[u0 + u];
-            const DCut L = Lcut[rep];
+            uint32_t member;
+            if (int_seg) member = int_seg[u0 + u];
+            else member = Lcut[rep].kind == kMember ? (uint32_t)Lcut[rep].seg : ~0u;
             uint32_t a = Lpos[(uint64_t)s * S + rep];
-            if (L.kind == kMember && (uint32_t)L.seg == s) a += 1;
+            if (member == s) a += 1;
             uint32_t b = Upos[(uint64_t)s * S + rep];
             if (b > n_s) b = n_s;  // defensive: a range never leaves its segment
             s_a[u] = a;
             s_b[u] = b;
             np = b > a ? ((b - 1) >> 1) - (a >> 1) + 1 : 0u;
         }
-        loc[k] = sum;
-        sum += np;
+        s_pre[u] = np;
     }
-    uint32_t tot;
-    const uint32_t incl = block_incl_scan<uint32_t>(sum, 0u, AddU32(), s_warp, tot);
-    const uint32_t ex = incl - sum;
+    __syncthreads();
+    uint32_t c[kPer] = {};
+    uint4* own = (uint4*)s_pre + 2 * threadIdx.x;
+    const bool mine = threadIdx.x * kPer < nu;
+    if (mine) {
+        const uint4 x = own[0], y = own[1];
+        c[0] = x.x; c[1] = x.y; c[2] = x.z; c[3] = x.w; c[4] = y.x; c[5] = y.y; c[6] = y.z; c[7] = y.w;
+    }
+    uint32_t sum = 0, tot;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) sum += c[k];
+    uint32_t run = block_incl_scan<uint32_t>(sum, 0u, AddU32(), s_warp, tot) - sum;
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
-        const uint32_t u = threadIdx.x * kPer + k;
-        if (u < nu) s_pre[u] = ex + loc[k];
+        const uint32_t x = c[k];
+        c[k] = run;
+        run += x;
     }
-    if (threadIdx.x == 0) s_pre[nu] = tot;
+    if (mine) {
+        own[0] = make_uint4(c[0], c[1], c[2], c[3]);
+        own[1] = make_uint4(c[4], c[5], c[6], c[7]);
+    }
+    if (threadIdx.x == 0) s_pre[nu] = tot;  // what a thread whose row holds this place writes there too
     __syncthreads();
     return tot;
 }
