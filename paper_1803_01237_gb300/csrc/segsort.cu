@@ -316,37 +316,6 @@ __device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t
                  "l"(gsrc), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
 }
-// In-place ascending sort of s[0..m) by the whole CTA: a bitonic network over
-// the next power of two P >= m in the form whose comparators all put the
-// smaller key at the lower index (the first step of every merge compares
-// mirrored positions), so that positions past m act as +infinity and are
-// never touched.  Ends with a barrier.
-template <int THREADS, typename T>
-__device__ __forceinline__ void cta_bitonic_sort(T* s, uint32_t m) {
-    uint32_t P = 1;
-    while (P < m) P <<= 1;
-    for (uint32_t k = 2; k <= P; k <<= 1) {
-        for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-            for (uint32_t t = threadIdx.x; t < (P >> 1); t += THREADS) {
-                uint32_t i, l;
-                if (j == (k >> 1)) {  // mirrored pairs of each k-block
-                    const uint32_t blk = t / j, r = t - blk * j;
-                    i = blk * k + r;
-                    l = blk * k + k - 1 - r;
-                } else {
-                    i = (t / j) * 2 * j + (t % j);
-                    l = i + j;
-                }
-                if (l < m) {
-                    const T x = s[i], y = s[l];
-                    if (y < x) { s[i] = y; s[l] = x; }
-                }
-            }
-            __syncthreads();
-        }
-    }
-}
-
 // CTAs per SM the register budget must allow: what their shared memory lets
 // an SM hold (with a payload; seven against six: 2^28 pairs 2.37 -> 2.30 ms.
 // Keys alone would spill for a ninth: 1.47 -> 1.58 ms).
@@ -1003,38 +972,68 @@ __device__ __forceinline__ PlanV plan_item(const uint64_t* seg_lo, const uint64_
     return v;
 }
 
-// Inclusive scan of PlanV over the CTA; returns the totals in tot.
-__device__ __forceinline__ void plan_scan(PlanV& v, PlanV& tot) {
+// From inclusive sums inside each warp (keys: the warp's sum, in lane 31) to
+// sums over the CTA's warps so far, and the CTA's totals in tot.  The keys are
+// only totalled.  Each warp adds up the others' sums with reductions (a loop
+// over the warps by every thread, and shuffles for the flags, took most of the
+// time: 4.2 million segments counted in 112 us, now 28, and written in 83, now
+// 32; one CTA of 1024 segments 7, now 4).
+__device__ __forceinline__ void plan_cross(PlanV& v, PlanV& tot) {
     __shared__ uint32_t s_c[5][32];
     __shared__ unsigned long long s_k[32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-#pragma unroll
-        for (int i = 0; i < 5; ++i) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, v.c[i], o);
-            if (lane >= o) v.c[i] += y;
-        }
-        const unsigned long long yk = __shfl_up_sync(0xffffffffu, v.keys, o);
-        if (lane >= o) v.keys += yk;
-    }
     if (lane == 31) {
 #pragma unroll
         for (int i = 0; i < 5; ++i) s_c[i][w] = v.c[i];
         s_k[w] = v.keys;
     }
     __syncthreads();
-    tot = PlanV{{0, 0, 0, 0, 0}, 0ull};
-    for (int j = 0; j < nw; ++j) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const uint32_t x = lane < nw ? s_c[i][lane] : 0u;
+        v.c[i] += __reduce_add_sync(0xffffffffu, lane < w ? x : 0u);
+        tot.c[i] = __reduce_add_sync(0xffffffffu, x);
+    }
+    unsigned long long k = lane < nw ? s_k[lane] : 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+    tot.keys = k;
+    __syncthreads();
+}
+// Inclusive scan of the CTA's items: flags by ballots, tiles and keys only in
+// warps that hold a large segment.
+__device__ __forceinline__ void plan_scan_items(PlanV& v, PlanV& tot) {
+    const uint32_t lane = threadIdx.x & 31, upto = 0xffffffffu >> (31 - lane);
+    uint32_t large = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        large = __ballot_sync(0xffffffffu, v.c[i] != 0u);
+        v.c[i] = __popc(large & upto);
+    }
+    if (large) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, v.c[4], o);
+            const unsigned long long yk = __shfl_up_sync(0xffffffffu, v.keys, o);
+            if (lane >= (uint32_t)o) { v.c[4] += y; v.keys += yk; }
+        }
+    }
+    plan_cross(v, tot);
+}
+// The same for the chunks' totals.
+__device__ __forceinline__ void plan_scan(PlanV& v, PlanV& tot) {
+    const uint32_t lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
-            if (j < w) v.c[i] += s_c[i][j];
-            tot.c[i] += s_c[i][j];
+            const uint32_t y = __shfl_up_sync(0xffffffffu, v.c[i], o);
+            if (lane >= (uint32_t)o) v.c[i] += y;
         }
-        if (j < w) v.keys += s_k[j];
-        tot.keys += s_k[j];
+        const unsigned long long yk = __shfl_up_sync(0xffffffffu, v.keys, o);
+        if (lane >= (uint32_t)o) v.keys += yk;
     }
-    __syncthreads();
+    plan_cross(v, tot);
 }
 
 __device__ __forceinline__ void blk_store(uint32_t* blk, uint32_t i, const PlanV& v) {
@@ -1055,7 +1054,7 @@ __device__ __forceinline__ PlanV blk_load(const uint32_t* blk, uint32_t i) {
 __global__ __launch_bounds__(1024) void k_plan_count(const uint64_t* __restrict__ seg_lo, const uint64_t* __restrict__ seg_hi,
                                                      uint64_t nseg, uint32_t* __restrict__ blk, uint32_t chip_max) {
     PlanV v = plan_item(seg_lo, seg_hi, nseg, (uint64_t)blockIdx.x * 1024 + threadIdx.x, chip_max), tot;
-    plan_scan(v, tot);
+    plan_scan_items(v, tot);
     if (threadIdx.x == 0) blk_store(blk, blockIdx.x, tot);
 }
 
@@ -1085,7 +1084,7 @@ __global__ __launch_bounds__(1024) void k_plan_scan(uint32_t nblk, uint32_t* __r
             PlanV ex;
 #pragma unroll
             for (int k = 0; k < 5; ++k) ex.c[k] = carry.c[k] + v.c[k] - v0.c[k];
-            ex.keys = carry.keys + v.keys - v0.keys;
+            ex.keys = 0ull;  // not used
             blk_store(blk, i, ex);
         }
 #pragma unroll
@@ -1145,7 +1144,7 @@ __global__ __launch_bounds__(1024) void k_plan_write(const uint64_t* __restrict_
     const PlanV item = plan_item(seg_lo, seg_hi, nseg, s, chip_max);
     if (s < nseg && seg_hi[s] - seg_lo[s] >= kMaxSegKeys) atomicOr(P.err, kDevErrSize);
     PlanV v = item, tot;
-    plan_scan(v, tot);
+    plan_scan_items(v, tot);
     const PlanV off = blk_load(blk, blockIdx.x);
     if (s < nseg) plan_entries(s, item, v, off, P);
     plan_tiles((uint32_t)s, off.c[4] + v.c[4] - item.c[4], item.c[4], P.tile_seg);
@@ -1165,7 +1164,7 @@ __global__ __launch_bounds__(1024) void k_plan_one(const uint64_t* __restrict__ 
         const PlanV item = plan_item(seg_lo, seg_hi, nseg, s, chip_max);
         if (s < nseg && seg_hi[s] - seg_lo[s] >= kMaxSegKeys) atomicOr(P.err, kDevErrSize);
         PlanV v = item, tot;
-        plan_scan(v, tot);
+        plan_scan_items(v, tot);
         if (s < nseg) plan_entries(s, item, v, carry, P);
         plan_tiles((uint32_t)s, carry.c[4] + v.c[4] - item.c[4], item.c[4], P.tile_seg);
 #pragma unroll
@@ -1225,6 +1224,58 @@ constexpr uint64_t kSplMax = 1ull << 19;
 // hide, and the 256 byte sub-buckets of a clustered one mostly fit the chip.
 constexpr uint64_t kSplMinKeys = 1ull << 22;
 constexpr uint64_t kSplMinSeg = 1ull << 15;
+// Sort of the sample by the CTA, eight words per thread in, s[0 .. 2047] out: a
+// bitonic network on rows of eight in registers, whose steps between threads of
+// a warp are shuffles; only the six steps between warps meet shared memory
+// (all 66 did: 4096 segments took 242 us, now 100).  Ends with a barrier.
+__device__ __forceinline__ void sort_sample(uint32_t (&v)[8], uint32_t* s) {
+    static_assert(kSplSample == 8 * 256, "eight words per thread");
+    const uint32_t tid = threadIdx.x;
+    sort_8(v);
+    if (tid & 1u) {  // descending
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t a = v[i];
+            v[i] = v[7 - i];
+            v[7 - i] = a;
+        }
+    }
+#pragma unroll
+    for (uint32_t k = 2; k <= 256; k *= 2) {  // runs of 8 k words from pairs of 4 k
+        const bool up = (tid & k) == 0u;
+#pragma unroll
+        for (uint32_t j = k / 2; j >= 1; j /= 2) {
+            const bool low = ((tid & j) == 0u) == up;
+            uint32_t o[8];
+            if (j >= 32) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) s[i * 256 + tid] = v[i];
+                __syncthreads();
+#pragma unroll
+                for (int i = 0; i < 8; ++i) o[i] = s[i * 256 + (tid ^ j)];
+                __syncthreads();
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) o[i] = __shfl_xor_sync(0xffffffffu, v[i], j);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = low ? min(v[i], o[i]) : max(v[i], o[i]);
+        }
+#pragma unroll
+        for (int j = 4; j >= 1; j /= 2)
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (!(i & j)) {
+                    const uint32_t a = min(v[i], v[i | j]), b = max(v[i], v[i | j]);
+                    v[i] = up ? a : b;
+                    v[i | j] = up ? b : a;
+                }
+    }
+    ((uint4*)s)[2 * tid] = make_uint4(v[0], v[1], v[2], v[3]);
+    ((uint4*)s)[2 * tid + 1] = make_uint4(v[4], v[5], v[6], v[7]);
+    __syncthreads();
+}
+
 __global__ __launch_bounds__(256) void k_seg_sample(const uint64_t* __restrict__ kin, const uint64_t* __restrict__ seg_lo,
                                                     const uint64_t* __restrict__ seg_hi,
                                                     const uint32_t* __restrict__ large_seg,
@@ -1232,7 +1283,7 @@ __global__ __launch_bounds__(256) void k_seg_sample(const uint64_t* __restrict__
                                                     uint32_t chip_max, uint32_t* __restrict__ spl_tab,
                                                     uint8_t* __restrict__ spl_mode) {
     constexpr int kPer = kSplSample / 256;
-    __shared__ uint32_t s_x[kSplSample];
+    __shared__ __align__(16) uint32_t s_x[kSplSample];
     __shared__ uint32_t s_h[kRadix];
     __shared__ unsigned long long s_or[8], s_and[8];
     __shared__ uint32_t s_sum[2];
@@ -1276,10 +1327,10 @@ __global__ __launch_bounds__(256) void k_seg_sample(const uint64_t* __restrict__
     const uint32_t crowded = s_sum[0];
     if (crowded < kSplSample / 4) return;  // uniform
     const int sft = max(0, 32 - __clzll((long long)o));
+    uint32_t x[kPer];
 #pragma unroll
-    for (int i = 0; i < kPer; ++i) s_x[tid + i * 256] = (uint32_t)(key[i] >> sft);
-    __syncthreads();
-    cta_bitonic_sort<256>(s_x, (uint32_t)kSplSample);
+    for (int i = 0; i < kPer; ++i) x[i] = (uint32_t)(key[i] >> sft);
+    sort_sample(x, s_x);
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
         const uint32_t j = tid + i * 256;
