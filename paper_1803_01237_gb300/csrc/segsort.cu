@@ -1639,8 +1639,10 @@ __global__ __launch_bounds__(256) void k_msd_prep(const uint64_t* __restrict__ s
     const uint32_t bal = __ballot_sync(0xffffffffu, large);
     if ((d & 31) == 0) large_mask[(uint64_t)id * 8 + (d >> 5)] = bal;
     if (d == 0) any_large[id] = 0u;
-    cmin[(uint64_t)id * kRadix + d] = ~0ull;
-    cmax[(uint64_t)id * kRadix + d] = 0ull;
+    if (chip_max != ~0u) {  // key ranges are gathered at this level
+        cmin[(uint64_t)id * kRadix + d] = ~0ull;
+        cmax[(uint64_t)id * kRadix + d] = 0ull;
+    }
     __syncthreads();
     if (bal && (d & 31) == 0) atomicOr(&any_large[id], 1u);
     uint32_t run = x;
