@@ -1480,39 +1480,62 @@ __global__ __launch_bounds__(256) void k_tile_stats(const uint64_t* __restrict__
 
 // Recount of the tiles of segments whose top varying byte (from the OR/AND of
 // the statistics pass) is not the speculative one: the histogram of that byte
-// into the tile's second row.  A unit of work is every kRecountUnits-th tile
-// of a segment, so the segments that need none (most) cost a check per unit
-// and not one per tile (2^28 keys in 1024 segments, none to do: 63 -> 11 us).
-constexpr uint32_t kRecountUnits = 8;
+// into the tile's second row.  CTA b owns tiles b, b + gridDim.x, ...; its 256
+// threads look at one each, so a level that needs none costs one chain of loads
+// (2^28 keys in 1024 segments: 63 us by a tile per step of a CTA, 6.4 here),
+// and a segment that needs one is spread over all CTAs however few segments
+// there are (keys below 2^40, 2^27 of them in one segment: the sort takes
+// 5.6 ms, 16.5 with eight CTAs per segment).
 __global__ __launch_bounds__(256) void k_tile_recount(
     const uint64_t* __restrict__ kin, const uint64_t* __restrict__ seg_lo, const uint64_t* __restrict__ seg_hi,
-    const uint32_t* __restrict__ counters, const uint32_t* __restrict__ large_seg, const uint32_t* __restrict__ tile_start,
-    uint16_t* __restrict__ tile_hist, uint8_t* __restrict__ tile_skew, const uint8_t* __restrict__ spl_mode,
-    const unsigned long long* __restrict__ vor, const unsigned long long* __restrict__ vand,
-    const uint32_t* __restrict__ spec, uint64_t flip_in) {
+    uint64_t nseg, const uint32_t* __restrict__ tile_start, const uint32_t* __restrict__ tile_seg,
+    const uint32_t* __restrict__ large_id, uint16_t* __restrict__ tile_hist, uint8_t* __restrict__ tile_skew,
+    const uint8_t* __restrict__ spl_mode, const unsigned long long* __restrict__ vor,
+    const unsigned long long* __restrict__ vand, const uint32_t* __restrict__ spec, uint64_t flip_in) {
     __shared__ uint32_t s_h[kRadix];
-    const uint64_t units = (uint64_t)counters[19] * kRecountUnits;
-    for (uint64_t unit = blockIdx.x; unit < units; unit += gridDim.x) {  // uniform per CTA
-        const uint32_t id = (uint32_t)(unit / kRecountUnits);
-        if (spl_mode && spl_mode[id]) continue;  // the statistics pass counted the splitter buckets
-        const unsigned long long vary = vor[id] ^ vand[id];
-        if (vary == 0ull) continue;
-        const uint32_t w = (uint32_t)(63 - __clzll((long long)vary)) >> 3;
-        if (w == spec[id]) continue;
-        const uint32_t s = large_seg[id], t0 = tile_start[s], t1 = tile_start[s + 1];
-        const uint64_t lo = seg_lo[s], n = seg_hi[s] - lo;
-        const int sh = 8 * (int)w;
-        for (uint32_t t = t0 + (uint32_t)(unit % kRecountUnits); t < t1; t += kRecountUnits) {
-            s_h[threadIdx.x] = 0;
-            __syncthreads();
-            const uint64_t a = (uint64_t)(t - t0) * kOsTile, b = min(n, a + kOsTile);
-#pragma unroll 4
-            for (uint64_t e = a + threadIdx.x; e < b; e += 256)
-                atomicAdd(&s_h[(uint32_t)((kin[lo + e] ^ flip_in) >> sh) & 255u], 1u);
-            __syncthreads();
-            tile_hist[(uint64_t)t * (2 * kRadix) + kRadix + threadIdx.x] = (uint16_t)s_h[threadIdx.x];
-            tile_skew_flag(s_h[threadIdx.x], tile_skew, t);  // ends with a barrier
+    __shared__ uint32_t s_todo[8];  // the CTA's tiles to count again, a bit each
+    __shared__ uint64_t s_at[256];   // their first keys
+    __shared__ uint16_t s_cnt[256];  // and numbers of them
+    __shared__ uint8_t s_byte[256];
+    const uint32_t total = tile_start[nseg];
+    for (uint64_t first = blockIdx.x; first < total; first += (uint64_t)256 * gridDim.x) {  // uniform per CTA
+        const uint64_t mine = first + (uint64_t)threadIdx.x * gridDim.x;
+        bool again = false;
+        if (mine < total) {
+            const uint32_t s = tile_seg[mine], id = large_id[s];
+            const unsigned long long vary = vor[id] ^ vand[id];
+            // on sampled splitters the statistics pass has counted the buckets
+            if (vary != 0ull && !(spl_mode && spl_mode[id])) {
+                const uint32_t w = (uint32_t)(63 - __clzll((long long)vary)) >> 3;
+                again = w != spec[id];
+                if (again) {
+                    const uint64_t a = seg_lo[s] + (mine - tile_start[s]) * kOsTile;
+                    s_at[threadIdx.x] = a;
+                    s_cnt[threadIdx.x] = (uint16_t)min((uint64_t)kOsTile, seg_hi[s] - a);
+                    s_byte[threadIdx.x] = (uint8_t)w;
+                }
+            }
         }
+        const uint32_t bal = __ballot_sync(0xffffffffu, again);
+        if ((threadIdx.x & 31) == 0) s_todo[threadIdx.x >> 5] = bal;
+        __syncthreads();
+        for (uint32_t v = 0; v < 8; ++v) {
+            for (uint32_t left = s_todo[v]; left; left &= left - 1) {
+                const uint32_t i = 32 * v + (uint32_t)(__ffs(left) - 1);
+                const uint32_t t = (uint32_t)(first + (uint64_t)i * gridDim.x), m = s_cnt[i];
+                const uint64_t* g = kin + s_at[i];
+                const int sh = 8 * (int)s_byte[i];
+                s_h[threadIdx.x] = 0;
+                __syncthreads();
+#pragma unroll 4
+                for (uint32_t e = threadIdx.x; e < m; e += 256)
+                    atomicAdd(&s_h[(uint32_t)((g[e] ^ flip_in) >> sh) & 255u], 1u);
+                __syncthreads();
+                tile_hist[(uint64_t)t * (2 * kRadix) + kRadix + threadIdx.x] = (uint16_t)s_h[threadIdx.x];
+                tile_skew_flag(s_h[threadIdx.x], tile_skew, t);  // ends with a barrier
+            }
+        }
+        __syncthreads();  // s_todo is written again
     }
 }
 
@@ -2187,9 +2210,9 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
                        ws.large_id, ws.tile_hist, ws.tile_skew, ws.vor, ws.vand, L.hint_lo, L.hint_mult, L.hint_hi,
                        prev_shift, ws.spec, L.flip_in, nullptr, nullptr, nullptr, 0u);
         if (!L.hint_lo)
-            HSS_LAUNCH(k_tile_recount, (unsigned)std::min<uint64_t>((uint64_t)n_large * kRecountUnits, (uint64_t)num_sms() * 8),
-                       256, 0, st, L.in, L.seg_lo, L.seg_hi, ws.counters, ws.large_seg, ws.tile_start, ws.tile_hist,
-                       ws.tile_skew, bysplit_level ? ws.spl_mode : nullptr, ws.vor, ws.vand, ws.spec, L.flip_in);
+            HSS_LAUNCH(k_tile_recount, (unsigned)std::min<uint64_t>(tiles, (uint64_t)num_sms() * 8), 256, 0, st, L.in, L.seg_lo,
+                       L.seg_hi, L.nseg, ws.tile_start, ws.tile_seg, ws.large_id, ws.tile_hist, ws.tile_skew,
+                       bysplit_level ? ws.spl_mode : nullptr, ws.vor, ws.vand, ws.spec, L.flip_in);
         HSS_LAUNCH(k_msd_prep, n_large, 256, 0, st, L.seg_lo, ws.large_seg, ws.counters, ws.tile_start, ws.tile_hist,
                    ws.vor, ws.vand, L.hint_lo, L.hint_mult, ws.msd_base, ws.msd_mult, ws.msd_shift[buf], ws.spec,
                    ws.direct, ws.sub_lo[buf], ws.sub_hi[buf], ws.tile_off, child_interp ? chip_max : 0xffffffffu,
