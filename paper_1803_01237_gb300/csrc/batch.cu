@@ -828,7 +828,12 @@ int run_batch(const void* d_keys, const uint32_t* d_payload, int key_type, const
         if (h.active == 0) break;
         ++round;
         const uint64_t Zc = h.Zc;
-        if (T.N_tot <= kSampWarpKeys * T.P_tot)
+        // A warp per segment where they are short on average, unless the
+        // longest, for which all others wait, is above four times that.  4096
+        // jobs of 2^14 keys and one longer job, four segments each, all rounds
+        // by warps and by CTAs: the one's segments 2^14 keys 1362, 1463 us;
+        // 2^17 keys 1413, 1500; 2^20 keys 1788, 1756; 2^24 keys 10630, 6900.
+        if (T.N_tot <= kSampWarpKeys * T.P_tot && T.max_seg <= 4 * kSampWarpKeys)
             HSS_LAUNCH(kb_sample_write<true>, (unsigned)cdivh(T.P_tot, kSampThreads / 32), kSampThreads, 0, st, T.P_tot,
                        keysA, jobs, jseg, seg_off, ctl, bitmap, seg_cnt, G, zoff, skey, sseg, sspos, siota);
         else
