@@ -1488,7 +1488,7 @@ __global__ __launch_bounds__(256) void k_tile_stats(const uint64_t* __restrict__
 // 5.6 ms, 16.5 with eight CTAs per segment).
 __global__ __launch_bounds__(256) void k_tile_recount(
     const uint64_t* __restrict__ kin, const uint64_t* __restrict__ seg_lo, const uint64_t* __restrict__ seg_hi,
-    uint64_t nseg, const uint32_t* __restrict__ tile_start, const uint32_t* __restrict__ tile_seg,
+    uint32_t tiles, const uint32_t* __restrict__ tile_start, const uint32_t* __restrict__ tile_seg,
     const uint32_t* __restrict__ large_id, uint16_t* __restrict__ tile_hist, uint8_t* __restrict__ tile_skew,
     const uint8_t* __restrict__ spl_mode, const unsigned long long* __restrict__ vor,
     const unsigned long long* __restrict__ vand, const uint32_t* __restrict__ spec, uint64_t flip_in) {
@@ -1497,11 +1497,10 @@ __global__ __launch_bounds__(256) void k_tile_recount(
     __shared__ uint64_t s_at[256];   // their first keys
     __shared__ uint16_t s_cnt[256];  // and numbers of them
     __shared__ uint8_t s_byte[256];
-    const uint32_t total = tile_start[nseg];
-    for (uint64_t first = blockIdx.x; first < total; first += (uint64_t)256 * gridDim.x) {  // uniform per CTA
+    for (uint64_t first = blockIdx.x; first < tiles; first += (uint64_t)256 * gridDim.x) {  // uniform per CTA
         const uint64_t mine = first + (uint64_t)threadIdx.x * gridDim.x;
         bool again = false;
-        if (mine < total) {
+        if (mine < tiles) {
             const uint32_t s = tile_seg[mine], id = large_id[s];
             const unsigned long long vary = vor[id] ^ vand[id];
             // on sampled splitters the statistics pass has counted the buckets
@@ -2211,7 +2210,7 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
                        prev_shift, ws.spec, L.flip_in, nullptr, nullptr, nullptr, 0u);
         if (!L.hint_lo)
             HSS_LAUNCH(k_tile_recount, (unsigned)std::min<uint64_t>(tiles, (uint64_t)num_sms() * 8), 256, 0, st, L.in, L.seg_lo,
-                       L.seg_hi, L.nseg, ws.tile_start, ws.tile_seg, ws.large_id, ws.tile_hist, ws.tile_skew,
+                       L.seg_hi, tiles, ws.tile_start, ws.tile_seg, ws.large_id, ws.tile_hist, ws.tile_skew,
                        bysplit_level ? ws.spl_mode : nullptr, ws.vor, ws.vand, ws.spec, L.flip_in);
         HSS_LAUNCH(k_msd_prep, n_large, 256, 0, st, L.seg_lo, ws.large_seg, ws.counters, ws.tile_start, ws.tile_hist,
                    ws.vor, ws.vand, L.hint_lo, L.hint_mult, ws.msd_base, ws.msd_mult, ws.msd_shift[buf], ws.spec,
