@@ -132,6 +132,13 @@ __global__ void k_cdf_init(hss_cdf_model* M, uint64_t seed, int feature, int key
     M->v[k] = 0.f;
 }
 
+// Feature and target of a training point.
+__device__ __forceinline__ float2 point_of(const hss_cdf_model* M, const uint64_t* __restrict__ keys,
+                                           const uint64_t* __restrict__ ranks, uint64_t b, double invN) {
+    const uint64_t flip = M->key_type == HSS_KEY_I64 ? kSignBit : 0ull;
+    return make_float2(feature_of(keys[b], M, flip), (float)((double)ranks[b] * invN));
+}
+
 // Features and targets of the training points, once per call: the feature map
 // is double precision (log2), which the steps would otherwise repeat.
 __global__ __launch_bounds__(kGradThreads) void k_cdf_points(const hss_cdf_model* __restrict__ M,
@@ -141,8 +148,7 @@ __global__ __launch_bounds__(kGradThreads) void k_cdf_points(const hss_cdf_model
     const uint32_t b = blockIdx.x * kGradThreads + threadIdx.x;
     if (b == 0) *arrived = 0u;
     if (b >= n) return;
-    const uint64_t flip = M->key_type == HSS_KEY_I64 ? kSignBit : 0ull;
-    pts[b] = make_float2(feature_of(keys[b], M, flip), (float)((double)ranks[b] * invN));
+    pts[b] = point_of(M, keys, ranks, b, invN);
 }
 
 // One step: the gradient of the mean squared error, and Adam.  Each CTA takes
@@ -155,7 +161,12 @@ __global__ __launch_bounds__(kGradThreads) void k_cdf_points(const hss_cdf_model
 // Bound by the latency of its dependent chains (four warps on an SM, a few
 // SMs).  4096 points: 78 us per step as two kernels that walked the 256 staged
 // rows one load at a time, here 19 us.
-__global__ __launch_bounds__(kGradThreads) void k_cdf_step(hss_cdf_model* M, const float2* __restrict__ pts, uint32_t n,
+// PTS: the points come from pts.  Without (a scratch buffer that has no room
+// for them, see Work) every step computes them from the keys and ranks.
+template <bool PTS>
+__global__ __launch_bounds__(kGradThreads) void k_cdf_step(hss_cdf_model* M, const float2* __restrict__ pts,
+                                                           const uint64_t* __restrict__ keys,
+                                                           const uint64_t* __restrict__ ranks, double invN, uint32_t n,
                                                            float inv_n, float* __restrict__ part,
                                                            uint32_t* __restrict__ arrived, float lr, int apply,
                                                            float* __restrict__ grad_out, float* __restrict__ loss_out) {
@@ -197,7 +208,7 @@ __global__ __launch_bounds__(kGradThreads) void k_cdf_step(hss_cdf_model* M, con
         float x = 0.f, d = 0.f;
         float h1[kH], h2[kH], dz1[kH];
         if (b < n) {
-            const float2 pt = pts[b];
+            const float2 pt = PTS ? pts[b] : point_of(M, keys, ranks, b, invN);
             x = pt.x;
             const float e = layers(th, x, h1, h2) - pt.y;
             d = 2.f * e * inv_n;
@@ -270,6 +281,7 @@ __global__ __launch_bounds__(kGradThreads) void k_cdf_step(hss_cdf_model* M, con
     if (lane == 0) { s_sum[w] = accD; s_sum[kGradThreads / 32 + w] = accL; }
     __syncthreads();
     float* out = part + (uint64_t)blockIdx.x * kPartStride;
+    const bool vec = PTS || ((uintptr_t)part & 15u) == 0;  // the partials lie on 16 bytes
     if (grp == 0) {
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
@@ -279,7 +291,12 @@ __global__ __launch_bounds__(kGradThreads) void k_cdf_step(hss_cdf_model* M, con
                 const float4 o = *(const float4*)(H1s + (g - 1) * 1024 + (i0 + p) * kH + j0);
                 v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
             }
-            *(float4*)(out + kOffW2 + (i0 + p) * kH + j0) = v;
+            float* o = out + kOffW2 + (i0 + p) * kH + j0;
+            if (vec) {
+                *(float4*)o = v;
+            } else {
+                o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+            }
         }
     }
     out[(w == 0 ? 0 : (w == 1 ? kOffB1 : (w == 2 ? kOffB2 : kOffW3))) + lane] = accS;
@@ -306,7 +323,12 @@ __global__ __launch_bounds__(kGradThreads) void k_cdf_step(hss_cdf_model* M, con
         s_c[tid] = (float)(1.0 - q);
     }
     const int G = (int)gridDim.x;
-    for (int k4 = tid; k4 < kPartStride / 4; k4 += kGradThreads) {
+    for (int k = tid; !vec && k < kPartStride; k += kGradThreads) {
+        float g = 0.f;
+        for (int c = 0; c < G; ++c) g += __ldcg(part + (uint64_t)c * kPartStride + k);
+        H1s[k] = g;
+    }
+    for (int k4 = tid; vec && k4 < kPartStride / 4; k4 += kGradThreads) {
         float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 16
         for (int c = 0; c < G; ++c) {
@@ -389,33 +411,61 @@ __global__ void k_cdf_propose(const hss_cdf_model* __restrict__ M, uint32_t p, u
     out[q] = bits ^ flip;
 }
 
-int grad_blocks(uint32_t n) {
-    return (int)std::max<uint32_t>(1, std::min<uint64_t>(kMaxGradBlocks, ((uint64_t)n + kGradThreads - 1) / kGradThreads));
-}
-
 size_t grad_smem() { return (size_t)(kP + 3 + 4 * kGradThreads * kStage + 2 * kGradThreads) * sizeof(float); }
 
-// Scratch: the CTAs' partials, the arrival counter, the points.
+uint32_t grad_blocks(uint32_t n, int points) {  // CTAs for n points, `points` to a CTA
+    return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(kMaxGradBlocks, ((uint64_t)n + points - 1) / points));
+}
+
+// Scratch of a call: the CTAs' partials, the arrival counter, the points.  A
+// buffer too small for that, but of the least size (a partial for every 256
+// points, 32 at most: independent of n from 8192 points on), holds that many
+// partials, the counter in the first one's padding, and no points.
 struct Work {
+    uint32_t blocks;
     float* part;
     uint32_t* arrived;
-    float2* pts;
-    size_t bytes;
-    Work(void* base, uint32_t n) {
-        const size_t p = (size_t)grad_blocks(n) * kPartStride * sizeof(float);  // a multiple of 16
-        char* q = (char*)(((uintptr_t)base + 15) & ~(uintptr_t)15);
-        part = (float*)q;
-        arrived = (uint32_t*)(q + p);
-        pts = (float2*)(q + p + 16);
-        bytes = 16 + p + 16 + (size_t)n * sizeof(float2);
+    float2* pts;  // null: none kept
+    static size_t parts(uint32_t blocks) { return (size_t)blocks * kPartStride * sizeof(float); }  // a multiple of 16
+    static size_t least(uint32_t n) { return parts(grad_blocks(n, 256)); }
+    static size_t bytes(uint32_t n) { return 16 + parts(grad_blocks(n, kGradThreads)) + 16 + (size_t)n * sizeof(float2); }
+    Work(void* base, size_t size, uint32_t n) {
+        if (size >= bytes(n)) {
+            blocks = grad_blocks(n, kGradThreads);
+            char* q = (char*)(((uintptr_t)base + 15) & ~(uintptr_t)15);
+            part = (float*)q;
+            arrived = (uint32_t*)(q + parts(blocks));
+            pts = (float2*)(q + parts(blocks) + 16);
+        } else {
+            blocks = grad_blocks(n, 256);
+            part = (float*)base;
+            arrived = (uint32_t*)(part + kP + 1);
+            pts = nullptr;
+        }
     }
 };
 
-int launch_points(const hss_cdf_model* M, const uint64_t* keys, const uint64_t* ranks, uint32_t n, uint64_t N,
-                  const Work& wk, cudaStream_t st) {
-    if (ensure_func_attrs((const void*)k_cdf_step, (int)grad_smem()) != cudaSuccess) return HSS_ERR_CUDA;
-    HSS_LAUNCH(k_cdf_points, (unsigned)(((uint64_t)n + kGradThreads - 1) / kGradThreads), kGradThreads, 0, st, M, keys, ranks,
-               n, 1.0 / (double)N, wk.pts, wk.arrived);
+// One call's steps: the points (or the counter alone), then a kernel per step.
+int run_steps(hss_cdf_model* M, const uint64_t* keys, const uint64_t* ranks, uint32_t n, uint64_t N, const Work& wk,
+              uint32_t steps, float lr, int apply, float* grad, float* loss, cudaStream_t st) {
+    const double invN = 1.0 / (double)N;
+    const float inv_n = (float)(1.0 / (double)n);
+    const void* fn = wk.pts ? (const void*)k_cdf_step<true> : (const void*)k_cdf_step<false>;
+    if (ensure_func_attrs(fn, (int)grad_smem()) != cudaSuccess) return HSS_ERR_CUDA;
+    if (wk.pts)
+        HSS_LAUNCH(k_cdf_points, (unsigned)(((uint64_t)n + kGradThreads - 1) / kGradThreads), kGradThreads, 0, st, M, keys,
+                   ranks, n, invN, wk.pts, wk.arrived);
+    else if (cudaMemsetAsync(wk.arrived, 0, sizeof(uint32_t), st) != cudaSuccess)
+        return HSS_ERR_CUDA;
+    for (uint32_t s = 0; s < steps; ++s) {
+        float* l = s + 1 == steps ? loss : nullptr;
+        if (wk.pts)
+            HSS_LAUNCH(k_cdf_step<true>, wk.blocks, kGradThreads, grad_smem(), st, M, wk.pts, nullptr, nullptr, invN, n, inv_n,
+                       wk.part, wk.arrived, lr, apply, grad, l);
+        else
+            HSS_LAUNCH(k_cdf_step<false>, wk.blocks, kGradThreads, grad_smem(), st, M, nullptr, keys, ranks, invN, n, inv_n,
+                       wk.part, wk.arrived, lr, apply, grad, l);
+    }
     return cudaGetLastError() == cudaSuccess ? HSS_OK : HSS_ERR_CUDA;
 }
 
@@ -440,7 +490,7 @@ int hss_cdf_set_weights(hss_cdf_model* d_model, int weights, void* stream) {
     return cudaGetLastError() == cudaSuccess ? HSS_OK : HSS_ERR_CUDA;
 }
 
-size_t hss_cdf_work_bytes(uint32_t n) { return Work(nullptr, n).bytes; }
+size_t hss_cdf_work_bytes(uint32_t n) { return Work::bytes(n); }
 
 int hss_cdf_init(hss_cdf_model* d_model, uint64_t seed, int feature, int key_type, uint64_t lo_key, uint64_t hi_key,
                  void* stream) {
@@ -456,29 +506,19 @@ int hss_cdf_init(hss_cdf_model* d_model, uint64_t seed, int feature, int key_typ
 int hss_cdf_grad(const hss_cdf_model* d_model, const void* d_keys, const uint64_t* d_ranks, uint32_t n, uint64_t N,
                  float* d_grad, float* d_loss, void* d_work, size_t work_bytes, void* stream) {
     if (!d_model || n == 0 || N == 0 || !d_keys || !d_ranks || !d_work) return HSS_ERR_INVALID;
-    if (work_bytes < hss_cdf_work_bytes(n)) return HSS_ERR_WORKSPACE;
+    if (work_bytes < Work::least(n)) return HSS_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
-    const Work wk(d_work, n);
-    const int rc = launch_points(d_model, (const uint64_t*)d_keys, d_ranks, n, N, wk, st);
-    if (rc != HSS_OK) return rc;
-    HSS_LAUNCH(k_cdf_step, grad_blocks(n), kGradThreads, grad_smem(), st, const_cast<hss_cdf_model*>(d_model), wk.pts, n,
-               (float)(1.0 / (double)n), wk.part, wk.arrived, 0.f, 0, d_grad, d_loss);
-    return cudaGetLastError() == cudaSuccess ? HSS_OK : HSS_ERR_CUDA;
+    return run_steps(const_cast<hss_cdf_model*>(d_model), (const uint64_t*)d_keys, d_ranks, n, N, Work(d_work, work_bytes, n), 1,
+                     0.f, 0, d_grad, d_loss, st);
 }
 
 int hss_cdf_train(hss_cdf_model* d_model, const void* d_keys, const uint64_t* d_ranks, uint32_t n, uint64_t N,
                   uint32_t steps, float lr, float* d_loss, void* d_work, size_t work_bytes, void* stream) {
     if (!d_model || n == 0 || N == 0 || !d_keys || !d_ranks || !d_work || !(lr > 0.f)) return HSS_ERR_INVALID;
-    if (work_bytes < hss_cdf_work_bytes(n)) return HSS_ERR_WORKSPACE;
+    if (work_bytes < Work::least(n)) return HSS_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     if (steps == 0) return HSS_OK;
-    const Work wk(d_work, n);
-    const int rc = launch_points(d_model, (const uint64_t*)d_keys, d_ranks, n, N, wk, st);
-    if (rc != HSS_OK) return rc;
-    for (uint32_t s = 0; s < steps; ++s)
-        HSS_LAUNCH(k_cdf_step, grad_blocks(n), kGradThreads, grad_smem(), st, d_model, wk.pts, n, (float)(1.0 / (double)n),
-                   wk.part, wk.arrived, lr, 1, nullptr, s + 1 == steps ? d_loss : nullptr);
-    return cudaGetLastError() == cudaSuccess ? HSS_OK : HSS_ERR_CUDA;
+    return run_steps(d_model, (const uint64_t*)d_keys, d_ranks, n, N, Work(d_work, work_bytes, n), steps, lr, 1, nullptr, d_loss, st);
 }
 
 int hss_cdf_eval(const hss_cdf_model* d_model, const void* d_keys, uint32_t n, float* d_y, void* stream) {
