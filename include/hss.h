@@ -519,8 +519,9 @@ typedef struct {
     /* Packing of small sub-buckets: after a split, runs of consecutive
      * sub-buckets that are sorted on chip are merged into one on-chip sort of
      * up to pack_keys keys (their keys are already in order between them, so
-     * sorting the run sorts each).  1 .. 4096; 0 = 1024; 1 packs nothing.
-     * 1024, the default, stands for 1536 at levels of 2^22 keys and more. */
+     * sorting the run sorts each).  1 .. 4096; 1 packs nothing; 0 (default):
+     * 1024, or 1536 at levels of 2^22 keys and more (hss_get_tuning reports
+     * 1024). */
     uint32_t pack_keys;
     /* First split of each segment of a local sort.  A sample of the segment
      * shows whether its top varying byte would crowd the keys into a few

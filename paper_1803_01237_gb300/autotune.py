@@ -47,7 +47,7 @@ class Choice:
     chip_max_keys: int = 4096
     child_interp: int = 0
     child_bucket_keys: int = 384
-    pack_keys: int = 1024
+    pack_keys: int = 0             # 0: by the level's size
     first_split: int = 0
 
     def flags(self) -> int:
@@ -68,7 +68,7 @@ def default_space(p: int):
     splitters (spatially clustered keys, e.g. Morton codes of a Plummer
     sphere, need one split level instead of three)."""
     over = [3.0, 5.0, 8.0, 12.0]
-    tiles = [(4096, 0, 384), (14336, 0, 384), (4096, 1, 384), (4096, 1, 768), (4096, 0, 384, 1024, 1)]
+    tiles = [(4096, 0, 384), (14336, 0, 384), (4096, 1, 384), (4096, 1, 768), (4096, 0, 384, 0, 1)]
     return over, tiles
 
 

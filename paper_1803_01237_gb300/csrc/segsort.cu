@@ -28,18 +28,23 @@ namespace hss {
 __host__ __device__ static inline uint64_t ceil_div(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// The default packing: packs that fill the first on-chip class where a level
-// has enough of them (merge of 2^28 pairs in 4096 buckets 4.44 -> 4.23 ms
-// against packs of 1024), smaller and more of them where SMs would stand idle
-// (2^15 keys: 71 us, with full packs 83).
+// Packing that nothing asked for (pack_keys 0): packs that fill the first
+// on-chip class where a level has enough of them (merge of 2^28 pairs in 4096
+// buckets 4.44 -> 4.23 ms against packs of 1024), smaller and more of them
+// where SMs would stand idle (2^15 keys: 71 us, with full packs 83).
+constexpr uint32_t kPackAuto = 0;
 constexpr uint32_t kPackDefault = 1024;
 constexpr uint64_t kPackMinKeys = 1ull << 22;
+static uint32_t pack_limit(uint32_t pack_keys, uint64_t keys_large) {
+    if (pack_keys != kPackAuto) return pack_keys;
+    return keys_large >= kPackMinKeys ? (uint32_t)kC0Cap : kPackDefault;
+}
 
 // Process-wide tuning (hss_set_tuning).
 static std::atomic<uint32_t> g_chip_max{(uint32_t)kC1Cap};
 static std::atomic<uint32_t> g_child_interp{0u};
 static std::atomic<uint32_t> g_child_keys{384u};
-static std::atomic<uint32_t> g_pack_keys{kPackDefault};
+static std::atomic<uint32_t> g_pack_keys{kPackAuto};
 static std::atomic<uint32_t> g_splitters{0u};
 static std::atomic<uint32_t> g_scatter{0u};
 
@@ -48,23 +53,22 @@ int set_tuning(const hss_tuning* t) {
         g_chip_max = (uint32_t)kC1Cap;
         g_child_interp = 0u;
         g_child_keys = 384u;
-        g_pack_keys = kPackDefault;
+        g_pack_keys = kPackAuto;
         g_splitters = 0u;
         g_scatter = 0u;
         return HSS_OK;
     }
     const uint32_t cm = t->chip_max_keys ? t->chip_max_keys : (uint32_t)kC1Cap;
     const uint32_t ck = t->child_bucket_keys ? t->child_bucket_keys : 384u;
-    const uint32_t pk = t->pack_keys ? t->pack_keys : kPackDefault;
     if ((cm != (uint32_t)kC1Cap && cm != (uint32_t)kSmallCap) || t->child_interp > 1u || ck < 128u || ck > 4096u ||
-        pk > 4096u || t->first_split > 1u || t->split_scatter > 1u)
+        t->pack_keys > 4096u || t->first_split > 1u || t->split_scatter > 1u)
         return HSS_ERR_INVALID;
     for (uint32_t r : t->reserved)
         if (r) return HSS_ERR_INVALID;
     g_chip_max = cm;
     g_child_interp = t->child_interp;
     g_child_keys = ck;
-    g_pack_keys = pk;
+    g_pack_keys = t->pack_keys;
     g_splitters = t->first_split;
     g_scatter = t->split_scatter;
     return HSS_OK;
@@ -74,7 +78,8 @@ void get_tuning(hss_tuning* t) {
     t->chip_max_keys = g_chip_max;
     t->child_interp = g_child_interp;
     t->child_bucket_keys = g_child_keys;
-    t->pack_keys = g_pack_keys;
+    const uint32_t pk = g_pack_keys;
+    t->pack_keys = pk == kPackAuto ? kPackDefault : pk;
     t->first_split = g_splitters;
     t->split_scatter = g_scatter;
 }
@@ -2216,7 +2221,7 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
                    ws.vor, ws.vand, L.hint_lo, L.hint_mult, ws.msd_base, ws.msd_mult, ws.msd_shift[buf], ws.spec,
                    ws.direct, ws.sub_lo[buf], ws.sub_hi[buf], ws.tile_off, child_interp ? chip_max : 0xffffffffu,
                    ws.large_mask, ws.any_large, ws.cmin[buf], ws.cmax[buf], chip_max,
-                   std::min(pack_keys == kPackDefault && keys_large >= kPackMinKeys ? (uint32_t)kC0Cap : pack_keys, chip_max),
+                   std::min(pack_limit(pack_keys, keys_large), chip_max),
                    bysplit_level ? ws.spl_mode : nullptr);
         // The split pass: level buffers alternate tmp, dst, tmp, ... after src.
         uint64_t* next = (L.depth & 1) ? dst : tmp;
