@@ -523,13 +523,14 @@ typedef struct {
      * 1024, or 1536 at levels of 2^22 keys and more (hss_get_tuning reports
      * 1024). */
     uint32_t pack_keys;
-    /* First split of each segment of a local sort.  A sample of the segment
-     * shows whether its top varying byte would crowd the keys into a few
-     * sub-buckets too large for the chip (Gaussian clusters, spatially
-     * clustered Morton codes): then the segment splits on 255 splitters taken
-     * from the sorted sample (a binary search per key) instead.  0 (default):
+    /* First split of each segment of a local sort: 0 on its top varying byte;
+     * 1: a sample of the segment shows whether that byte would crowd the keys
+     * into a few sub-buckets too large for the chip (Gaussian clusters,
+     * spatially clustered Morton codes), and then the segment splits on 255
+     * splitters taken from the sorted sample (a binary search per key) instead.
+     * Where no tuning is set (hss_set_tuning never called, or last with NULL),
      * calls of 2^22 keys and more in segments of 2^15 keys and more on average
-     * are sampled; 1: every local sort is. */
+     * are sampled, others split on the byte; hss_get_tuning reports 0 then. */
     uint32_t first_split;
     /* How the split pass writes a tile: 0 stages the tile in shared memory in
      * digit order and writes each digit's run with consecutive stores; 1
@@ -541,8 +542,8 @@ typedef struct {
     uint32_t reserved[2];        /* zero */
 } hss_tuning;
 
-/* Set the tuning (NULL restores the defaults); HSS_ERR_INVALID for a value
- * out of range.  Calls already enqueued keep the tuning they started with. */
+/* Set the tuning (NULL restores the defaults, the choices by size among
+ * them); HSS_ERR_INVALID for a value out of range.  Calls already enqueued keep the tuning they started with. */
 int hss_set_tuning(const hss_tuning* t);
 int hss_get_tuning(hss_tuning* t);
 

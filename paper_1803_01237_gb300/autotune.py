@@ -54,10 +54,18 @@ class Choice:
         return int(self.hist_flags) | (hss.FLAG_HOST_ROUNDS if self.host_rounds else 0)
 
     def apply(self):
-        """Set the process-wide sort tiling; returns (oversample, flags) for the calls."""
-        hss.set_tuning(self.chip_max_keys, self.child_interp, self.child_bucket_keys, self.pack_keys,
-                       self.first_split)
+        """Set the process-wide sort tiling; returns (oversample, flags) for the
+        calls.  The default tiling is the library's own, whose first split
+        and packing go by the sizes of a call."""
+        tiling = (self.chip_max_keys, self.child_interp, self.child_bucket_keys, self.pack_keys, self.first_split)
+        if tiling == _DEFAULT_TILING:
+            hss.reset_tuning()
+        else:
+            hss.set_tuning(*tiling)
         return float(self.oversample), self.flags()
+
+
+_DEFAULT_TILING = (4096, 0, 384, 0, 0)
 
 
 def default_space(p: int):

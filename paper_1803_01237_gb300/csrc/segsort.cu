@@ -40,12 +40,17 @@ static uint32_t pack_limit(uint32_t pack_keys, uint64_t keys_large) {
     return keys_large >= kPackMinKeys ? (uint32_t)kC0Cap : kPackDefault;
 }
 
+// First splits of local sorts: on the top varying byte, on sampled splitters
+// where the sample calls for them, or (nothing asked for) by the call's size
+// (kSplMinKeys, kSplMinSeg).
+constexpr uint32_t kFirstByte = 0, kFirstSampled = 1, kFirstAuto = 2;
+
 // Process-wide tuning (hss_set_tuning).
 static std::atomic<uint32_t> g_chip_max{(uint32_t)kC1Cap};
 static std::atomic<uint32_t> g_child_interp{0u};
 static std::atomic<uint32_t> g_child_keys{384u};
 static std::atomic<uint32_t> g_pack_keys{kPackAuto};
-static std::atomic<uint32_t> g_splitters{0u};
+static std::atomic<uint32_t> g_splitters{kFirstAuto};
 static std::atomic<uint32_t> g_scatter{0u};
 
 int set_tuning(const hss_tuning* t) {
@@ -54,14 +59,14 @@ int set_tuning(const hss_tuning* t) {
         g_child_interp = 0u;
         g_child_keys = 384u;
         g_pack_keys = kPackAuto;
-        g_splitters = 0u;
+        g_splitters = kFirstAuto;
         g_scatter = 0u;
         return HSS_OK;
     }
     const uint32_t cm = t->chip_max_keys ? t->chip_max_keys : (uint32_t)kC1Cap;
     const uint32_t ck = t->child_bucket_keys ? t->child_bucket_keys : 384u;
     if ((cm != (uint32_t)kC1Cap && cm != (uint32_t)kSmallCap) || t->child_interp > 1u || ck < 128u || ck > 4096u ||
-        t->pack_keys > 4096u || t->first_split > 1u || t->split_scatter > 1u)
+        t->pack_keys > 4096u || t->first_split > kFirstSampled || t->split_scatter > 1u)
         return HSS_ERR_INVALID;
     for (uint32_t r : t->reserved)
         if (r) return HSS_ERR_INVALID;
@@ -80,7 +85,7 @@ void get_tuning(hss_tuning* t) {
     t->child_bucket_keys = g_child_keys;
     const uint32_t pk = g_pack_keys;
     t->pack_keys = pk == kPackAuto ? kPackDefault : pk;
-    t->first_split = g_splitters;
+    t->first_split = g_splitters == kFirstSampled ? kFirstSampled : kFirstByte;
     t->split_scatter = g_scatter;
 }
 
@@ -2134,7 +2139,7 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
     const bool child_interp = g_child_interp.load() != 0u;
     const uint32_t child_keys = g_child_keys.load();
     const uint32_t pack_keys = g_pack_keys.load();
-    const bool use_splitters = g_splitters.load() != 0u;
+    const uint32_t first_split = g_splitters.load();
     const uint32_t scatter = g_scatter.load();
     volatile uint32_t* mapped = nullptr;  // host view of the planning counts
     uint32_t* mapped_dev = nullptr;        // the kernel's view
@@ -2197,7 +2202,8 @@ static cudaError_t segsort_t(const uint64_t* src, uint64_t* dst, uint64_t* tmp, 
         // The first split of a level-0 segment may take sampled splitters
         // (skewed keys); later levels and hinted splits keep their digits.
         const bool bysplit_level = L.depth == 0 && !L.hint_lo && n_large <= ws.max_spl &&
-                                   (use_splitters || (keys_large >= kSplMinKeys && keys_large / n_large >= kSplMinSeg));
+                                   (first_split == kFirstSampled || (first_split == kFirstAuto && keys_large >= kSplMinKeys &&
+                                                                      keys_large / n_large >= kSplMinSeg));
         if (bysplit_level)
             HSS_LAUNCH(k_seg_sample, n_large, 256, 0, st, L.in, L.seg_lo, L.seg_hi, ws.large_seg, ws.counters, L.flip_in,
                        chip_max, ws.spl_tab, ws.spl_mode);

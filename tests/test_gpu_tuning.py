@@ -49,3 +49,30 @@ def test_pack_keys(hss, asked, limit):
     w = ws[: ws.numel() // 4 * 4].view(torch.int32).cpu().numpy()
     at = np.flatnonzero(w[:-4] == expect)
     assert any((w[i + 1:i + 5] == 0).all() for i in at)
+
+
+@pytest.mark.parametrize("asked", [None, 0, 1])
+@pytest.mark.parametrize("p", [P, 512])
+def test_first_split(hss, asked, p):
+    """A sample is one launch: of every local sort (1), of none (0), and where
+    nothing was asked for, of segments of 2^15 keys and more."""
+    keys = torch.randint(-(1 << 62), 1 << 62, (N,), device="cuda") * 2
+
+    def launches():
+        before = hss.launch_count()
+        hss.local_sort(keys, p)
+        torch.cuda.synchronize()
+        return hss.launch_count() - before
+
+    hss.set_tuning(first_split=0)
+    plain = launches()
+    hss.set_tuning(first_split=1)
+    sampled = launches()
+    assert sampled == plain + 1
+    if asked is None:
+        hss.reset_tuning()
+    else:
+        hss.set_tuning(first_split=asked)
+    assert hss.get_tuning()["first_split"] == (asked or 0)
+    by_size = sampled if N // p >= 1 << 15 else plain
+    assert launches() == (by_size if asked is None else sampled if asked else plain)
