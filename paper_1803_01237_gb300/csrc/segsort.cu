@@ -360,11 +360,13 @@ constexpr int chip_min_blocks() { return THREADS <= 128 ? (PAY ? 7 : 8) : (THREA
 //    stable order of equal keys; where their keys are found out of order the
 //    run is sorted by (key, position).
 // A group above kChipMaxGroup words that is left holds one key value (keys
-// alone): its order is free.  The refining ends: a count that takes a crowded
-// group's places from its own range leaves no part wider than 2/57 of it, so
-// thirteen of them use up 64 bits (one more order of magnitude covers the
-// positions of a payload's equal keys), and a count without that follows only
-// where the largest group shrank to a quarter, at most seven times.
+// alone): its order is free.  The refining ends after kChipRefines counts at
+// most.  A count from the groups' own ranges cuts every group above kChipRefine
+// keys into 25 parts or more, none wider than 2/25 of its range, so 18 of them
+// use up the keys' 64 bits and 4 the 14 bits of the positions (a payload's
+// equal keys).  One count takes positions over the whole segment, and the
+// others, the first and those that follow where the largest group shrank to a
+// quarter and is still above kChipRefine, are five.
 //
 // Bound by shared-memory wavefronts and issue slots together (67% and 66% of
 // their peaks; about 34 wavefronts and 146 instructions per key of a warp): the
@@ -375,9 +377,7 @@ constexpr int chip_min_blocks() { return THREADS <= 128 ? (PAY ? 7 : 8) : (THREA
 // 2^28 uniform keys in buckets of about 1024: 2.28 ms with an insertion sort
 // per thread over 64-bit keys (60 wavefronts, 204 instructions), 1.5 ms here;
 // 2^28 Morton keys with a payload in segments of 2^14, whose groups crowd:
-// 57.9 ms (most of it in the LSD kernel), 6.6 ms.  Refining by a group's own
-// ranges leaves the LSD kernel nothing of these inputs (packs that span the gap
-// between two clusters used to end there: 1.3 ms per 2^28 pairs).
+// 57.9 ms (most of it in digit passes that took the crowded segments), 6.6 ms.
 // ---------------------------------------------------------------------------
 // Exclusive scan in place of 2 NW 16-bit counters packed in NW shared words
 // (counter 2i in the low half of word i) by a CTA of T threads, and the
@@ -450,7 +450,21 @@ __device__ __forceinline__ void sort_8(uint32_t (&k)[8]) {
 
 constexpr uint32_t kChipRefine = 24;    // a larger group: count again on the refined groups
 constexpr uint32_t kChipMaxGroup = 56;  // the largest group the window rounds order (start mod 64 is unambiguous)
-constexpr int kChipRefines = 32;  // never reached (see above)
+// Counts from a group's own range until a range of `bits` bits is one value
+// (32 bits of a key are looked at: the last factor is the part cut off), and
+// the bound on all counts (see above).
+constexpr int range_counts(int bits) {
+    int c = 0;
+    for (double r = (double)(1ull << (bits - 1)) * 2.0; r >= 1.0; r *= 2.0 / (kChipRefine + 1) * (1.0 + 0x1p-26)) ++c;
+    return c;
+}
+constexpr int other_counts() {
+    int c = 1;
+    for (uint32_t most = kSmallCap / 4; most > kChipRefine; most /= 4) ++c;
+    return c;
+}
+constexpr int kChipRefines = range_counts(64) + range_counts(14) + 1 + other_counts();
+static_assert(range_counts(64) == 18 && range_counts(14) == 4 && other_counts() == 5, "as the comment above counts them");
 constexpr uint32_t kChipRounds = (kChipMaxGroup + 2) / 4 + 3;  // rounds that order the largest group, and the one that finds it so
 constexpr int kStartBits = 6;
 
