@@ -595,8 +595,10 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
         const bool late = !mbar_wait(s_bar, phase);
         phase ^= 1u;
         if (__syncthreads_or(late)) {  // uniform; not expected: a bulk copy that never landed
-            if (tid == 0) atomicOr(err, kDevErrTimeout);
-            cur.ok = false;
+            if (tid == 0) {
+                atomicOr(err, kDevErrTimeout);
+                mbar_wait(s_bar, phase ^ 1u);  // the CTA's memory stays until the copy is done, or once more the limit
+            }
             break;
         }
         // Range of the high words (of the low words when those are all equal).
@@ -1842,7 +1844,10 @@ __global__ __launch_bounds__(split_threads<PAY>(), PAY ? 3 : 5) void k_split(con
     cp_async_wait_all();
     __syncthreads();  // the barrier is initialised, the small copies have landed
     if (__syncthreads_or(!mbar_wait(&s_bar, 0u))) {  // uniform; not expected: a bulk copy that never landed
-        if (tid == 0) atomicOr(A.err, kDevErrTimeout);
+        if (tid == 0) {
+            atomicOr(A.err, kDevErrTimeout);
+            mbar_wait(&s_bar, 0u);  // the CTA's memory stays until the copy is done, or once more the limit
+        }
         return;
     }
     const uint64_t* keys = s_keys + hd;
