@@ -320,6 +320,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     }
     return false;
 }
+// Orders ordinary accesses to shared memory, seen by the calling thread, before
+// the bulk copies that it issues next.
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 __device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
                      smem_u32(sdst)),
@@ -559,6 +562,7 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
             pm = ((d.n - ph) >> 2) << 2;
         }
         if (tid == 0) {
+            fence_proxy_async();  // the last segment was read, and its ends written, where the next one goes
             mbar_arrive_expect_tx(s_bar, m * 8u + pm * 4u);
             if (m) bulk_load(s_key + 2 * hd, g + hd, m * 8u, s_bar);
             if (SPAY && pm) bulk_load(s_pay + po + ph, gp + ph, pm * 4u, s_bar);
