@@ -321,7 +321,7 @@ def run_gpu(args):
     o = out[:: max(1, N // (1 << 20))].cpu().numpy().view(np.uint64)
     sorted_ok = bool(np.all(o[:-1] <= o[1:]))
 
-    # roofline of the dominant kernel: the one-sweep split pass reads and
+    # roofline of the dominant kernel: the split pass reads and
     # writes every key of the segments it splits once (16 B per key)
     peak, peak_kind = _measured_peaks()
     avg_pass_ms = pass_ms / max(pass_launches, 1)
@@ -371,7 +371,7 @@ def run_gpu(args):
                    "l2": "inputs (2 GiB keys per distribution) larger than L2; no flush between steps",
                    "parallelism": "replicas only" if world > 1 else "single GPU"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                     "traffic": traffic, "kernel": "k_split (one-sweep MSD scatter, 16 B/key)",
+                     "traffic": traffic, "kernel": "k_split (MSD scatter, 16 B/key)",
                      "bytes_per_launch": bytes_per_pass,
                      "peak_source": f"{peak_kind} hbm_gbs", "avg_launch_ms": avg_pass_ms,
                      "launches": pass_launches},

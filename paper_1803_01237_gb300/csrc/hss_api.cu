@@ -133,8 +133,8 @@ struct Layout {
 
 static const uint64_t kMaxN = 1ull << 40;
 static const uint32_t kMaxP = 1u << 22;
-// A segment or bucket holds fewer than 2^30 keys: the look-back words of the
-// split pack a digit's count into 30 bits and in-segment positions are u32.
+// A segment or bucket holds fewer than 2^30 keys: in-segment positions are u32,
+// with room for the sums that the kernels make of them.
 static const uint64_t kMaxSeg = 1ull << 30;
 
 // Every processor segment of N keys over p processors is below the limit.

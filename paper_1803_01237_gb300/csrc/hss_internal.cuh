@@ -4,7 +4,6 @@
 #include <cstdint>
 #include <cstddef>
 #include <cuda_runtime.h>
-#include <cuda/atomic>
 
 #include "hss.h"
 
@@ -21,8 +20,8 @@ constexpr uint32_t kDevErrSize = 4u;  // a segment of 2^30 keys or more (reporte
 constexpr uint64_t kMaxSegKeys = 1ull << 30;
 
 // No kernel of the library waits on another CTA or kernel (the split pass
-// takes its tile offsets from a scan, not a look-back), so kDevErrTimeout is
-// set by none today; the status it maps to stays part of the ABI.
+// takes its tile offsets from a scan).  kDevErrTimeout: a CTA's own bulk copy
+// had not landed within the limit of its wait.
 
 // Cut kinds, ordered so that comparison by (kind class, key, seg, spos) is the
 // tag order of Sec. 6.1.
@@ -93,18 +92,6 @@ __device__ __forceinline__ void sample_words(uint64_t seed, uint32_t seg, uint32
     const Philox4 x = philox4x32_10(m, seg, round, 0u, (uint32_t)seed, (uint32_t)(seed >> 32));
     even = ((uint64_t)x.v[1] << 32) | x.v[0];
     odd = ((uint64_t)x.v[3] << 32) | x.v[2];
-}
-
-// ---------------------------------------------------------------------------
-// Relaxed device-scope atomics for the decoupled look-back status words.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t ld_relaxed(uint32_t* p) {
-    cuda::atomic_ref<uint32_t, cuda::thread_scope_device> r(*p);
-    return r.load(cuda::memory_order_relaxed);
-}
-__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
-    cuda::atomic_ref<uint32_t, cuda::thread_scope_device> r(*p);
-    r.store(v, cuda::memory_order_relaxed);
 }
 
 // Launch accounting: every kernel launch of the library goes through this.

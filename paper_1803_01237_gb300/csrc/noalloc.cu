@@ -2,7 +2,7 @@
 //
 // hss_local_sort_noalloc runs the same segmented radix sort as hss_local_sort,
 // but takes its scratch (the ping-pong key/payload buffers, the segment
-// offsets, the digit offsets and the look-back words) from one fixed array
+// offsets, the digit counts and offsets) from one fixed array
 // that lives in the library's device image instead of from a caller
 // workspace.  The array is kNoAllocScratchBytes per device and stays resident
 // on every device that loads the library until the process exits.
@@ -70,7 +70,7 @@ extern "C" int hss_local_sort_noalloc(const void* d_keys, const uint32_t* d_payl
     uint32_t* err = (uint32_t*)(b + o_err);
     uint64_t* seg_off = (uint64_t*)(b + o_seg);
     // The array keeps the previous call's contents: zero the error word here;
-    // the sort zeroes its own counters and look-back words before use.
+    // the sort writes the rest of its scratch before it reads it.
     if (cudaMemsetAsync(err, 0, 256, st) != cudaSuccess) return HSS_ERR_CUDA;
     if (fill_even_offsets(seg_off, N, p, st) != cudaSuccess) return HSS_ERR_CUDA;
     SegSortWs ws = segsort_ws_carve(b + o_ws, N1, p, err);

@@ -830,11 +830,10 @@ __global__ void k_ctl_init(RoundCtl* ctl, uint64_t seed, uint32_t max_rounds) {
     ctl->form = kFormSearch;
 }
 
-__global__ void k_ctl_record(RoundCtl* ctl, uint32_t rounds, int32_t status, uint64_t last_z) {
+__global__ void k_ctl_record(RoundCtl* ctl, uint32_t rounds, int32_t status) {
     if (threadIdx.x == 0) {
         ctl->round = rounds;
         ctl->status = status;
-        (void)last_z;
     }
 }
 
@@ -1273,7 +1272,7 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
     out->rounds = j;
     out->status = status;
     {   // the same record the device-driven loop leaves, for hss_call_stats
-        HSS_LAUNCH(k_ctl_record, 1, 64, 0, st, ws.ctl, j, status, out->sample_size[j > 0 ? j - 1 : 0]);
+        HSS_LAUNCH(k_ctl_record, 1, 64, 0, st, ws.ctl, j, status);
         HSS_TRY(cudaMemcpyAsync(ws.ctl->hist_Z, out->sample_size, sizeof(out->sample_size), cudaMemcpyHostToDevice, st));
         HSS_TRY(cudaMemcpyAsync(ws.ctl->hist_gamma, out->gamma, sizeof(out->gamma), cudaMemcpyHostToDevice, st));
         HSS_TRY(cudaMemcpyAsync(ws.ctl->hist_unres, out->unresolved, sizeof(out->unresolved), cudaMemcpyHostToDevice, st));

@@ -2,11 +2,12 @@
 // bucket ranges, the local merge).
 //
 // Design for sm_103a:
-//  * A segment of at most 14336 keys is sorted by one CTA on chip (k_chip): its
+//  * A segment of at most 4096 keys is sorted by one CTA on chip (k_chip): its
 //    keys (and payload) are copied from HBM once into shared memory, counted
 //    into groups that follow their distribution, ordered inside the groups as
 //    32-bit words in registers, and written once (16 B of HBM traffic per key).
-//    Three CTA shapes by segment size (128, 256, 1024 threads).
+//    CTA shapes by segment size: 128 and 256 threads, and 1024 for segments of
+//    up to 14336 keys where the tuning keeps them whole or the call has no more.
 //  * A larger segment takes one read pass for statistics (digit counts and the
 //    OR/AND of its keys) and one stable scatter on its first-split
 //    digit (its top varying byte, or an interpolation of the key range the
@@ -371,8 +372,8 @@ constexpr int chip_min_blocks() { return THREADS <= 128 ? (PAY ? 7 : 8) : (THREA
 // others, the first and those that follow where the largest group shrank to a
 // quarter and is still above kChipRefine, are five.
 //
-// Bound by shared-memory wavefronts and issue slots together (67% and 66% of
-// their peaks; about 34 wavefronts and 146 instructions per key of a warp): the
+// Bound by shared-memory wavefronts and issue slots together (65% and 66% of
+// their peaks; about 34 wavefronts and 144 instructions per key of a warp): the
 // counting atomics, the group-start and key gathers and the word scatter each
 // meet random banks.  Words of 32 bits instead of the keys themselves halve
 // the scatter's wavefronts and make a comparator two instructions (six for 64
@@ -992,7 +993,7 @@ __device__ __forceinline__ PlanV plan_item(const uint64_t* seg_lo, const uint64_
         } else if (n <= (uint64_t)chip_max) {
             v.c[2] = 1;
         } else if (n >= kMaxSegKeys) {
-            // too large for the split's 30-bit counts: left unsorted, reported by k_plan_write
+            // above the limit on a segment: left unsorted, reported where the entries are written
         } else {
             v.c[3] = 1;
             v.c[4] = (uint32_t)ceil_div(n, kOsTile);
@@ -1763,7 +1764,7 @@ constexpr size_t split_smem(bool gather) {
 // tile is then written run by run through it.  So no thread holds its keys in
 // registers across the ranking (64 registers and half the warps of an SM
 // before), and shared memory sees 2 bytes per key scattered instead of 9 (13).
-// Bound by shared-memory wavefronts (80% of their peak keys alone, 74% with a
+// Bound by shared-memory wavefronts (87% of their peak keys alone, 74% with a
 // payload: the counting atomics, the index scatter and the key gather meet
 // random banks).  2^28 keys, 256-way: keys alone 1.10 -> 0.90 ms, with a
 // payload 2.50 -> 1.95 ms.  Keys alone with 512 threads: 6% slower.

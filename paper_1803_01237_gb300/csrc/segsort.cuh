@@ -1,7 +1,8 @@
 // segsort.cuh -- stable segmented radix sort of 64-bit keys (+ u32 payload).
 //
 // Segments are given by a device array seg_off[nseg+1] of u64 offsets.  A
-// segment of at most kSmallCap keys is sorted by one CTA entirely on chip.  A
+// segment of at most kC1Cap keys (kSmallCap where the tuning, or a call of no
+// more keys, has it so) is sorted by one CTA entirely on chip.  A
 // larger segment is split by one most-significant-digit pass (per-tile digit
 // counts, a scan into per-tile offsets, then a scatter of every tile) on its top
 // varying 8-bit window into 256 sub-buckets, which are sorted the same way,
@@ -16,12 +17,12 @@ namespace hss {
 constexpr int kRadixBits = 8;
 constexpr int kRadix = 256;
 // Levels of the split recursion: byte splits need at most 8 (one per byte of
-// the key) and one more to copy single-valued sub-buckets; interpolated splits
+// the key), a first split on sampled splitters comes before them, and one more
+// copies single-valued sub-buckets; interpolated splits
 // of sub-buckets choose their width to finish within the limit.
 constexpr int kMaxDepth = 16;
 
 constexpr int kOsThreads = 256;
-constexpr int kOsWarps = kOsThreads / 32;
 constexpr int kOsItems = 16;
 constexpr int kOsTile = kOsThreads * kOsItems;  // 4096 keys per split tile
 
@@ -34,7 +35,7 @@ constexpr int kC1Cap = kC1Threads * kC1Items;
 constexpr int kSmallCap = kC2Threads * kC2Items;
 
 struct SegSortWs {
-    uint64_t max_large;    // bound on segments larger than kSmallCap at any depth
+    uint64_t max_large;    // bound on segments larger than kC1Cap at any depth
     uint64_t max_list;     // bound on the length of any segment list
     uint64_t max_tiles;
     uint32_t* tile_start;  // [max_list + 1]
@@ -51,7 +52,7 @@ struct SegSortWs {
     uint32_t* msd_shift[2];  // [max_large] split window (bits) of each large segment, by level parity
     uint32_t* spec;        // [max_large] byte counted speculatively by the statistics pass
     uint64_t* msd_base;    // [max_large] digit = ((key >> shift) - base) & 255, or
-    uint64_t* msd_mult;    // [max_large] when mult != 0: digit = mulhi(key - base, mult)
+    uint64_t* msd_mult;    // [max_large] when mult != 0: digit = interp_digit(key - base, mult)
     uint32_t* direct;      // [max_large] all keys equal: copy to the output
     uint64_t* sub_lo[2];   // [max_large * 256] sub-bucket bounds, double-buffered by depth
     uint64_t* sub_hi[2];
