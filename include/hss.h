@@ -72,8 +72,8 @@ extern "C" {
 /* Histogram form of the splitter rounds (Sec. 3.3 step 2; the result is the
  * same either way).  By default each round chooses: with few keys of a
  * segment between two probes (one per probe and segment at most in round 1, an
- * eighth later; 2^24 positions at least) each segment is walked along the
- * sorted probes; when all its probes share one interval (round 1) and searching every segment for every probe
+ * eighth later, and one where a segment's keys crowd most, as in sorted input;
+ * 2^24 positions at least) each segment is walked along the sorted probes; when all its probes share one interval (round 1) and searching every segment for every probe
  * (Z p log2(N/p) dependent loads) would cost more than eight reads of the
  * keys (four from 2^26 positions on), a staged form ranks blocks of sorted probes against the keys between
  * the block's first and last probe, staged in shared memory; else every

@@ -121,11 +121,43 @@ RoundWs rounds_ws_carve(void* base, uint64_t N, uint64_t p, uint64_t cap, uint32
 
 // ---------------------------------------------------------------------------
 // Initial state: every splitter interval is (-inf, +inf).
+// With ctl non-null, also how far segments crowd their keys into a part of the
+// key range (an input that is sorted, or sorted in runs or by blocks, where an
+// even share of all keys between two probes is a segment's whole share or
+// none): the largest ratio of a segment's keys per rank in its own range to
+// those of the input, by the ranks of the range in four segments.  A warp per
+// segment beside the others' stores: nothing to be seen of it in the kernel's
+// time.  Segments of one value, or of a few keys, do not count.
 // ---------------------------------------------------------------------------
+constexpr uint32_t kConcMin = 64;  // keys
+__device__ __forceinline__ void crowding(const uint64_t* __restrict__ skeys, const uint64_t* __restrict__ seg_off, uint64_t s,
+                                         uint32_t p, uint64_t N, RoundCtl* ctl) {
+    const uint64_t off = seg_off[s];
+    const uint32_t n = (uint32_t)(seg_off[s + 1] - off), lane = threadIdx.x;
+    if (n < kConcMin) return;  // uniform per warp
+    const uint64_t lo = skeys[off], hi = skeys[off + n - 1];
+    if (lo == hi) return;
+    const uint64_t t = (uint64_t)(2 * ((lane >> 1) & 3u) + 1) * p / 8, a = seg_off[t];  // p >= 4
+    const uint32_t len = (uint32_t)(seg_off[t + 1] - a);
+    const uint32_t c = lane & 1u ? count_below(skeys + a, len, hi, false) : count_below(skeys + a, len, lo, true);
+    uint32_t in = __shfl_down_sync(0xffffffffu, c, 1) - c;  // even lanes: the reference's keys in [lo, hi]
+    float covered = (float)in, of = (float)len;
+#pragma unroll
+    for (int o = 2; o <= 4; o *= 2) {
+        covered += __shfl_xor_sync(0xffffffffu, covered, o);
+        of += __shfl_xor_sync(0xffffffffu, of, o);
+    }
+    if (lane != 0) return;
+    const float conc = (float)n * (float)p / (float)N * of / fmaxf(covered, 0.5f);
+    if (conc > 2.f) atomicMax((int*)&ctl->conc, __float_as_int(conc));  // of positive floats, as their bits
+}
+
 __global__ void k_rounds_init(const uint64_t* __restrict__ seg_off, uint32_t S, uint64_t N, DCut* Lcut, DCut* Ucut,
-                              uint32_t* Lpos, uint32_t* Upos) {
+                              uint32_t* Lpos, uint32_t* Upos, const uint64_t* __restrict__ skeys, uint32_t p,
+                              RoundCtl* ctl) {
     const uint64_t s = blockIdx.x;
     const uint32_t i = blockIdx.y * blockDim.x + threadIdx.x;
+    if (ctl && blockIdx.y == 0 && threadIdx.x < 32) crowding(skeys, seg_off, s, p, N, ctl);
     if (i >= S) return;
     const uint32_t n = (uint32_t)(seg_off[s + 1] - seg_off[s]);
     Lpos[s * S + i] = 0;
@@ -311,7 +343,10 @@ constexpr int kHistSegPerBlock = 64;  // k_rank_cuts
 // the chip.  One interval, p = 4096, round 1 (keys per probe and segment:
 // staged, walk): 0.4: 685, 373 us; 0.8: 777, 680; 1.6: 880, 1650.  Many
 // intervals, each begun by loads of its own (search, walk): 0.04: 298, 271;
-// 0.08: 344, 313; 0.15: 367, 370; 0.3: 413, 461.  The staged form pays when the
+// 0.08: 344, 313; 0.15: 367, 370; 0.3: 413, 461.  Where the input is sorted, in
+// whole or by parts, a segment holds all the keys between some probes, and its
+// lane walks alone while the warp waits: 2^24 sorted keys, p = 4096, partition
+// 4262 us with walks, 2520 without (shuffled keys 2670, with walks).  The staged form pays when the
 // searches (Z p log2(N/p) dependent loads) would cost several reads of the keys:
 // eight, or four where its CTAs (one per 2^15 positions) come in several waves
 // (2^28 keys, p = 4096, five reads: 1564 us searched, 1088 staged; 2^26 keys,
@@ -320,16 +355,18 @@ constexpr uint32_t kFormSearch = 0, kFormStaged = 1, kFormWalk = 2;
 constexpr double kWalkMin = (double)(1ull << 24);   // positions per round, at least
 constexpr double kStagedWaves = (double)(1ull << 26);  // positions
 constexpr double kWalkKeysOne = 1.0, kWalkKeysMany = 0.125;  // keys per position, at most
+constexpr double kWalkKeysCrowded = 1.0;  // the same where a segment's keys crowd most
+__host__ __device__ __forceinline__ bool walk_pays(double positions, uint32_t nint, double gamma, float conc) {
+    return positions >= kWalkMin && gamma <= (nint == 1 ? kWalkKeysOne : kWalkKeysMany) * positions &&
+           gamma * (double)conc <= kWalkKeysCrowded * positions;
+}
 __host__ __device__ __forceinline__ bool staged_pays(double Z, uint64_t N, uint32_t p) {
     const double reads = Z * (double)p * log2((double)N / (double)p + 2.0) / (double)N;
     return reads >= 8.0 || (reads >= 4.0 && Z * (double)p >= kStagedWaves);
 }
 __host__ __device__ __forceinline__ uint32_t hist_form(double Z, uint64_t N, uint32_t p, uint32_t nint, double gamma,
-                                                       uint32_t hist_mode) {
-    const double positions = Z * (double)p;
-    if (hist_mode == kHistAuto && positions >= kWalkMin &&
-        gamma <= (nint == 1 ? kWalkKeysOne : kWalkKeysMany) * positions)
-        return kFormWalk;
+                                                       float conc, uint32_t hist_mode) {
+    if (hist_mode == kHistAuto && walk_pays(Z * (double)p, nint, gamma, conc)) return kFormWalk;
     const bool staged = nint == 1 && hist_mode != kHistProbe && (hist_mode == kHistStaged || staged_pays(Z, N, p));
     return staged ? kFormStaged : kFormSearch;
 }
@@ -630,8 +667,9 @@ __global__ void k_prop_load(const uint64_t* __restrict__ prop, uint32_t nprop, u
 
 __global__ void k_prop_probes(uint32_t nprop, const uint64_t* __restrict__ okey_sorted, uint64_t* __restrict__ pkey,
                               int32_t* __restrict__ pseg, uint32_t* __restrict__ pspos, uint32_t* __restrict__ pint,
-                              uint64_t* __restrict__ prank) {
+                              uint64_t* __restrict__ prank, RoundCtl* ctl, uint64_t N, uint32_t p, uint32_t hist_mode) {
     const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k == 0) ctl->form = hist_form((double)nprop, N, p, 1u, (double)N, ctl->conc, hist_mode);
     if (k >= nprop) return;
     pkey[k] = okey_sorted[k]; pseg[k] = -1; pspos[k] = 0; prank[k] = 0; pint[k] = 0;
 }
@@ -854,7 +892,7 @@ __device__ void round_decide(RoundCtl* ctl, uint64_t cap, uint64_t N, uint32_t p
             ctl->status = HSS_ERR_CAPACITY;
         } else {
             // the histogram form of this round, as the host loop chooses it
-            ctl->form = hist_form((double)Z, N, p, ctl->nint, (double)ctl->gamma, hist_mode);
+            ctl->form = hist_form((double)Z, N, p, ctl->nint, (double)ctl->gamma, ctl->conc, hist_mode);
             go = 1;
         }
     }
@@ -943,6 +981,26 @@ static void enqueue_update(const RoundWs& ws, uint32_t S, uint64_t N, uint32_t N
                schedule, T_ovr, all_ovr, ws.int_T, ws.int_all, ws.int_seg);
 }
 
+// The histogram whose form the device has chosen (ctl->form): the forms that at
+// most `most` probes can take, Ze of them expected.
+static void enqueue_forms(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uint32_t p, uint32_t S, uint64_t most,
+                          double Ze, uint32_t hist_mode, const RoundWs& ws, cudaStream_t st) {
+    if (hist_mode == kHistStaged || (hist_mode == kHistAuto && staged_pays((double)most, N, p)))
+        HSS_LAUNCH(k_histogram_staged, dim3((unsigned)cdiv(most, kStgProbes), (unsigned)cdiv(p, kStgSegs)), kStgThreads, 0,
+                   st, skeys, d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, kZFromCtl,
+                   ws.prank, ws.probe_pos, ws.cap, ws.sws.err, ws.ctl);
+    if (hist_mode == kHistAuto && (double)most * (double)p >= kWalkMin) {
+        const uint32_t chunk = walk_chunk(Ze, p);
+        HSS_LAUNCH(k_histogram_walk, dim3((unsigned)cdiv(most, chunk), (unsigned)cdiv(p, kWalkThreads)), kWalkThreads, 0,
+                   st, skeys, d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, ws.pint,
+                   kZFromCtl, ws.prank, ws.probe_pos, ws.cap, ws.sws.err, ws.ctl, chunk);
+    }
+    const uint32_t per_warp = hist_per_warp(Ze, p);
+    HSS_LAUNCH(k_histogram, dim3((unsigned)cdiv(most, 32), (unsigned)cdiv(p, 8 * per_warp)), 256, 0, st, skeys, d_seg_off, p,
+               S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, ws.pint, kZFromCtl, ws.prank, ws.probe_pos,
+               ws.cap, ws.sws.err, ws.ctl, per_warp);
+}
+
 bool device_loop_possible(uint64_t cap, uint32_t schedule) {
     // the probe sort of a round must run without host planning (one segment
     // of at most the on-chip capacity), and the threshold must come from the
@@ -969,22 +1027,7 @@ cudaError_t enqueue_device_round(const uint64_t* skeys, const uint64_t* d_seg_of
     if (e != cudaSuccess) return e;
     HSS_LAUNCH(k_probe_build, (unsigned)cdiv(cap, 256), 256, 0, st, kZFromCtl, ws.skey_sorted, ws.sperm, ws.sseg,
                ws.sspos, ws.Ucut, ws.int_rep, ws.ctl, ws.pkey, ws.pseg, ws.pspos, ws.pint, ws.prank);
-    // the forms that a round of at most cap probes can take
-    if (hist_mode == kHistStaged || (hist_mode == kHistAuto && staged_pays((double)cap, N, p)))
-        HSS_LAUNCH(k_histogram_staged, dim3((unsigned)cdiv(cap, kStgProbes), (unsigned)cdiv(p, kStgSegs)), kStgThreads, 0,
-                   st, skeys, d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, kZFromCtl,
-                   ws.prank, ws.probe_pos, cap, ws.sws.err, ws.ctl);
-    const double Ze = (double)oversample * (double)NB;  // probes expected
-    if (hist_mode == kHistAuto && (double)cap * (double)p >= kWalkMin) {
-        const uint32_t chunk = walk_chunk(Ze, p);
-        HSS_LAUNCH(k_histogram_walk, dim3((unsigned)cdiv(cap, chunk), (unsigned)cdiv(p, kWalkThreads)), kWalkThreads, 0,
-                   st, skeys, d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, ws.pint,
-                   kZFromCtl, ws.prank, ws.probe_pos, cap, ws.sws.err, ws.ctl, chunk);
-    }
-    const uint32_t per_warp = hist_per_warp(Ze, p);
-    HSS_LAUNCH(k_histogram, dim3((unsigned)cdiv(cap, 32), (unsigned)cdiv(p, 8 * per_warp)), 256, 0, st, skeys, d_seg_off, p,
-               S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, ws.pint, kZFromCtl, ws.prank, ws.probe_pos, cap,
-               ws.sws.err, ws.ctl, per_warp);
+    enqueue_forms(skeys, d_seg_off, N, p, S, cap, (double)oversample * (double)NB, hist_mode, ws, st);
     enqueue_update(ws, S, N, NB, kZFromCtl, tol, oversample, schedule, 0ull, 0u, st);
     if ((e = enqueue_sampling(ws, d_seg_off, N, p, S, 0ull, 0u, st, per_interval, true)) != cudaSuccess) return e;
     HSS_LAUNCH(k_count_scan<true>, 1, 1024, 0, st, ws.seg_cnt, p, ws.seg_cnt_off, cap, ws.ctl, N, hist_mode, loop);
@@ -1159,8 +1202,8 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
                    schedule, Tq, allq, ws.int_T, ws.int_all, ws.int_seg);
     };
     // The histogram of Z probes in nint intervals of gamma keys.
-    auto histogram = [&](uint64_t Z, uint32_t nint, uint64_t gamma) -> cudaError_t {
-        const uint32_t form = hist_form((double)Z, N, p, nint, (double)gamma, hist_mode);
+    auto histogram = [&](uint64_t Z, uint32_t nint, uint64_t gamma, float conc) -> cudaError_t {
+        const uint32_t form = hist_form((double)Z, N, p, nint, (double)gamma, conc, hist_mode);
         if (form == kFormStaged) {
             HSS_LAUNCH(k_histogram_staged, dim3((unsigned)cdiv(Z, kStgProbes), (unsigned)cdiv(p, kStgSegs)), kStgThreads, 0,
                        st, skeys, d_seg_off, p, S, ws.Lpos, ws.Upos, ws.int_rep, ws.pkey, ws.pseg, ws.pspos, Z, ws.prank,
@@ -1188,7 +1231,10 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
         return HSS_OK;
     }
     const unsigned sblk = (unsigned)cdiv(S, 256);
-    HSS_LAUNCH(k_rounds_init, dim3(p, sblk), 256, 0, st, d_seg_off, S, N, ws.Lcut, ws.Ucut, ws.Lpos, ws.Upos);
+    // how far segments crowd their keys is asked where a round may walk them
+    const bool may_walk = hist_mode == kHistAuto && p >= 4 && (double)ws.cap * (double)p >= kWalkMin;
+    HSS_LAUNCH(k_rounds_init, dim3(p, sblk), 256, 0, st, d_seg_off, S, N, ws.Lcut, ws.Ucut, ws.Lpos, ws.Upos, skeys, p,
+               may_walk ? ws.ctl : nullptr);
     intervals(1);
     if (nprop > 0) {
         // Proposed cuts: sorted, ranked in every segment, offered to L/U.
@@ -1198,8 +1244,9 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
         HSS_TRY(segsort(ws.skey, ws.skey_sorted, ws.stmp, nullptr, nullptr, nullptr, nprop, 1, ws.ctl->seg_off_z, false,
                         false, ws.sws, st, nullptr));
         HSS_LAUNCH(k_prop_probes, (unsigned)cdiv(nprop, 256), 256, 0, st, nprop, ws.skey_sorted, ws.pkey, ws.pseg,
-                   ws.pspos, ws.pint, ws.prank);
-        HSS_TRY(histogram((uint64_t)nprop, 1u, N));
+                   ws.pspos, ws.pint, ws.prank, ws.ctl, N, p, hist_mode);
+        enqueue_forms(skeys, d_seg_off, N, p, S, nprop, (double)nprop, hist_mode, ws, st);
+        HSS_TRY(cudaGetLastError());
         HSS_LAUNCH(k_update, sblk, 256, 0, st, S, N, NB, ws.pkey, ws.pseg, ws.pspos, ws.prank, (uint64_t)nprop,
                    (int32_t)kNonMember, ws.Lcut, ws.Ucut, ws.chgL, ws.chgU, ws.ctl);
         HSS_LAUNCH(k_update_pos, p, 256, 0, st, S, ws.chgL, ws.chgU, ws.probe_pos, ws.cap, ws.Lpos, ws.Upos);
@@ -1255,7 +1302,7 @@ int run_rounds(const uint64_t* skeys, const uint64_t* d_seg_off, uint64_t N, uin
                             false, ws.sws, st, nullptr));
             HSS_LAUNCH(k_probe_build, (unsigned)cdiv(Z, 256), 256, 0, st, Z, ws.skey_sorted, ws.sperm, ws.sseg, ws.sspos,
                        ws.Ucut, ws.int_rep, ws.ctl, ws.pkey, ws.pseg, ws.pspos, ws.pint, ws.prank);
-            HSS_TRY(histogram(Z, h.nint, h.gamma));
+            HSS_TRY(histogram(Z, h.nint, h.gamma, h.conc));
             uint64_t Tq;
             uint32_t allq;
             threshold(j + 1, Tq, allq);

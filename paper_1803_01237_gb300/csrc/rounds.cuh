@@ -23,7 +23,7 @@ struct RoundCtl {
     uint32_t form;         // form of the next histogram
     uint64_t seed;         // Philox key of the sampling
     uint32_t max_rounds;
-    uint32_t pad;
+    float conc;            // how far the segments' keys crowd into parts of the key range (see k_rounds_init)
     uint64_t hist_Z[HSS_MAX_ROUNDS];
     uint64_t hist_gamma[HSS_MAX_ROUNDS];
     uint64_t hist_unres[HSS_MAX_ROUNDS + 1];
