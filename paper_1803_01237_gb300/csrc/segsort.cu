@@ -340,6 +340,7 @@ constexpr int chip_min_blocks() { return THREADS <= 128 ? (PAY ? 7 : 8) : (THREA
 // On-chip sort of segments with min_n < n <= max_n keys (n <= CAP), with or
 // without a payload, taken from `list` (compact ids, count at *nlist) or, when
 // list is null, from all nseg segments: the stable sort by (key, position).
+// whole: the segments are the caller's, not sub-buckets of a split.
 //
 // One bulk copy brings the keys (and the payload) into shared memory, where
 // they stay until they are written in order; what is sorted is one 32-bit
@@ -453,6 +454,7 @@ __device__ __forceinline__ void sort_8(uint32_t (&k)[8]) {
 }
 
 constexpr uint32_t kChipRefine = 24;    // a larger group: count again on the refined groups
+constexpr uint32_t kFewShare = 16;      // a group above this part of the segment may be one of a few values
 constexpr uint32_t kChipMaxGroup = 56;  // the largest group the window rounds order (start mod 64 is unambiguous)
 // Counts from a group's own range until a range of `bits` bits is one value
 // (32 bits of a key are looked at: the last factor is the part cut off), and
@@ -499,7 +501,7 @@ template <bool PAY, int THREADS, int CAP, int R>
 __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_chip(
     const uint64_t* kin, uint64_t* kout, const uint32_t* pin, uint32_t* pout, const uint64_t* __restrict__ seg_lo,
     const uint64_t* __restrict__ seg_hi, const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist,
-    uint64_t nseg, uint32_t min_n, uint32_t max_n, uint64_t flip_in, uint64_t flip_out,
+    uint64_t nseg, uint32_t min_n, uint32_t max_n, uint64_t flip_in, uint64_t flip_out, uint32_t whole,
     uint32_t* __restrict__ err) {
     constexpr int ITEMS = CAP / THREADS;
     constexpr int WARPS = THREADS / 32;
@@ -699,7 +701,23 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
                         if (s_start[d + 1] - a > kChipRefine) body(i, e, s_w + a);
                     });
                 };
-                if (it > 0 && 4u * mx > before) {
+                bool look = it > 0 && 4u * mx > before;
+                if (!PAY && it == 0 && (CAP > 2048 || whole) && kFewShare * mx > n) {
+                    // A few values make groups of one value each, which another
+                    // count leaves as they are, every key at the same counter.
+                    // Where no two neighbouring items of a thread share a group
+                    // and not their place, look first (4096 segments of 4096
+                    // keys, 2 or 16 values: 236 -> 201, 218 -> 192 us).  Packs
+                    // of the smallest class are left out: they seldom hold a few
+                    // values, and clusters would pay for the barrier.
+                    bool spread = false;
+#pragma unroll
+                    for (int i = 0; i + 1 < ITEMS; ++i)
+                        if ((uint32_t)(tid + (i + 1) * THREADS) < n)
+                            spread = spread || (((dp[i] ^ dp[i + 1]) & kGroupMask) == 0u && fr[i] != fr[i + 1]);
+                    look = __syncthreads_or(spread) == 0;
+                }
+                if (look) {
                     // Crowded groups of one key value each are in order (keys
                     // alone), or the window rounds put them in order.
                     each_crowded([&](int i, uint32_t e, uint32_t* r) {
@@ -715,7 +733,7 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
                         const uint32_t unit = 0xffffffffu / n;
                         tried_pos = true;
                         each_crowded([&](int i, uint32_t e, uint32_t*) { fr[i] = e * unit; });
-                    } else {
+                    } else if (it > 0) {
                         // the group's key range (high words, then the low
                         // words at its ends) and positions
                         each_crowded([&](int i, uint32_t, uint32_t* r) {
@@ -2089,7 +2107,7 @@ template <bool PAY, int THREADS, int CAP, int R>
 static cudaError_t launch_chip(const uint64_t* in, uint64_t* out, const uint32_t* pin, uint32_t* pout,
                                const uint64_t* seg_lo, const uint64_t* seg_hi, const uint32_t* list,
                                const uint32_t* nlist, uint64_t count, uint64_t nseg, uint32_t min_n, uint32_t max_n,
-                               uint64_t fin, uint64_t fout, uint32_t* err, cudaStream_t st) {
+                               uint64_t fin, uint64_t fout, uint32_t whole, uint32_t* err, cudaStream_t st) {
     constexpr size_t smem = chip_smem<PAY, THREADS, CAP, R>();
     const void* fn = (const void*)k_chip<PAY, THREADS, CAP, R>;
     {
@@ -2101,7 +2119,7 @@ static cudaError_t launch_chip(const uint64_t* in, uint64_t* out, const uint32_t
     const uint64_t grid = std::min<uint64_t>(count, (uint64_t)num_sms() * per_sm);
     if (grid == 0) return cudaSuccess;
     HSS_LAUNCH((k_chip<PAY, THREADS, CAP, R>), (unsigned)grid, THREADS, smem, st, in, out, pin, pout, seg_lo, seg_hi, list,
-               nlist, nseg, min_n, max_n, fin, fout, err);
+               nlist, nseg, min_n, max_n, fin, fout, whole, err);
     return cudaGetLastError();
 }
 
@@ -2125,12 +2143,12 @@ static cudaError_t chip_class(int c, const Level& L, uint64_t* dst, uint32_t* pd
                               const SegSortWs& ws, cudaStream_t st) {
     if (c == 0)
         return launch_chip<PAY, kC0Threads, kC0Cap, 1024>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
-                                                          L.nseg, lo_n, hi_n, L.flip_in, fout, ws.err, st);
+                                                          L.nseg, lo_n, hi_n, L.flip_in, fout, L.depth == 0, ws.err, st);
     if (c == 1)
         return launch_chip<PAY, kC1Threads, kC1Cap, 4096>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
-                                                          L.nseg, lo_n, hi_n, L.flip_in, fout, ws.err, st);
+                                                          L.nseg, lo_n, hi_n, L.flip_in, fout, L.depth == 0, ws.err, st);
     return launch_chip<PAY, kC2Threads, kSmallCap, 8192>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
-                                                         L.nseg, lo_n, hi_n, L.flip_in, fout, ws.err, st);
+                                                         L.nseg, lo_n, hi_n, L.flip_in, fout, L.depth == 0, ws.err, st);
 }
 
 // This thread's mapped pinned buffer for the planning counts (allocated once

@@ -1,4 +1,7 @@
-"""Segments of a few distinct values: equal keys with a payload through the split."""
+"""Segments of a few distinct values, sorted on chip: result at the edges of the
+classes and of the share that makes the sort look at the groups first, one
+value among many, equal keys with a payload through the split, and the cost
+beside that of shuffled distinct keys."""
 import numpy as np
 import pytest
 
@@ -20,6 +23,27 @@ def _check(k, p, payload, key_type="i64"):
     assert np.array_equal(keys.cpu().numpy(), kv[want])
     if payload:
         assert np.array_equal(pout.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("payload", [False, True])
+@pytest.mark.parametrize("values", [2, 3, 15, 16, 17, 33])
+@pytest.mark.parametrize("n,p", [(30, 1), (1536, 1), (4096 * 3, 3), (2796 * 7 + 5, 7), (14336, 1), (1000 * 20, 20)])
+def test_few_values(n, p, values, payload):
+    g = torch.Generator(device="cuda").manual_seed(n + values)
+    v = torch.randint(-(1 << 62), 1 << 62, (values,), device="cuda", generator=g)
+    v[-1] = v[0] + 1  # two of them share their high word, and mostly their group
+    _check(v[torch.randint(0, values, (n,), device="cuda", generator=g)], p, payload)
+
+
+@pytest.mark.parametrize("payload", [False, True])
+@pytest.mark.parametrize("others", [1, 40, 900])
+def test_one_value_among_many(others, payload):
+    """The large group is one value, the crowded rest is not, or is not crowded."""
+    g = torch.Generator(device="cuda").manual_seed(others)
+    k = torch.full((4096 * 5,), 1 << 40, dtype=torch.int64, device="cuda")
+    at = torch.randperm(k.numel(), device="cuda", generator=g)[: 5 * others]
+    k[at] = (1 << 41) + torch.randint(0, 1 << 20, (5 * others,), device="cuda", generator=g)
+    _check(k, 5, payload)
 
 
 @pytest.mark.parametrize("key_type", ["u64", "i64"])
@@ -63,3 +87,18 @@ def test_equal_keys_cost_no_more_without_a_ranking():
     out, pout = torch.empty_like(k), torch.empty_like(pay)
     alone = _best_ms(lambda: hss.local_sort(k, 1024, key_type="i64", out=out))
     assert _best_ms(lambda: hss.local_sort(k, 1024, payload=pay, key_type="i64", out=out, out_payload=pout)) < 1.55 * alone
+
+
+@pytest.mark.parametrize("p", [4096, 16384])
+def test_two_values_cost(p):
+    """Two values meet two counters, shuffled distinct keys a thousand: 1.5 times
+    the time (1.9 with a second count)."""
+    from paper_1803_01237_gb300 import hss
+
+    g = torch.Generator(device="cuda").manual_seed(3)
+    n = 1 << 26
+    k = torch.randint(-(1 << 62), 1 << 62, (n,), device="cuda", generator=g)
+    out = torch.empty_like(k)
+    distinct = _best_ms(lambda: hss.local_sort(k, 4 * p, key_type="i64", out=out))
+    two = (k & 1) << 50
+    assert _best_ms(lambda: hss.local_sort(two, 4 * p, key_type="i64", out=out)) < 1.7 * distinct
