@@ -340,7 +340,7 @@ constexpr int chip_min_blocks() { return THREADS <= 128 ? (PAY ? 7 : 8) : (THREA
 // On-chip sort of segments with min_n < n <= max_n keys (n <= CAP), with or
 // without a payload, taken from `list` (compact ids, count at *nlist) or, when
 // list is null, from all nseg segments: the stable sort by (key, position).
-// whole: the segments are the caller's, not sub-buckets of a split.
+// FEW: segments of a few values are looked for (see below).
 //
 // One bulk copy brings the keys (and the payload) into shared memory, where
 // they stay until they are written in order; what is sorted is one 32-bit
@@ -497,11 +497,11 @@ constexpr size_t chip_smem() {
            2 * (size_t)chip_windows<THREADS, CAP>() * (THREADS / 32) * 4 * 4 + 4 * 4 + 8 + 16;
 }
 
-template <bool PAY, int THREADS, int CAP, int R>
+template <bool PAY, int THREADS, int CAP, int R, bool FEW>
 __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_chip(
     const uint64_t* kin, uint64_t* kout, const uint32_t* pin, uint32_t* pout, const uint64_t* __restrict__ seg_lo,
     const uint64_t* __restrict__ seg_hi, const uint32_t* __restrict__ list, const uint32_t* __restrict__ nlist,
-    uint64_t nseg, uint32_t min_n, uint32_t max_n, uint64_t flip_in, uint64_t flip_out, uint32_t whole,
+    uint64_t nseg, uint32_t min_n, uint32_t max_n, uint64_t flip_in, uint64_t flip_out,
     uint32_t* __restrict__ err) {
     constexpr int ITEMS = CAP / THREADS;
     constexpr int WARPS = THREADS / 32;
@@ -702,14 +702,12 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
                     });
                 };
                 bool look = it > 0 && 4u * mx > before;
-                if (!PAY && it == 0 && (CAP > 2048 || whole) && kFewShare * mx > n) {
+                if (FEW && it == 0 && kFewShare * mx > n) {
                     // A few values make groups of one value each, which another
                     // count leaves as they are, every key at the same counter.
                     // Where no two neighbouring items of a thread share a group
                     // and not their place, look first (4096 segments of 4096
-                    // keys, 2 or 16 values: 236 -> 201, 218 -> 192 us).  Packs
-                    // of the smallest class are left out: they seldom hold a few
-                    // values, and clusters would pay for the barrier.
+                    // keys, 2 or 16 values: 236 -> 201, 218 -> 192 us).
                     bool spread = false;
 #pragma unroll
                     for (int i = 0; i + 1 < ITEMS; ++i)
@@ -733,7 +731,7 @@ __global__ __launch_bounds__(THREADS, chip_min_blocks<PAY, THREADS>()) void k_ch
                         const uint32_t unit = 0xffffffffu / n;
                         tried_pos = true;
                         each_crowded([&](int i, uint32_t e, uint32_t*) { fr[i] = e * unit; });
-                    } else if (it > 0) {
+                    } else if (!FEW || it > 0) {
                         // the group's key range (high words, then the low
                         // words at its ends) and positions
                         each_crowded([&](int i, uint32_t, uint32_t* r) {
@@ -2103,13 +2101,13 @@ cudaError_t fill_even_offsets(uint64_t* d_seg_off, uint64_t N, uint64_t p, cudaS
 // ---------------------------------------------------------------------------
 static int num_sms() { return device_sm_count(); }
 
-template <bool PAY, int THREADS, int CAP, int R>
+template <bool PAY, int THREADS, int CAP, int R, bool FEW>
 static cudaError_t launch_chip(const uint64_t* in, uint64_t* out, const uint32_t* pin, uint32_t* pout,
                                const uint64_t* seg_lo, const uint64_t* seg_hi, const uint32_t* list,
                                const uint32_t* nlist, uint64_t count, uint64_t nseg, uint32_t min_n, uint32_t max_n,
-                               uint64_t fin, uint64_t fout, uint32_t whole, uint32_t* err, cudaStream_t st) {
+                               uint64_t fin, uint64_t fout, uint32_t* err, cudaStream_t st) {
     constexpr size_t smem = chip_smem<PAY, THREADS, CAP, R>();
-    const void* fn = (const void*)k_chip<PAY, THREADS, CAP, R>;
+    const void* fn = (const void*)k_chip<PAY, THREADS, CAP, R, FEW>;
     {
         // all of L1 as shared memory: the CTAs per SM are limited by their buffers
         const cudaError_t e = ensure_func_attrs(fn, (int)smem, 100);
@@ -2118,8 +2116,8 @@ static cudaError_t launch_chip(const uint64_t* in, uint64_t* out, const uint32_t
     const int per_sm = resident_ctas(fn, THREADS, smem);
     const uint64_t grid = std::min<uint64_t>(count, (uint64_t)num_sms() * per_sm);
     if (grid == 0) return cudaSuccess;
-    HSS_LAUNCH((k_chip<PAY, THREADS, CAP, R>), (unsigned)grid, THREADS, smem, st, in, out, pin, pout, seg_lo, seg_hi, list,
-               nlist, nseg, min_n, max_n, fin, fout, whole, err);
+    HSS_LAUNCH((k_chip<PAY, THREADS, CAP, R, FEW>), (unsigned)grid, THREADS, smem, st, in, out, pin, pout, seg_lo, seg_hi, list,
+               nlist, nseg, min_n, max_n, fin, fout, err);
     return cudaGetLastError();
 }
 
@@ -2136,19 +2134,26 @@ struct Level {
     const uint64_t* hint_hi = nullptr;  // largest key of each segment, when known
 };
 
-// The on-chip sort of the segments of one size class.
+// The on-chip sort of the segments of one size class.  Segments of a few values
+// are looked for with keys alone (a payload's positions are counted anyway), but
+// not among the packs of a split in the smallest class: they seldom hold a few
+// values, and uniform and clustered keys took 0.4% longer for the code and the
+// barrier.
 template <bool PAY>
 static cudaError_t chip_class(int c, const Level& L, uint64_t* dst, uint32_t* pdst, const uint32_t* list,
                               const uint32_t* nlist, uint64_t count, uint32_t lo_n, uint32_t hi_n, uint64_t fout,
                               const SegSortWs& ws, cudaStream_t st) {
+    if (c == 0 && !PAY && L.depth == 0)
+        return launch_chip<PAY, kC0Threads, kC0Cap, 1024, !PAY>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist,
+                                                                count, L.nseg, lo_n, hi_n, L.flip_in, fout, ws.err, st);
     if (c == 0)
-        return launch_chip<PAY, kC0Threads, kC0Cap, 1024>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
-                                                          L.nseg, lo_n, hi_n, L.flip_in, fout, L.depth == 0, ws.err, st);
+        return launch_chip<PAY, kC0Threads, kC0Cap, 1024, false>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist,
+                                                                 count, L.nseg, lo_n, hi_n, L.flip_in, fout, ws.err, st);
     if (c == 1)
-        return launch_chip<PAY, kC1Threads, kC1Cap, 4096>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
-                                                          L.nseg, lo_n, hi_n, L.flip_in, fout, L.depth == 0, ws.err, st);
-    return launch_chip<PAY, kC2Threads, kSmallCap, 8192>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist, count,
-                                                         L.nseg, lo_n, hi_n, L.flip_in, fout, L.depth == 0, ws.err, st);
+        return launch_chip<PAY, kC1Threads, kC1Cap, 4096, !PAY>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist,
+                                                                count, L.nseg, lo_n, hi_n, L.flip_in, fout, ws.err, st);
+    return launch_chip<PAY, kC2Threads, kSmallCap, 8192, !PAY>(L.in, dst, L.pin, pdst, L.seg_lo, L.seg_hi, list, nlist,
+                                                               count, L.nseg, lo_n, hi_n, L.flip_in, fout, ws.err, st);
 }
 
 // This thread's mapped pinned buffer for the planning counts (allocated once
