@@ -373,7 +373,7 @@ constexpr int chip_min_blocks() { return THREADS <= 128 ? (PAY ? 7 : 8) : (THREA
 // others, the first and those that follow where the largest group shrank to a
 // quarter and is still above kChipRefine, are five.
 //
-// Bound by shared-memory wavefronts and issue slots together (64% and 65% of
+// Bound by shared-memory wavefronts and issue slots together (65% and 66% of
 // their peaks; about 34 wavefronts and 144 instructions per key of a warp): the
 // counting atomics, the group-start and key gathers and the word scatter each
 // meet random banks.  Words of 32 bits instead of the keys themselves halve
